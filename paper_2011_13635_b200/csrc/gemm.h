@@ -1,6 +1,6 @@
 // Dense contraction with the step's fused epilogue; see mslt_gemm_desc in mslt.h.
 //   D[z][m][n] = epilogue(alpha * sum_k A[z](m,k) * B[z](n,k))
-// dtype 0: fp32 CUDA-core kernel (gemm_simt.cu); dtype 1: bf16 tcgen05 kernel (gemm_tc.cu).
+// dtype 0: fp32 CUDA-core kernel (gemm_f32.cu); dtype 1: bf16 tcgen05 kernel (gemm_tc.cu).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -13,6 +13,7 @@ namespace mslt {
 // with a message in `err` (at least 256 bytes).
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err);
 
+int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err);
 

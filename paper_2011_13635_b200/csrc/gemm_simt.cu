@@ -1,8 +1,7 @@
-// CUDA-core contraction for the fp32 path (and for any element type as a plain-ALU kernel):
+// CUDA-core contraction of bf16 operands, a debugging aid (MSLT_BF16_CUDA_CORES=1, see gemm.cu):
 // 64x64 output tile per block, 16-deep k slices in shared memory, 4x4 outputs per thread,
-// fp32 accumulation in k order.  Operands are addressed by (row stride, k stride), so forward,
-// input-gradient and weight-gradient products and the batched attention products all run here
-// without transposed copies.  TF32 tensor cores are not used: the fp32 path is held to 1e-4.
+// fp32 accumulation in k order.  Operands are addressed by (row stride, k stride), so every
+// layout of the step runs here without transposed copies.
 #include <stdio.h>
 
 #include "common.cuh"
@@ -96,8 +95,7 @@ int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
     snprintf(err, 256, "gemm: grid too large for the CUDA-core kernel");
     return MSLT_ERR_SIZE;
   }
-  if (d.dtype == 1) gemm_simt_kernel<bf16><<<grid, 256, 0, st>>>(d);
-  else gemm_simt_kernel<float><<<grid, 256, 0, st>>>(d);
+  gemm_simt_kernel<bf16><<<grid, 256, 0, st>>>(d);
   return 0;
 }
 

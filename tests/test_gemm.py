@@ -237,3 +237,36 @@ def test_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
     ref = a.double() @ b.double().t()
     assert (out.double() - ref).abs().max() / ref.abs().max() < 6e-3
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("shape,majors", [
+    ((1024, 768, 768), ("k", "k")),      # 32 x 32 tiles
+    ((1024, 2304, 96), ("k", "k")),      # 128 x 128 tiles
+    ((160, 768, 2500), ("k", "mn")),     # k split over a cluster, last slice ragged
+    ((2304, 760, 1000), ("mn", "mn")),   # 64 x 64 tiles in clusters, ragged columns
+    ((3000, 760, 200), ("mn", "mn")),    # 128 x 128 tiles, ragged both ways
+    ((33, 31, 260), ("mn", "k")), ((1, 1, 1), ("k", "k"))])
+def test_fp32_tiles_and_cluster_splits(shape, majors):
+    """Every tile size and k split that the fp32 kernel's rule chooses, with remainders.  Sums of K
+    products of unit normals: the error of a running fp32 sum grows as sqrt(K) * 2^-24 of its range."""
+    wgrad = majors == ("mn", "mn")
+    _run(0, *shape, *majors, bias=not wgrad, d_fp32=True, accumulate=wgrad)
+
+
+def test_fp32_unaligned_operands_take_the_element_wise_copies():
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    M, N, K, ld = 70, 41, 67, 71                    # odd pitch and odd base: no 16-byte access anywhere
+    g = torch.Generator(device="cuda").manual_seed(3)
+    A, B = torch.randn(M * ld + 1, generator=g, device="cuda"), torch.randn(N * ld + 1, generator=g, device="cuda")
+    D = torch.zeros(M, N, device="cuda")
+    d = Bd.GemmDesc()
+    d.dtype, d.M, d.N, d.K, d.batch, d.hdiv, d.alpha = 0, M, N, K, 1, 1, 1.0
+    d.A, d.a_rs, d.a_ks = A.data_ptr() + 4, ld, 1
+    d.B, d.b_rs, d.b_ks = B.data_ptr() + 4, ld, 1
+    d.D, d.ldd, d.d_fp32 = D.data_ptr(), N, 1
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Bd.mslt_op_gemm(d, torch.cuda.current_stream().cuda_stream, status)
+    a, b = A[1:].view(M, ld)[:, :K].double(), B[1:].view(N, ld)[:, :K].double()
+    ref = a @ b.t()
+    assert ((D.double() - ref).abs().max() / ref.abs().max()).item() < 2e-5
