@@ -140,6 +140,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
   const int n_my = ((int)blockIdx.x < p.items) ? (p.items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (warp == 0 && lane == 0 && !p.starve) {
@@ -419,6 +420,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
   const int nqt = (p.S + 127) >> 7;   // query tiles per (sequence, head); key blocks likewise
   const int nzh = p.items / nqt;      // (sequence, head) pairs
   // Keys at or beyond the sequence's length have probability 0: an item covers only the
@@ -818,6 +820,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
   const int n_my = ((int)blockIdx.x < p.items) ? (p.items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (warp == 0 && lane == 0 && !p.starve) {
@@ -1129,7 +1132,7 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
     rc = attn_opt_in(attn_fwd_long_kernel, &adev->attr_long, smem_optin, err);
     if (rc) return rc;
     const int grid_long = p.items < num_sms ? p.items : num_sms;
-    attn_fwd_long_kernel<<<grid_long, AL_THREADS, smem_long, st>>>(mq.map, mk.map, mv.map, p);
+    launch_pdl(attn_fwd_long_kernel, grid_long, AL_THREADS, smem_long, st, mq.map, mk.map, mv.map, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
     g_attn_launches++;
@@ -1140,7 +1143,7 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   rc = attn_opt_in(attn_fwd_kernel, &adev->attr_fwd, smem_optin, err);
   if (rc) return rc;
   const int grid = p.items < num_sms ? p.items : num_sms;
-  attn_fwd_kernel<<<grid, NUM_THREADS, smem_bytes, st>>>(mq.map, mk.map, mv.map, p);
+  launch_pdl(attn_fwd_kernel, grid, NUM_THREADS, smem_bytes, st, mq.map, mk.map, mv.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches++;
@@ -1198,7 +1201,7 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
   rc = attn_opt_in(attn_bwd_kernel, &adev->attr_bwd, smem_optin, err);
   if (rc) return rc;
   const int grid = p.items < num_sms ? p.items : num_sms;
-  attn_bwd_kernel<<<grid, NUM_THREADS, smem_bytes, st>>>(mq.map, mk.map, mv.map, mc.map, mp.map, p);
+  launch_pdl(attn_bwd_kernel, grid, NUM_THREADS, smem_bytes, st, mq.map, mk.map, mv.map, mc.map, mp.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches++;

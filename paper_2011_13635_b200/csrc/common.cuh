@@ -5,7 +5,34 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 typedef __nv_bfloat16 bf16;
+
+// Programmatic dependent launch.  Every kernel of the library is launched with launch_pdl (or the
+// same attribute), so it may be set up while its predecessor in the stream drains, and begins with
+// pdl_begin: wait until the predecessor has completed and its writes are visible, then let the
+// successor be set up.  Since every kernel waits, completion is transitive along the stream.
+// A kernel may do work that touches no global memory before it calls this.  Measured: the gap
+// between two kernels of a step falls from 2.0-2.6 us to about 1 us.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... Par, typename... Arg>
+inline cudaError_t launch_pdl(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Arg&&... arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Arg>(arg)...);
+}
 
 // bits of the device status word
 enum : int {

@@ -170,6 +170,7 @@ gemm_f32_kernel(const F32Params p) {
   constexpr int STAGE = (BMT + BNT) * FK;  // floats
   static_assert(BMT * BNT <= STAGE * STAGES, "the partial tile reuses the ring");
   extern __shared__ __align__(128) float f32_ring[];
+  pdl_begin();
   const mslt_gemm_desc& d = p.d;
   const int rank = blockIdx.x % p.splits, nt = blockIdx.x / p.splits;
   const int z = blockIdx.z, zo = z / d.hdiv, zi = z - zo * d.hdiv;
@@ -358,13 +359,15 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   cfg.blockDim = dim3(kThreads[t]);
   cfg.dynamicSmemBytes = (size_t)2 * tile * FK * 4 * kStages[t];
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = s;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = s;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = s > 1 ? 1 : 0;
+  cfg.numAttrs = s > 1 ? 2 : 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kF32[t][amn][bmn][vec], p);
   if (e != cudaSuccess) { snprintf(err, 256, "gemm: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   return 0;

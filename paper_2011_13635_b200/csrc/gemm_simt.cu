@@ -11,6 +11,7 @@ namespace mslt {
 
 template <typename T>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(mslt_gemm_desc d) {
+  pdl_begin();
   __shared__ float As[16][64 + 4];
   __shared__ float Bs[16][64 + 4];
   const int z = blockIdx.z;
@@ -95,7 +96,7 @@ int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
     snprintf(err, 256, "gemm: grid too large for the CUDA-core kernel");
     return MSLT_ERR_SIZE;
   }
-  gemm_simt_kernel<bf16><<<grid, 256, 0, st>>>(d);
+  launch_pdl(gemm_simt_kernel<bf16>, grid, 256, 0, st, d);
   return 0;
 }
 

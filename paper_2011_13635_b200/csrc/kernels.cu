@@ -77,6 +77,7 @@ template <typename T, int NV, int ROWS>
 __global__ void __launch_bounds__(256)
 ln_fwd_kernel(const T* __restrict__ z, const float* __restrict__ gamma, const float* __restrict__ beta,
               T* __restrict__ y, float* __restrict__ stats, int rows, int H, float eps) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   typedef typename VecT<T>::Raw Raw;
   const int lane = threadIdx.x & 31;
@@ -186,6 +187,7 @@ embed_ln_kernel(const int* __restrict__ tokens, const int* __restrict__ segments
                 const float* __restrict__ beta, T* __restrict__ y, T* __restrict__ zstash,
                 float* __restrict__ stats, int rows, int S, int H, int V, float eps,
                 int* __restrict__ status) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   constexpr int NV = LN_MAXE / VN;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(NSLICE * RG * 32, 1)
 ln_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ z, const float* __restrict__ stats,
               const float* __restrict__ gamma, T* __restrict__ dz, float* __restrict__ dgamma,
               float* __restrict__ dbeta, float* __restrict__ dbias, int rows, int H) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   constexpr int LR = LN_BWD_ROWS;  // rows a warp has in flight
   typedef typename VecT<T>::Raw Raw;
@@ -389,6 +392,7 @@ template <typename T, int LPR, int NV>
 __global__ void __launch_bounds__(256)
 softmax_fwd_kernel(const T* __restrict__ sc, T* __restrict__ p, const int* __restrict__ seq_lens,
                    int rows, int S, int rows_per_seq, float scale) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   typedef typename VecT<T>::Raw Raw;
   constexpr int GPW = 32 / LPR;
@@ -473,6 +477,7 @@ softmax_fwd_kernel(const T* __restrict__ sc, T* __restrict__ p, const int* __res
 template <typename T, int LPR, int NV>
 __global__ void __launch_bounds__(256)
 softmax_bwd_kernel(T* __restrict__ dp, const T* __restrict__ p, int rows, int S, float scale) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   typedef typename VecT<T>::Raw Raw;
   constexpr int GPW = 32 / LPR;  // groups per warp
@@ -538,6 +543,7 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
                                      int* __restrict__ rowsrc, int* __restrict__ rowlabel,
                                      int* __restrict__ n_valid, float* __restrict__ inv_n,
                                      int* __restrict__ status) {
+  pdl_begin();
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -573,6 +579,7 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
 template <typename T>
 __global__ void gather_rows_kernel(const T* __restrict__ x, const int* __restrict__ rowsrc,
                                    T* __restrict__ out, int R, int H) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   const int r = blockIdx.x;
   const int src = rowsrc[r];
@@ -593,6 +600,7 @@ __global__ void gather_rows_kernel(const T* __restrict__ x, const int* __restric
 template <typename T>
 __global__ void scatter_rows_kernel(const T* __restrict__ d, const int* __restrict__ rowsrc,
                                     T* __restrict__ dx, int P, int H) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   const int b = blockIdx.x;
   for (int c = threadIdx.x * VN; c < H; c += blockDim.x * VN) {
@@ -619,6 +627,7 @@ __global__ void __launch_bounds__(256)
 cross_entropy_kernel(const float* __restrict__ logits, int64_t ldl, const int* __restrict__ rowlabel,
                      const float* __restrict__ inv_n, T* __restrict__ dlogits, int64_t ldd,
                      float* __restrict__ nll, int V) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   __shared__ float sm[8], ss[8];
   __shared__ float s_lse;
@@ -702,6 +711,7 @@ __global__ void __launch_bounds__(1024)
 cross_entropy_regs_kernel(const float* __restrict__ logits, int64_t ldl, const int* __restrict__ rowlabel,
                           const float* __restrict__ inv_n, T* __restrict__ dlogits, int64_t ldd,
                           float* __restrict__ nll, int V) {
+  pdl_begin();
   __shared__ float red[32];
   __shared__ float bcast;
   const int r = blockIdx.x, tid = threadIdx.x;
@@ -784,6 +794,7 @@ cross_entropy_regs_kernel(const float* __restrict__ logits, int64_t ldl, const i
 
 __global__ void loss_reduce_kernel(const float* __restrict__ nll, int R,
                                    const float* __restrict__ inv_n, float* __restrict__ loss) {
+  pdl_begin();
   __shared__ float part[32];
   float s = 0.f;
   for (int r = threadIdx.x; r < R; r += blockDim.x) s += nll[r];
@@ -798,6 +809,7 @@ __global__ void loss_reduce_kernel(const float* __restrict__ nll, int R,
 }
 
 __global__ void override_inv_n_kernel(const int* __restrict__ total_valid, float* __restrict__ inv_n) {
+  pdl_begin();
   const int n = *total_valid;
   *inv_n = n > 0 ? 1.0f / (float)n : 0.f;
 }
@@ -809,6 +821,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 colsum_kernel(const T* __restrict__ x, int64_t ld, int rows, int N, int rows_per_block,
               float* __restrict__ out) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   __shared__ float red[8][32 * VN];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -858,6 +871,7 @@ constexpr int ES_MAX_SLOTS = 2048;  // chunk slots: at most T / ES_CHUNK + (toke
 __global__ void __launch_bounds__(ES_BLOCK)
 embed_sort_count_kernel(const int* __restrict__ tokens, int T, int V, int nb, int* __restrict__ counts,
                         int* __restrict__ rank) {
+  pdl_begin();
   __shared__ int tk[ES_BLOCK];
   const int t = blockIdx.x * ES_BLOCK + threadIdx.x;
   int tok = t < T ? tokens[t] : -1;
@@ -876,6 +890,7 @@ embed_sort_count_kernel(const int* __restrict__ tokens, int T, int V, int nb, in
 __global__ void __launch_bounds__(256)
 embed_sort_prefix_kernel(int* __restrict__ counts, int nb, int V, int* __restrict__ total,
                          int* __restrict__ start_local, int* __restrict__ blocksum, int* __restrict__ hot) {
+  pdl_begin();
   __shared__ int part[256];
   const int v = blockIdx.x * 256 + threadIdx.x;
   int run = 0;
@@ -918,6 +933,7 @@ embed_sort_prefix_kernel(int* __restrict__ counts, int nb, int V, int* __restric
 // exclusive scan of the block sums (at most 1024 blocks of 256 tokens) in place
 __global__ void __launch_bounds__(1024)
 embed_sort_scan_kernel(int* __restrict__ blocksum, int n) {
+  pdl_begin();
   __shared__ int part[1024];
   const int mine = threadIdx.x < n ? blocksum[threadIdx.x] : 0;
   part[threadIdx.x] = mine;
@@ -935,6 +951,7 @@ __global__ void embed_sort_place_kernel(const int* __restrict__ tokens, int T, i
                                         const int* __restrict__ counts, const int* __restrict__ rank,
                                         const int* __restrict__ start_local, const int* __restrict__ blockoff,
                                         int* __restrict__ order) {
+  pdl_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= T) return;
   int tok = tokens[t];
@@ -993,6 +1010,7 @@ __global__ void __launch_bounds__(256)
 embed_word_grad_kernel(const T* __restrict__ dz, const int* __restrict__ order, const int* __restrict__ start_local,
                        const int* __restrict__ blockoff, const int* __restrict__ total,
                        float* __restrict__ dword, int H, int V) {
+  pdl_begin();
   extern __shared__ float es_part[];  // [G][H]
   for (int v = blockIdx.x; v < V; v += gridDim.x) {
     const int n = total[v];
@@ -1008,6 +1026,7 @@ embed_word_hot_chunk_kernel(const T* __restrict__ dz, const int* __restrict__ or
                             const int* __restrict__ start_local, const int* __restrict__ blockoff,
                             const int* __restrict__ total, const int* __restrict__ hot,
                             float* __restrict__ partial, int H) {
+  pdl_begin();
   extern __shared__ float es_part[];
   const int slot = blockIdx.x;
   if (slot >= min(hot[0], ES_MAX_SLOTS)) return;
@@ -1020,6 +1039,7 @@ embed_word_hot_chunk_kernel(const T* __restrict__ dz, const int* __restrict__ or
 // second half: block = frequent token, dword[v, :] += its chunks' partial sums in chunk order
 __global__ void embed_word_hot_sum_kernel(const int* __restrict__ total, const int* __restrict__ hot,
                                           const float* __restrict__ partial, float* __restrict__ dword, int H) {
+  pdl_begin();
   const int h = blockIdx.x;
   if (h >= min(hot[1], ES_MAX_SLOTS / 2)) return;
   const int v = hot[2 + 2 * ES_MAX_SLOTS + 2 * h], base = hot[2 + 2 * ES_MAX_SLOTS + 2 * h + 1];
@@ -1036,6 +1056,7 @@ __global__ void embed_word_hot_sum_kernel(const int* __restrict__ total, const i
 template <typename T>
 __global__ void __launch_bounds__(256)
 embed_pos_grad_kernel(const T* __restrict__ dz, float* __restrict__ dpos, int B, int S, int H) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   __shared__ float part[8][32 * VN];
   const int s = blockIdx.x;
@@ -1082,6 +1103,7 @@ embed_pos_grad_kernel(const T* __restrict__ dz, float* __restrict__ dpos, int B,
 // there, so that a captured step (CUDA graph) replays with the right values.
 __global__ void adam_tick_kernel(int* __restrict__ t, float* __restrict__ bc, float beta1, float beta2,
                                  int bias_correction) {
+  pdl_begin();
   const int n = *t + 1;
   *t = n;
   bc[0] = bias_correction ? (float)(1.0 / (1.0 - pow((double)beta1, (double)n))) : 1.f;
@@ -1092,6 +1114,7 @@ __global__ void __launch_bounds__(256)
 adam_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w,
             const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
             bf16* __restrict__ wb, AdamHyper h, const float* __restrict__ bc) {
+  pdl_begin();
   h.bc1 = bc[0];
   h.bc2 = bc[1];
   const AdamChunk ch = chunks[blockIdx.x];
@@ -1134,6 +1157,7 @@ adam_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w,
 // ---------------------------------------------------------------------------------------
 __global__ void nsp_prepare_kernel(const int* __restrict__ labels, int B, int S, int* __restrict__ rowsrc,
                                    float* __restrict__ inv_n, const int* __restrict__ total_valid) {
+  pdl_begin();
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -1155,6 +1179,7 @@ __global__ void __launch_bounds__(128)
 nsp_head_kernel(const T* __restrict__ pooled, const float* __restrict__ wn, const float* __restrict__ bn,
                 const int* __restrict__ labels, const float* __restrict__ inv_n, T* __restrict__ dup,
                 float* __restrict__ dwn, float* __restrict__ dbn, float* __restrict__ loss, int H) {
+  pdl_begin();
   const int b = blockIdx.x;
   const T* pr = pooled + (int64_t)b * H;
   float s0 = 0.f, s1 = 0.f;
@@ -1196,6 +1221,7 @@ nsp_head_kernel(const T* __restrict__ pooled, const float* __restrict__ wn, cons
 // y = tanh(x), elementwise
 template <typename T>
 __global__ void tanh_kernel(const T* __restrict__ x, T* __restrict__ y, int64_t n) {
+  pdl_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = from_f<T>(tanhf(to_f<T>(x[i])));
 }
@@ -1206,6 +1232,7 @@ template <typename T>
 __global__ void __launch_bounds__(128)
 type_grad_kernel(const T* __restrict__ dz, const int* __restrict__ segments, float* __restrict__ dtype,
                  int rows, int H, int rows_per_block) {
+  pdl_begin();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= H) return;
   const int r0 = blockIdx.y * rows_per_block, r1 = min(rows, r0 + rows_per_block);
@@ -1224,6 +1251,7 @@ __global__ void __launch_bounds__(256)
 lamb_moments_kernel(const AdamChunk* __restrict__ chunks, const float* __restrict__ w,
                     const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v, AdamHyper h,
                     const float* __restrict__ bc, float* __restrict__ norms) {
+  pdl_begin();
   h.bc1 = bc[0];
   h.bc2 = bc[1];
   const AdamChunk ch = chunks[blockIdx.x];
@@ -1270,6 +1298,7 @@ __global__ void __launch_bounds__(256)
 lamb_apply_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w, const float* __restrict__ m,
                   const float* __restrict__ v, bf16* __restrict__ wb, AdamHyper h,
                   const float* __restrict__ bc, const float* __restrict__ norms) {
+  pdl_begin();
   h.bc1 = bc[0];
   h.bc2 = bc[1];
   const AdamChunk ch = chunks[blockIdx.x];
@@ -1301,6 +1330,7 @@ lamb_apply_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w, c
 // d[i] *= gelu'(u[i]) (MLM transform backward)
 template <typename T>
 __global__ void dgelu_kernel(T* __restrict__ d, const T* __restrict__ u, int64_t n) {
+  pdl_begin();
   constexpr int VN = VecT<T>::N;
   for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * VN; i < n;
        i += (int64_t)gridDim.x * blockDim.x * VN) {
@@ -1314,6 +1344,7 @@ __global__ void dgelu_kernel(T* __restrict__ d, const T* __restrict__ u, int64_t
 }
 
 __global__ void f32_to_bf16_kernel(const float* __restrict__ src, bf16* __restrict__ dst, int64_t n) {
+  pdl_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     dst[i] = __float2bfloat16_rn(src[i]);
@@ -1334,7 +1365,7 @@ void launch_ln_fwd(bool bf, const void* z, const float* gamma, const float* beta
   const int vn = bf ? 8 : 4;
   const int nv = (H + 32 * vn - 1) / (32 * vn);
 #define LN_FWD(NV, ROWS)                                                                             \
-  DISPATCH_T(bf, (ln_fwd_kernel<T, NV, ROWS><<<div_up(rows, 4 * ROWS), 128, 0, st>>>(                  \
+  DISPATCH_T(bf, (launch_pdl(ln_fwd_kernel<T, NV, ROWS>, div_up(rows, 4 * ROWS), 128, 0, st,                   \
                      (const T*)z, gamma, beta, (T*)y, stats, rows, H, eps)))
   if (nv <= 1) LN_FWD(1, 4);
   else if (nv <= 2) LN_FWD(2, 2);
@@ -1349,7 +1380,7 @@ void launch_embed_ln(bool bf, const int* tokens, const int* segments, const void
                      const void* type, const float* gamma, const float* beta, void* y, void* zstash,
                      float* stats, int rows, int S, int H, int V, float eps, int* status, cudaStream_t st) {
   if (rows <= 0) return;
-  DISPATCH_T(bf, (embed_ln_kernel<T><<<div_up(rows, 8), 256, 0, st>>>(
+  DISPATCH_T(bf, (launch_pdl(embed_ln_kernel<T>, div_up(rows, 8), 256, 0, st, 
                      tokens, segments, (const T*)word, (const T*)pos, (const T*)type, gamma, beta, (T*)y,
                      (T*)zstash, stats, rows, S, H, V, eps, status)));
 }
@@ -1365,7 +1396,7 @@ void launch_ln_bwd(bool bf, const void* dy, const void* z, const float* stats, c
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // one block per SM walks the rows: the column sums end in one atomic per column and block
 #define LN_BWD(NS, RG)                                                                                   \
-  DISPATCH_T(bf, (ln_bwd_kernel<T, NS, RG, 4><<<std::min(div_up(rows, RG * 4), sms), NS * RG * 32, 0, st>>>( \
+  DISPATCH_T(bf, (launch_pdl(ln_bwd_kernel<T, NS, RG, 4>, std::min(div_up(rows, RG * 4), sms), NS * RG * 32, 0, st,  \
                      (const T*)dy, (const T*)z, stats, gamma, (T*)dz, dgamma, dbeta, dbias, rows, H)))
   if (nslice <= 1) LN_BWD(1, 8);
   else if (nslice <= 2) LN_BWD(2, 6);
@@ -1382,7 +1413,7 @@ void launch_softmax_fwd(bool bf, const void* sc, void* p, const int* seq_lens, i
   const int vn = bf ? 8 : 4;
   const int nvec = (S + vn - 1) / vn;  // 16-byte vectors per row
 #define SM_FWD(LPR, NV)                                                                        \
-  DISPATCH_T(bf, (softmax_fwd_kernel<T, LPR, NV><<<div_up(rows, 8 * (32 / LPR) * 2), 256, 0, st>>>( \
+  DISPATCH_T(bf, (launch_pdl(softmax_fwd_kernel<T, LPR, NV>, div_up(rows, 8 * (32 / LPR) * 2), 256, 0, st,  \
                      (const T*)sc, (T*)p, seq_lens, rows, S, rows_per_seq, scale)))
   if (nvec <= 16) SM_FWD(16, 1);
   else if (nvec <= 32) SM_FWD(32, 1);
@@ -1397,7 +1428,7 @@ void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float
   const int vn = bf ? 8 : 4;
   const int nvec = (S + vn - 1) / vn;  // 16-byte vectors per row
 #define SM_BWD(LPR, NV)                                                                        \
-  DISPATCH_T(bf, (softmax_bwd_kernel<T, LPR, NV><<<div_up(rows, 8 * (32 / LPR) * 2), 256, 0, st>>>( \
+  DISPATCH_T(bf, (launch_pdl(softmax_bwd_kernel<T, LPR, NV>, div_up(rows, 8 * (32 / LPR) * 2), 256, 0, st,  \
                      (T*)dp, (const T*)p, rows, S, scale)))
   if (nvec <= 16) SM_BWD(16, 1);
   else if (nvec <= 32) SM_BWD(32, 1);
@@ -1409,20 +1440,20 @@ void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float
 void launch_slots_prepare(const int* positions, const int* labels, const int* seq_lens, int B,
                           int S, int P, int V, int* rowsrc, int* rowlabel, int* n_valid,
                           float* inv_n, int* status, cudaStream_t st) {
-  slots_prepare_kernel<<<1, 256, 0, st>>>(positions, labels, seq_lens, B, S, P, V, rowsrc, rowlabel,
+  launch_pdl(slots_prepare_kernel, 1, 256, 0, st, positions, labels, seq_lens, B, S, P, V, rowsrc, rowlabel,
                                           n_valid, inv_n, status);
 }
 
 void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, int R, int H,
                         cudaStream_t st) {
   if (R <= 0) return;
-  DISPATCH_T(bf, (gather_rows_kernel<T><<<R, 128, 0, st>>>((const T*)x, rowsrc, (T*)out, R, H)));
+  DISPATCH_T(bf, (launch_pdl(gather_rows_kernel<T>, R, 128, 0, st, (const T*)x, rowsrc, (T*)out, R, H)));
 }
 
 void launch_scatter_rows(bool bf, const void* d, const int* rowsrc, void* dx, int B, int P, int H,
                          cudaStream_t st) {
   if (B <= 0 || P <= 0) return;
-  DISPATCH_T(bf, (scatter_rows_kernel<T><<<B, 128, 0, st>>>((const T*)d, rowsrc, (T*)dx, P, H)));
+  DISPATCH_T(bf, (launch_pdl(scatter_rows_kernel<T>, B, 128, 0, st, (const T*)d, rowsrc, (T*)dx, P, H)));
 }
 
 void launch_cross_entropy(bool bf, const float* logits, int64_t ldl, const int* rowlabel,
@@ -1430,19 +1461,19 @@ void launch_cross_entropy(bool bf, const float* logits, int64_t ldl, const int* 
                           cudaStream_t st) {
   if (R <= 0) return;
   if (ldl <= CE_REG_V4 * 1024 * 4)
-    DISPATCH_T(bf, (cross_entropy_regs_kernel<T><<<R, 1024, 0, st>>>(logits, ldl, rowlabel, inv_n,
+    DISPATCH_T(bf, (launch_pdl(cross_entropy_regs_kernel<T>, R, 1024, 0, st, logits, ldl, rowlabel, inv_n,
                                                                      (T*)dlogits, ldd, nll, V)));
   else
-    DISPATCH_T(bf, (cross_entropy_kernel<T><<<R, 256, 0, st>>>(logits, ldl, rowlabel, inv_n,
+    DISPATCH_T(bf, (launch_pdl(cross_entropy_kernel<T>, R, 256, 0, st, logits, ldl, rowlabel, inv_n,
                                                               (T*)dlogits, ldd, nll, V)));
 }
 
 void launch_override_inv_n(const int* total_valid, float* inv_n, cudaStream_t st) {
-  override_inv_n_kernel<<<1, 1, 0, st>>>(total_valid, inv_n);
+  launch_pdl(override_inv_n_kernel, 1, 1, 0, st, total_valid, inv_n);
 }
 
 void launch_loss_reduce(const float* nll, int R, const float* inv_n, float* loss, cudaStream_t st) {
-  loss_reduce_kernel<<<1, 1024, 0, st>>>(nll, R, inv_n, loss);
+  launch_pdl(loss_reduce_kernel, 1, 1024, 0, st, nll, R, inv_n, loss);
 }
 
 void launch_colsum(bool bf, const void* x, int64_t ld, int rows, int N, float* out,
@@ -1453,7 +1484,7 @@ void launch_colsum(bool bf, const void* x, int64_t ld, int rows, int N, float* o
   int gy = std::max(1, std::min(div_up(rows, 64), (148 * 4 + gx - 1) / gx));
   const int rpb = div_up(rows, gy);
   gy = div_up(rows, rpb);
-  DISPATCH_T(bf, (colsum_kernel<T><<<dim3(gx, gy), 256, 0, st>>>((const T*)x, ld, rows, N, rpb, out)));
+  DISPATCH_T(bf, (launch_pdl(colsum_kernel<T>, dim3(gx, gy), 256, 0, st, (const T*)x, ld, rows, N, rpb, out)));
 }
 
 void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float* dword, float* dpos, int B, int S,
@@ -1464,66 +1495,66 @@ void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float*
   const int nb = div_up(T, ES_BLOCK), vb = div_up(V, 256);
   cudaMemsetAsync(counts, 0, (size_t)nb * V * sizeof(int), st);
   cudaMemsetAsync(hot, 0, 2 * sizeof(int), st);
-  embed_sort_count_kernel<<<nb, ES_BLOCK, 0, st>>>(tokens, T, V, nb, counts, rank);
-  embed_sort_prefix_kernel<<<vb, 256, 0, st>>>(counts, nb, V, total, start, blocksum, hot);
-  embed_sort_scan_kernel<<<1, 1024, 0, st>>>(blocksum, vb);
-  embed_sort_place_kernel<<<div_up(T, 256), 256, 0, st>>>(tokens, T, V, nb, counts, rank, start, blocksum, order);
+  launch_pdl(embed_sort_count_kernel, nb, ES_BLOCK, 0, st, tokens, T, V, nb, counts, rank);
+  launch_pdl(embed_sort_prefix_kernel, vb, 256, 0, st, counts, nb, V, total, start, blocksum, hot);
+  launch_pdl(embed_sort_scan_kernel, 1, 1024, 0, st, blocksum, vb);
+  launch_pdl(embed_sort_place_kernel, div_up(T, 256), 256, 0, st, tokens, T, V, nb, counts, rank, start, blocksum, order);
   const int vn = bf ? 8 : 4;
   const size_t smem = (size_t)(1024 / (H / vn)) * H * sizeof(float), smem_small = (size_t)(256 / (H / vn)) * H * sizeof(float);
   // at most T / ES_CHUNK tokens have more than ES_CHUNK rows, and they have at most 2 T / ES_CHUNK chunks
   const int max_hot = std::min(ES_MAX_SLOTS / 2, T / ES_CHUNK), max_slots = std::min(ES_MAX_SLOTS, 2 * (T / ES_CHUNK));
-  DISPATCH_T(bf, (embed_word_grad_kernel<T><<<div_up(V, ES_TOKENS), 256, smem_small, st>>>(
+  DISPATCH_T(bf, (launch_pdl(embed_word_grad_kernel<T>, div_up(V, ES_TOKENS), 256, smem_small, st, 
                      (const T*)dz, order, start, blocksum, total, dword, H, V)));
   if (max_slots > 0) {
-    DISPATCH_T(bf, (embed_word_hot_chunk_kernel<T><<<max_slots, 1024, smem, st>>>((const T*)dz, order, start, blocksum,
+    DISPATCH_T(bf, (launch_pdl(embed_word_hot_chunk_kernel<T>, max_slots, 1024, smem, st, (const T*)dz, order, start, blocksum,
                                                                               total, hot, partial, H)));
-    embed_word_hot_sum_kernel<<<max_hot, 256, 0, st>>>(total, hot, partial, dword, H);
+    launch_pdl(embed_word_hot_sum_kernel, max_hot, 256, 0, st, total, hot, partial, dword, H);
   }
-  DISPATCH_T(bf, (embed_pos_grad_kernel<T><<<dim3(S, div_up(H, 32 * vn)), 256, 0, st>>>((const T*)dz, dpos, B, S, H)));
+  DISPATCH_T(bf, (launch_pdl(embed_pos_grad_kernel<T>, dim3(S, div_up(H, 32 * vn)), 256, 0, st, (const T*)dz, dpos, B, S, H)));
 }
 
 void launch_adam(const AdamChunk* chunks, int n_chunks, float* w, const float* g, float* m, float* v,
                  void* wb, const AdamHyper& h, int* t_dev, float* bc_dev, int bias_correction,
                  cudaStream_t st) {
-  adam_tick_kernel<<<1, 1, 0, st>>>(t_dev, bc_dev, h.beta1, h.beta2, bias_correction);
+  launch_pdl(adam_tick_kernel, 1, 1, 0, st, t_dev, bc_dev, h.beta1, h.beta2, bias_correction);
   if (n_chunks <= 0) return;
-  adam_kernel<<<n_chunks, 256, 0, st>>>(chunks, w, g, m, v, (bf16*)wb, h, bc_dev);
+  launch_pdl(adam_kernel, n_chunks, 256, 0, st, chunks, w, g, m, v, (bf16*)wb, h, bc_dev);
 }
 
 void launch_lamb(const AdamChunk* chunks, int n_chunks, float* w, const float* g, float* m, float* v,
                  void* wb, const AdamHyper& h, int* t_dev, float* bc_dev, int bias_correction,
                  float* norms, int n_tensors, cudaStream_t st) {
-  adam_tick_kernel<<<1, 1, 0, st>>>(t_dev, bc_dev, h.beta1, h.beta2, bias_correction);
+  launch_pdl(adam_tick_kernel, 1, 1, 0, st, t_dev, bc_dev, h.beta1, h.beta2, bias_correction);
   if (n_chunks <= 0) return;
   cudaMemsetAsync(norms, 0, (size_t)n_tensors * 2 * sizeof(float), st);
-  lamb_moments_kernel<<<n_chunks, 256, 0, st>>>(chunks, w, g, m, v, h, bc_dev, norms);
-  lamb_apply_kernel<<<n_chunks, 256, 0, st>>>(chunks, w, m, v, (bf16*)wb, h, bc_dev, norms);
+  launch_pdl(lamb_moments_kernel, n_chunks, 256, 0, st, chunks, w, g, m, v, h, bc_dev, norms);
+  launch_pdl(lamb_apply_kernel, n_chunks, 256, 0, st, chunks, w, m, v, (bf16*)wb, h, bc_dev, norms);
 }
 
 void launch_nsp_prepare(const int* labels, int B, int S, int* rowsrc, float* inv_n, const int* total_valid,
                         cudaStream_t st) {
-  nsp_prepare_kernel<<<1, 128, 0, st>>>(labels, B, S, rowsrc, inv_n, total_valid);
+  launch_pdl(nsp_prepare_kernel, 1, 128, 0, st, labels, B, S, rowsrc, inv_n, total_valid);
 }
 
 void launch_nsp_head(bool bf, const void* pooled, const float* wn, const float* bn, const int* labels,
                      const float* inv_n, void* dup, float* dwn, float* dbn, float* loss, int B, int H,
                      cudaStream_t st) {
   if (B <= 0) return;
-  DISPATCH_T(bf, (nsp_head_kernel<T><<<B, 128, 0, st>>>((const T*)pooled, wn, bn, labels, inv_n, (T*)dup, dwn, dbn,
+  DISPATCH_T(bf, (launch_pdl(nsp_head_kernel<T>, B, 128, 0, st, (const T*)pooled, wn, bn, labels, inv_n, (T*)dup, dwn, dbn,
                                                        loss, H)));
 }
 
 void launch_tanh(bool bf, const void* x, void* y, int64_t n, cudaStream_t st) {
   if (n <= 0) return;
   int blocks = (int)std::min<int64_t>((n + 255) / 256, 148 * 8);
-  DISPATCH_T(bf, (tanh_kernel<T><<<blocks, 256, 0, st>>>((const T*)x, (T*)y, n)));
+  DISPATCH_T(bf, (launch_pdl(tanh_kernel<T>, blocks, 256, 0, st, (const T*)x, (T*)y, n)));
 }
 
 void launch_type_grad(bool bf, const void* dz, const int* segments, float* dtype, int rows, int H,
                       cudaStream_t st) {
   if (rows <= 0) return;
   const int rpb = 512;
-  DISPATCH_T(bf, (type_grad_kernel<T><<<dim3(div_up(H, 128), div_up(rows, rpb)), 128, 0, st>>>(
+  DISPATCH_T(bf, (launch_pdl(type_grad_kernel<T>, dim3(div_up(H, 128), div_up(rows, rpb)), 128, 0, st, 
                      (const T*)dz, segments, dtype, rows, H, rpb)));
 }
 
@@ -1531,13 +1562,13 @@ void launch_dgelu(bool bf, void* d, const void* u, int64_t n, cudaStream_t st) {
   if (n <= 0) return;
   const int vn = bf ? 8 : 4;
   int blocks = (int)std::min<int64_t>((n / vn + 255) / 256, 148 * 8);
-  DISPATCH_T(bf, (dgelu_kernel<T><<<blocks, 256, 0, st>>>((T*)d, (const T*)u, n)));
+  DISPATCH_T(bf, (launch_pdl(dgelu_kernel<T>, blocks, 256, 0, st, (T*)d, (const T*)u, n)));
 }
 
 void launch_f32_to_bf16(const float* src, void* dst, int64_t n, cudaStream_t st) {
   if (n <= 0) return;
   int blocks = (int)std::min<int64_t>((n + 255) / 256, 148 * 8);
-  f32_to_bf16_kernel<<<blocks, 256, 0, st>>>(src, (bf16*)dst, n);
+  launch_pdl(f32_to_bf16_kernel, blocks, 256, 0, st, src, (bf16*)dst, n);
 }
 
 }  // namespace mslt

@@ -30,6 +30,7 @@ int op_fail(int code, const char* fmt, ...) {
 // labels >= V are treated as "ignore" after raising the status bit; counts the valid rows
 __global__ void count_labels_kernel(const int* __restrict__ labels, int R, int V, int* __restrict__ rowlabel,
                                     int* __restrict__ n_valid, float* __restrict__ inv_n) {
+  pdl_begin();
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -74,7 +75,7 @@ int run_ce(int dtype, const float* logits, int64_t ldl, const int32_t* labels, i
   int* rowlabel = (int*)scratch + R;
   int* n_valid = (int*)scratch + 2 * (size_t)R;
   float* inv_n = (float*)scratch + 2 * (size_t)R + 1;
-  count_labels_kernel<<<1, 256, 0, st>>>(labels, R, V, rowlabel, n_valid, inv_n);
+  launch_pdl(count_labels_kernel, 1, 256, 0, st, labels, R, V, rowlabel, n_valid, inv_n);
   launch_cross_entropy(dtype == 1, logits, ldl, rowlabel, inv_n, dlogits, ldd, nll, R, V, st);
   launch_loss_reduce(nll, R, inv_n, loss, st);
   cudaError_t e = cudaGetLastError();
