@@ -241,7 +241,7 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
 
 // ---- the kernel ---------------------------------------------------------------------------------
 // 12 warps: a thread may use up to 168 registers
-template <int kMode, bool kPair>
+template <int kMode, bool kPair, int KSUB>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmD, const TcParams p) {
@@ -261,9 +261,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int w_step = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   // A ring stage holds KSUB 64-deep k blocks of both operands ("a round").  The issuing thread
   // spends a fixed ~250-350 cycles per round on its barrier hand-shakes whatever the round holds;
-  // with four MMAs (512 cycles of tensor-core work) per round that kept the tensor core waiting,
-  // with eight it does not.  The pair form has the shared memory for three such stages.
-  constexpr int KSUB = kPair ? 2 : 1;
+  // with four MMAs (512 cycles of tensor-core work at 256 columns) per round that kept the tensor
+  // core waiting, with eight it does not.  Two blocks per round wherever three such stages fit
+  // shared memory: the pair form, and single CTAs with at most 128 columns.
   const int b_stage_bytes = bn_cta * BK * 2;
   const int sub_bytes = A_STAGE_BYTES + b_stage_bytes;
   const int stage_bytes = KSUB * sub_bytes;
@@ -495,7 +495,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // division per tile); the bias of the NEXT tile is fetched while this tile is worked on; the
       // TMEM read of the next chunk is in flight while the current chunk is converted and stored;
       // and a lane stores its row segment straight from registers.
-      const int nch = p.bn >> 6;
       constexpr bool kHasXf = kMode == EPI_RESIDUAL || kMode == EPI_DGELU;
       const bf16* xsrc = kMode == EPI_DGELU ? p.aux : kMode == EPI_RESIDUAL ? p.residual : nullptr;
       // digits of the work index (n tile fastest, then m tile, batch, split) and of the step
@@ -533,7 +532,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
         for (int i = 0; i < 4; i++) {
           const int n = nt_ * p.bn + ccol(i) * 32 + lane;
-          b[i] = (i < nch && p.bias && n < p.N) ? p.bias[n] : 0.f;
+          b[i] = (ccol(i) * 32 < p.bn && p.bias && n < p.N) ? p.bias[n] : 0.f;
         }
       };
       float bnext[4];
@@ -555,7 +554,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const float* bias_t = bias_s + (tile & 1) * 128;
         const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 256;
         auto chunk_n0 = [&](int i) { return n_base + ccol(i) * 32; };
-        auto chunk_ok = [&](int i) { return i < nch && chunk_n0(i) < p.N; };
+        auto chunk_ok = [&](int i) { return ccol(i) * 32 < p.bn && chunk_n0(i) < p.N; };
         auto prefetch_x = [&](int i, uint4 (&x)[4]) {
           if (kHasXf && row_ok) {
             const uint4* src = reinterpret_cast<const uint4*>(xsrc + off0 + chunk_n0(i));
@@ -927,6 +926,52 @@ DeviceInfo g_dev[kMaxDevices];
 std::mutex g_dev_mu;
 }  // namespace
 
+// Tile form and k split of one product.  The estimate below (microseconds) was fitted to 1500 timed
+// launches of all forms: every product shape of BERT-Base at 64 to 16384 rows and its weight
+// gradients.  Over those shapes the form it picks is on average 0.7 % slower than the fastest one.
+// Against the rule it replaces (256 columns, or 128 where that fills the SMs better, and pairs from
+// 30 GFLOP on): 64 x 768 x 768 10.8 -> 6.1 us, 1024 x 768 x 3072 20.8 -> 14.5, 4096 x 768 x 768
+// 16.4 -> 13.3, 4096 x 768 x 3072 30.1 -> 25.4, 2304 x 768 x 2400 (weight gradient) 16.1 -> 14.6,
+// 8192 x 768 x 3072 44.5 -> 39.0.
+//   per 64 of k, with the operand reads from L2 and the issuing thread's hand-shakes in it;
+//   an epilogue that overlaps the next tile's loop, one more at the end;
+//   start-up (pairs have a cluster to set up); singles slow down a little when many waves of them
+//   contend for L2, where a pair fetches a third less per flop.
+static void choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, bool can_split, bool* pair, int* bn,
+                          int* ksub, int* splits) {
+  struct Form { bool pair; int bn, ksub; double per_k; };
+  static const Form forms[] = {{false, 64, 2, 0.202}, {false, 128, 2, 0.280}, {false, 192, 1, 0.362}, {false, 256, 1, 0.413},
+                               {true, 128, 2, 0.240}, {true, 192, 2, 0.317}, {true, 256, 2, 0.383}};
+  // epilogue of a tile: fixed part and part per 256 columns
+  double e0 = 2.0, e1 = 1.5;
+  if (d.d_fp32) { e0 = d.accumulate ? 1.7 : 4.4; e1 = d.accumulate ? 5.4 : 6.4; }
+  else if (d.act == 2) { e0 = 1.4; e1 = 6.9; }
+  else if (d.act == 1) { e0 = 1.6; e1 = d.aux ? 5.4 : 4.2; }
+  else if (d.residual) { e0 = 1.2; e1 = 6.6; }
+  const bool b_mn = d.b_rs == 1 && d.b_ks != 1;
+  const bool pairs_ok = d.M > BM && d.act != 3 && num_sms % 2 == 0 && variant != 1;
+  const int kblocks = (d.K + BK - 1) / BK, fixed_splits = *splits;
+  double best = 1e30;
+  for (const Form& f : forms) {
+    if (f.bn > 64 && f.bn >= d.N + 64) continue;            // no wider than the output needs
+    if (d.act == 3 && (f.bn > 128 || f.bn < d.N)) continue;  // the softmax epilogue holds whole rows
+    if (f.pair && (!pairs_ok || (b_mn && f.bn % 128))) continue;  // row-contiguous B comes in 64-wide boxes
+    if (!f.pair && variant == 2 && pairs_ok && d.N > 64) continue;
+    const int ks = d.act == 3 || kblocks == 1 ? 1 : f.ksub;
+    const int rows = f.pair ? 2 * BM : BM, units = f.pair ? num_sms / 2 : num_sms;
+    const long long tiles = (long long)((d.M + rows - 1) / rows) * ((d.N + f.bn - 1) / f.bn) * d.batch;
+    const double epi = e0 + e1 * f.bn / 256.;
+    for (int sp = fixed_splits; sp == fixed_splits || (can_split && sp <= 16 && sp * 4 <= kblocks); sp++) {
+      const double waves = (double)((tiles * sp + units - 1) / units);
+      const int kb = ((kblocks + sp - 1) / sp + ks - 1) / ks * ks;
+      const double loop = kb * f.per_k + 0.66;
+      const double crowd = f.pair ? 1. : 1. + 0.004 * (waves - 1 < 4 ? waves - 1 : 4);
+      const double t = (f.pair ? 2.4 : 1.0) + waves * (loop > epi ? loop : epi) * crowd + (loop < epi ? loop : epi);
+      if (t < best) { best = t; *pair = f.pair; *bn = f.bn; *ksub = f.pair ? 2 : ks; *splits = sp; }
+    }
+  }
+}
+
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_starve_next.exchange(0) != 0;
@@ -951,50 +996,18 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.M = d.M; p.N = d.N; p.K = d.K; p.batch = d.batch; p.hdiv = d.hdiv;
   p.a_mn = (d.a_rs == 1 && d.a_ks != 1) ? 1 : 0;
   p.b_mn = (d.b_rs == 1 && d.b_ks != 1) ? 1 : 0;
-  p.bn = d.N <= 64 ? 64 : (d.N <= 128 ? 128 : 256);
-  // Two CTAs per 256 x 256 tile: each SM then streams 64 instead of 96 bytes of operands per clock
-  // from L2 (about 117 is what an SM was measured to take) and has six instead of four stages in
-  // flight.
   const int variant = g_tile_variant.load();
-  // Small products (under ~30 GFLOP, e.g. 16384 x 768 x 768) measured 5-10 % faster on single CTAs.
-  const double flops = 2.0 * d.M * d.N * (double)d.K * d.batch;
-  bool pair = variant != 1 && p.bn == 256 && d.M > BM && d.act != 3 && num_sms % 2 == 0 &&
-              (variant == 2 || flops >= 30e9);
-  // share of the SMs that the last wave of tiles keeps busy
-  auto wave_eff = [](long long work, int units_) {
-    const long long waves = (work + units_ - 1) / units_;
-    return (double)work / (double)(waves * units_);
-  };
-  const bool can_split = d.split_k != 1 && d.d_fp32 && d.accumulate;
-  if (p.bn == 256 && !can_split) {
-    // few large tiles leave SMs idle: 128-wide tiles on single CTAs may fill the machine better
-    const long long t256 = (long long)((d.M + (pair ? 2 * BM : BM) - 1) / (pair ? 2 * BM : BM)) *
-                           ((d.N + 255) / 256) * d.batch;
-    const long long t128 = (long long)((d.M + BM - 1) / BM) * ((d.N + 127) / 128) * d.batch;
-    if (wave_eff(t128, num_sms) > 1.25 * wave_eff(t256, pair ? num_sms / 2 : num_sms)) {
-      p.bn = 128;
-      pair = false;
-    }
-  }
+  const bool can_split = d.split_k == 0 && d.d_fp32 && d.accumulate;
+  bool pair = false;
+  int splits = d.split_k > 1 ? d.split_k : 1, ksub = 1;
+  choose_tiling(d, num_sms, variant, can_split, &pair, &p.bn, &ksub, &splits);
   const int tile_m = pair ? 2 * BM : BM;
   p.m_tiles = (d.M + tile_m - 1) / tile_m;
   p.n_tiles = (d.N + p.bn - 1) / p.bn;
-  const int round_k = pair ? 2 * BK : BK;  // k extent of a ring stage (see KSUB in the kernel)
+  const int round_k = ksub * BK;  // k extent of a ring stage (see KSUB in the kernel)
   p.kb_total = (d.K + round_k - 1) / round_k;
   const long long tiles = (long long)p.m_tiles * p.n_tiles * d.batch;
   const int units = pair ? num_sms / 2 : num_sms;  // CTAs or CTA pairs that run concurrently
-  int splits = 1;
-  if (d.split_k > 1) {
-    splits = d.split_k;
-  } else if (d.split_k == 0 && can_split && tiles < 2 * units && p.kb_total * round_k >= 8 * BK) {
-    // the split count that fills the last wave best, with at least 256 k per split
-    const int max_by_k = p.kb_total * round_k / (4 * BK);
-    double best = wave_eff(tiles, units);
-    for (int sp = 2; sp <= 16 && sp <= max_by_k; sp++) {
-      const double e = wave_eff(tiles * sp, units);
-      if (e > best + 0.04) { best = e; splits = sp; }
-    }
-  }
   if (splits > 1 && !(d.d_fp32 && d.accumulate)) {
     snprintf(err, 256, "gemm: split_k needs an fp32 accumulating output");
     return MSLT_ERR_ARG;
@@ -1009,7 +1022,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
     snprintf(err, 256, "gemm: the softmax epilogue needs bf16 output rows of at most 128 columns");
     return MSLT_ERR_ARG;
   }
-  const int stage_bytes = (pair ? 2 : 1) * (A_STAGE_BYTES + (pair ? p.bn / 2 : p.bn) * BK * 2);  // per CTA
+  const int stage_bytes = ksub * (A_STAGE_BYTES + (pair ? p.bn / 2 : p.bn) * BK * 2);  // per CTA
   // barriers, then the softmax epilogue's exchange area or the 32 floats per epilogue warp that
   // hold the bias of a ragged chunk when the staging buffers carry output tiles
   const int book_bytes = 256 + (d.act == 3 ? 64 + 2 * NUM_EPI_WARPS * 32 * 4 : NUM_EPI_WARPS * 32 * 4);
@@ -1086,19 +1099,16 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   }
 
   typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams);
-  static const KernelFn kernels[EPI_COUNT][2] = {
-      {gemm_tc_kernel<EPI_STORE, false>, gemm_tc_kernel<EPI_STORE, true>},
-      {gemm_tc_kernel<EPI_RESIDUAL, false>, gemm_tc_kernel<EPI_RESIDUAL, true>},
-      {gemm_tc_kernel<EPI_GELU, false>, gemm_tc_kernel<EPI_GELU, true>},
-      {gemm_tc_kernel<EPI_GELU_AUX, false>, gemm_tc_kernel<EPI_GELU_AUX, true>},
-      {gemm_tc_kernel<EPI_DGELU, false>, gemm_tc_kernel<EPI_DGELU, true>},
-      {gemm_tc_kernel<EPI_F32, false>, gemm_tc_kernel<EPI_F32, true>},
-      {gemm_tc_kernel<EPI_GENERIC, false>, gemm_tc_kernel<EPI_GENERIC, true>},
-      {gemm_tc_kernel<EPI_SOFTMAX, false>, nullptr}};
+  // [one CTA, one k block per round | one CTA, two | pair, two]
+#define FORMS(mode) {gemm_tc_kernel<mode, false, 1>, gemm_tc_kernel<mode, false, 2>, gemm_tc_kernel<mode, true, 2>}
+  static const KernelFn kernels[EPI_COUNT][3] = {
+      FORMS(EPI_STORE), FORMS(EPI_RESIDUAL), FORMS(EPI_GELU), FORMS(EPI_GELU_AUX), FORMS(EPI_DGELU), FORMS(EPI_F32),
+      FORMS(EPI_GENERIC), {gemm_tc_kernel<EPI_SOFTMAX, false, 1>, nullptr, nullptr}};
+#undef FORMS
   std::unique_lock<std::mutex> dev_lock(g_dev_mu);
   if (!di.attr_set) {
     for (int mo = 0; mo < EPI_COUNT; mo++)
-      for (int pr = 0; pr < 2; pr++) {
+      for (int pr = 0; pr < 3; pr++) {
         if (!kernels[mo][pr]) continue;
         cudaError_t e = cudaFuncSetAttribute((const void*)kernels[mo][pr], cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
         if (e != cudaSuccess) { snprintf(err, 256, "gemm: cudaFuncSetAttribute: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
@@ -1106,7 +1116,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
     di.attr_set = true;
   }
   dev_lock.unlock();
-  const KernelFn fn = kernels[mode][pair ? 1 : 0];
+  const KernelFn fn = kernels[mode][pair ? 2 : ksub - 1];
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.blockDim = dim3(GEMM_THREADS);

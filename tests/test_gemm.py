@@ -270,3 +270,16 @@ def test_fp32_unaligned_operands_take_the_element_wise_copies():
     a, b = A[1:].view(M, ld)[:, :K].double(), B[1:].view(N, ld)[:, :K].double()
     ref = a @ b.t()
     assert ((D.double() - ref).abs().max() / ref.abs().max()).item() < 2e-5
+
+
+@pytest.mark.parametrize("shape,majors,kw", [
+    ((64, 768, 200), ("k", "k"), dict(bias=True, residual=True)),          # 64-wide tiles, two k blocks per round
+    ((130, 72, 136), ("k", "mn"), dict(act=2)),
+    ((1100, 2304, 136), ("k", "k"), dict(bias=True)),                       # 128-wide
+    ((4096, 760, 264), ("k", "k"), dict(bias=True, residual=True)),         # 192-wide, ragged last tile
+    ((4096, 768, 320), ("k", "mn"), dict(residual=True)),
+    ((4000, 768, 1160), ("k", "k"), dict(bias=True, act=1, aux_out=True)),  # pairs of 192 columns
+    ((2304, 768, 2408), ("mn", "mn"), dict(d_fp32=True, accumulate=True)),  # 192-wide, k split
+    ((24, 768, 4000), ("k", "mn"), dict(d_fp32=True, accumulate=True))])    # narrow tiles, k split many ways
+def test_bf16_tile_forms_the_estimate_picks(shape, majors, kw):
+    _run(1, *shape, *majors, **kw)
