@@ -1013,7 +1013,9 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
     return MSLT_ERR_ARG;
   }
   if (splits > p.kb_total) splits = p.kb_total;
-  p.kb_per_split = (p.kb_total + splits - 1) / splits;
+  // a split is a whole number of 128-deep slices in every form, so that the partial sums of a given
+  // split count do not depend on the tile form
+  p.kb_per_split = ((d.K + 2 * BK - 1) / (2 * BK) + splits - 1) / splits * (2 / ksub);
   p.splits = (p.kb_total + p.kb_per_split - 1) / p.kb_per_split;
   const long long total = tiles * p.splits;
   if (total > 0x7fffffffll) { snprintf(err, 256, "gemm: too many tiles"); return MSLT_ERR_SIZE; }

@@ -108,7 +108,7 @@ struct mslt_ctx {
   Workspace ws;
   int n_chunks;
   int64_t launches;
-  int Vp;
+  int Vp, num_sms;
   bool timing;
   cudaEvent_t ev[6];
   float phase_ms[5];
@@ -609,6 +609,25 @@ int head_forward(mslt_ctx* c, const void* x, int R, bool save) {
   return 0;
 }
 
+// Split count of the vocabulary-long contraction of the head's input gradient: the number that fills
+// the last wave of 256 x 256 tiles on CTA pairs.  Fixed here rather than left to the contraction's
+// own estimate, because this sum is rounded to bf16 and feeds the whole backward pass: with a fixed
+// count its rounding does not change with the tile form.  Small products keep the estimate.
+int dtm_splits(const mslt_ctx* c, int R) {
+  const int H = c->a.hidden, V = c->a.vocab;
+  if (2.0 * R * H * (double)V < 30e9 || H <= 128 || R <= 128) return 0;
+  const long long tiles = (long long)((R + 255) / 256) * ((H + 255) / 256), units = c->num_sms / 2;
+  int splits = 1;
+  double best = 0.;
+  for (int sp = 1; sp <= 16 && sp * 256 <= V; sp++) {
+    if (sp > 1 && tiles >= 2 * units) break;
+    const long long waves = (tiles * sp + units - 1) / units;
+    const double e = (double)(tiles * sp) / (double)(waves * units);
+    if (sp == 1 || e > best + 0.04) { best = e; splits = sp; }
+  }
+  return splits;
+}
+
 int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
   const int H = c->a.hidden, V = c->a.vocab, R = B * P, Vp = c->Vp;
   Workspace& w = c->ws;
@@ -622,6 +641,7 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
       // with fp32 partial sums, then round once to bf16
       CUDA_TRY(cudaMemsetAsync(w.dtm32, 0, (size_t)R * H * 4, c->st));
       g.d.D = w.dtm32; g.d.ldd = H; g.d.d_fp32 = 1; g.d.accumulate = 1;
+      g.d.split_k = dtm_splits(c, R);
       TRY(run_gemm(c, g.d));
       KL(PC_OTHER, 6.0 * R * H, launch_f32_to_bf16(w.dtm32, w.dtm, (int64_t)R * H, c->st));
     } else {
@@ -759,6 +779,10 @@ int mslt_create(const mslt_arch* arch, void* dev_params, size_t param_bytes, voi
   c->pending_update = false;
   memset(c->prof, 0, sizeof(c->prof));
   c->Vp = (int)pad_to(arch->vocab, 8);
+  int dev = 0;
+  c->num_sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, dev);
   build_tensor_table(*arch, c->tensors, c->n_elems);
   for (size_t i = 0; i < c->tensors.size(); i++) c->by_name[c->tensors[i].name] = (int)i;
   plan_workspace(*arch, c->tensors, (char*)dev_workspace, c->ws);
