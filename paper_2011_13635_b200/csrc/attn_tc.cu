@@ -38,6 +38,10 @@ struct AttnParams {
   int S, heads, items;
   float scale;
   const int* seq_lens;
+  const int* cu;      // packed rows: sequence b holds rows cu[b] .. cu[b] + len - 1 of qkv and C; null = b * S
+  const int* rows;    // packed: {rows in use, the same rounded up}; C's rows between the two are zeroed
+  float* lse;         // long rows: log2 of the row's sum of exponentials, [A][lse_ld] by row; or null
+  long long lse_ld;
   bf16* P;            // [B, A, S, S] or null
   long long p_bo, p_bi;
   bf16* C;            // element (b, i, h, e) at C + b * c_bo + h * c_bi + i * c_ld + e
@@ -72,6 +76,16 @@ inline int row_fast(const void* ptr, long long ld_elems) {
   return (((uintptr_t)ptr & 31) == 0 && (ld_elems * 2) % 32 == 0) ? 1 : 0;
 }
 
+// Packed batches: the rows between the last sequence and the next tile boundary belong to nobody.
+// They are zeroed, because later products read whole tiles.  Called by the threads of warps 2..9.
+__device__ __forceinline__ void zero_tail_rows(bf16* base, long long ld, long long width, const int* rows) {
+  const int r0 = rows[0], n = rows[1] - r0;
+  const long long vecs = width / 8;
+  const long long step = (long long)gridDim.x * (NUM_EPI_WARPS * 32);
+  for (long long i = (long long)blockIdx.x * (NUM_EPI_WARPS * 32) + threadIdx.x - 64; i < n * vecs; i += step)
+    *reinterpret_cast<uint4*>(base + (r0 + i / vecs) * ld + (i % vecs) * 8) = make_uint4(0, 0, 0, 0);
+}
+
 // Four 32-column reads of a row in flight together, one wait for all.
 __device__ __forceinline__ void tc_ld128(uint32_t taddr, float2 (&v)[4][16]) {
   uint32_t r0[32], r1[32], r2[32], r3[32];
@@ -98,6 +112,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+template <bool kPacked>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -155,16 +170,17 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const uint32_t fb = smem_u32(&full_bar[s]);
       mbar_expect_tx(fb, AT_STAGE_BYTES);
       const uint32_t sq = smem_u32(smem + (size_t)s * AT_STAGE_BYTES);
+      const int row0 = kPacked ? p.cu[zo] : 0, zseq = kPacked ? 0 : zo;
       int c[4];
-      c[0] = 0; c[p.q_perm[0]] = 0; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zo;
+      c[0] = 0; c[p.q_perm[0]] = row0; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zseq;
       tma_load_4d(sq, &tmQ, fb, c[0], c[1], c[2], c[3]);
-      c[0] = 0; c[p.k_perm[0]] = 0; c[p.k_perm[1]] = zi; c[p.k_perm[2]] = zo;
+      c[0] = 0; c[p.k_perm[0]] = row0; c[p.k_perm[1]] = zi; c[p.k_perm[2]] = zseq;
       tma_load_4d(sq + AT_TILE_BYTES, &tmK, fb, c[0], c[1], c[2], c[3]);
       // V is read with the head dimension contiguous: two boxes of 64 keys
-      c[0] = 0; c[p.v_perm[1]] = zi; c[p.v_perm[2]] = zo;
-      c[p.v_perm[0]] = 0;
+      c[0] = 0; c[p.v_perm[1]] = zi; c[p.v_perm[2]] = zseq;
+      c[p.v_perm[0]] = row0;
       tma_load_4d(sq + 2 * AT_TILE_BYTES, &tmV, fb, c[0], c[1], c[2], c[3]);
-      c[p.v_perm[0]] = 64;
+      c[p.v_perm[0]] = row0 + 64;
       tma_load_4d(sq + 2 * AT_TILE_BYTES + AT_TILE_BYTES / 2, &tmV, fb, c[0], c[1], c[2], c[3]);
       issued = i + 1;
     }
@@ -317,7 +333,15 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&pready_bar[g]));
+      const int rlim = kPacked ? len : p.S;  // rows of the item that exist
       if (p.P != nullptr) {
+        // the backward pass reads whole S x S blocks: rows that do not exist are stored as zeros
+        if (kPacked && r >= rlim) {
+#pragma unroll
+          for (int c = 0; c < 4; c++)
+#pragma unroll
+            for (int j = 0; j < 16; j++) v[c][j] = make_float2(0.f, 0.f);
+        }
         bf16* pg = p.P + zo * p.p_bo + zi * p.p_bi;
         if (p.fast_p) {  // S a multiple of 32: whole 32-column pieces only
           if (r < p.S) {
@@ -338,17 +362,18 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_ld32(orow, v[0]);
       tc_ld32(orow + 32, v[1]);
       tc_fence_before();
-      bf16* cg = p.C + zo * p.c_bo + zi * p.c_bi;
+      bf16* cg = p.C + (kPacked ? p.cu[zo] * p.c_ld : zo * p.c_bo) + zi * p.c_bi;
       if (p.fast_c) {
-        if (r < p.S) {
+        if (r < rlim) {
           store_row32_bf16(cg + (long long)r * p.c_ld, v[0]);
           store_row32_bf16(cg + (long long)r * p.c_ld + 32, v[1]);
         }
       } else {
-        stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, p.S, 64, p.vec_ok_c);
-        stage_store_bf16(stg, lane, v[1], cg, p.c_ld, q * 32, 32, p.S, 64, p.vec_ok_c);
+        stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, rlim, 64, p.vec_ok_c);
+        stage_store_bf16(stg, lane, v[1], cg, p.c_ld, q * 32, 32, rlim, 64, p.vec_ok_c);
       }
     }
+    if (kPacked) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
   }
 
   tc_fence_before();
@@ -382,6 +407,7 @@ constexpr int AL_P_BYTES = 2 * AT_TILE_BYTES;    // P_j as an MMA operand: 32 KB
 constexpr int AL_BARS_PER_GROUP = 4 + 2 * AL_RING + 6;
 constexpr long long AL_GROUP_SKEW_CYCLES = 2000;
 
+template <bool kPacked>
 __global__ void __launch_bounds__(AL_THREADS, 1)
 attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -463,8 +489,9 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const int nkb = (len + 127) >> 7;
       if (!mbar_wait(qempty, (ig & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
       ig++;
+      const int row0 = kPacked ? p.cu[zo] : 0, zseq = kPacked ? 0 : zo;
       int c[4];
-      c[0] = 0; c[p.q_perm[0]] = qt * 128; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zo;
+      c[0] = 0; c[p.q_perm[0]] = row0 + qt * 128; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zseq;
       mbar_expect_tx(qfull, AT_TILE_BYTES);
       tma_load_4d(smem_u32(my_q), &tmQ, qfull, c[0], c[1], c[2], c[3]);
       for (int idx = 0; idx < 3 * nkb; idx++, tt++) {
@@ -484,7 +511,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         mbar_expect_tx(fb, AT_TILE_BYTES);
         const int* perm = is_v ? p.v_perm : p.k_perm;
         c[0] = 0; c[1] = 0; c[2] = 0; c[3] = 0;
-        c[perm[0]] = j * 128; c[perm[1]] = zi; c[perm[2]] = zo;
+        c[perm[0]] = row0 + j * 128; c[perm[1]] = zi; c[perm[2]] = zseq;
         tma_load_4d(smem_u32(my_ring + (size_t)slot * AT_TILE_BYTES), is_v ? &tmV : &tmK, fb, c[0], c[1], c[2], c[3]);
       }
     }
@@ -587,9 +614,12 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const int zo = zh / p.heads, zi = zh - zo * p.heads;
       const int len = item_len(zo);
       float2 v[4][16];
-      bf16* cg = p.C + zo * p.c_bo + zi * p.c_bi + (long long)qt * 128 * p.c_ld;
+      const int row0 = kPacked ? p.cu[zo] : zo * p.S;
+      const int rlim = kPacked ? len : p.S;  // rows of the sequence that exist
+      bf16* cg = p.C + (long long)(row0 + qt * 128) * p.c_ld + zi * p.c_bi;
       bf16* pg = want_p ? p.P + zo * p.p_bo + zi * p.p_bi + (long long)qt * 128 * p.S : nullptr;
       if (qt * 128 >= len) {
+        if (kPacked) continue;
         // a query tile in the padding: zero context rows (finite, so that masked reads stay harmless)
 #pragma unroll
         for (int e = 0; e < 16; e++) v[0][e] = make_float2(0.f, 0.f);
@@ -724,6 +754,8 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(oempty);
+      if (p.lse && qt * 128 + r < rlim)
+        p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = mr * sl2 + log2f(want_p ? l : ls.x + ls.y);
       if (!want_p) {
         const float2 il = splat2(1.0f / (ls.x + ls.y));
 #pragma unroll
@@ -733,15 +765,16 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         }
       }
       if (p.fast_c) {
-        if (qt * 128 + r < p.S) {
+        if (qt * 128 + r < rlim) {
           store_row32_bf16(cg + (long long)r * p.c_ld, v[0]);
           store_row32_bf16(cg + (long long)r * p.c_ld + 32, v[1]);
         }
       } else {
-        stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, p.S - qt * 128, 64, p.vec_ok_c);
-        stage_store_bf16(stg, lane, v[1], cg, p.c_ld, q * 32, 32, p.S - qt * 128, 64, p.vec_ok_c);
+        stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, rlim - qt * 128, 64, p.vec_ok_c);
+        stage_store_bf16(stg, lane, v[1], cg, p.c_ld, q * 32, 32, rlim - qt * 128, 64, p.vec_ok_c);
       }
     }
+    if (kPacked) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
   }
 
   tc_fence_before();
@@ -769,6 +802,9 @@ constexpr uint32_t AB_GROUP_COLS = 192;
 struct AttnBwdParams {
   int S, heads, items;
   float scale;
+  const int* seq_lens;  // with cu / rows: packed rows, as in the forward kernels
+  const int* cu;
+  const int* rows;
   bf16* dQKV;         // element (b, i, which, h, e) at dQKV + b * g_bo + i * g_ld + which * H + h * 64 + e
   long long g_ld, g_bo, H;
   int vec_ok, fast;
@@ -835,14 +871,15 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const uint32_t fb = smem_u32(&full_bar[s]);
       mbar_expect_tx(fb, AB_STAGE_BYTES);
       const uint32_t base = smem_u32(smem + (size_t)s * AB_STAGE_BYTES);
+      const int row0 = p.cu ? p.cu[zo] : 0, zseq = p.cu ? 0 : zo;
       int c[4];
-      c[0] = 0; c[p.q_perm[0]] = 0; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zo;
+      c[0] = 0; c[p.q_perm[0]] = row0; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zseq;
       tma_load_4d(base, &tmQ, fb, c[0], c[1], c[2], c[3]);
-      c[0] = 0; c[p.k_perm[0]] = 0; c[p.k_perm[1]] = zi; c[p.k_perm[2]] = zo;
+      c[0] = 0; c[p.k_perm[0]] = row0; c[p.k_perm[1]] = zi; c[p.k_perm[2]] = zseq;
       tma_load_4d(base + AT_TILE_BYTES, &tmK, fb, c[0], c[1], c[2], c[3]);
-      c[0] = 0; c[p.v_perm[0]] = 0; c[p.v_perm[1]] = zi; c[p.v_perm[2]] = zo;
+      c[0] = 0; c[p.v_perm[0]] = row0; c[p.v_perm[1]] = zi; c[p.v_perm[2]] = zseq;
       tma_load_4d(base + 2 * AT_TILE_BYTES, &tmV, fb, c[0], c[1], c[2], c[3]);
-      c[0] = 0; c[p.c_perm[0]] = 0; c[p.c_perm[1]] = zi; c[p.c_perm[2]] = zo;
+      c[0] = 0; c[p.c_perm[0]] = row0; c[p.c_perm[1]] = zi; c[p.c_perm[2]] = zseq;
       tma_load_4d(base + 3 * AT_TILE_BYTES, &tmC, fb, c[0], c[1], c[2], c[3]);
       // P: two tiles of 64 keys, each 128 query rows of 128 bytes
       c[p.p_perm[0]] = 0; c[p.p_perm[1]] = zi; c[p.p_perm[2]] = zo;
@@ -992,18 +1029,19 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&dsready_bar[g]));
-      bf16* gq = p.dQKV + zo * p.g_bo + zi * 64;
+      const int rlim = p.cu ? min(max(p.seq_lens[zo], 1), p.S) : p.S;  // rows of the item that exist
+      bf16* gq = p.dQKV + (p.cu ? p.cu[zo] * p.g_ld : zo * p.g_bo) + zi * 64;
       // dV (complete since dP was): key r, 64 columns
       tc_ld32(trow + 128, v[0]);
       tc_ld32(trow + 160, v[1]);
       if (p.fast) {
-        if (r < p.S) {
+        if (r < rlim) {
           store_row32_bf16(gq + 2 * p.H + (long long)r * p.g_ld, v[0]);
           store_row32_bf16(gq + 2 * p.H + (long long)r * p.g_ld + 32, v[1]);
         }
       } else {
-        stage_store_bf16(stg, lane, v[0], gq + 2 * p.H, p.g_ld, q * 32, 0, p.S, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[1], gq + 2 * p.H, p.g_ld, q * 32, 32, p.S, 64, p.vec_ok);
+        stage_store_bf16(stg, lane, v[0], gq + 2 * p.H, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
+        stage_store_bf16(stg, lane, v[1], gq + 2 * p.H, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
       }
       if (!mbar_wait(smem_u32(&gfull_bar[g]), use & 1, abort_flag, p.status)) { ok = false; break; }
       tc_fence_after();
@@ -1013,7 +1051,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[g]));
       if (p.fast) {
-        if (r < p.S) {
+        if (r < rlim) {
           bf16* row = gq + (long long)r * p.g_ld;
           store_row32_bf16(row, v[0]);
           store_row32_bf16(row + 32, v[1]);
@@ -1021,12 +1059,13 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           store_row32_bf16(row + p.H + 32, v[3]);
         }
       } else {
-        stage_store_bf16(stg, lane, v[0], gq, p.g_ld, q * 32, 0, p.S, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[1], gq, p.g_ld, q * 32, 32, p.S, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[2], gq + p.H, p.g_ld, q * 32, 0, p.S, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[3], gq + p.H, p.g_ld, q * 32, 32, p.S, 64, p.vec_ok);
+        stage_store_bf16(stg, lane, v[0], gq, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
+        stage_store_bf16(stg, lane, v[1], gq, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
+        stage_store_bf16(stg, lane, v[2], gq + p.H, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
+        stage_store_bf16(stg, lane, v[3], gq + p.H, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
       }
     }
+    if (p.cu) zero_tail_rows(p.dQKV, p.g_ld, p.g_ld, p.rows);
   }
 
   tc_fence_before();
@@ -1037,6 +1076,347 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(AT_TMEM_COLS)
                  : "memory");
   }
+}
+
+// ---- backward for rows of 129..512 keys -----------------------------------------------------------
+// The probabilities are formed again from the scores and the forward's row sums (lse), so they never
+// reach memory: with P, dP and dS as [S, S] matrices in HBM the backward of a layer of 16 x 16 heads x
+// 512 keys took 184 us in four batched products and a softmax pass.
+//   P = 2^(scale log2e S - lse),  dS = P o (dP - delta) scale,  delta = rowsum(dC o C)
+// Two kernels of the same form.  kQ = false: an item is (sequence, head, tile of 128 keys), the loop
+// runs over query tiles and accumulates dV += P^T dC and dK += dS^T Q.  kQ = true: an item is a tile of
+// 128 queries, the loop runs over key tiles and accumulates dQ += dS K.  The second forms S and dP once
+// more (2 of 7 products) and in return needs no sums across CTAs: same bits on every run.
+//   warp 0: TMA producer (the item's two fixed tiles, a ring of three pairs of loop tiles)
+//   warp 1: one thread issues S and dP of a pair, then the accumulating products of the pair before
+//   warps 2-9: two warps per TMEM lane quarter, 64 columns each; a thread owns half a query row.
+// Tensor memory: S 128 columns, dP 128, accumulators 2 x 64.  Bound by the serial chain of a pair
+// (products, tensor-memory reads, exponentials, P and dS to shared memory): the products of the next
+// pair run while this one is worked on.
+constexpr int BL_RING = 3;
+constexpr uint32_t BL_ACC_COL = 256;
+
+struct AttnBwdLongParams {
+  int S, heads, items;
+  float scale;
+  const int* seq_lens;
+  const int* cu;
+  const int* rows;
+  const float* lse;
+  const float* delta;
+  long long ld;       // rows of one head in lse and delta
+  bf16* dQKV;
+  long long g_ld, H;
+  int q_perm[3], k_perm[3], v_perm[3], c_perm[3];
+  long long wait_limit;
+  int starve;
+  int* status;
+  uint32_t idesc_s, idesc_kv, idesc_q;
+};
+
+template <bool kQ>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmC,
+                     const AttnBwdLongParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  // fixed tiles: K, V of the item (kQ: Q, dC); ring stage: Q, dC of a query tile (kQ: K, V of a key tile)
+  uint8_t* ring_smem = smem + 2 * AT_TILE_BYTES;
+  uint8_t* p_smem = ring_smem + BL_RING * 2 * AT_TILE_BYTES;   // P, not used by kQ
+  uint8_t* ds_smem = p_smem + (kQ ? 0 : 2 * AT_TILE_BYTES);    // dS
+  uint64_t* bars = (uint64_t*)(ds_smem + 2 * AT_TILE_BYTES);
+  uint64_t* rfull_bar = bars;                    // [BL_RING]
+  uint64_t* rempty_bar = bars + BL_RING;         // [BL_RING]
+  uint64_t* misc = bars + 2 * BL_RING;
+  const uint32_t ffull = smem_u32(&misc[0]), fempty = smem_u32(&misc[1]);    // fixed tiles
+  const uint32_t sfull = smem_u32(&misc[2]), sempty = smem_u32(&misc[3]);    // S and dP of a pair
+  const uint32_t pready = smem_u32(&misc[4]), pfree = smem_u32(&misc[5]);    // P and dS in shared memory
+  const uint32_t accfull = smem_u32(&misc[6]), accempty = smem_u32(&misc[7]);
+  uint32_t* tmem_slot = (uint32_t*)(misc + 8);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < BL_RING; s++) {
+      mbar_init(smem_u32(&rfull_bar[s]), 1);
+      mbar_init(smem_u32(&rempty_bar[s]), 1);
+    }
+    mbar_init(ffull, 1); mbar_init(fempty, 1);
+    mbar_init(sfull, 1); mbar_init(sempty, NUM_EPI_WARPS);
+    mbar_init(pready, NUM_EPI_WARPS); mbar_init(pfree, 1);
+    mbar_init(accfull, 1); mbar_init(accempty, NUM_EPI_WARPS);
+    *abort_flag = 0;
+    *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(AT_TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
+  const int nt = (p.S + 127) >> 7, nzh = p.items / nt;
+  auto item_len = [&](int zo) {
+    int len = p.cu ? p.seq_lens[zo] : p.S;
+    return min(max(len, 1), p.S);
+  };
+  auto row_base = [&](int zo) { return p.cu ? p.cu[zo] : zo * p.S; };
+
+  if (warp == 0 && lane == 0 && !p.starve) {
+    // ------------------------------- TMA producer -------------------------------
+    bool ok = true;
+    uint32_t rt = 0, ni = 0;
+    auto load = [&](const CUtensorMap* map, const int (&perm)[3], uint32_t dst, uint32_t bar, int row, int zi) {
+      int c[4] = {0, 0, 0, 0};
+      c[perm[0]] = row; c[perm[1]] = zi;
+      tma_load_4d(dst, map, bar, c[0], c[1], c[2], c[3]);
+    };
+    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
+      const int tile = w / nzh, zh = w - tile * nzh;  // tile slowest: those that may be padding come last
+      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+      const int len = item_len(zo), row0 = row_base(zo);
+      if (tile * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      if (!mbar_wait(fempty, (ni & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+      ni++;
+      mbar_expect_tx(ffull, 2 * AT_TILE_BYTES);
+      const uint32_t f0 = smem_u32(smem);
+      load(kQ ? &tmQ : &tmK, kQ ? p.q_perm : p.k_perm, f0, ffull, row0 + tile * 128, zi);
+      load(kQ ? &tmC : &tmV, kQ ? p.c_perm : p.v_perm, f0 + AT_TILE_BYTES, ffull, row0 + tile * 128, zi);
+      for (int t = 0; t < n; t++, rt++) {
+        const uint32_t slot = rt % BL_RING, round = rt / BL_RING;
+        if (!mbar_wait(smem_u32(&rempty_bar[slot]), (round & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        const uint32_t fb = smem_u32(&rfull_bar[slot]);
+        mbar_expect_tx(fb, 2 * AT_TILE_BYTES);
+        const uint32_t r0 = smem_u32(ring_smem + (size_t)slot * 2 * AT_TILE_BYTES);
+        load(kQ ? &tmK : &tmQ, kQ ? p.k_perm : p.q_perm, r0, fb, row0 + t * 128, zi);
+        load(kQ ? &tmV : &tmC, kQ ? p.v_perm : p.c_perm, r0 + AT_TILE_BYTES, fb, row0 + t * 128, zi);
+      }
+    }
+    if (!ok || *abort_flag) {  // give the copies in flight time to land before the CTA leaves
+      const long long t0 = now_cycles();
+      while (now_cycles() - t0 < 4000000ll) {}
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ------------------------------- MMA issuer -------------------------------
+    bool ok = true;
+    const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);
+    const uint32_t lbo_k = (uint32_t)make_smem_desc(0, 16);               // k-contiguous operand
+    const uint32_t lbo_mn1 = (uint32_t)make_smem_desc(0, 8192);           // rows = k, one 64-wide m/n block
+    const uint32_t lbo_mn2 = (uint32_t)make_smem_desc(0, AT_TILE_BYTES);  // two 64-wide blocks 16 KB apart
+    auto addr16 = [](uint32_t a) { return (a & 0x3FFFFu) >> 4; };
+    constexpr uint32_t KS_K = UMMA_K * 2 / 16, KS_MN = UMMA_K * 128 / 16;
+    constexpr uint32_t KB_MN = 8192 / 16, KB_K = AT_TILE_BYTES / 16;
+    auto mma_k128 = [&](uint32_t d_tmem, uint32_t a_lo, uint32_t a_kb, uint32_t a_ks, uint32_t b_lo, uint32_t idesc,
+                        bool first) {  // contraction over 128 = 2 x 4 x 16, B with rows = k
+#pragma unroll
+      for (int kb = 0; kb < 2; kb++)
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          const uint64_t ad = ((uint64_t)hi << 32) | (a_lo + kb * a_kb + k * a_ks);
+          const uint64_t bd = ((uint64_t)hi << 32) | (b_lo + kb * KB_MN + k * KS_MN);
+          tc_mma(d_tmem, ad, bd, idesc, (first && kb == 0 && k == 0) ? 0u : 1u);
+        }
+    };
+    auto mma_k64 = [&](uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr) {  // both operands k-contiguous
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const uint64_t ad = ((uint64_t)hi << 32) | ((lbo_k | addr16(a_addr)) + k * KS_K);
+        const uint64_t bd = ((uint64_t)hi << 32) | ((lbo_k | addr16(b_addr)) + k * KS_K);
+        tc_mma(d_tmem, ad, bd, p.idesc_s, k > 0 ? 1u : 0u);
+      }
+    };
+    const uint32_t f0 = smem_u32(smem), pa = addr16(smem_u32(p_smem)), da = addr16(smem_u32(ds_smem));
+    uint32_t rt = 0, np = 0, ni = 0;  // score pairs (= ring tiles), accumulated pairs, items
+    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
+      const int tile = w / nzh, zh = w - tile * nzh;
+      const int len = item_len(zh / p.heads);
+      if (tile * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      if (!mbar_wait(ffull, ni & 1, abort_flag, p.status)) { ok = false; break; }
+      auto accumulate = [&](int t) -> bool {  // the accumulating products of pair t of this item
+        if (!mbar_wait(pready, np & 1, abort_flag, p.status)) return false;
+        if (t == 0 && !mbar_wait(accempty, (ni & 1) ^ 1, abort_flag, p.status)) return false;
+        tc_fence_after();
+        const uint32_t slot = np % BL_RING;
+        const uint32_t r0 = smem_u32(ring_smem + (size_t)slot * 2 * AT_TILE_BYTES);
+        const uint32_t acc = tmem_base + BL_ACC_COL;
+        if (kQ) {
+          mma_k128(acc, lbo_k | da, KB_K, KS_K, lbo_mn1 | addr16(r0), p.idesc_q, t == 0);  // dQ += dS K
+        } else {
+          mma_k128(acc, lbo_mn2 | pa, KB_MN, KS_MN, lbo_mn1 | addr16(r0 + AT_TILE_BYTES), p.idesc_kv, t == 0);  // dV += P^T dC
+          mma_k128(acc + 64, lbo_mn2 | da, KB_MN, KS_MN, lbo_mn1 | addr16(r0), p.idesc_kv, t == 0);             // dK += dS^T Q
+        }
+        tc_commit(pfree);
+        tc_commit(smem_u32(&rempty_bar[slot]));
+        np++;
+        return true;
+      };
+      for (int t = 0; t < n && ok; t++, rt++) {
+        const uint32_t slot = rt % BL_RING, round = rt / BL_RING;
+        if (!mbar_wait(smem_u32(&rfull_bar[slot]), round & 1, abort_flag, p.status)) { ok = false; break; }
+        if (!mbar_wait(sempty, (rt & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t r0 = smem_u32(ring_smem + (size_t)slot * 2 * AT_TILE_BYTES);
+        mma_k64(tmem_base, kQ ? f0 : r0, kQ ? r0 : f0);                                   // S = Q K^T
+        mma_k64(tmem_base + 128, (kQ ? f0 : r0) + AT_TILE_BYTES, (kQ ? r0 : f0) + AT_TILE_BYTES);  // dP = dC V^T
+        tc_commit(sfull);
+        if (t > 0) ok = accumulate(t - 1);
+      }
+      if (ok) ok = accumulate(n - 1);
+      if (ok) {
+        tc_commit(accfull);
+        tc_commit(fempty);
+      }
+      ni++;
+    }
+    if (!ok || *abort_flag) {
+      // make sure no MMA is still writing tensor memory before it is freed
+      tc_commit(sfull);
+      const long long t0 = now_cycles();
+      while (now_cycles() - t0 < 2000000ll) {}
+    }
+  } else if (warp >= 2) {
+    // ------------------------------- softmax-backward warps -------------------------------
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int r = q * 32 + lane;
+    const float sl2 = p.scale * 1.4426950408889634f;
+    const float2 k2 = splat2(sl2), sc2 = splat2(p.scale);
+    const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+    bool ok = true;
+    uint32_t sp = 0, ni = 0;
+    uint8_t* prow = p_smem + half * AT_TILE_BYTES + r * 128;
+    uint8_t* drow = ds_smem + half * AT_TILE_BYTES + r * 128;
+    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
+      const int tile = w / nzh, zh = w - tile * nzh;
+      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+      const int len = item_len(zo);
+      if (tile * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      const long long row0 = row_base(zo);
+      for (int t = 0; t < n && ok; t++) {
+        const int qrow = (kQ ? tile : t) * 128 + r, key0 = (kQ ? t : tile) * 128 + half * 64;
+        // a row beyond the sequence gets probability 2^-inf = 0 everywhere
+        float nl = -INFINITY, nd = 0.f;
+        if (qrow < len) {
+          nl = -p.lse[zi * p.ld + row0 + qrow];
+          nd = -p.delta[zi * p.ld + row0 + qrow];
+        }
+        const float2 nl2 = splat2(nl), nd2 = splat2(nd);
+        if (!mbar_wait(sfull, sp & 1, abort_flag, p.status)) { ok = false; break; }
+        tc_fence_after();
+        uint32_t s0[32], s1[32], d0[32], d1[32];
+        tc_ld32_issue(trow + half * 64, s0);
+        tc_ld32_issue(trow + half * 64 + 32, s1);
+        tc_ld32_issue(trow + 128 + half * 64, d0);
+        tc_ld32_issue(trow + 128 + half * 64 + 32, d1);
+        tc_ld32_wait(s0);
+        tc_ld32_wait(s1);
+        tc_ld32_wait(d0);
+        tc_ld32_wait(d1);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sempty);
+        // P and dS as bf16 pairs, kept in the registers of S and dP
+        auto work = [&](uint32_t (&s)[32], uint32_t (&d)[32], int k0) {
+          const bool edge = k0 + 32 > len;
+#pragma unroll
+          for (int j = 0; j < 16; j++) {
+            const float2 a = __ffma2_rn(make_float2(__uint_as_float(s[2 * j]), __uint_as_float(s[2 * j + 1])), k2, nl2);
+            float2 pr = make_float2(fast_exp2(a.x), fast_exp2(a.y));
+            if (edge) {
+              if (k0 + 2 * j >= len) pr.x = 0.f;
+              if (k0 + 2 * j + 1 >= len) pr.y = 0.f;
+            }
+            const float2 dp = __fadd2_rn(make_float2(__uint_as_float(d[2 * j]), __uint_as_float(d[2 * j + 1])), nd2);
+            const __nv_bfloat162 ds = __float22bfloat162_rn(__fmul2_rn(__fmul2_rn(dp, sc2), pr));
+            const __nv_bfloat162 pb = __float22bfloat162_rn(pr);
+            s[j] = *reinterpret_cast<const uint32_t*>(&pb);
+            d[j] = *reinterpret_cast<const uint32_t*>(&ds);
+          }
+        };
+        work(s0, d0, key0);
+        work(s1, d1, key0 + 32);
+        // the accumulating products of the pair before have read P and dS
+        if (!mbar_wait(pfree, (sp & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        sp++;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          const int u0 = (c ^ (r & 7)) << 4, u1 = ((4 + c) ^ (r & 7)) << 4;
+          if (!kQ) {
+            *reinterpret_cast<uint4*>(prow + u0) = make_uint4(s0[4 * c], s0[4 * c + 1], s0[4 * c + 2], s0[4 * c + 3]);
+            *reinterpret_cast<uint4*>(prow + u1) = make_uint4(s1[4 * c], s1[4 * c + 1], s1[4 * c + 2], s1[4 * c + 3]);
+          }
+          *reinterpret_cast<uint4*>(drow + u0) = make_uint4(d0[4 * c], d0[4 * c + 1], d0[4 * c + 2], d0[4 * c + 3]);
+          *reinterpret_cast<uint4*>(drow + u1) = make_uint4(d1[4 * c], d1[4 * c + 1], d1[4 * c + 2], d1[4 * c + 3]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(pready);
+      }
+      if (!ok) break;
+      // the item's gradients: row r of its tile
+      if (!mbar_wait(accfull, ni & 1, abort_flag, p.status)) { ok = false; break; }
+      ni++;
+      tc_fence_after();
+      float2 v0[16], v1[16];
+      const uint32_t acol = BL_ACC_COL + (kQ ? half * 32 : half * 64);
+      tc_ld32(trow + acol, v0);
+      if (!kQ) tc_ld32(trow + acol + 32, v1);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(accempty);
+      if (tile * 128 + r < len) {
+        bf16* g = p.dQKV + (row0 + tile * 128 + r) * p.g_ld + zi * 64;
+        if (kQ) {
+          store_row32_bf16(g + half * 32, v0);
+        } else {
+          g += half ? p.H : 2 * p.H;  // the first accumulator is dV, the second dK
+          store_row32_bf16(g, v0);
+          store_row32_bf16(g + 32, v1);
+        }
+      }
+    }
+    if (kQ && p.cu) zero_tail_rows(p.dQKV, p.g_ld, p.g_ld, p.rows);
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(AT_TMEM_COLS)
+                 : "memory");
+  }
+}
+
+// delta[h][row] = sum over the head's 64 columns of dC o C.  Eight lanes share a head's row.
+__global__ void __launch_bounds__(256)
+attn_delta_kernel(const bf16* __restrict__ c, const bf16* __restrict__ dc, float* __restrict__ delta, int rows, int heads,
+                  long long ld, const int* __restrict__ rows_dev) {
+  pdl_begin();
+  if (rows_dev) rows = min(rows, rows_dev[0]);
+  const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  const long long unit = i >> 3;  // (row, head)
+  const long long row = unit / heads;
+  const int h = (int)(unit - row * heads);
+  float s = 0.f;
+  if (row < rows) {
+    float a[8], b[8];
+    VecT<bf16>::load(c + unit * 64 + (i & 7) * 8, a);
+    VecT<bf16>::load(dc + unit * 64 + (i & 7) * 8, b);
+#pragma unroll
+    for (int e = 0; e < 8; e++) s = fmaf(a[e], b[e], s);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((i & 7) == 0 && row < rows) delta[h * ld + row] = s;
 }
 
 }  // namespace
@@ -1050,7 +1430,8 @@ namespace {
 // per-device facts and one-time kernel attributes (a process may drive several GPUs)
 struct AttnDevice {
   int num_sms = 0, smem_optin = 0;
-  bool attr_fwd = false, attr_long = false, attr_bwd = false;
+  bool attr_fwd[2] = {false, false}, attr_long[2] = {false, false};
+  bool attr_bwd = false, attr_bwd_kv = false, attr_bwd_q = false;
 };
 constexpr int kMaxDevices = 64;
 AttnDevice g_adev[kMaxDevices];
@@ -1083,7 +1464,7 @@ int attn_opt_in(K kernel, bool* done, int smem_optin, char* err) {
 }  // namespace
 
 int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens, int B, int S, int A, int d,
-                    float scale, int* status, cudaStream_t st, char* err) {
+                    float scale, int* status, cudaStream_t st, char* err, const int* cu, const int* rows, float* lse) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_attn_starve.exchange(0) != 0;
   AttnDevice* adev = attn_device(err);
@@ -1098,6 +1479,12 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   AttnParams p;
   memset(&p, 0, sizeof(p));
   p.S = S; p.heads = A; p.items = B * A * (long_rows ? (S + 127) / 128 : 1); p.scale = scale; p.seq_lens = seq_lens;
+  p.cu = cu; p.rows = rows;
+  p.lse = lse; p.lse_ld = (long long)B * S;
+  if ((cu && (!seq_lens || !rows)) || (cu && long_rows && probs) || (lse && !long_rows)) {
+    snprintf(err, 256, "attention: packed rows need lengths and row counts; long packed rows store no probabilities");
+    return MSLT_ERR_ARG;
+  }
   p.P = (bf16*)probs; p.p_bo = (long long)A * S * S; p.p_bi = (long long)S * S;
   p.C = (bf16*)ctx; p.c_ld = H; p.c_bo = (long long)S * H; p.c_bi = d;
   p.vec_ok_p = (S % 8 == 0 && ((uintptr_t)probs & 15) == 0) ? 1 : 0;
@@ -1114,25 +1501,29 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   p.idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
   p.idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
   const bf16* base = (const bf16*)qkv;
+  // packed rows: one long run of rows, a sequence being an offset into it
+  const long long mrows = cu ? (long long)B * S : S, mbo = cu ? 0 : (long long)S * 3 * H;
+  const int mseqs = cu ? 1 : B;
   MapVal mq, mk, mv;
-  int rc = get_map(base, S, d, 3 * H, 1, (long long)S * 3 * H, d, A, B, BM, &mq, err);
+  int rc = get_map(base, mrows, d, 3 * H, 1, mbo, d, A, mseqs, BM, &mq, err);
   if (rc) return rc;
-  rc = get_map(base + H, S, d, 3 * H, 1, (long long)S * 3 * H, d, A, B, BM, &mk, err);
+  rc = get_map(base + H, mrows, d, 3 * H, 1, mbo, d, A, mseqs, BM, &mk, err);
   if (rc) return rc;
   // V: the short kernel reads it as two boxes of 64 keys with the head width contiguous; the long
   // one as one box of 128 key rows, which are the same bytes in shared memory
-  if (long_rows) rc = get_map(base + 2 * H, S, d, 3 * H, 1, (long long)S * 3 * H, d, A, B, BM, &mv, err);
-  else rc = get_map(base + 2 * H, d, S, 1, 3 * H, (long long)S * 3 * H, d, A, B, 64, &mv, err);
+  if (long_rows) rc = get_map(base + 2 * H, mrows, d, 3 * H, 1, mbo, d, A, mseqs, BM, &mv, err);
+  else rc = get_map(base + 2 * H, d, mrows, 1, 3 * H, mbo, d, A, mseqs, 64, &mv, err);
   if (rc) return rc;
   for (int i = 0; i < 3; i++) { p.q_perm[i] = mq.perm[i]; p.k_perm[i] = mk.perm[i]; p.v_perm[i] = mv.perm[i]; }
   if (long_rows) {
     const size_t smem_long = 2 * (size_t)AT_TILE_BYTES + 2 * (size_t)AL_RING * AT_TILE_BYTES + 2 * (size_t)AL_P_BYTES +
                              NUM_EPI_WARPS * AT_STAGING + 1024 + 512;
     if ((int)smem_long > smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
-    rc = attn_opt_in(attn_fwd_long_kernel, &adev->attr_long, smem_optin, err);
+    const auto kernel = cu ? attn_fwd_long_kernel<true> : attn_fwd_long_kernel<false>;
+    rc = attn_opt_in(kernel, &adev->attr_long[cu != nullptr], smem_optin, err);
     if (rc) return rc;
     const int grid_long = p.items < num_sms ? p.items : num_sms;
-    launch_pdl(attn_fwd_long_kernel, grid_long, AL_THREADS, smem_long, st, mq.map, mk.map, mv.map, p);
+    launch_pdl(kernel, grid_long, AL_THREADS, smem_long, st, mq.map, mk.map, mv.map, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
     g_attn_launches++;
@@ -1140,10 +1531,11 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   }
   const size_t smem_bytes = (size_t)AT_STAGES * AT_STAGE_BYTES + NUM_EPI_WARPS * AT_STAGING + 1024 + 256;
   if ((int)smem_bytes > smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
-  rc = attn_opt_in(attn_fwd_kernel, &adev->attr_fwd, smem_optin, err);
+  const auto kernel = cu ? attn_fwd_kernel<true> : attn_fwd_kernel<false>;
+  rc = attn_opt_in(kernel, &adev->attr_fwd[cu != nullptr], smem_optin, err);
   if (rc) return rc;
   const int grid = p.items < num_sms ? p.items : num_sms;
-  launch_pdl(attn_fwd_kernel, grid, NUM_THREADS, smem_bytes, st, mq.map, mk.map, mv.map, p);
+  launch_pdl(kernel, grid, NUM_THREADS, smem_bytes, st, mq.map, mk.map, mv.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches++;
@@ -1151,7 +1543,8 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
 }
 
 int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* dqkv, int B, int S, int A, int d,
-                    float scale, int* status, cudaStream_t st, char* err) {
+                    float scale, int* status, cudaStream_t st, char* err, const int* seq_lens, const int* cu,
+                    const int* rows) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_attn_starve.exchange(0) != 0;
   AttnDevice* adev = attn_device(err);
@@ -1181,14 +1574,17 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
   p.idesc_dq = common | (1u << 16) | ((uint32_t)(64 >> 3) << 17);
   p.idesc_dk = common | (1u << 15) | (1u << 16) | ((uint32_t)(64 >> 3) << 17);
   const bf16* base = (const bf16*)qkv;
+  const long long mrows = cu ? (long long)B * S : S;
+  const int mseqs = cu ? 1 : B;
+  p.seq_lens = seq_lens; p.cu = cu; p.rows = rows;
   MapVal mq, mk, mv, mc, mp;
-  int rc = get_map(base, S, d, 3 * H, 1, (long long)S * 3 * H, d, A, B, BM, &mq, err);
+  int rc = get_map(base, mrows, d, 3 * H, 1, cu ? 0 : (long long)S * 3 * H, d, A, mseqs, BM, &mq, err);
   if (rc) return rc;
-  rc = get_map(base + H, S, d, 3 * H, 1, (long long)S * 3 * H, d, A, B, BM, &mk, err);
+  rc = get_map(base + H, mrows, d, 3 * H, 1, cu ? 0 : (long long)S * 3 * H, d, A, mseqs, BM, &mk, err);
   if (rc) return rc;
-  rc = get_map(base + 2 * H, S, d, 3 * H, 1, (long long)S * 3 * H, d, A, B, BM, &mv, err);
+  rc = get_map(base + 2 * H, mrows, d, 3 * H, 1, cu ? 0 : (long long)S * 3 * H, d, A, mseqs, BM, &mv, err);
   if (rc) return rc;
-  rc = get_map(dctx, S, d, H, 1, (long long)S * H, d, A, B, BM, &mc, err);
+  rc = get_map(dctx, mrows, d, H, 1, cu ? 0 : (long long)S * H, d, A, mseqs, BM, &mc, err);
   if (rc) return rc;
   rc = get_map(probs, S, S, S, 1, (long long)A * S * S, (long long)S * S, A, B, BM, &mp, err);
   if (rc) return rc;
@@ -1205,6 +1601,56 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches++;
+  return 0;
+}
+
+int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, const float* lse, float* delta,
+                         void* dqkv, int B, int S, int A, float scale, int* status, cudaStream_t st, char* err,
+                         const int* seq_lens, const int* cu, const int* rows) {
+  const bool starve = g_attn_starve.exchange(0) != 0;
+  AttnDevice* adev = attn_device(err);
+  if (!adev) return MSLT_ERR_CUDA;
+  if (S < 1 || S > 512 || B < 1 || A < 1 || !status || !lse || !delta || (cu && (!seq_lens || !rows))) {
+    snprintf(err, 256, "attention backward: bad arguments");
+    return MSLT_ERR_ARG;
+  }
+  const long long H = (long long)A * 64, T = (long long)B * S;
+  AttnBwdLongParams p;
+  memset(&p, 0, sizeof(p));
+  p.S = S; p.heads = A; p.items = B * A * ((S + 127) / 128); p.scale = scale;
+  p.seq_lens = seq_lens; p.cu = cu; p.rows = rows; p.lse = lse; p.delta = delta; p.ld = T;
+  p.dQKV = (bf16*)dqkv; p.g_ld = 3 * H; p.H = H;
+  p.wait_limit = starve ? 40000000ll : WAIT_LIMIT_CYCLES;
+  p.starve = starve ? 1 : 0;
+  p.status = status;
+  const uint32_t common = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
+  p.idesc_s = common | ((uint32_t)(128 >> 3) << 17);
+  p.idesc_kv = common | (1u << 15) | (1u << 16) | ((uint32_t)(64 >> 3) << 17);
+  p.idesc_q = common | (1u << 16) | ((uint32_t)(64 >> 3) << 17);
+  const bf16* base = (const bf16*)qkv;
+  MapVal mq, mk, mv, mc;
+  int rc = get_map(base, T, 64, 3 * H, 1, 0, 64, A, 1, BM, &mq, err);
+  if (!rc) rc = get_map(base + H, T, 64, 3 * H, 1, 0, 64, A, 1, BM, &mk, err);
+  if (!rc) rc = get_map(base + 2 * H, T, 64, 3 * H, 1, 0, 64, A, 1, BM, &mv, err);
+  if (!rc) rc = get_map(dctx, T, 64, H, 1, 0, 64, A, 1, BM, &mc, err);
+  if (rc) return rc;
+  for (int i = 0; i < 3; i++) {
+    p.q_perm[i] = mq.perm[i]; p.k_perm[i] = mk.perm[i]; p.v_perm[i] = mv.perm[i]; p.c_perm[i] = mc.perm[i];
+  }
+  const size_t smem_kv = (size_t)(2 + 2 * BL_RING + 4) * AT_TILE_BYTES + 1024 + 256;
+  const size_t smem_q = (size_t)(2 + 2 * BL_RING + 2) * AT_TILE_BYTES + 1024 + 256;
+  if ((int)smem_kv > adev->smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
+  rc = attn_opt_in(attn_bwd_long_kernel<false>, &adev->attr_bwd_kv, adev->smem_optin, err);
+  if (!rc) rc = attn_opt_in(attn_bwd_long_kernel<true>, &adev->attr_bwd_q, adev->smem_optin, err);
+  if (rc) return rc;
+  const int grid = p.items < adev->num_sms ? p.items : adev->num_sms;
+  launch_pdl(attn_delta_kernel, (unsigned)((T * A * 8 + 255) / 256), 256, 0, st, (const bf16*)ctx, (const bf16*)dctx,
+             delta, (int)T, A, T, rows);
+  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS, smem_kv, st, mq.map, mk.map, mv.map, mc.map, p);
+  launch_pdl(attn_bwd_long_kernel<true>, grid, NUM_THREADS, smem_q, st, mq.map, mk.map, mv.map, mc.map, p);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
+  g_attn_launches += 3;
   return 0;
 }
 

@@ -11,11 +11,14 @@ namespace mslt {
 // Enqueues the contraction on `st`.  `status` is a device word that a tensor-core kernel ORs an
 // error bit into when one of its bounded waits runs out.  Returns 0, or a negative mslt_status
 // with a message in `err` (at least 256 bytes).
-int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err);
+// rows (dtype 1 only, may be null): device count <= M, or <= K with rows_are_k, of the rows that hold
+// anything; work is cut to it (row results beyond it are not written).
+int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows = nullptr,
+                int rows_are_k = 0);
 
 int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
-int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err);
+int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k);
 
 // Test hook: the next tensor-core launch gets a producer that issues no copies and a wait limit of
 // about 20 ms, so that its first wait runs out and the give-up path is exercised.
@@ -28,13 +31,25 @@ void gemm_tc_set_variant(int variant);
 // qkv is the fused projection [B*S, 3*A*d] (queries, keys, values; head h in columns h*d..);
 // probs ([B, A, S, S], may be null: not written) and ctx ([B*S, A*d]) are outputs.  `status` as for
 // gemm_launch.  Returns 0 or a negative mslt_status with a message in `err`.
+// cu (with rows, both device): the batch is packed, sequence b holds rows cu[b] .. cu[b] + len - 1 of
+// qkv and ctx (allocated for B*S rows); rows = {rows in use, rounded up}: ctx between the two is zeroed.
+// probs then still are [B, A, S, S], with zero rows where there is no query.
+// lse (more than 128 keys): [A, B*S] by row, log2 of the row's sum of exponentials, for the backward.
 int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens, int B, int S, int A, int d,
-                    float scale, int* status, cudaStream_t st, char* err);
+                    float scale, int* status, cudaStream_t st, char* err, const int* cu = nullptr,
+                    const int* rows = nullptr, float* lse = nullptr);
 // Its backward: dqkv ([B*S, 3*A*d], queries | keys | values like qkv) from the saved probabilities
 // and the gradient of the context dctx ([B*S, A*d]); S a multiple of 8.
 //   dV = P^T dC,  dP = dC V^T,  dS = P o (dP - rowsum(dP o P)) * scale,  dQ = dS K,  dK = dS^T Q
 int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* dqkv, int B, int S, int A, int d,
-                    float scale, int* status, cudaStream_t st, char* err);
+                    float scale, int* status, cudaStream_t st, char* err, const int* seq_lens = nullptr,
+                    const int* cu = nullptr, const int* rows = nullptr);
+// The backward for 129 to 512 keys: no stored probabilities, they are formed again from lse.  ctx is the
+// forward's output, delta [A, B*S] scratch (per row and head: sum of dctx o ctx).  Without cu every
+// sequence has S rows.  Three launches.
+int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, const float* lse, float* delta,
+                         void* dqkv, int B, int S, int A, float scale, int* status, cudaStream_t st, char* err,
+                         const int* seq_lens, const int* cu, const int* rows);
 long long attn_launches();
 // Test hook like gemm_tc_starve_next, for the next attention launch (forward or backward).
 void attn_starve_next(int on);

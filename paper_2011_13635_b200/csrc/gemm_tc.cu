@@ -57,6 +57,8 @@ struct TcParams {
   int act;
   bf16* aux;
   const bf16* residual;
+  const int* rows;      // device count that replaces M (or K, rows_are_k) as far as work goes, or null
+  int rows_are_k;
   const int* seq_lens;  // act 3: valid keys per outer batch index, or null
   long long wait_limit; // SM cycles a wait may take before the CTA gives up
   int starve;           // test hook: the producer issues no copies, so the first wait runs out
@@ -317,7 +319,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
 
-  const int tiles_per_z = p.m_tiles * p.n_tiles;
+  // The number of rows that hold anything may be known on the device only (batches with padding are
+  // kept packed): the tile list is then cut to it.  Rows between that count and M stay unwritten.
+  int m_tiles = p.m_tiles, kb_total = p.kb_total, kb_per_split = p.kb_per_split, total_work = p.total_work;
+  if (p.rows != nullptr) {
+    const int rows = *p.rows;
+    if (p.rows_are_k) {
+      kb_total = (rows + KSUB * BK - 1) / (KSUB * BK);
+      kb_per_split = ((rows + 2 * BK - 1) / (2 * BK) + p.splits - 1) / p.splits * (2 / KSUB);
+      total_work = m_tiles * p.n_tiles * p.batch * ((kb_total + kb_per_split - 1) / kb_per_split);
+    } else {
+      m_tiles = (rows + mt_rows - 1) / mt_rows;
+      total_work = m_tiles * p.n_tiles * p.batch * p.splits;
+    }
+  }
+  const int tiles_per_z = m_tiles * p.n_tiles;
   const int per_split = tiles_per_z * p.batch;
 
   if ((warp == 0 || warp == 2 || warp == 3) && lane == 0 && !p.starve) {
@@ -338,15 +354,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t full0 = smem_u32(&full_bar[0]), empty0 = smem_u32(&empty_bar[0]);
     const uint32_t tx_bytes = kPair ? 2 * stage_bytes : stage_bytes;
     const int a_boxes = p.a_mn ? BM / 64 : 1, b_boxes = p.b_mn ? bn_cta / 64 : 1;
-    for (int w = w_first; w < p.total_work && ok; w += w_step) {
+    for (int w = w_first; w < total_work && ok; w += w_step) {
       const int split = w / per_split;
       int r = w - split * per_split;
       const int z = r / tiles_per_z;
       r -= z * tiles_per_z;
       const int mt = r / p.n_tiles, nt = r - mt * p.n_tiles;
       const int zo = z / p.hdiv, zi = z - zo * p.hdiv;
-      const int kb0 = split * p.kb_per_split;
-      const int kb1 = min(p.kb_total, kb0 + p.kb_per_split);
+      const int kb0 = split * kb_per_split;
+      const int kb1 = min(kb_total, kb0 + kb_per_split);
       const int row0 = mt * mt_rows + (int)cta_rank * BM;
       const int col0 = nt * p.bn + (int)cta_rank * bn_cta;
       int ca[4], cb[4];
@@ -430,10 +446,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // of the current block, and its answer is only read afterwards: `ready` for the next ring
     // slot, `acc_free` for the next work item's accumulator.
     uint32_t ready = 0, acc_free = 0;
-    for (int w = w_first; w < p.total_work && ok; w += w_step, tile++) {
+    for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
       const int split = w / per_split;
-      const int kb0 = split * p.kb_per_split;
-      const int kb1 = min(p.kb_total, kb0 + p.kb_per_split);
+      const int kb0 = split * kb_per_split;
+      const int kb1 = min(kb_total, kb0 + kb_per_split);
       const uint32_t acc = tile & 1, use = tile >> 1;
       if (!acc_free && !mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
       acc_free = 0;
@@ -446,7 +462,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         uint32_t s1 = s + 1, ph1 = ph;
         if (s1 == (uint32_t)p.stages) { s1 = 0; ph1 ^= 1; }
         ready = mbar_try_wait(full0 + s1 * 8, ph1) ? 1u : 0u;
-        if (kb == kb1 - 1 && w + w_step < p.total_work) {
+        if (kb == kb1 - 1 && w + w_step < total_work) {
           const uint32_t nt = tile + 1;
           acc_free = mbar_try_wait(smem_u32(&tempty_bar[nt & 1]), ((nt >> 1) & 1) ^ 1) ? 1u : 0u;
         }
@@ -514,8 +530,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         int c = nt_ >= p.n_tiles ? 1 : 0;
         nt_ -= c ? p.n_tiles : 0;
         mt_ += d_mt + c;
-        c = mt_ >= p.m_tiles ? 1 : 0;
-        mt_ -= c ? p.m_tiles : 0;
+        c = mt_ >= m_tiles ? 1 : 0;
+        mt_ -= c ? m_tiles : 0;
         z_ += d_z + c;
         c = z_ >= p.batch ? 1 : 0;
         z_ -= c ? p.batch : 0;
@@ -536,13 +552,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       };
       float bnext[4];
-      if (w_first < p.total_work && !tma_out) {
+      if (w_first < total_work && !tma_out) {
         fetch_bias(nt, bnext);
 #pragma unroll
         for (int i = 0; i < 4; i++) bias_s[i * 32 + lane] = bnext[i];
         __syncwarp();
       }
-      for (int w = w_first; w < p.total_work && ok; w += w_step, tile++) {
+      for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
         const int zo = p.hdiv == 1 ? z : z / p.hdiv, zi = p.hdiv == 1 ? 0 : z - zo * p.hdiv;
         const uint32_t acc = tile & 1, use = tile >> 1;
         const int m_warp = mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
@@ -565,7 +581,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // the next work item and its bias (the loads travel while this tile is worked on)
         int nt2 = nt, mt2 = mt, z2 = z, sp2 = sp;
         advance(nt2, mt2, z2, sp2);
-        const bool more = w + w_step < p.total_work && !tma_out;  // (of interest to the bias hand-over only)
+        const bool more = w + w_step < total_work && !tma_out;  // (of interest to the bias hand-over only)
         if (more) fetch_bias(nt2, bnext);
         uint4 x[4];
         const bool c0ok = chunk_ok(0);
@@ -657,7 +673,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         nt = nt2; mt = mt2; z = z2; sp = sp2;
       }
     } else
-    for (int w = w_first; w < p.total_work && ok; w += w_step, tile++) {
+    for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
       const int split = w / per_split;
       int r = w - split * per_split;
       const int z = r / tiles_per_z;
@@ -972,7 +988,7 @@ static void choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, boo
   }
 }
 
-int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err) {
+int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_starve_next.exchange(0) != 0;
   int dev = 0;
@@ -1048,6 +1064,8 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.d_fp32 = d.d_fp32; p.accumulate = d.accumulate; p.alpha = d.alpha; p.bias = d.bias; p.act = d.act;
   p.aux = (bf16*)d.aux; p.residual = (const bf16*)d.residual; p.status = status;
   p.seq_lens = d.seq_lens;
+  p.rows = rows;
+  p.rows_are_k = rows_are_k;
   p.wait_limit = WAIT_LIMIT_CYCLES;
   if (starve) {  // armed by mslt_debug_starve_next_gemm
     p.starve = 1;

@@ -76,8 +76,10 @@ __device__ __forceinline__ void ln_finish_row(float (&x)[LN_MAXE], int lane, int
 template <typename T, int NV, int ROWS>
 __global__ void __launch_bounds__(256)
 ln_fwd_kernel(const T* __restrict__ z, const float* __restrict__ gamma, const float* __restrict__ beta,
-              T* __restrict__ y, float* __restrict__ stats, int rows, int H, float eps) {
+              T* __restrict__ y, float* __restrict__ stats, int rows, int H, float eps,
+              const int* __restrict__ rows_dev) {
   pdl_begin();
+  if (rows_dev != nullptr) rows = rows_dev[1];
   constexpr int VN = VecT<T>::N;
   typedef typename VecT<T>::Raw Raw;
   const int lane = threadIdx.x & 31;
@@ -186,28 +188,48 @@ embed_ln_kernel(const int* __restrict__ tokens, const int* __restrict__ segments
                 const float* __restrict__ gamma,
                 const float* __restrict__ beta, T* __restrict__ y, T* __restrict__ zstash,
                 float* __restrict__ stats, int rows, int S, int H, int V, float eps,
-                int* __restrict__ status) {
+                int* __restrict__ status, const int* __restrict__ cu, const int* __restrict__ rows_dev, int B,
+                int* __restrict__ ptok, int* __restrict__ pseg) {
   pdl_begin();
+  if (rows_dev != nullptr) rows = rows_dev[1];
   constexpr int VN = VecT<T>::N;
   constexpr int NV = LN_MAXE / VN;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
-  int tok = tokens[row];
+  // packed rows: row -> (sequence, position) by bisection of the sequences' first rows; the rows that
+  // fill up the last tile read token 0 at position 0
+  int src = row, at = row % S;
+  if (cu != nullptr) {
+    src = -1;
+    at = 0;
+    if (row < rows_dev[0]) {
+      int lo = 0, hi = B;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (cu[mid] <= row) lo = mid; else hi = mid;
+      }
+      at = row - cu[lo];
+      src = lo * S + at;
+    }
+  }
+  int tok = src >= 0 ? tokens[src] : 0;
   if (tok < 0 || tok >= V) {
     if (lane == 0) atomicOr(status, ST_BAD_TOKEN);
     tok = 0;
   }
+  if (ptok != nullptr && lane == 0) ptok[row] = src >= 0 ? tok : -1;
   const T* wr = word + (int64_t)tok * H;
-  const T* pr = pos + (int64_t)(row % S) * H;
+  const T* pr = pos + (int64_t)at * H;
   // segment (token-type) row: table of two rows; ids outside {0, 1} are reported and read as 0
   const T* tr = nullptr;
   if (type != nullptr) {
-    int sg = segments ? segments[row] : 0;
+    int sg = segments && src >= 0 ? segments[src] : 0;
     if (sg < 0 || sg > 1) {
       if (lane == 0) atomicOr(status, ST_BAD_TOKEN);
       sg = 0;
     }
+    if (pseg != nullptr && lane == 0) pseg[row] = sg;
     tr = type + (int64_t)sg * H;
   }
   float x[LN_MAXE];
@@ -250,8 +272,10 @@ template <typename T, int NSLICE, int RG, int LN_BWD_ROWS>
 __global__ void __launch_bounds__(NSLICE * RG * 32, 1)
 ln_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ z, const float* __restrict__ stats,
               const float* __restrict__ gamma, T* __restrict__ dz, float* __restrict__ dgamma,
-              float* __restrict__ dbeta, float* __restrict__ dbias, int rows, int H) {
+              float* __restrict__ dbeta, float* __restrict__ dbias, int rows, int H,
+              const int* __restrict__ rows_dev) {
   pdl_begin();
+  if (rows_dev != nullptr) rows = rows_dev[1];
   constexpr int VN = VecT<T>::N;
   constexpr int LR = LN_BWD_ROWS;  // rows a warp has in flight
   typedef typename VecT<T>::Raw Raw;
@@ -542,9 +566,45 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
                                      const int* __restrict__ seq_lens, int B, int S, int P, int V,
                                      int* __restrict__ rowsrc, int* __restrict__ rowlabel,
                                      int* __restrict__ n_valid, float* __restrict__ inv_n,
-                                     int* __restrict__ status) {
+                                     int* __restrict__ status, int* __restrict__ cu, int* __restrict__ rows) {
   pdl_begin();
   __shared__ int cnt;
+  if (cu != nullptr) {
+    // packed batch: first row of every sequence, and {rows in use, the same rounded up to a tile}
+    __shared__ int warp_sums[32];
+    __shared__ int base;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (threadIdx.x == 0) base = 0;
+    for (int b0 = 0; b0 < B; b0 += blockDim.x) {
+      const int b = b0 + (int)threadIdx.x;
+      const int len = b < B ? min(max(seq_lens[b], 1), S) : 0;
+      int incl = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane == 31) warp_sums[warp] = incl;
+      __syncthreads();
+      int before = base;
+      for (int w = 0; w < warp; w++) before += warp_sums[w];
+      if (b < B) cu[b] = before + incl - len;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        int t = base;
+        for (int w = 0; w < nw; w++) t += warp_sums[w];
+        base = t;
+      }
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+      cu[B] = base;
+      rows[0] = base;
+      rows[1] = min((base + 127) / 128 * 128, B * S);
+    }
+    if (positions == nullptr) return;  // the layout was all that was asked for
+    __syncthreads();
+  }
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
   int local = 0, bad = 0;
@@ -558,7 +618,7 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
     if (seq_lens != nullptr) len = min(max(seq_lens[b], 1), S);
     if (pos >= len) { bad |= ST_BAD_POSITION; ok = false; }
     if (lab >= V) { bad |= ST_BAD_LABEL; ok = false; }
-    rowsrc[r] = ok ? b * S + pos : -1;
+    rowsrc[r] = ok ? (cu ? cu[b] : b * S) + pos : -1;
     rowlabel[r] = ok ? lab : -1;
     local += ok ? 1 : 0;
   }
@@ -593,6 +653,23 @@ __global__ void gather_rows_kernel(const T* __restrict__ x, const int* __restric
     }
     VecT<T>::store(out + (int64_t)r * H + c, t);
   }
+}
+
+// out[b, s, :] = x[cu[b] + s, :], zero where s is at or beyond the sequence's length; a warp per row
+template <typename T>
+__global__ void __launch_bounds__(256)
+unpack_rows_kernel(const T* __restrict__ x, const int* __restrict__ cu, T* __restrict__ out, int rows, int S, int H) {
+  pdl_begin();
+  constexpr int VN = VecT<T>::N;
+  typedef typename VecT<T>::Raw Raw;
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row >= rows) return;
+  const int b = row / S, s = row - b * S;
+  const int r0 = cu[b];
+  const bool in = s < cu[b + 1] - r0;
+  const Raw zero = {};
+  for (int c = (threadIdx.x & 31) * VN; c < H; c += 32 * VN)
+    *reinterpret_cast<Raw*>(out + (int64_t)row * H + c) = in ? VecT<T>::load_raw(x + (int64_t)(r0 + s) * H + c) : zero;
 }
 
 // dx[rowsrc[r],:] += d[r,:]; one block per sequence walks its slots in order, so repeated
@@ -820,8 +897,12 @@ __global__ void override_inv_n_kernel(const int* __restrict__ total_valid, float
 template <typename T>
 __global__ void __launch_bounds__(256)
 colsum_kernel(const T* __restrict__ x, int64_t ld, int rows, int N, int rows_per_block,
-              float* __restrict__ out) {
+              float* __restrict__ out, const int* __restrict__ rows_dev) {
   pdl_begin();
+  if (rows_dev != nullptr) {  // the blocks share out the rows in use
+    rows = rows_dev[1];
+    rows_per_block = (rows + gridDim.y - 1) / gridDim.y;
+  }
   constexpr int VN = VecT<T>::N;
   __shared__ float red[8][32 * VN];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -870,10 +951,11 @@ constexpr int ES_MAX_SLOTS = 2048;  // chunk slots: at most T / ES_CHUNK + (toke
 // counts is laid out [V][nb] so that a token's per-block counts are contiguous
 __global__ void __launch_bounds__(ES_BLOCK)
 embed_sort_count_kernel(const int* __restrict__ tokens, int T, int V, int nb, int* __restrict__ counts,
-                        int* __restrict__ rank) {
+                        int* __restrict__ rank, const int* __restrict__ rows_dev) {
   pdl_begin();
   __shared__ int tk[ES_BLOCK];
   const int t = blockIdx.x * ES_BLOCK + threadIdx.x;
+  if (rows_dev != nullptr) T = rows_dev[0];
   int tok = t < T ? tokens[t] : -1;
   if (t < T && (tok < 0 || tok >= V)) tok = 0;
   tk[threadIdx.x] = tok;
@@ -950,8 +1032,9 @@ embed_sort_scan_kernel(int* __restrict__ blocksum, int n) {
 __global__ void embed_sort_place_kernel(const int* __restrict__ tokens, int T, int V, int nb,
                                         const int* __restrict__ counts, const int* __restrict__ rank,
                                         const int* __restrict__ start_local, const int* __restrict__ blockoff,
-                                        int* __restrict__ order) {
+                                        int* __restrict__ order, const int* __restrict__ rows_dev) {
   pdl_begin();
+  if (rows_dev != nullptr) T = rows_dev[0];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= T) return;
   int tok = tokens[t];
@@ -1055,7 +1138,8 @@ __global__ void embed_word_hot_sum_kernel(const int* __restrict__ total, const i
 // column threads times 8 row groups over the batch, combined in shared memory in a fixed order.
 template <typename T>
 __global__ void __launch_bounds__(256)
-embed_pos_grad_kernel(const T* __restrict__ dz, float* __restrict__ dpos, int B, int S, int H) {
+embed_pos_grad_kernel(const T* __restrict__ dz, float* __restrict__ dpos, int B, int S, int H,
+                      const int* __restrict__ cu) {
   pdl_begin();
   constexpr int VN = VecT<T>::N;
   __shared__ float part[8][32 * VN];
@@ -1065,7 +1149,16 @@ embed_pos_grad_kernel(const T* __restrict__ dz, float* __restrict__ dpos, int B,
   float acc[VN];
 #pragma unroll
   for (int e = 0; e < VN; e++) acc[e] = 0.f;
-  if (c < H) {
+  if (c < H && cu != nullptr) {  // packed rows: the sequences long enough to have this position
+    for (int b = g; b < B; b += 8) {
+      const int r0 = cu[b];
+      if (s >= cu[b + 1] - r0) continue;
+      float a[VN];
+      VecT<T>::load(dz + (int64_t)(r0 + s) * H + c, a);
+#pragma unroll
+      for (int e = 0; e < VN; e++) acc[e] += a[e];
+    }
+  } else if (c < H) {
     int b = g;
     for (; b + 24 < B; b += 32) {
       float a[4][VN];
@@ -1156,14 +1249,15 @@ adam_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w,
 // at the pooler's pre-activation: dup = (dlogit . Wn) * (1 - pooled^2).
 // ---------------------------------------------------------------------------------------
 __global__ void nsp_prepare_kernel(const int* __restrict__ labels, int B, int S, int* __restrict__ rowsrc,
-                                   float* __restrict__ inv_n, const int* __restrict__ total_valid) {
+                                   float* __restrict__ inv_n, const int* __restrict__ total_valid,
+                                   const int* __restrict__ cu) {
   pdl_begin();
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
   int local = 0;
   for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    rowsrc[b] = b * S;  // the first token of sequence b
+    rowsrc[b] = cu ? cu[b] : b * S;  // the first token of sequence b
     local += (labels != nullptr && labels[b] >= 0 && labels[b] <= 1) ? 1 : 0;
   }
   if (local) atomicAdd(&cnt, local);
@@ -1231,8 +1325,9 @@ __global__ void tanh_kernel(const T* __restrict__ x, T* __restrict__ y, int64_t 
 template <typename T>
 __global__ void __launch_bounds__(128)
 type_grad_kernel(const T* __restrict__ dz, const int* __restrict__ segments, float* __restrict__ dtype,
-                 int rows, int H, int rows_per_block) {
+                 int rows, int H, int rows_per_block, const int* __restrict__ rows_dev) {
   pdl_begin();
+  if (rows_dev != nullptr) rows = rows_dev[0];
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= H) return;
   const int r0 = blockIdx.y * rows_per_block, r1 = min(rows, r0 + rows_per_block);
@@ -1360,13 +1455,13 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ src, bf16* __restri
   } while (0)
 
 void launch_ln_fwd(bool bf, const void* z, const float* gamma, const float* beta, void* y,
-                   float* stats, int rows, int H, float eps, cudaStream_t st) {
+                   float* stats, int rows, int H, float eps, cudaStream_t st, const int* rows_dev) {
   if (rows <= 0) return;
   const int vn = bf ? 8 : 4;
   const int nv = (H + 32 * vn - 1) / (32 * vn);
 #define LN_FWD(NV, ROWS)                                                                             \
   DISPATCH_T(bf, (launch_pdl(ln_fwd_kernel<T, NV, ROWS>, div_up(rows, 4 * ROWS), 128, 0, st,                   \
-                     (const T*)z, gamma, beta, (T*)y, stats, rows, H, eps)))
+                     (const T*)z, gamma, beta, (T*)y, stats, rows, H, eps, rows_dev)))
   if (nv <= 1) LN_FWD(1, 4);
   else if (nv <= 2) LN_FWD(2, 2);
   else if (nv <= 3) LN_FWD(3, 2);
@@ -1378,15 +1473,17 @@ void launch_ln_fwd(bool bf, const void* z, const float* gamma, const float* beta
 
 void launch_embed_ln(bool bf, const int* tokens, const int* segments, const void* word, const void* pos,
                      const void* type, const float* gamma, const float* beta, void* y, void* zstash,
-                     float* stats, int rows, int S, int H, int V, float eps, int* status, cudaStream_t st) {
+                     float* stats, int rows, int S, int H, int V, float eps, int* status, cudaStream_t st,
+                     const int* cu, const int* rows_dev, int* ptok, int* pseg) {
   if (rows <= 0) return;
   DISPATCH_T(bf, (launch_pdl(embed_ln_kernel<T>, div_up(rows, 8), 256, 0, st, 
                      tokens, segments, (const T*)word, (const T*)pos, (const T*)type, gamma, beta, (T*)y,
-                     (T*)zstash, stats, rows, S, H, V, eps, status)));
+                     (T*)zstash, stats, rows, S, H, V, eps, status, cu, rows_dev, rows / S, ptok, pseg)));
 }
 
 void launch_ln_bwd(bool bf, const void* dy, const void* z, const float* stats, const float* gamma,
-                   void* dz, float* dgamma, float* dbeta, float* dbias, int rows, int H, cudaStream_t st) {
+                   void* dz, float* dgamma, float* dbeta, float* dbias, int rows, int H, cudaStream_t st,
+                   const int* rows_dev) {
   if (rows <= 0) return;
   // warps per row: one 16-byte vector per lane; row groups fill the block up to 12-16 warps
   const int vn = bf ? 8 : 4;
@@ -1397,7 +1494,7 @@ void launch_ln_bwd(bool bf, const void* dy, const void* z, const float* stats, c
   // one block per SM walks the rows: the column sums end in one atomic per column and block
 #define LN_BWD(NS, RG)                                                                                   \
   DISPATCH_T(bf, (launch_pdl(ln_bwd_kernel<T, NS, RG, 4>, std::min(div_up(rows, RG * 4), sms), NS * RG * 32, 0, st,  \
-                     (const T*)dy, (const T*)z, stats, gamma, (T*)dz, dgamma, dbeta, dbias, rows, H)))
+                     (const T*)dy, (const T*)z, stats, gamma, (T*)dz, dgamma, dbeta, dbias, rows, H, rows_dev)))
   if (nslice <= 1) LN_BWD(1, 8);
   else if (nslice <= 2) LN_BWD(2, 6);
   else if (nslice <= 3) LN_BWD(3, 4);
@@ -1439,15 +1536,19 @@ void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float
 
 void launch_slots_prepare(const int* positions, const int* labels, const int* seq_lens, int B,
                           int S, int P, int V, int* rowsrc, int* rowlabel, int* n_valid,
-                          float* inv_n, int* status, cudaStream_t st) {
-  launch_pdl(slots_prepare_kernel, 1, 256, 0, st, positions, labels, seq_lens, B, S, P, V, rowsrc, rowlabel,
-                                          n_valid, inv_n, status);
+                          float* inv_n, int* status, cudaStream_t st, int* cu, int* rows) {
+  launch_pdl(slots_prepare_kernel, 1, cu || B * P > 1024 ? 1024 : 256, 0, st, positions, labels, seq_lens, B, S, P, V,
+             rowsrc, rowlabel, n_valid, inv_n, status, cu, rows);
 }
 
 void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, int R, int H,
                         cudaStream_t st) {
   if (R <= 0) return;
   DISPATCH_T(bf, (launch_pdl(gather_rows_kernel<T>, R, 128, 0, st, (const T*)x, rowsrc, (T*)out, R, H)));
+}
+
+void launch_unpack_rows(bool bf, const void* x, const int* cu, void* out, int B, int S, int H, cudaStream_t st) {
+  DISPATCH_T(bf, (launch_pdl(unpack_rows_kernel<T>, div_up(B * S, 8), 256, 0, st, (const T*)x, cu, (T*)out, B * S, S, H)));
 }
 
 void launch_scatter_rows(bool bf, const void* d, const int* rowsrc, void* dx, int B, int P, int H,
@@ -1477,28 +1578,29 @@ void launch_loss_reduce(const float* nll, int R, const float* inv_n, float* loss
 }
 
 void launch_colsum(bool bf, const void* x, int64_t ld, int rows, int N, float* out,
-                   cudaStream_t st) {
+                   cudaStream_t st, const int* rows_dev) {
   if (rows <= 0 || N <= 0) return;
   const int vn = bf ? 8 : 4;
   const int gx = div_up(N, 32 * vn);
   int gy = std::max(1, std::min(div_up(rows, 64), (148 * 4 + gx - 1) / gx));
   const int rpb = div_up(rows, gy);
   gy = div_up(rows, rpb);
-  DISPATCH_T(bf, (launch_pdl(colsum_kernel<T>, dim3(gx, gy), 256, 0, st, (const T*)x, ld, rows, N, rpb, out)));
+  DISPATCH_T(bf, (launch_pdl(colsum_kernel<T>, dim3(gx, gy), 256, 0, st, (const T*)x, ld, rows, N, rpb, out, rows_dev)));
 }
 
 void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float* dword, float* dpos, int B, int S,
                               int H, int V, int* counts, int* total, int* start, int* rank, int* order,
-                              int* blocksum, int* hot, float* partial, cudaStream_t st) {
+                              int* blocksum, int* hot, float* partial, cudaStream_t st, const int* cu,
+                              const int* rows_dev) {
   const int T = B * S;
   if (T <= 0) return;
   const int nb = div_up(T, ES_BLOCK), vb = div_up(V, 256);
   cudaMemsetAsync(counts, 0, (size_t)nb * V * sizeof(int), st);
   cudaMemsetAsync(hot, 0, 2 * sizeof(int), st);
-  launch_pdl(embed_sort_count_kernel, nb, ES_BLOCK, 0, st, tokens, T, V, nb, counts, rank);
+  launch_pdl(embed_sort_count_kernel, nb, ES_BLOCK, 0, st, tokens, T, V, nb, counts, rank, rows_dev);
   launch_pdl(embed_sort_prefix_kernel, vb, 256, 0, st, counts, nb, V, total, start, blocksum, hot);
   launch_pdl(embed_sort_scan_kernel, 1, 1024, 0, st, blocksum, vb);
-  launch_pdl(embed_sort_place_kernel, div_up(T, 256), 256, 0, st, tokens, T, V, nb, counts, rank, start, blocksum, order);
+  launch_pdl(embed_sort_place_kernel, div_up(T, 256), 256, 0, st, tokens, T, V, nb, counts, rank, start, blocksum, order, rows_dev);
   const int vn = bf ? 8 : 4;
   const size_t smem = (size_t)(1024 / (H / vn)) * H * sizeof(float), smem_small = (size_t)(256 / (H / vn)) * H * sizeof(float);
   // at most T / ES_CHUNK tokens have more than ES_CHUNK rows, and they have at most 2 T / ES_CHUNK chunks
@@ -1510,7 +1612,7 @@ void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float*
                                                                               total, hot, partial, H)));
     launch_pdl(embed_word_hot_sum_kernel, max_hot, 256, 0, st, total, hot, partial, dword, H);
   }
-  DISPATCH_T(bf, (launch_pdl(embed_pos_grad_kernel<T>, dim3(S, div_up(H, 32 * vn)), 256, 0, st, (const T*)dz, dpos, B, S, H)));
+  DISPATCH_T(bf, (launch_pdl(embed_pos_grad_kernel<T>, dim3(S, div_up(H, 32 * vn)), 256, 0, st, (const T*)dz, dpos, B, S, H, cu)));
 }
 
 void launch_adam(const AdamChunk* chunks, int n_chunks, float* w, const float* g, float* m, float* v,
@@ -1532,8 +1634,8 @@ void launch_lamb(const AdamChunk* chunks, int n_chunks, float* w, const float* g
 }
 
 void launch_nsp_prepare(const int* labels, int B, int S, int* rowsrc, float* inv_n, const int* total_valid,
-                        cudaStream_t st) {
-  launch_pdl(nsp_prepare_kernel, 1, 128, 0, st, labels, B, S, rowsrc, inv_n, total_valid);
+                        cudaStream_t st, const int* cu) {
+  launch_pdl(nsp_prepare_kernel, 1, 128, 0, st, labels, B, S, rowsrc, inv_n, total_valid, cu);
 }
 
 void launch_nsp_head(bool bf, const void* pooled, const float* wn, const float* bn, const int* labels,
@@ -1551,11 +1653,11 @@ void launch_tanh(bool bf, const void* x, void* y, int64_t n, cudaStream_t st) {
 }
 
 void launch_type_grad(bool bf, const void* dz, const int* segments, float* dtype, int rows, int H,
-                      cudaStream_t st) {
+                      cudaStream_t st, const int* rows_dev) {
   if (rows <= 0) return;
   const int rpb = 512;
   DISPATCH_T(bf, (launch_pdl(type_grad_kernel<T>, dim3(div_up(H, 128), div_up(rows, rpb)), 128, 0, st, 
-                     (const T*)dz, segments, dtype, rows, H, rpb)));
+                     (const T*)dz, segments, dtype, rows, H, rpb, rows_dev)));
 }
 
 void launch_dgelu(bool bf, void* d, const void* u, int64_t n, cudaStream_t st) {

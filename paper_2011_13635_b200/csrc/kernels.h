@@ -20,21 +20,31 @@ struct AdamHyper {
   float bc1, bc2;    // bias corrections 1 / (1 - beta^t), or 1: filled on the device
 };
 
+// Packed batches.  A batch whose sequences have lengths is kept without its padding: sequence b holds
+// rows cu[b] .. cu[b + 1] - 1 of every activation, rows_dev (device) = {rows in use, the same rounded up
+// to a tile of 128}.  The launchers below then get the allocated row count for their grid and work on the
+// rows in use only; null = every row.
 void launch_ln_fwd(bool bf, const void* z, const float* gamma, const float* beta, void* y,
-                   float* stats, int rows, int H, float eps, cudaStream_t st);
-// segments / type: segment ids and the two-row segment table, or null (no segment term)
+                   float* stats, int rows, int H, float eps, cudaStream_t st, const int* rows_dev = nullptr);
+// segments / type: segment ids and the two-row segment table, or null (no segment term).  rows = B * S.
+// Packed: ptok (and pseg) receive the token id (segment) of every packed row, -1 past the last.
 void launch_embed_ln(bool bf, const int* tokens, const int* segments, const void* word, const void* pos,
                      const void* type, const float* gamma, const float* beta, void* y, void* zstash,
-                     float* stats, int rows, int S, int H, int V, float eps, int* status, cudaStream_t st);
+                     float* stats, int rows, int S, int H, int V, float eps, int* status, cudaStream_t st,
+                     const int* cu = nullptr, const int* rows_dev = nullptr, int* ptok = nullptr, int* pseg = nullptr);
 void launch_ln_bwd(bool bf, const void* dy, const void* z, const float* stats, const float* gamma,
-                   void* dz, float* dgamma, float* dbeta, float* dbias, int rows, int H, cudaStream_t st);
+                   void* dz, float* dgamma, float* dbeta, float* dbias, int rows, int H, cudaStream_t st,
+                   const int* rows_dev = nullptr);
 void launch_softmax_fwd(bool bf, const void* sc, void* p, const int* seq_lens, int rows, int S,
                         int rows_per_seq, float scale, cudaStream_t st);
 void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float scale,
                         cudaStream_t st);
+// cu, rows (outputs, with seq_lens): the packed layout; positions null: only that
 void launch_slots_prepare(const int* positions, const int* labels, const int* seq_lens, int B,
                           int S, int P, int V, int* rowsrc, int* rowlabel, int* n_valid,
-                          float* inv_n, int* status, cudaStream_t st);
+                          float* inv_n, int* status, cudaStream_t st, int* cu = nullptr, int* rows = nullptr);
+// out [B, S, H] from packed rows; zero past a sequence's length
+void launch_unpack_rows(bool bf, const void* x, const int* cu, void* out, int B, int S, int H, cudaStream_t st);
 void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, int R, int H,
                         cudaStream_t st);
 void launch_scatter_rows(bool bf, const void* d, const int* rowsrc, void* dx, int B, int P, int H,
@@ -46,7 +56,7 @@ void launch_cross_entropy(bool bf, const float* logits, int64_t ldl, const int* 
 void launch_loss_reduce(const float* nll, int R, const float* inv_n, float* loss, cudaStream_t st);
 // out[n] += sum over rows; N a multiple of the 16-byte vector width, out has room for N floats
 void launch_colsum(bool bf, const void* x, int64_t ld, int rows, int N, float* out,
-                   cudaStream_t st);
+                   cudaStream_t st, const int* rows_dev = nullptr);
 // The embedding gradients without hot-row atomics and with run-to-run identical bits: counting sort
 // of the rows by token id, one block per token id, batch sum per position.  Needs H / (16 bytes of
 // activation) <= 1024 column threads and V <= 262144.  Scratch: counts [ceil(T/256) * V], total [V],
@@ -54,7 +64,8 @@ void launch_colsum(bool bf, const void* x, int64_t ld, int rows, int N, float* o
 // needs T <= 65536 and H / (16-byte vector) <= 256.  Nine launches.
 void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float* dword, float* dpos, int B, int S,
                               int H, int V, int* counts, int* total, int* start, int* rank, int* order,
-                              int* blocksum, int* hot, float* partial, cudaStream_t st);
+                              int* blocksum, int* hot, float* partial, cudaStream_t st, const int* cu = nullptr,
+                              const int* rows_dev = nullptr);
 // t_dev: step count in device memory (incremented here); bc_dev: two floats that receive the bias
 // corrections of this step
 void launch_adam(const AdamChunk* chunks, int n_chunks, float* w, const float* g, float* m, float* v,
@@ -73,14 +84,14 @@ void launch_lamb(const AdamChunk* chunks, int n_chunks, float* w, const float* g
 // added to *loss, gradients of the classifier added to dwn [2,H] / dbn [2], and dup [B,H] = gradient
 // at the pooler's pre-activation (tanh derivative included).
 void launch_nsp_prepare(const int* labels, int B, int S, int* rowsrc, float* inv_n, const int* total_valid,
-                        cudaStream_t st);
+                        cudaStream_t st, const int* cu = nullptr);
 void launch_nsp_head(bool bf, const void* pooled, const float* wn, const float* bn, const int* labels,
                      const float* inv_n, void* dup, float* dwn, float* dbn, float* loss, int B, int H,
                      cudaStream_t st);
 void launch_tanh(bool bf, const void* x, void* y, int64_t n, cudaStream_t st);
 // dtype[seg[t], :] += dz[t, :] for the two-row segment table
 void launch_type_grad(bool bf, const void* dz, const int* segments, float* dtype, int rows, int H,
-                      cudaStream_t st);
+                      cudaStream_t st, const int* rows_dev = nullptr);
 // data-parallel steps: the loss normaliser becomes 1 / *total_valid (0 when that count is 0)
 void launch_override_inv_n(const int* total_valid, float* inv_n, cudaStream_t st);
 void launch_dgelu(bool bf, void* d, const void* u, int64_t n, cudaStream_t st);

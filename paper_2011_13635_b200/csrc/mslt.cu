@@ -83,6 +83,7 @@ struct Workspace {
   char *hm, *ut, *gt, *tm, *dlogits, *dtm, *dgt, *dhm;
   int *es_counts, *es_total, *es_start, *es_rank, *es_order, *es_blocksum, *es_hot;
   float* es_partial;  // embedding backward: rows sorted by token id
+  int *cu, *rows, *ptok, *pseg;             // packed batches: see kernels.h
   int* nsp_rowsrc;                          // NSP head: first-token row of every sequence
   char *cls, *up, *pooled, *dup, *dcls;     // [B,H] each
   float *hst, *logits, *nll, *dtm32;
@@ -107,6 +108,8 @@ struct mslt_ctx {
   int64_t emb_off, emb_cnt, layer0_off, layer_cnt, layer_mat_cnt, head_off, head_cnt;
   Workspace ws;
   int n_chunks;
+  // this call's batch is packed (its sequences have lengths): first rows and row counts on the device
+  const int *cu, *rows;
   int64_t launches;
   int Vp, num_sms;
   bool timing;
@@ -234,6 +237,10 @@ void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char
   const int64_t Vp = pad_to(a.vocab, 8);
   const int64_t P2 = (int64_t)a.max_batch * A * a.max_seq * a.max_seq;
   w.scalars = (int*)take(256);
+  w.cu = (int*)take(((int64_t)a.max_batch + 1) * 4);
+  w.rows = (int*)take(2 * 4);
+  w.ptok = (int*)take(T * 4);
+  w.pseg = (int*)take(T * 4);
   w.rowsrc = (int*)take(R * 4);
   w.rowlabel = (int*)take(R * 4);
   w.max_chunks = 0;
@@ -371,13 +378,17 @@ bool getenv_unfused_attention() {
   return v;
 }
 
-// scores, masked softmax and context of one layer in one kernel (bf16, head width 64, S <= 128)
-int run_attention(mslt_ctx* c, const void* qkv, void* probs, void* ctx, const int* seq_lens, int B, int S,
+// bf16 attention runs in the fused kernels (head width 64 and S <= 512 are checked at creation)
+bool fused_attention(const mslt_ctx* c) { return c->bf && !getenv_cuda_cores() && !getenv_unfused_attention(); }
+
+// scores, masked softmax and context of one layer in one kernel; for the backward pass either the
+// probabilities (S <= 128) or the rows' sums of exponentials (lse)
+int run_attention(mslt_ctx* c, const void* qkv, void* probs, float* lse, void* ctx, const int* seq_lens, int B, int S,
                   int A, int d, float scale) {
   char err[256] = "";
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
-  int rc = attn_fwd_launch(qkv, probs, ctx, seq_lens, B, S, A, d, scale, c->ws.scalars, c->st, err);
+  int rc = attn_fwd_launch(qkv, probs, ctx, seq_lens, B, S, A, d, scale, c->ws.scalars, c->st, err, c->cu, c->rows, lse);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({1, 4.0 * B * A * (double)S * S * d});
@@ -387,28 +398,31 @@ int run_attention(mslt_ctx* c, const void* qkv, void* probs, void* ctx, const in
   return 0;
 }
 
-int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const void* dctx, void* dqkv, int B,
-                      int S, int A, int d, float scale) {
+int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const void* ctx, const void* dctx, void* dqkv,
+                      const int* seq_lens, int B, int S, int A, int d, float scale) {
   char err[256] = "";
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
-  int rc = attn_bwd_launch(qkv, probs, dctx, dqkv, B, S, A, d, scale, c->ws.scalars, c->st, err);
+  // rows of more than 128 keys keep their sums of exponentials in the place of the probabilities
+  int rc = S <= 128 ? attn_bwd_launch(qkv, probs, dctx, dqkv, B, S, A, d, scale, c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows)
+                    : attn_bwd_long_launch(qkv, ctx, dctx, (const float*)probs, (float*)c->ws.dp, dqkv, B, S, A, scale,
+                                           c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({1, 8.0 * B * A * (double)S * S * d});
   }
   if (rc) return fail(rc, "%s", err);
-  c->launches++;
+  c->launches += S <= 128 ? 1 : 3;
   return 0;
 }
 
-int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d) {
+int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, int rows_are_k = 0) {
   if (d.M <= 0 || d.N <= 0 || d.K <= 0 || d.batch <= 0) return 0;
   char err[256] = "";
   const int64_t before = gemm_launches();
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
-  int rc = gemm_launch(d, c->ws.scalars, c->st, err);
+  int rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({d.batch > 1 ? 1 : 0, 2.0 * d.M * d.N * (double)d.K * d.batch});
@@ -421,7 +435,7 @@ int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d) {
 // Y[T,N] = X[T,K] * W[N,K]^T (+ bias) with optional GELU / residual
 int linear_fwd(mslt_ctx* c, const void* x, int T, int K, int64_t w_off, int64_t b_off, int N,
                void* y, int act, void* aux, const void* residual, bool out_fp32 = false,
-               int64_t ldd = 0) {
+               int64_t ldd = 0, const int* rows = nullptr) {
   Lin g(c, T, N, K);
   g.d.A = x; g.d.a_rs = K; g.d.a_ks = 1;
   g.d.B = Wc(c, w_off); g.d.b_rs = K; g.d.b_ks = 1;
@@ -429,29 +443,29 @@ int linear_fwd(mslt_ctx* c, const void* x, int T, int K, int64_t w_off, int64_t 
   g.d.bias = Wv(c, b_off);
   g.d.act = act; g.d.aux = aux; g.d.residual = residual;
   g.d.d_fp32 = out_fp32 ? 1 : 0;
-  return run_gemm(c, g.d);
+  return run_gemm(c, g.d, rows);
 }
 
 // dX[T,K] = dY[T,N] * W[N,K]  (optionally * gelu'(aux), + residual)
 int linear_dgrad(mslt_ctx* c, const void* dy, int T, int N, int64_t lda, int64_t w_off, int K,
-                 void* dx, int act, void* aux, const void* residual) {
+                 void* dx, int act, void* aux, const void* residual, const int* rows = nullptr) {
   Lin g(c, T, K, N);
   g.d.A = dy; g.d.a_rs = lda; g.d.a_ks = 1;
   g.d.B = Wc(c, w_off); g.d.b_rs = 1; g.d.b_ks = K;
   g.d.D = dx; g.d.ldd = K;
   g.d.act = act; g.d.aux = aux; g.d.residual = residual;
-  return run_gemm(c, g.d);
+  return run_gemm(c, g.d, rows);
 }
 
 // dW[N,K] += dY[T,N]^T * X[T,K]   (fp32, into the zeroed gradient arena)
 int linear_wgrad(mslt_ctx* c, const void* dy, int T, int N, int64_t lddy, const void* x, int K,
-                 int64_t w_off) {
+                 int64_t w_off, const int* rows = nullptr) {
   Lin g(c, N, K, T);
   g.d.A = dy; g.d.a_rs = 1; g.d.a_ks = lddy;
   g.d.B = x; g.d.b_rs = 1; g.d.b_ks = K;
   g.d.D = G(c, w_off); g.d.ldd = K;
   g.d.d_fp32 = 1; g.d.accumulate = 1;
-  return run_gemm(c, g.d);
+  return run_gemm(c, g.d, rows, 1);
 }
 
 #define TRY(x)        \
@@ -490,10 +504,11 @@ int layer_forward(mslt_ctx* c, int l, const void* x, LayerBuf& b, void* out, boo
   const int E = c->esz;
   const float scale = 1.0f / sqrtf((float)d);
   TRY(linear_fwd(c, x, T, H, toff(c, l, "qkv.weight"), toff(c, l, "qkv.bias"), 3 * H, b.qkv, 0,
-                 nullptr, nullptr));
-  if (c->bf && S <= 512 && d == 64 && !getenv_cuda_cores() && !getenv_unfused_attention()) {
+                 nullptr, nullptr, false, 0, c->rows));
+  if (fused_attention(c)) {
     // the probabilities go to memory only where the backward pass will read them
-    TRY(run_attention(c, b.qkv, save ? b.p : nullptr, b.c, seq_lens, B, S, A, d, scale));
+    TRY(run_attention(c, b.qkv, save && S <= 128 ? b.p : nullptr, save && S > 128 ? (float*)b.p : nullptr, b.c, seq_lens, B,
+                      S, A, d, scale));
   } else {
     {  // scores[b,h,i,j] = q_i . k_j / sqrt(d)
       Lin g(c, S, S, d);
@@ -519,40 +534,40 @@ int layer_forward(mslt_ctx* c, int l, const void* x, LayerBuf& b, void* out, boo
       TRY(run_gemm(c, g.d));
     }
   }
-  TRY(linear_fwd(c, b.c, T, H, toff(c, l, "out.weight"), toff(c, l, "out.bias"), H, b.z1, 0, nullptr, x));
+  TRY(linear_fwd(c, b.c, T, H, toff(c, l, "out.weight"), toff(c, l, "out.bias"), H, b.z1, 0, nullptr, x, false, 0, c->rows));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_ln_fwd(c->bf, b.z1, Wv(c, toff(c, l, "ln1.gamma")), Wv(c, toff(c, l, "ln1.beta")), b.y,
-                   save ? b.st1 : nullptr, T, H, c->a.ln_eps, c->st));
+                   save ? b.st1 : nullptr, T, H, c->a.ln_eps, c->st, c->rows));
   TRY(linear_fwd(c, b.y, T, H, toff(c, l, "ffn1.weight"), toff(c, l, "ffn1.bias"), F, b.g, 1,
-                 save ? b.u : nullptr, nullptr));
-  TRY(linear_fwd(c, b.g, T, F, toff(c, l, "ffn2.weight"), toff(c, l, "ffn2.bias"), H, b.z2, 0, nullptr, b.y));
+                 save ? b.u : nullptr, nullptr, false, 0, c->rows));
+  TRY(linear_fwd(c, b.g, T, F, toff(c, l, "ffn2.weight"), toff(c, l, "ffn2.bias"), H, b.z2, 0, nullptr, b.y, false, 0, c->rows));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_ln_fwd(c->bf, b.z2, Wv(c, toff(c, l, "ln2.gamma")), Wv(c, toff(c, l, "ln2.beta")), out,
-                   save ? b.st2 : nullptr, T, H, c->a.ln_eps, c->st));
+                   save ? b.st2 : nullptr, T, H, c->a.ln_eps, c->st, c->rows));
   return 0;
 }
 
 // ---- one encoder layer, backward -------------------------------------------------------------------
 // dx: gradient w.r.t. the layer output; dx_out (if need_dx): gradient w.r.t. its input x_in.
 int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void* dx, void* dx_out,
-                   bool need_dx, int B, int S) {
+                   bool need_dx, int B, int S, const int* seq_lens) {
   const int H = c->a.hidden, F = c->a.ffn, A = c->a.heads, d = H / A, T = B * S;
   const int E = c->esz;
   Workspace& w = c->ws;
   const float scale = 1.0f / sqrtf((float)d);
   KL(PC_LN_BWD, 3.0 * T * H * c->esz, launch_ln_bwd(c->bf, dx, b.z2, b.st2, Wv(c, toff(c, l, "ln2.gamma")), w.dz2,
-                   G(c, toff(c, l, "ln2.gamma")), G(c, toff(c, l, "ln2.beta")), G(c, toff(c, l, "ffn2.bias")), T, H, c->st));
-  TRY(linear_wgrad(c, w.dz2, T, H, H, b.g, F, toff(c, l, "ffn2.weight")));
-  TRY(linear_dgrad(c, w.dz2, T, H, H, toff(c, l, "ffn2.weight"), F, w.dg, 2, b.u, nullptr));
-  TRY(linear_wgrad(c, w.dg, T, F, F, b.y, H, toff(c, l, "ffn1.weight")));
-  KL(PC_COLSUM, 1.0 * T * F * c->esz, launch_colsum(c->bf, w.dg, F, T, F, G(c, toff(c, l, "ffn1.bias")), c->st));
-  TRY(linear_dgrad(c, w.dg, T, F, F, toff(c, l, "ffn1.weight"), H, w.dy, 0, nullptr, w.dz2));
+                   G(c, toff(c, l, "ln2.gamma")), G(c, toff(c, l, "ln2.beta")), G(c, toff(c, l, "ffn2.bias")), T, H, c->st, c->rows));
+  TRY(linear_wgrad(c, w.dz2, T, H, H, b.g, F, toff(c, l, "ffn2.weight"), c->rows));
+  TRY(linear_dgrad(c, w.dz2, T, H, H, toff(c, l, "ffn2.weight"), F, w.dg, 2, b.u, nullptr, c->rows));
+  TRY(linear_wgrad(c, w.dg, T, F, F, b.y, H, toff(c, l, "ffn1.weight"), c->rows));
+  KL(PC_COLSUM, 1.0 * T * F * c->esz, launch_colsum(c->bf, w.dg, F, T, F, G(c, toff(c, l, "ffn1.bias")), c->st, c->rows));
+  TRY(linear_dgrad(c, w.dg, T, F, F, toff(c, l, "ffn1.weight"), H, w.dy, 0, nullptr, w.dz2, c->rows));
   KL(PC_LN_BWD, 3.0 * T * H * c->esz, launch_ln_bwd(c->bf, w.dy, b.z1, b.st1, Wv(c, toff(c, l, "ln1.gamma")), w.dz1,
-                   G(c, toff(c, l, "ln1.gamma")), G(c, toff(c, l, "ln1.beta")), G(c, toff(c, l, "out.bias")), T, H, c->st));
-  TRY(linear_wgrad(c, w.dz1, T, H, H, b.c, H, toff(c, l, "out.weight")));
-  TRY(linear_dgrad(c, w.dz1, T, H, H, toff(c, l, "out.weight"), H, w.dc, 0, nullptr, nullptr));
+                   G(c, toff(c, l, "ln1.gamma")), G(c, toff(c, l, "ln1.beta")), G(c, toff(c, l, "out.bias")), T, H, c->st, c->rows));
+  TRY(linear_wgrad(c, w.dz1, T, H, H, b.c, H, toff(c, l, "out.weight"), c->rows));
+  TRY(linear_dgrad(c, w.dz1, T, H, H, toff(c, l, "out.weight"), H, w.dc, 0, nullptr, nullptr, c->rows));
   const int64_t qs = (int64_t)S * 3 * H, ps = (int64_t)A * S * S, cs = (int64_t)S * H;
-  if (c->bf && S <= 128 && S % 8 == 0 && d == 64 && !getenv_cuda_cores() && !getenv_unfused_attention()) {
+  if (fused_attention(c)) {
     // dV, dP, softmax backward, dQ and dK of the layer in one kernel
-    TRY(run_attention_bwd(c, b.qkv, b.p, w.dc, w.dqkv, B, S, A, d, scale));
+    TRY(run_attention_bwd(c, b.qkv, b.p, b.c, w.dc, w.dqkv, seq_lens, B, S, A, d, scale));
   } else {
     {  // dV[j,:] = sum_i p[i,j] dC[i,:]
       Lin g(c, S, d, S);
@@ -588,10 +603,10 @@ int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void
       TRY(run_gemm(c, g.d));
     }
   }
-  TRY(linear_wgrad(c, w.dqkv, T, 3 * H, 3 * H, x_in, H, toff(c, l, "qkv.weight")));
-  KL(PC_COLSUM, 3.0 * T * H * c->esz, launch_colsum(c->bf, w.dqkv, 3 * H, T, 3 * H, G(c, toff(c, l, "qkv.bias")), c->st));
+  TRY(linear_wgrad(c, w.dqkv, T, 3 * H, 3 * H, x_in, H, toff(c, l, "qkv.weight"), c->rows));
+  KL(PC_COLSUM, 3.0 * T * H * c->esz, launch_colsum(c->bf, w.dqkv, 3 * H, T, 3 * H, G(c, toff(c, l, "qkv.bias")), c->st, c->rows));
   if (need_dx)  // the frozen boundary stops here: nothing below needs a gradient
-    TRY(linear_dgrad(c, w.dqkv, T, 3 * H, 3 * H, toff(c, l, "qkv.weight"), H, dx_out, 0, nullptr, w.dz1));
+    TRY(linear_dgrad(c, w.dqkv, T, 3 * H, 3 * H, toff(c, l, "qkv.weight"), H, dx_out, 0, nullptr, w.dz1, c->rows));
   return 0;
 }
 
@@ -711,6 +726,15 @@ int check_batch(mslt_ctx* c, int B, int S, int P) {
   return 0;
 }
 
+// A batch with sequence lengths is kept packed on the bf16 path: only the tokens that exist are embedded
+// and take part in the products (25 to 38 % of a batch with lengths spread over a factor of two to four
+// is padding).  Decided per call; the row count itself stays on the device.
+void pack_batch(mslt_ctx* c, const int* seq_lens) {
+  const bool on = seq_lens != nullptr && fused_attention(c);
+  c->cu = on ? c->ws.cu : nullptr;
+  c->rows = on ? c->ws.rows : nullptr;
+}
+
 int finish(mslt_ctx* c, float* loss_out) {
   CUDA_TRY(cudaGetLastError());
   if (!loss_out) return 0;
@@ -777,6 +801,7 @@ int mslt_create(const mslt_arch* arch, void* dev_params, size_t param_bytes, voi
   c->bucket_user = nullptr;
   c->comm_done = nullptr;
   c->pending_update = false;
+  c->cu = c->rows = nullptr;
   memset(c->prof, 0, sizeof(c->prof));
   c->Vp = (int)pad_to(arch->vocab, 8);
   int dev = 0;
@@ -894,8 +919,9 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
   CUDA_TRY(cudaMemsetAsync(w.scalars, 0, 16, c->st));
   c->prec.clear();
   mark(c, 0);
+  pack_batch(c, d_seq_lens);
   KL(PC_OTHER, 16.0 * B * P, launch_slots_prepare(d_pos, d_lab, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel, w.scalars + 1,
-                          inv_n, status, c->st));
+                          inv_n, status, c->st, c->cu ? w.cu : nullptr, w.rows));
   if (d_total_valid)  // the mean runs over the valid slots of every rank's batch
     KL(PC_OTHER, 8.0, launch_override_inv_n(d_total_valid, inv_n, c->st));
   // embeddings, then the frozen prefix: forward only, two buffers, nothing kept but the output
@@ -903,7 +929,7 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
                      c->a.nsp ? Wc(c, toff(c, -1, "emb.type")) : nullptr,
                      Wv(c, toff(c, -1, "emb.ln.gamma")), Wv(c, toff(c, -1, "emb.ln.beta")), w.xa,
                      full ? w.z0 : nullptr, full ? w.st0 : nullptr, T, S, H, V, c->a.ln_eps, status,
-                     c->st));
+                     c->st, c->cu, c->rows, c->cu ? w.ptok : nullptr, c->cu ? w.pseg : nullptr));
   char* cur = w.xa;
   for (int l = 0; l < first; l++) {
     char* out = cur == w.xa ? w.xb : w.xa;
@@ -926,7 +952,7 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
   if (nsp) {
     // second objective, forward: pooled = tanh(Wp x_L[b, 0] + bp)
     const int32_t* nsp_total = d_total_valid ? d_total_valid + 1 : nullptr;
-    KL(PC_OTHER, 8.0 * B, launch_nsp_prepare(d_nsp_lab, B, S, w.nsp_rowsrc, nsp_inv_n, nsp_total, c->st));
+    KL(PC_OTHER, 8.0 * B, launch_nsp_prepare(d_nsp_lab, B, S, w.nsp_rowsrc, nsp_inv_n, nsp_total, c->st, c->cu));
     KL(PC_OTHER, 2.0 * B * H * c->esz, launch_gather_rows(c->bf, cur, w.nsp_rowsrc, w.cls, B, H, c->st));
     TRY(linear_fwd(c, w.cls, B, H, toff(c, -1, "head.pooler.weight"), toff(c, -1, "head.pooler.bias"), H, w.up, 0,
                    nullptr, nullptr));
@@ -952,22 +978,22 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
   for (int l = c->L - 1; l >= first; l--) {
     const void* x_in = l == first ? (const void*)boundary : (const void*)w.layer[l - 1 - first].xout;
     const bool need_dx = l > first || full;
-    TRY(layer_backward(c, l, x_in, w.layer[l - first], dx, dx_other, need_dx, B, S));
+    TRY(layer_backward(c, l, x_in, w.layer[l - first], dx, dx_other, need_dx, B, S, d_seq_lens));
     if (need_dx) std::swap(dx, dx_other);
     if (l % group_of(c->a) == 0)  // the lowest layer of a parameter block completes its gradients
       TRY(bucket_done(c, (c->L - l) / group_of(c->a)));
   }
   if (full) {
     KL(PC_LN_BWD, 3.0 * T * H * c->esz, launch_ln_bwd(c->bf, dx, w.z0, w.st0, Wv(c, toff(c, -1, "emb.ln.gamma")), w.dz2,
-                     G(c, toff(c, -1, "emb.ln.gamma")), G(c, toff(c, -1, "emb.ln.beta")), nullptr, T, H, c->st));
+                     G(c, toff(c, -1, "emb.ln.gamma")), G(c, toff(c, -1, "emb.ln.beta")), nullptr, T, H, c->st, c->rows));
     // rows grouped by token id (counting sort), one block per id, batch sum per position: no hot-row
     // atomics, same bits on every run
-    KL(PC_OTHER, 2.0 * T * H * c->esz, launch_embed_grad_sorted(c->bf, w.dz2, d_tokens, G(c, toff(c, -1, "emb.word")),
+    KL(PC_OTHER, 2.0 * T * H * c->esz, launch_embed_grad_sorted(c->bf, w.dz2, c->cu ? w.ptok : d_tokens, G(c, toff(c, -1, "emb.word")),
                             G(c, toff(c, -1, "emb.pos")), B, S, H, V, w.es_counts, w.es_total, w.es_start,
-                            w.es_rank, w.es_order, w.es_blocksum, w.es_hot, w.es_partial, c->st));
+                            w.es_rank, w.es_order, w.es_blocksum, w.es_hot, w.es_partial, c->st, c->cu, c->rows));
     c->launches += 8;
     if (c->a.nsp)
-      KL(PC_OTHER, 1.0 * T * H * c->esz, launch_type_grad(c->bf, w.dz2, d_seg, G(c, toff(c, -1, "emb.type")), T, H, c->st));
+      KL(PC_OTHER, 1.0 * T * H * c->esz, launch_type_grad(c->bf, w.dz2, c->cu ? w.pseg : d_seg, G(c, toff(c, -1, "emb.type")), T, H, c->st, c->rows));
     TRY(bucket_done(c, c->top_k / group_of(c->a) + 1));
   }
   mark(c, 4);
@@ -1083,20 +1109,23 @@ int mslt_forward(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens
   Workspace& w = c->ws;
   const int H = c->a.hidden, V = c->a.vocab, T = B * S;
   CUDA_TRY(cudaMemsetAsync(w.scalars, 0, 16, c->st));
-  if (head)
-    KL(PC_OTHER, 8.0 * B * P, launch_slots_prepare(d_pos, nullptr, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel,
-                            w.scalars + 1, (float*)(w.scalars + 2), w.scalars, c->st));
+  pack_batch(c, d_seq_lens);
+  if (head || c->cu)
+    KL(PC_OTHER, 8.0 * B * P, launch_slots_prepare(head ? d_pos : nullptr, nullptr, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel,
+                            w.scalars + 1, (float*)(w.scalars + 2), w.scalars, c->st, c->cu ? w.cu : nullptr, w.rows));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_embed_ln(c->bf, d_tokens, nullptr, Wc(c, toff(c, -1, "emb.word")), Wc(c, toff(c, -1, "emb.pos")),
                      c->a.nsp ? Wc(c, toff(c, -1, "emb.type")) : nullptr,
                      Wv(c, toff(c, -1, "emb.ln.gamma")), Wv(c, toff(c, -1, "emb.ln.beta")), w.xa,
-                     nullptr, nullptr, T, S, H, V, c->a.ln_eps, w.scalars, c->st));
+                     nullptr, nullptr, T, S, H, V, c->a.ln_eps, w.scalars, c->st, c->cu, c->rows));
   char* cur = w.xa;
   for (int l = 0; l < c->L; l++) {
     char* out = cur == w.xa ? w.xb : w.xa;
     TRY(layer_forward(c, l, cur, w.scratch, out, false, B, S, d_seq_lens));
     cur = out;
   }
-  if (d_hidden_out)
+  if (d_hidden_out && c->cu)
+    KL(PC_OTHER, 2.0 * T * H * c->esz, launch_unpack_rows(c->bf, cur, c->cu, d_hidden_out, B, S, H, c->st));
+  else if (d_hidden_out)
     CUDA_TRY(cudaMemcpyAsync(d_hidden_out, cur, (size_t)T * H * c->esz, cudaMemcpyDeviceToDevice, c->st));
   if (head) {
     TRY(head_forward(c, cur, B * P, false));

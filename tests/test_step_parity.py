@@ -185,3 +185,33 @@ def test_bf16_step_with_unfused_attention_in_a_child_process():
         counts[unfused] = int(r.stdout.strip().split()[-1])
     # two launches per layer forward become three, one per trainable layer backward becomes five
     assert counts["1"] > counts["0"]
+
+
+@pytest.mark.parametrize("seq,varlen,nsp", [(128, (1, 128), False), (136, (1, 136), True), (256, (120, 256), False),
+                                            (512, (60, 512), False), (136, None, False), (384, None, False)])
+def test_bf16_packed_batches_and_long_row_backward(seq, varlen, nsp):
+    """Batches with lengths run without their padding, rows of more than 128 keys recompute their
+    probabilities in the backward pass: lengths of 1, ragged last tiles, every layer and the
+    embeddings trained, and the same without lengths."""
+    cfg = I.StageConfig("packed", hidden=192, heads=3, ffn=320, vocab=1037, max_pos=512, layers=2, trainable=2,
+                        batch=5, seq=seq, pred=9, dtype="bf16", varlen=varlen, seed_index=31, nsp=nsp)
+    if nsp:
+        _run_nsp(cfg, steps=2, lr=1e-4)
+    else:
+        _run(cfg, steps=2, lr=1e-4)
+
+
+def test_bf16_forward_zeroes_the_padding_of_a_packed_batch():
+    import torch
+    cfg = I.scaled(I.CONFIGS["base_stage"], layers=1, trainable=1, batch=3, varlen=(20, 128))
+    m, oracle = PT.build_pair(cfg, lr=1e-3)
+    tok, lens, pos, lab = I.make_batch(cfg)
+    d_tok, d_lens = PT.to_cuda(torch, tok, lens)
+    hidden, _ = m.mslt_forward(d_tok, d_lens)
+    hidden = hidden.float().cpu().numpy()
+    h_ref, _ = oracle.forward(tok, lens, pos)
+    for b in range(cfg.batch):
+        n = int(lens[b])
+        assert PT.max_rel(hidden[b, :n], h_ref[b, :n]) < PT.TOL["bf16"]["hidden"]
+        assert not hidden[b, n:].any()
+    m.close()
