@@ -1,0 +1,92 @@
+// Shared by the two fp32 contraction kernels (CUDA cores, and tensor cores on split operands): launch
+// parameters, the fused epilogue, and the addition of partial tiles inside a cluster.
+#pragma once
+#include "common.cuh"
+#include "gemm.h"
+
+namespace mslt {
+namespace {
+
+struct F32Params {
+  mslt_gemm_desc d;
+  int splits, kb_per_split, n_tiles;
+  int vec_out;  // D, aux, residual and bias rows allow 16-byte access
+};
+
+__device__ __forceinline__ uint32_t f32_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int m, int n, float4 v4) {
+  const mslt_gemm_desc& d = p.d;
+  if (m >= d.M || n >= d.N) return;
+  const int64_t o = zoff + (int64_t)m * d.ldd + n;
+  float v[4] = {d.alpha * v4.x, d.alpha * v4.y, d.alpha * v4.z, d.alpha * v4.w};
+  float* D = (float*)d.D;
+  if (p.vec_out && n + 4 <= d.N) {
+    if (d.bias) {
+      const float4 b = *reinterpret_cast<const float4*>(d.bias + n);
+      v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
+    }
+    if (d.act == 1) {
+      if (d.aux) *reinterpret_cast<float4*>((float*)d.aux + o) = make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+      for (int e = 0; e < 4; e++) v[e] = gelu_f(v[e]);
+    } else if (d.act == 2) {
+      const float4 u = *reinterpret_cast<const float4*>((const float*)d.aux + o);
+      v[0] *= gelu_grad_f(u.x); v[1] *= gelu_grad_f(u.y); v[2] *= gelu_grad_f(u.z); v[3] *= gelu_grad_f(u.w);
+    }
+    if (d.residual) {
+      const float4 r = *reinterpret_cast<const float4*>((const float*)d.residual + o);
+      v[0] += r.x; v[1] += r.y; v[2] += r.z; v[3] += r.w;
+    }
+    if (d.accumulate)
+      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(D + o), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+    else *reinterpret_cast<float4*>(D + o) = make_float4(v[0], v[1], v[2], v[3]);
+    return;
+  }
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    if (n + e >= d.N) return;
+    float x = v[e];
+    if (d.bias) x += d.bias[n + e];
+    if (d.act == 1) {
+      if (d.aux) ((float*)d.aux)[o + e] = x;
+      x = gelu_f(x);
+    } else if (d.act == 2) {
+      x *= gelu_grad_f(((const float*)d.aux)[o + e]);
+    }
+    if (d.residual) x += ((const float*)d.residual)[o + e];
+    if (d.accumulate) atomicAdd(D + o + e, x); else D[o + e] = x;
+  }
+}
+
+// Partial tiles [BMT][BNT] (rows PITCH floats apart) of the blocks of a cluster are added in rank order;
+// each block finishes its share of the rows.  Without a split the tile just leaves through the epilogue.
+template <int BMT, int BNT, int NT, int PITCH = BNT>
+__device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int rank, float* tile, int64_t zoff, int m0, int n0) {
+  const uint32_t base = f32_smem(tile);
+  if (p.splits == 1) __syncthreads();
+  else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  const int share = BMT / p.splits;
+  for (int idx = threadIdx.x; idx < share * (BNT / 4); idx += NT) {
+    const int r = rank * share + idx / (BNT / 4), c = (idx % (BNT / 4)) * 4;
+    const uint32_t at = base + (uint32_t)(r * PITCH + c) * 4u;
+    if (p.splits == 1) {
+      epilogue4(p, zoff, m0 + r, n0 + c, *reinterpret_cast<const float4*>(tile + r * PITCH + c));
+      continue;
+    }
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < p.splits; q++) {
+      uint32_t far;
+      float4 t;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(far) : "r"(at), "r"(q));
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(far) : "memory");
+      s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+    }
+    epilogue4(p, zoff, m0 + r, n0 + c, s);
+  }
+  // no block leaves while its tile is read
+  if (p.splits > 1) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+}  // namespace
+}  // namespace mslt

@@ -83,6 +83,7 @@ struct Workspace {
   char *hm, *ut, *gt, *tm, *dlogits, *dtm, *dgt, *dhm;
   int *es_counts, *es_total, *es_start, *es_rank, *es_order, *es_blocksum, *es_hot;
   float* es_partial;  // embedding backward: rows sorted by token id
+  char *x3a, *x3b, *x3e;                    // fp32: bf16 planes of a product's operands, of the word table
   int *cu, *rows, *ptok, *pseg;             // packed batches: see kernels.h
   int* nsp_rowsrc;                          // NSP head: first-token row of every sequence
   char *cls, *up, *pooled, *dup, *dcls;     // [B,H] each
@@ -110,6 +111,8 @@ struct mslt_ctx {
   int n_chunks;
   // this call's batch is packed (its sequences have lengths): first rows and row counts on the device
   const int *cu, *rows;
+  const void* a_split;  // fp32: left operand whose planes the last product left in x3a
+  bool emb_split;       // fp32: x3e holds the planes of this call's word table
   int64_t launches;
   int Vp, num_sms;
   bool timing;
@@ -237,6 +240,12 @@ void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char
   const int64_t Vp = pad_to(a.vocab, 8);
   const int64_t P2 = (int64_t)a.max_batch * A * a.max_seq * a.max_seq;
   w.scalars = (int*)take(256);
+  if (a.dtype == 0) {
+    const int64_t wide = std::max(3 * H, F);
+    w.x3a = take(std::max(T * wide, R * std::max(Vp, H)) * 6);
+    w.x3b = take(std::max(std::max(wide * H, R * H), T * std::max(F, H)) * 6);
+    w.x3e = take((int64_t)a.vocab * H * 6);
+  }
   w.cu = (int*)take(((int64_t)a.max_batch + 1) * 4);
   w.rows = (int*)take(2 * 4);
   w.ptok = (int*)take(T * 4);
@@ -416,13 +425,42 @@ int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const voi
   return 0;
 }
 
-int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, int rows_are_k = 0) {
+// fp32 products that are large enough run on the tensor cores (gemm_f32x3.cu) on operands split into bf16
+// planes.  reuse_a: A is, unchanged, the left operand of the product before this one, so its planes may
+// still be there.  b_is_emb: B is the word table, whose planes are kept for the rest of the call.
+int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_emb, bool* done) {
+  *done = false;
+  const bool a_ready = reuse_a && c->a_split == d.A, b_ready = b_is_emb && c->emb_split;
+  c->a_split = a_ready ? d.A : nullptr;
+  if (!gemm_f32x3_wins(d, (a_ready ? 1 : 0) | (b_ready ? 2 : 0))) return 0;
+  Workspace& w = c->ws;
+  char* pb = b_is_emb ? w.x3e : w.x3b;
+  // the operands' storage, pitch included
+  const int64_t na = d.a_ks == 1 ? d.M * d.a_rs : d.K * d.a_ks, nb = d.b_ks == 1 ? d.N * d.b_rs : d.K * d.b_ks;
+  if (!a_ready) { launch_split3((const float*)d.A, w.x3a, na, c->st); c->launches++; }
+  if (!b_ready) { launch_split3((const float*)d.B, pb, nb, c->st); c->launches++; }
+  c->a_split = d.A;
+  if (b_is_emb) c->emb_split = true;
+  char err[256] = "";
+  int rc = gemm_f32x3_launch(d, w.x3a, pb, w.scalars, c->st, err);
+  if (rc) return fail(rc, "%s", err);
+  c->launches++;
+  *done = true;
+  return 0;
+}
+
+int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, int rows_are_k = 0, bool reuse_a = false,
+             bool b_is_emb = false) {
   if (d.M <= 0 || d.N <= 0 || d.K <= 0 || d.batch <= 0) return 0;
   char err[256] = "";
   const int64_t before = gemm_launches();
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
-  int rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k);
+  int rc = 0;
+  bool done = false;
+  if (!c->bf) rc = run_gemm_x3(c, d, reuse_a, b_is_emb, &done);
+  if (rc) return rc;
+  if (!done) rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({d.batch > 1 ? 1 : 0, 2.0 * d.M * d.N * (double)d.K * d.batch});
@@ -443,7 +481,7 @@ int linear_fwd(mslt_ctx* c, const void* x, int T, int K, int64_t w_off, int64_t 
   g.d.bias = Wv(c, b_off);
   g.d.act = act; g.d.aux = aux; g.d.residual = residual;
   g.d.d_fp32 = out_fp32 ? 1 : 0;
-  return run_gemm(c, g.d, rows);
+  return run_gemm(c, g.d, rows, 0, false, w_off == 0);  // the word table is the arena's first tensor
 }
 
 // dX[T,K] = dY[T,N] * W[N,K]  (optionally * gelu'(aux), + residual)
@@ -454,7 +492,7 @@ int linear_dgrad(mslt_ctx* c, const void* dy, int T, int N, int64_t lda, int64_t
   g.d.B = Wc(c, w_off); g.d.b_rs = 1; g.d.b_ks = K;
   g.d.D = dx; g.d.ldd = K;
   g.d.act = act; g.d.aux = aux; g.d.residual = residual;
-  return run_gemm(c, g.d, rows);
+  return run_gemm(c, g.d, rows, 0, true);  // its weight gradient, from the same dY, has just run
 }
 
 // dW[N,K] += dY[T,N]^T * X[T,K]   (fp32, into the zeroed gradient arena)
@@ -661,7 +699,7 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
       KL(PC_OTHER, 6.0 * R * H, launch_f32_to_bf16(w.dtm32, w.dtm, (int64_t)R * H, c->st));
     } else {
       g.d.D = w.dtm; g.d.ldd = H;
-      TRY(run_gemm(c, g.d));
+      TRY(run_gemm(c, g.d, nullptr, 0, false, true));
     }
   }
   if (full) {  // the shared word embedding moves only while every layer is trainable
@@ -669,7 +707,7 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
     g.d.A = w.dlogits; g.d.a_rs = 1; g.d.a_ks = Vp;
     g.d.B = w.tm; g.d.b_rs = 1; g.d.b_ks = H;
     g.d.D = G(c, toff(c, -1, "emb.word")); g.d.ldd = H; g.d.d_fp32 = 1; g.d.accumulate = 1;
-    TRY(run_gemm(c, g.d));
+    TRY(run_gemm(c, g.d, nullptr, 0, true));
   }
   KL(PC_LN_BWD, 3.0 * R * H * c->esz, launch_ln_bwd(c->bf, w.dtm, w.gt, w.hst, Wv(c, toff(c, -1, "head.ln.gamma")), w.dgt,
                    G(c, toff(c, -1, "head.ln.gamma")), G(c, toff(c, -1, "head.ln.beta")), nullptr, R, H, c->st));
@@ -730,6 +768,8 @@ int check_batch(mslt_ctx* c, int B, int S, int P) {
 // and take part in the products (25 to 38 % of a batch with lengths spread over a factor of two to four
 // is padding).  Decided per call; the row count itself stays on the device.
 void pack_batch(mslt_ctx* c, const int* seq_lens) {
+  c->a_split = nullptr;
+  c->emb_split = false;
   const bool on = seq_lens != nullptr && fused_attention(c);
   c->cu = on ? c->ws.cu : nullptr;
   c->rows = on ? c->ws.rows : nullptr;
@@ -802,6 +842,8 @@ int mslt_create(const mslt_arch* arch, void* dev_params, size_t param_bytes, voi
   c->comm_done = nullptr;
   c->pending_update = false;
   c->cu = c->rows = nullptr;
+  c->a_split = nullptr;
+  c->emb_split = false;
   memset(c->prof, 0, sizeof(c->prof));
   c->Vp = (int)pad_to(arch->vocab, 8);
   int dev = 0;

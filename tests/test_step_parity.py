@@ -215,3 +215,13 @@ def test_bf16_forward_zeroes_the_padding_of_a_packed_batch():
         assert PT.max_rel(hidden[b, :n], h_ref[b, :n]) < PT.TOL["bf16"]["hidden"]
         assert not hidden[b, n:].any()
     m.close()
+
+
+@pytest.mark.parametrize("layers,trainable,batch,seq", [(2, 1, 3, 72), (1, 1, 9, 128)])
+def test_fp32_base_shapes_on_split_operands(layers, trainable, batch, seq):
+    """BERT-Base widths in fp32: the linear products are large enough for the tensor-core form on
+    operands split into bf16 planes (ragged rows, k split over clusters, the vocabulary-long
+    contractions), held to the fp32 tolerances."""
+    cfg = I.scaled(I.CONFIGS["base_stage"], layers=layers, trainable=trainable, batch=batch, seq=seq, pred=11,
+                   dtype="fp32", varlen=(seq // 3, seq))
+    _run(cfg, steps=2, lr=1e-3)
