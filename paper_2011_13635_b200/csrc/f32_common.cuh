@@ -60,8 +60,9 @@ __device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int 
 }
 
 // Partial tiles [BMT][BNT] (rows PITCH floats apart) of the blocks of a cluster are added in rank order;
-// each block finishes its share of the rows.  Without a split the tile just leaves through the epilogue.
-template <int BMT, int BNT, int NT, int PITCH = BNT>
+// each block finishes its share of the rows.  A block may itself hold KG partial tiles, one after the
+// other.  Without a split the tile just leaves through the epilogue.
+template <int BMT, int BNT, int NT, int PITCH = BNT, int KG = 1>
 __device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int rank, float* tile, int64_t zoff, int m0, int n0) {
   const uint32_t base = f32_smem(tile);
   if (p.splits == 1) __syncthreads();
@@ -70,17 +71,24 @@ __device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int r
   for (int idx = threadIdx.x; idx < share * (BNT / 4); idx += NT) {
     const int r = rank * share + idx / (BNT / 4), c = (idx % (BNT / 4)) * 4;
     const uint32_t at = base + (uint32_t)(r * PITCH + c) * 4u;
-    if (p.splits == 1) {
-      epilogue4(p, zoff, m0 + r, n0 + c, *reinterpret_cast<const float4*>(tile + r * PITCH + c));
-      continue;
-    }
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int q = 0; q < p.splits; q++) {
+    if (p.splits == 1) {
+#pragma unroll
+      for (int g = 0; g < KG; g++) {
+        const float4 t = *reinterpret_cast<const float4*>(tile + g * BMT * PITCH + r * PITCH + c);
+        s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+      }
+    }
+    for (int q = 0; q < (p.splits > 1 ? p.splits : 0); q++) {
       uint32_t far;
-      float4 t;
       asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(far) : "r"(at), "r"(q));
-      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(far) : "memory");
-      s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+#pragma unroll
+      for (int g = 0; g < KG; g++) {
+        float4 t;
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(far + g * BMT * PITCH * 4) : "memory");
+        s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+      }
     }
     epilogue4(p, zoff, m0 + r, n0 + c, s);
   }

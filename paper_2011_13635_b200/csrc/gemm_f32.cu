@@ -4,8 +4,9 @@
 // 768 98.6 us, input gradient 1024 x 768 x 3072 120 us, weight gradients 3072 x 768 x 1024 92 us,
 // 160 x 768 x 30528 262 us; an average product of that step took 171 us in the 64 x 64 kernel with
 // unpipelined loads that this one replaces, one of the smallest configuration (512 x 128 x 512) 20 us,
-// now below 6.  The fp32 pipe is 50-67 % busy; 16 warps per SM with fragments of one k (128 registers),
-// packed multiply-adds along k and slices of 16 were no faster.
+// then 6, and with four groups of warps sharing the k of a 32 x 32 tile 3.1 to 6.0.  The fp32 pipe is
+// 50-67 % busy at 128 x 128; 16 warps per SM with fragments of one k (128 registers), packed
+// multiply-adds along k and slices of 16 were no faster.
 //
 // Bound by the fp32 pipe (128 lanes per SM) where there is work for every SM, by the serial chain of
 // k slices where there is not.  A block owns an output tile (128 x 128, 64 x 64 or 32 x 32) and walks
@@ -87,13 +88,15 @@ struct SliceLoader {
 
 __device__ __forceinline__ float pick(const float4& v, int e) { return e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w)); }
 
-// TM x TN outputs per thread; a warp is 4 (rows) x 8 (columns) threads, a block WM x WN warps.
-template <int TM, int TN, int WM, int WN, int STAGES, bool AMN, bool BMN, bool VEC>
-__global__ void __launch_bounds__(WM * WN * 32)
+// TM x TN outputs per thread; a warp is 4 (rows) x 8 (columns) threads, a tile WM x WN warps.  KG groups
+// of such warps share the k of every slice and add their tiles at the end: a small tile alone on an SM
+// is bound by the chain of multiply-adds of its few warps (32 x 32 with KG = 1: 34 cycles per k).
+template <int TM, int TN, int WM, int WN, int KG, int STAGES, bool AMN, bool BMN, bool VEC>
+__global__ void __launch_bounds__(WM * WN * KG * 32)
 gemm_f32_kernel(const F32Params p) {
-  constexpr int NT = WM * WN * 32, BMT = WM * 4 * TM, BNT = WN * 8 * TN;
+  constexpr int NT = WM * WN * KG * 32, BMT = WM * 4 * TM, BNT = WN * 8 * TN;
   constexpr int STAGE = (BMT + BNT) * FK;  // floats
-  static_assert(BMT * BNT <= STAGE * STAGES, "the partial tile reuses the ring");
+  static_assert(KG * BMT * BNT <= STAGE * STAGES, "the partial tile reuses the ring");
   extern __shared__ __align__(128) float f32_ring[];
   pdl_begin();
   const mslt_gemm_desc& d = p.d;
@@ -103,7 +106,7 @@ gemm_f32_kernel(const F32Params p) {
   const float* B = (const float*)d.B + zo * d.b_bo + zi * d.b_bi;
   const int64_t zoff = zo * d.d_bo + zi * d.d_bi;
   const int m0 = blockIdx.y * BMT, n0 = nt * BNT;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % (WM * WN), kg = (threadIdx.x >> 5) / (WM * WN);
   const int lr = lane >> 3, lc = lane & 7;
   const int row_t = (warp / WN) * 4 * TM + lr * 4, col_t = (warp % WN) * 8 * TN + lc * 4;
   const int kb_total = (d.K + FK - 1) / FK;
@@ -143,7 +146,8 @@ gemm_f32_kernel(const F32Params p) {
       return *reinterpret_cast<const float4*>(t + r * FK + 4 * (q ^ ((r >> 2) & 7)));
     };
 #pragma unroll
-    for (int q = 0; q < FK / 4; q++) {
+    for (int qi = 0; qi < FK / 4 / KG; qi++) {
+      const int q = kg * (FK / 4 / KG) + qi;
       // fragments of four k: a k-contiguous operand gives four k of one row per 16 bytes, a
       // row-contiguous one four rows of one k
       float4 a[TM], b[TN];
@@ -183,7 +187,7 @@ gemm_f32_kernel(const F32Params p) {
   }
   auto out4 = [&](int i, int h) { return make_float4(acc[i][2 * h].x, acc[i][2 * h].y, acc[i][2 * h + 1].x, acc[i][2 * h + 1].y); };
   cp_wait<0>();
-  if (p.splits == 1) {
+  if (KG == 1 && p.splits == 1) {
 #pragma unroll
     for (int i = 0; i < TM; i++)
 #pragma unroll
@@ -196,8 +200,8 @@ gemm_f32_kernel(const F32Params p) {
   for (int i = 0; i < TM; i++)
 #pragma unroll
     for (int h = 0; h < TN / 4; h++)
-      *reinterpret_cast<float4*>(f32_ring + (row_t + (i >> 2) * 16 + (i & 3)) * BNT + col_t + h * 32) = out4(i, h);
-  cluster_add_and_finish<BMT, BNT, NT>(p, rank, f32_ring, zoff, m0, n0);
+      *reinterpret_cast<float4*>(f32_ring + kg * BMT * BNT + (row_t + (i >> 2) * 16 + (i & 3)) * BNT + col_t + h * 32) = out4(i, h);
+  cluster_add_and_finish<BMT, BNT, NT, BNT, KG>(p, rank, f32_ring, zoff, m0, n0);
 }
 
 typedef void (*F32Fn)(const F32Params);
@@ -207,9 +211,10 @@ typedef void (*F32Fn)(const F32Params);
     {gemm_f32_kernel<__VA_ARGS__, false, true, false>, gemm_f32_kernel<__VA_ARGS__, false, true, true>}},    \
    {{gemm_f32_kernel<__VA_ARGS__, true, false, false>, gemm_f32_kernel<__VA_ARGS__, true, false, true>},     \
     {gemm_f32_kernel<__VA_ARGS__, true, true, false>, gemm_f32_kernel<__VA_ARGS__, true, true, true>}}}
-const F32Fn kF32[3][2][2][2] = {F32_SET(8, 8, 4, 2, 3), F32_SET(8, 8, 2, 1, 3), F32_SET(4, 4, 2, 1, 4)};
+// 128 x 128, 64 x 64, 32 x 32 with shared k (few tiles), 32 x 32 (many, in batches)
+const F32Fn kF32[4][2][2][2] = {F32_SET(8, 8, 4, 2, 1, 3), F32_SET(8, 8, 2, 1, 1, 3), F32_SET(4, 4, 2, 1, 4, 6), F32_SET(4, 4, 2, 1, 1, 4)};
 #undef F32_SET
-constexpr int kTile[3] = {128, 64, 32}, kThreads[3] = {256, 64, 64}, kStages[3] = {3, 3, 4};
+constexpr int kTile[4] = {128, 64, 32, 32}, kThreads[4] = {256, 64, 256, 64}, kStages[4] = {3, 3, 6, 4};
 
 constexpr int kMaxDevices = 64;
 struct { int sms = 0; } g_dev[kMaxDevices];
@@ -231,7 +236,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   {
     std::lock_guard<std::mutex> lock(g_dev_mu);
     if (g_dev[dev].sms == 0) {
-      for (int t = 0; t < 3; t++)
+      for (int t = 0; t < 4; t++)
         for (int i = 0; i < 8; i++) {
           cudaError_t e = cudaFuncSetAttribute((const void*)kF32[t][i >> 2][(i >> 1) & 1][i & 1], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                2 * kTile[t] * FK * 4 * kStages[t]);
@@ -247,21 +252,26 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   // every product of BERT-Base at 1024 tokens and of the small configurations.  A block alone on an
   // SM takes `alone` cycles per k, n blocks share the fp32 pipe at `share` cycles each: measured 58 %
   // of the pipe for 128 x 128 (k-contiguous B), 67 % (row-contiguous B, packed multiply-adds), 60 %
-  // for 64 x 64 (row-contiguous B only: 45 % otherwise), 50 % for 32 x 32.
+  // for 64 x 64 (row-contiguous B only: 45 % otherwise); 32 x 32 is bound by its chain of slices.
   const bool amn = d.a_rs == 1 && d.a_ks != 1, bmn = d.b_rs == 1 && d.b_ks != 1;
   const int kb_total = (d.K + FK - 1) / FK;
   int t = 2, s = 1;
   double best = 1e30;
-  for (int ti = 0; ti < 3; ti++) {
+  for (int ti = 0; ti < 4; ti++) {
     const long long tiles = (long long)((d.M + kTile[ti] - 1) / kTile[ti]) * ((d.N + kTile[ti] - 1) / kTile[ti]) * d.batch;
-    const double share = ti == 0 ? (bmn ? 190. : 220.) : ti == 1 ? (bmn ? 53. : 72.) : 16.;
-    const double alone = ti == 0 ? share : ti == 1 ? 130. : 34., per_block = ti == 0 ? 3000. : ti == 1 ? 600. : 150.,
-                 per_split = ti == 0 ? 6000. : ti == 1 ? 1500. : 400.;  // exchange of the partial tile
+    const double share = ti == 0 ? (bmn ? 190. : 220.) : ti == 1 ? (bmn ? 53. : 72.) : ti == 2 ? (bmn ? 16. : 22.) : 16.;
+    // products with a batch read short rows of wide matrices: 64 x 64 took 22.8 us on 96 x (128 x 128 x 64)
+    // inside a step, 32 x 32 without shared k 11.2
+    if (ti == 1 && d.batch > 1) continue;
+    const double alone = ti == 0 ? share : ti == 1 ? 130. : ti == 2 ? 23. : 34.;
+    const double per_block = ti == 0 ? 3000. : ti == 1 ? 600. : ti == 2 ? 700. : 150.;
     for (int si = 1; si <= 8 && (si == 1 || kb_total >= si); si *= 2) {
+      const double per_split = ti == 0 ? 6000. : ti == 1 ? 1500. : ti == 2 ? 1000. + 400. * si : 2000.;  // exchange of the partial tile
       // one 128 x 128 block fits an SM, so clusters of four and eight leave SMs of a GPC unused
       const int units = ti == 0 && si >= 4 ? sms * (si == 4 ? 8 : 7) / 9 : sms;
       const double n = (double)((tiles * si + units - 1) / units);
-      const double c = (kb_total + si - 1) / si * FK * (n * share > alone ? n * share : alone) + n * (per_block + (si > 1 ? per_split : 0.));
+      const double c = (kb_total + si - 1) / si * FK * (n * share > alone ? n * share : alone) + n * (per_block + (si > 1 ? per_split : 0.)) +
+                       (ti == 3 ? 3000. : 0.);  // its short rows of threads start and end slowly
       if (c < best) { best = c; t = ti; s = si; }
     }
   }
