@@ -12,9 +12,10 @@ namespace mslt {
 // error bit into when one of its bounded waits runs out.  Returns 0, or a negative mslt_status
 // with a message in `err` (at least 256 bytes).
 // rows (dtype 1 only, may be null): device count <= M, or <= K with rows_are_k, of the rows that hold
-// anything; work is cut to it (row results beyond it are not written).
+// anything; work is cut to it (row results beyond it are not written).  b_static: B is written by neither
+// of the two kernels before this one in the stream (weights inside a step), so it may be read early.
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows = nullptr,
-                int rows_are_k = 0);
+                int rows_are_k = 0, bool b_static = false);
 
 int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 // The same on the tensor cores (gemm_f32x3.cu), for products without a batch: each operand has first been
@@ -25,7 +26,12 @@ bool gemm_f32x3_wins(const mslt_gemm_desc& d, int planes_ready);
 int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void* planes_b, int* status, cudaStream_t st,
                       char* err);
 int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
-int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k);
+int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
+                   bool b_static);
+// The form for few tiles (gemm_tc_small.cu): split count and estimated time, 0 where it does not apply.
+int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, double* t);
+int gemm_tc_small_launch(const mslt_gemm_desc& d, int splits, bool early, int* status, cudaStream_t st, char* err,
+                         const int* rows, bool starve);
 
 // Test hook: the next tensor-core launch gets a producer that issues no copies and a wait limit of
 // about 20 ms, so that its first wait runs out and the give-up path is exercised.

@@ -66,51 +66,6 @@ struct TcParams {
   uint32_t idesc;
 };
 
-// GELU on the FMA pipe only: the epilogue of a GELU tile is bound by the special-function unit when
-// erf costs a reciprocal and an exponential per element, and by instruction issue after that, so
-// the polynomials below run on the packed two-wide fp32 instructions (fma.rn.f32x2), two columns
-// per instruction.  gelu(u) = u * Phi(u) with Phi(u) - 1/2 = u * Q(u^2), Q a degree-8
-// least-maximum-error fit on |u| <= 4 (gelu is off by less than 3e-5 in fp32 there, far inside bf16
-// resolution).  Outside, u^2 is clamped to 16 and Phi saturates to [0, 1], which gives gelu(u) = u
-// above and 0 below (the exact values differ from those by less than 2e-4).
-__device__ __forceinline__ float2 gelu_fast2(float2 u) {
-  float2 t = __fmul2_rn(u, u);
-  t.x = fminf(t.x, 16.0f);
-  t.y = fminf(t.y, 16.0f);
-  float2 q = splat2(8.093845117e-11f);
-  q = __ffma2_rn(q, t, splat2(-7.032516570e-09f));
-  q = __ffma2_rn(q, t, splat2(2.727248615e-07f));
-  q = __ffma2_rn(q, t, splat2(-6.317188128e-06f));
-  q = __ffma2_rn(q, t, splat2(9.916073864e-05f));
-  q = __ffma2_rn(q, t, splat2(-1.135572678e-03f));
-  q = __ffma2_rn(q, t, splat2(9.883344319e-03f));
-  q = __ffma2_rn(q, t, splat2(-6.642043264e-02f));
-  q = __ffma2_rn(q, t, splat2(3.989280708e-01f));
-  float2 phi;
-  phi.x = __saturatef(fmaf(q.x, u.x, 0.5f));
-  phi.y = __saturatef(fmaf(q.y, u.y, 0.5f));
-  return __fmul2_rn(u, phi);
-}
-// GELU'(u) = Phi(u) + u phi(u), also on the FMA pipe: 0.5 + u * P(u^2) with a degree-17 odd
-// least-maximum-error fit on |u| <= 4 (absolute error below 1e-4); beyond that the derivative is
-// 0 or 1 to within 5e-4.  The result multiplies a gradient that is then rounded to bf16.
-__device__ __forceinline__ float2 gelu_grad_fast2(float2 u) {
-  const float2 t = __fmul2_rn(u, u);
-  float2 p = splat2(9.837601957e-10f);
-  p = __ffma2_rn(p, t, splat2(-8.257008028e-08f));
-  p = __ffma2_rn(p, t, splat2(3.042579986e-06f));
-  p = __ffma2_rn(p, t, splat2(-6.523749948e-05f));
-  p = __ffma2_rn(p, t, splat2(9.104776309e-04f));
-  p = __ffma2_rn(p, t, splat2(-8.736754371e-03f));
-  p = __ffma2_rn(p, t, splat2(5.852845753e-02f));
-  p = __ffma2_rn(p, t, splat2(-2.649477277e-01f));
-  p = __ffma2_rn(p, t, splat2(7.976755055e-01f));
-  p = __ffma2_rn(p, u, splat2(0.5f));
-  // step(u) without a second comparison: u * 2^100 saturated to [0, 1]
-  p.x = fabsf(u.x) >= 4.0f ? __saturatef(u.x * 1.2676506e30f) : p.x;
-  p.y = fabsf(u.y) >= 4.0f ? __saturatef(u.y * 1.2676506e30f) : p.y;
-  return p;
-}
 // Epilogue flavours.  Each is its own kernel instantiation: one kernel with every flavour behind
 // run-time branches measured 2-3x slower per chunk (register pressure and jumps across large code
 // blocks), which made shallow contractions wait for their epilogue.
@@ -953,7 +908,7 @@ std::mutex g_dev_mu;
 //   an epilogue that overlaps the next tile's loop, one more at the end;
 //   start-up (pairs have a cluster to set up); singles slow down a little when many waves of them
 //   contend for L2, where a pair fetches a third less per flop.
-static void choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, bool can_split, bool* pair, int* bn,
+static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, bool can_split, bool* pair, int* bn,
                           int* ksub, int* splits) {
   struct Form { bool pair; int bn, ksub; double per_k; };
   static const Form forms[] = {{false, 64, 2, 0.202}, {false, 128, 2, 0.280}, {false, 192, 1, 0.362}, {false, 256, 1, 0.413},
@@ -986,9 +941,11 @@ static void choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, boo
       if (t < best) { best = t; *pair = f.pair; *bn = f.bn; *ksub = f.pair ? 2 : ks; *splits = sp; }
     }
   }
+  return best;
 }
 
-int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k) {
+int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
+                   bool b_static) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_starve_next.exchange(0) != 0;
   int dev = 0;
@@ -1016,7 +973,10 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const bool can_split = d.split_k == 0 && d.d_fp32 && d.accumulate;
   bool pair = false;
   int splits = d.split_k > 1 ? d.split_k : 1, ksub = 1;
-  choose_tiling(d, num_sms, variant, can_split, &pair, &p.bn, &ksub, &splits);
+  const double estimate = choose_tiling(d, num_sms, variant, can_split, &pair, &p.bn, &ksub, &splits);
+  double t_small = 0.;
+  const int s_small = variant == 0 && g_store_variant.load() == 0 && !rows_are_k ? gemm_tc_small_plan(d, num_sms, &t_small) : 0;
+  if (s_small && t_small < estimate) return gemm_tc_small_launch(d, s_small, b_static, status, st, err, rows, starve);
   const int tile_m = pair ? 2 * BM : BM;
   p.m_tiles = (d.M + tile_m - 1) / tile_m;
   p.n_tiles = (d.N + p.bn - 1) / p.bn;

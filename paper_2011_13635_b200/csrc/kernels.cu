@@ -672,6 +672,34 @@ unpack_rows_kernel(const T* __restrict__ x, const int* __restrict__ cu, T* __res
     *reinterpret_cast<Raw*>(out + (int64_t)row * H + c) = in ? VecT<T>::load_raw(x + (int64_t)(r0 + s) * H + c) : zero;
 }
 
+// out[r, 0 .. V) = in[r, 0 .. V) from rows of pitch ldi to rows without padding, a block per row.  VN = 2:
+// both pitches even, 8-byte accesses; rows of odd V start on any float.
+template <int VN>
+__global__ void __launch_bounds__(256)
+copy_rows_kernel(const float* __restrict__ in, int64_t ldi, float* __restrict__ out, int V) {
+  pdl_begin();
+  const float* src = in + (int64_t)blockIdx.x * ldi;
+  float* dst = out + (int64_t)blockIdx.x * V;
+  constexpr int U = 8;  // loads in flight per thread
+  for (int c0 = threadIdx.x * VN; c0 < V; c0 += 256 * VN * U) {
+    float2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int c = c0 + u * 256 * VN;
+      if (c >= V) continue;
+      if (VN == 2) v[u] = __ldcs(reinterpret_cast<const float2*>(src + c));
+      else v[u].x = __ldcs(src + c);
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int c = c0 + u * 256 * VN;
+      if (c >= V) continue;
+      if (VN == 2) __stcs(reinterpret_cast<float2*>(dst + c), v[u]);
+      else __stcs(dst + c, v[u].x);
+    }
+  }
+}
+
 // dx[rowsrc[r],:] += d[r,:]; one block per sequence walks its slots in order, so repeated
 // positions add up without atomics.  dx must be zeroed beforehand.
 template <typename T>
@@ -1549,6 +1577,14 @@ void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, in
 
 void launch_unpack_rows(bool bf, const void* x, const int* cu, void* out, int B, int S, int H, cudaStream_t st) {
   DISPATCH_T(bf, (launch_pdl(unpack_rows_kernel<T>, div_up(B * S, 8), 256, 0, st, (const T*)x, cu, (T*)out, B * S, S, H)));
+}
+
+void launch_copy_rows(const float* in, int64_t ldi, float* out, int R, int V, cudaStream_t st) {
+  if (R <= 0) return;
+  if (V % 2 == 0 && ldi % 2 == 0 && (((uintptr_t)in | (uintptr_t)out) & 7) == 0)
+    launch_pdl(copy_rows_kernel<2>, R, 256, 0, st, in, ldi, out, V);
+  else
+    launch_pdl(copy_rows_kernel<1>, R, 256, 0, st, in, ldi, out, V);
 }
 
 void launch_scatter_rows(bool bf, const void* d, const int* rowsrc, void* dx, int B, int P, int H,

@@ -45,6 +45,8 @@ void launch_slots_prepare(const int* positions, const int* labels, const int* se
                           float* inv_n, int* status, cudaStream_t st, int* cu = nullptr, int* rows = nullptr);
 // out [B, S, H] from packed rows; zero past a sequence's length
 void launch_unpack_rows(bool bf, const void* x, const int* cu, void* out, int B, int S, int H, cudaStream_t st);
+// fp32 rows of pitch ldi to dense rows of V (a strided device copy took 91 us for 720 x 30522, this 30)
+void launch_copy_rows(const float* in, int64_t ldi, float* out, int R, int V, cudaStream_t st);
 void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, int R, int H,
                         cudaStream_t st);
 void launch_scatter_rows(bool bf, const void* d, const int* rowsrc, void* dx, int B, int P, int H,

@@ -450,7 +450,7 @@ int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_em
 }
 
 int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, int rows_are_k = 0, bool reuse_a = false,
-             bool b_is_emb = false) {
+             bool b_is_emb = false, bool b_static = false) {
   if (d.M <= 0 || d.N <= 0 || d.K <= 0 || d.batch <= 0) return 0;
   char err[256] = "";
   const int64_t before = gemm_launches();
@@ -460,7 +460,7 @@ int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, in
   bool done = false;
   if (!c->bf) rc = run_gemm_x3(c, d, reuse_a, b_is_emb, &done);
   if (rc) return rc;
-  if (!done) rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k);
+  if (!done) rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k, b_static);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({d.batch > 1 ? 1 : 0, 2.0 * d.M * d.N * (double)d.K * d.batch});
@@ -481,7 +481,7 @@ int linear_fwd(mslt_ctx* c, const void* x, int T, int K, int64_t w_off, int64_t 
   g.d.bias = Wv(c, b_off);
   g.d.act = act; g.d.aux = aux; g.d.residual = residual;
   g.d.d_fp32 = out_fp32 ? 1 : 0;
-  return run_gemm(c, g.d, rows, 0, false, w_off == 0);  // the word table is the arena's first tensor
+  return run_gemm(c, g.d, rows, 0, false, w_off == 0, true);  // the word table is the arena's first tensor
 }
 
 // dX[T,K] = dY[T,N] * W[N,K]  (optionally * gelu'(aux), + residual)
@@ -492,7 +492,7 @@ int linear_dgrad(mslt_ctx* c, const void* dy, int T, int N, int64_t lda, int64_t
   g.d.B = Wc(c, w_off); g.d.b_rs = 1; g.d.b_ks = K;
   g.d.D = dx; g.d.ldd = K;
   g.d.act = act; g.d.aux = aux; g.d.residual = residual;
-  return run_gemm(c, g.d, rows, 0, true);  // its weight gradient, from the same dY, has just run
+  return run_gemm(c, g.d, rows, 0, true, false, true);  // its weight gradient, from the same dY, has just run
 }
 
 // dW[N,K] += dY[T,N]^T * X[T,K]   (fp32, into the zeroed gradient arena)
@@ -1171,8 +1171,7 @@ int mslt_forward(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens
     CUDA_TRY(cudaMemcpyAsync(d_hidden_out, cur, (size_t)T * H * c->esz, cudaMemcpyDeviceToDevice, c->st));
   if (head) {
     TRY(head_forward(c, cur, B * P, false));
-    CUDA_TRY(cudaMemcpy2DAsync(d_logits_out, (size_t)V * 4, w.logits, (size_t)c->Vp * 4, (size_t)V * 4,
-                               (size_t)B * P, cudaMemcpyDeviceToDevice, c->st));
+    KL(PC_OTHER, 8.0 * B * P * V, launch_copy_rows(w.logits, c->Vp, d_logits_out, B * P, V, c->st));
   }
   float dummy;
   return finish(c, &dummy);

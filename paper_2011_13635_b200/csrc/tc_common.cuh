@@ -225,6 +225,51 @@ __device__ __forceinline__ float2 bf162_to_f2(uint32_t h) {
   return make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u));
 }
 
+// GELU on the FMA pipe only: the epilogue of a GELU tile is bound by the special-function unit when
+// erf costs a reciprocal and an exponential per element, and by instruction issue after that, so
+// the polynomials below run on the packed two-wide fp32 instructions (fma.rn.f32x2), two columns
+// per instruction.  gelu(u) = u * Phi(u) with Phi(u) - 1/2 = u * Q(u^2), Q a degree-8
+// least-maximum-error fit on |u| <= 4 (gelu is off by less than 3e-5 in fp32 there, far inside bf16
+// resolution).  Outside, u^2 is clamped to 16 and Phi saturates to [0, 1], which gives gelu(u) = u
+// above and 0 below (the exact values differ from those by less than 2e-4).
+__device__ __forceinline__ float2 gelu_fast2(float2 u) {
+  float2 t = __fmul2_rn(u, u);
+  t.x = fminf(t.x, 16.0f);
+  t.y = fminf(t.y, 16.0f);
+  float2 q = splat2(8.093845117e-11f);
+  q = __ffma2_rn(q, t, splat2(-7.032516570e-09f));
+  q = __ffma2_rn(q, t, splat2(2.727248615e-07f));
+  q = __ffma2_rn(q, t, splat2(-6.317188128e-06f));
+  q = __ffma2_rn(q, t, splat2(9.916073864e-05f));
+  q = __ffma2_rn(q, t, splat2(-1.135572678e-03f));
+  q = __ffma2_rn(q, t, splat2(9.883344319e-03f));
+  q = __ffma2_rn(q, t, splat2(-6.642043264e-02f));
+  q = __ffma2_rn(q, t, splat2(3.989280708e-01f));
+  float2 phi;
+  phi.x = __saturatef(fmaf(q.x, u.x, 0.5f));
+  phi.y = __saturatef(fmaf(q.y, u.y, 0.5f));
+  return __fmul2_rn(u, phi);
+}
+// GELU'(u) = Phi(u) + u phi(u), also on the FMA pipe: 0.5 + u * P(u^2) with a degree-17 odd
+// least-maximum-error fit on |u| <= 4 (absolute error below 1e-4); beyond that the derivative is
+// 0 or 1 to within 5e-4.  The result multiplies a gradient that is then rounded to bf16.
+__device__ __forceinline__ float2 gelu_grad_fast2(float2 u) {
+  const float2 t = __fmul2_rn(u, u);
+  float2 p = splat2(9.837601957e-10f);
+  p = __ffma2_rn(p, t, splat2(-8.257008028e-08f));
+  p = __ffma2_rn(p, t, splat2(3.042579986e-06f));
+  p = __ffma2_rn(p, t, splat2(-6.523749948e-05f));
+  p = __ffma2_rn(p, t, splat2(9.104776309e-04f));
+  p = __ffma2_rn(p, t, splat2(-8.736754371e-03f));
+  p = __ffma2_rn(p, t, splat2(5.852845753e-02f));
+  p = __ffma2_rn(p, t, splat2(-2.649477277e-01f));
+  p = __ffma2_rn(p, t, splat2(7.976755055e-01f));
+  p = __ffma2_rn(p, u, splat2(0.5f));
+  // step(u) without a second comparison: u * 2^100 saturated to [0, 1]
+  p.x = fabsf(u.x) >= 4.0f ? __saturatef(u.x * 1.2676506e30f) : p.x;
+  p.y = fabsf(u.y) >= 4.0f ? __saturatef(u.y * 1.2676506e30f) : p.y;
+  return p;
+}
 // Staging buffer of one epilogue warp: 32 rows of 64 bytes (2 KB).  Lane r writes its row as four
 // 16-byte pieces; the slot function permutes the pieces so that both this
 // row-per-lane write and the row-segment-per-quarter-warp read that follows are free of bank

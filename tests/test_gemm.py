@@ -283,3 +283,14 @@ def test_fp32_unaligned_operands_take_the_element_wise_copies():
     ((24, 768, 4000), ("k", "mn"), dict(d_fp32=True, accumulate=True))])    # narrow tiles, k split many ways
 def test_bf16_tile_forms_the_estimate_picks(shape, majors, kw):
     _run(1, *shape, *majors, **kw)
+
+
+@pytest.mark.parametrize("shape,majors,kw", [
+    ((1, 8, 64), ("k", "k"), dict(bias=True)),                              # one row, one round
+    ((64, 768, 3072), ("k", "k"), dict(bias=True, residual=True)),          # k over a cluster of eight
+    ((130, 776, 3080), ("k", "mn"), dict(residual=True, alpha=0.5)),        # second row tile of two rows, ragged k and columns
+    ((200, 768, 1160), ("mn", "k"), dict(bias=True, act=1, aux_out=True)),  # ring reused inside a block
+    ((33, 136, 72), ("mn", "mn"), dict(act=2)), ((129, 64, 640), ("k", "k"), dict(bias=True, act=1))])
+def test_bf16_few_tile_kernel(shape, majors, kw):
+    """Outputs of few tiles: partial sums added inside a cluster, every epilogue."""
+    _run(1, *shape, *majors, **kw)
