@@ -386,15 +386,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   }
 }
 
-// ---- forward for rows of 129..512 keys -----------------------------------------------------------
+// ---- forward for rows of 129..512 keys that stores the probabilities (single-kernel entry point) -----------------------------------------------------------
 // A work item is (sequence, head, tile of 128 queries); the keys come in blocks of 128.  The scores
-// of a row do not fit tensor memory next to the context, so an item runs two passes over the key
-// blocks.  When the probabilities are wanted: pass 1 forms the row maximum and the sum of
-// exponentials (S = Q K_j^T only), pass 2 forms the scores again, writes P_j = exp(.)/sum as bf16
-// and accumulates C += P_j V_j: an exact softmax with no rescaling of the context, and
-// probabilities that can be stored as they are.  When they are not wanted (a frozen layer), pass 1
-// forms the maximum only, pass 2 uses exp(s - max) as it is, sums it on the way, and the context
-// is divided by the sum at the end: half the exponentials.
+// of a row do not fit tensor memory next to two context accumulators, so an item runs two passes over
+// the key blocks: pass 1 forms the row maximum and the sum of exponentials (S = Q K_j^T only), pass 2
+// forms the scores again, writes P_j = exp(.)/sum as bf16 and accumulates C += P_j V_j: probabilities
+// that can be stored as they are.
 // Each of the two softmax groups owns every second item of the CTA, whole: its own Q tile, ring of
 // K / V tiles, score and context accumulators, P block, producer thread and MMA-issuing thread.  A
 // thread owns one query row of its group's item through all key blocks, so nothing is exchanged
@@ -407,7 +404,6 @@ constexpr int AL_P_BYTES = 2 * AT_TILE_BYTES;    // P_j as an MMA operand: 32 KB
 constexpr int AL_BARS_PER_GROUP = 4 + 2 * AL_RING + 6;
 constexpr long long AL_GROUP_SKEW_CYCLES = 2000;
 
-template <bool kPacked>
 __global__ void __launch_bounds__(AL_THREADS, 1)
 attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -471,7 +467,6 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   uint8_t* my_q = q_smem + g * AT_TILE_BYTES;
   uint8_t* my_ring = ring_smem + (size_t)g * AL_RING * AT_TILE_BYTES;
   uint8_t* my_p = p_smem + (size_t)g * AL_P_BYTES;
-  const bool want_p = p.P != nullptr;
   // Tiles of an item in the order the MMA thread uses them: pass 1: K_0 .. K_{n-1}; pass 2: K_0, then
   // (K_j, V_{j-1}) for j = 1 .. n-1, then V_{n-1} (the scores of block j are issued before the second
   // product of block j - 1, which has to wait for that block's probabilities).
@@ -489,9 +484,8 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const int nkb = (len + 127) >> 7;
       if (!mbar_wait(qempty, (ig & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
       ig++;
-      const int row0 = kPacked ? p.cu[zo] : 0, zseq = kPacked ? 0 : zo;
       int c[4];
-      c[0] = 0; c[p.q_perm[0]] = row0 + qt * 128; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zseq;
+      c[0] = 0; c[p.q_perm[0]] = qt * 128; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zo;
       mbar_expect_tx(qfull, AT_TILE_BYTES);
       tma_load_4d(smem_u32(my_q), &tmQ, qfull, c[0], c[1], c[2], c[3]);
       for (int idx = 0; idx < 3 * nkb; idx++, tt++) {
@@ -511,7 +505,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         mbar_expect_tx(fb, AT_TILE_BYTES);
         const int* perm = is_v ? p.v_perm : p.k_perm;
         c[0] = 0; c[1] = 0; c[2] = 0; c[3] = 0;
-        c[perm[0]] = row0 + j * 128; c[perm[1]] = zi; c[perm[2]] = zseq;
+        c[perm[0]] = j * 128; c[perm[1]] = zi; c[perm[2]] = zo;
         tma_load_4d(smem_u32(my_ring + (size_t)slot * AT_TILE_BYTES), is_v ? &tmV : &tmK, fb, c[0], c[1], c[2], c[3]);
       }
     }
@@ -614,20 +608,16 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const int zo = zh / p.heads, zi = zh - zo * p.heads;
       const int len = item_len(zo);
       float2 v[4][16];
-      const int row0 = kPacked ? p.cu[zo] : zo * p.S;
-      const int rlim = kPacked ? len : p.S;  // rows of the sequence that exist
-      bf16* cg = p.C + (long long)(row0 + qt * 128) * p.c_ld + zi * p.c_bi;
-      bf16* pg = want_p ? p.P + zo * p.p_bo + zi * p.p_bi + (long long)qt * 128 * p.S : nullptr;
+      bf16* cg = p.C + zo * p.c_bo + zi * p.c_bi + (long long)qt * 128 * p.c_ld;
+      bf16* pg = p.P + zo * p.p_bo + zi * p.p_bi + (long long)qt * 128 * p.S;
       if (qt * 128 >= len) {
-        if (kPacked) continue;
         // a query tile in the padding: zero context rows (finite, so that masked reads stay harmless)
 #pragma unroll
         for (int e = 0; e < 16; e++) v[0][e] = make_float2(0.f, 0.f);
         stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, p.S - qt * 128, 64, p.vec_ok_c);
         stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 32, p.S - qt * 128, 64, p.vec_ok_c);
-        if (pg != nullptr)
-          for (int n0 = 0; n0 < p.S; n0 += 32)
-            stage_store_bf16(stg, lane, v[0], pg, p.S, q * 32, n0, p.S - qt * 128, p.S, p.vec_ok_p);
+        for (int n0 = 0; n0 < p.S; n0 += 32)
+          stage_store_bf16(stg, lane, v[0], pg, p.S, q * 32, n0, p.S - qt * 128, p.S, p.vec_ok_p);
         continue;
       }
       const int nkb = (len + 127) >> 7;
@@ -658,14 +648,14 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         bm = fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3]));
         return true;
       };
-      // pass 1: running maximum of the raw scores; with probabilities wanted also the running sum
+      // pass 1: running maximum of the raw scores and running sum
       // of 2^((s - max) * scale * log2 e)
       float mr = -INFINITY, l = 0.f;
       for (int j = 0; j < nkb && ok; j++) {
         float bm;
         if (!load_block(j, bm)) { ok = false; break; }
         const float mn = fmaxf(mr, bm);
-        if (want_p && mn != -INFINITY) {
+        if (mn != -INFINITY) {
           const float2 nm2 = splat2(-mn * sl2);
           float2 sc[4];
 #pragma unroll
@@ -685,8 +675,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       if (!ok) break;
       // mr is finite: at least one key of the row is valid
       const float2 nM2 = splat2(-mr * sl2);
-      const float2 inv = splat2(want_p ? 1.0f / l : 1.0f);
-      float2 ls = make_float2(0.f, 0.f);  // without stored probabilities: the sum, formed in pass 2
+      const float2 inv = splat2(1.0f / l);
       // pass 2
       for (int j = 0; j < nkb && ok; j++) {
         float bm;
@@ -697,12 +686,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
           for (int e = 0; e < 16; e++) {
             const float2 a = __ffma2_rn(v[c][e], k2, nM2);
             const float2 ex = make_float2(fast_exp2(a.x), fast_exp2(a.y));
-            if (want_p) {
-              v[c][e] = __fmul2_rn(ex, inv);
-            } else {
-              v[c][e] = ex;
-              ls = __fadd2_rn(ls, ex);
-            }
+            v[c][e] = __fmul2_rn(ex, inv);
           }
         // the group's P block is free once its previous second product has read it
         if (!mbar_wait(pfree, (pv & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
@@ -754,24 +738,306 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(oempty);
-      if (p.lse && qt * 128 + r < rlim)
-        p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = mr * sl2 + log2f(want_p ? l : ls.x + ls.y);
-      if (!want_p) {
-        const float2 il = splat2(1.0f / (ls.x + ls.y));
-#pragma unroll
-        for (int e = 0; e < 16; e++) {
-          v[0][e] = __fmul2_rn(v[0][e], il);
-          v[1][e] = __fmul2_rn(v[1][e], il);
-        }
-      }
       if (p.fast_c) {
-        if (qt * 128 + r < rlim) {
+        if (qt * 128 + r < p.S) {
           store_row32_bf16(cg + (long long)r * p.c_ld, v[0]);
           store_row32_bf16(cg + (long long)r * p.c_ld + 32, v[1]);
         }
       } else {
-        stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, rlim - qt * 128, 64, p.vec_ok_c);
-        stage_store_bf16(stg, lane, v[1], cg, p.c_ld, q * 32, 32, rlim - qt * 128, 64, p.vec_ok_c);
+        stage_store_bf16(stg, lane, v[0], cg, p.c_ld, q * 32, 0, p.S - qt * 128, 64, p.vec_ok_c);
+        stage_store_bf16(stg, lane, v[1], cg, p.c_ld, q * 32, 32, p.S - qt * 128, 64, p.vec_ok_c);
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(AT_TMEM_COLS)
+                 : "memory");
+  }
+}
+
+// ---- forward for rows of 129..512 keys, no probabilities stored -----------------------------------
+// A work item is (sequence, head, tile of 128 queries).  Tensor memory holds the scores of a whole row
+// (four blocks of 128 keys), so they are formed once: all eight softmax warps read them twice, first for
+// the row maximum, then for the exponentials, and the context accumulates over columns whose scores have
+// been used up (block 0 when there are four blocks, else the upper half of the unused block 3).
+// A thread owns one query row's half of every key block; the two halves of a row exchange maximum and
+// sum through shared memory.  P_j goes to one of two shared-memory blocks as the second product's operand.
+//   warp 0: TMA producer (Q tile, ring of K and V tiles: K_0 .. K_{n-1}, V_0 .. V_{n-1})
+//   warp 1: MMA issuer: the next item's scores are issued behind this item's last second product, so they
+//           are ready when the softmax warps have stored the context
+// Bound by the exponential unit (16 a clock: 1024 cycles per block) and the passes around it.  The form
+// before, with two groups of warps on items of their own and the scores formed twice, took 12.9 k cycles
+// per item of four blocks.
+constexpr int AR_RING = 8;
+constexpr int AR_BARS = 2 + 2 * AR_RING + 1 + 2 * 2 + 2;
+
+template <bool kPacked>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                     const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* ring_smem = smem + AT_TILE_BYTES;                  // Q first
+  uint8_t* p_smem = ring_smem + AR_RING * AT_TILE_BYTES;      // two blocks of P, 32 KB each
+  float* xch = (float*)(p_smem + 4 * AT_TILE_BYTES);          // [2][NUM_EPI_WARPS][32] maxima, sums
+  volatile int* xflag = (volatile int*)(xch + 2 * NUM_EPI_WARPS * 32);
+  uint64_t* bars = (uint64_t*)(xflag + NUM_EPI_WARPS);
+  const uint32_t qfull = smem_u32(&bars[0]), qempty = smem_u32(&bars[1]);
+  const uint32_t tfull0 = smem_u32(&bars[2]), tempty0 = smem_u32(&bars[2 + AR_RING]);
+  const uint32_t sfull = smem_u32(&bars[2 + 2 * AR_RING]);
+  const uint32_t pready0 = smem_u32(&bars[3 + 2 * AR_RING]), pfree0 = smem_u32(&bars[5 + 2 * AR_RING]);  // [2] each
+  const uint32_t ofull = smem_u32(&bars[7 + 2 * AR_RING]), oempty = smem_u32(&bars[8 + 2 * AR_RING]);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 9 + 2 * AR_RING);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    mbar_init(qfull, 1); mbar_init(qempty, 1); mbar_init(sfull, 1); mbar_init(ofull, 1);
+    mbar_init(oempty, NUM_EPI_WARPS);
+    for (int s = 0; s < AR_RING; s++) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 1); }
+    for (int b = 0; b < 2; b++) { mbar_init(pready0 + 8 * b, NUM_EPI_WARPS); mbar_init(pfree0 + 8 * b, 1); }
+    for (int i = 0; i < NUM_EPI_WARPS; i++) xflag[i] = 0;
+    *abort_flag = 0;
+    *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(AT_TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
+  const int nzh = p.items / ((p.S + 127) >> 7);  // (sequence, head) pairs; the query tile is the slow index
+  auto item_len = [&](int zo) {
+    int len = p.seq_lens ? p.seq_lens[zo] : p.S;
+    return min(max(len, 1), p.S);
+  };
+  // column of the context accumulator, and the key block it lies in
+  auto o_block = [](int n) { return n == 4 ? 0 : 3; };
+  auto o_col = [](int n) { return n == 4 ? 0u : 448u; };
+
+  if (warp == 0 && lane == 0 && !p.starve) {
+    // ------------------------------- TMA producer -------------------------------
+    bool ok = true;
+    uint32_t tt = 0, ig = 0;
+    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
+      const int qt = w / nzh, zh = w - qt * nzh;
+      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+      const int len = item_len(zo);
+      if (qt * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      const int row0 = kPacked ? p.cu[zo] : 0, zseq = kPacked ? 0 : zo;
+      if (!mbar_wait(qempty, (ig & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+      ig++;
+      int c[4];
+      c[0] = 0; c[p.q_perm[0]] = row0 + qt * 128; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zseq;
+      mbar_expect_tx(qfull, AT_TILE_BYTES);
+      tma_load_4d(smem_u32(smem), &tmQ, qfull, c[0], c[1], c[2], c[3]);
+      for (int i = 0; i < 2 * n; i++, tt++) {
+        const bool is_v = i >= n;
+        const uint32_t slot = tt % AR_RING, round = tt / AR_RING;
+        if (!mbar_wait(tempty0 + 8 * slot, (round & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        mbar_expect_tx(tfull0 + 8 * slot, AT_TILE_BYTES);
+        const int* perm = is_v ? p.v_perm : p.k_perm;
+        c[0] = 0; c[perm[0]] = row0 + (is_v ? i - n : i) * 128; c[perm[1]] = zi; c[perm[2]] = zseq;
+        tma_load_4d(smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES), is_v ? &tmV : &tmK, tfull0 + 8 * slot, c[0], c[1], c[2], c[3]);
+      }
+    }
+    if (!ok || *abort_flag) {  // give the copies in flight time to land before the CTA leaves
+      const long long t0 = now_cycles();
+      while (now_cycles() - t0 < 4000000ll) {}
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ------------------------------- MMA issuer -------------------------------
+    bool ok = true;
+    const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);
+    const uint32_t lbo_mn_lo = (uint32_t)make_smem_desc(0, 64 * BK * 2);
+    const uint32_t q_lo = (uint32_t)make_smem_desc(smem_u32(smem), 16);
+    uint32_t tt = 0, pv = 0, ig = 0;  // ring tiles, second products, items
+    int n_prev = 0;
+    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
+      const int qt = w / nzh, zh = w - qt * nzh;
+      const int len = item_len(zh / p.heads);
+      if (qt * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      if (!mbar_wait(qfull, ig & 1, abort_flag, p.status)) { ok = false; break; }
+      auto scores = [&](int j) -> bool {  // S_j = Q K_j^T
+        const uint32_t pos = tt + j, slot = pos % AR_RING;
+        if (!mbar_wait(tfull0 + 8 * slot, (pos / AR_RING) & 1, abort_flag, p.status)) return false;
+        tc_fence_after();
+        const uint32_t k_lo = (uint32_t)make_smem_desc(smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES), 16);
+#pragma unroll
+        for (int k = 0; k < BK / UMMA_K; k++) {
+          const uint64_t ad = ((uint64_t)hi << 32) | (q_lo + k * (UMMA_K * 2 / 16));
+          const uint64_t bd = ((uint64_t)hi << 32) | (k_lo + k * (UMMA_K * 2 / 16));
+          tc_mma(tmem_base + j * 128, ad, bd, p.idesc_s, k > 0 ? 1u : 0u);
+        }
+        tc_commit(tempty0 + 8 * slot);
+        return true;
+      };
+      // The scores of the item before have been read (its P blocks were waited for below); only the block
+      // its context lies in has to wait until that context has been read.
+      const int held = n_prev ? o_block(n_prev) : -1;
+      for (int j = 0; j < n && ok; j++)
+        if (j != held) ok = scores(j);
+      if (ok && n_prev && !mbar_wait(oempty, (ig & 1) ^ 1, abort_flag, p.status)) ok = false;
+      if (ok && held >= 0 && held < n) ok = scores(held);
+      if (!ok) break;
+      tc_commit(sfull);
+      tc_commit(qempty);
+      tt += n;
+      for (int j = 0; j < n; j++, pv++, tt++) {  // C (+)= P_j V_j
+        const uint32_t slot = tt % AR_RING, b = pv & 1;
+        if (!mbar_wait(pready0 + 8 * b, (pv >> 1) & 1, abort_flag, p.status) ||
+            !mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t p_lo = (uint32_t)make_smem_desc(smem_u32(p_smem + b * 2 * AT_TILE_BYTES), 16);
+        const uint32_t v_lo = lbo_mn_lo | ((smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES) & 0x3FFFFu) >> 4);
+#pragma unroll
+        for (int kb = 0; kb < 2; kb++)
+#pragma unroll
+          for (int k = 0; k < BK / UMMA_K; k++) {
+            const uint64_t ad = ((uint64_t)hi << 32) | (p_lo + kb * (AT_TILE_BYTES / 16) + k * (UMMA_K * 2 / 16));
+            const uint64_t bd = ((uint64_t)hi << 32) | (v_lo + kb * (AT_TILE_BYTES / 2 / 16) + k * (UMMA_K * 128 / 16));
+            tc_mma(tmem_base + o_col(n), ad, bd, p.idesc_o, (j > 0 || kb > 0 || k > 0) ? 1u : 0u);
+          }
+        tc_commit(pfree0 + 8 * b);
+        tc_commit(tempty0 + 8 * slot);
+      }
+      if (ok) tc_commit(ofull);
+      ig++;
+      n_prev = n;
+    }
+    if (!ok || *abort_flag) {  // make sure no MMA is still writing tensor memory before it is freed
+      tc_commit(sfull);
+      const long long t0 = now_cycles();
+      while (now_cycles() - t0 < 2000000ll) {}
+    }
+  } else if (warp >= 2) {
+    // ------------------------------- softmax warps -------------------------------
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int me = q * 2 + half, other = me ^ 1;
+    const int r = q * 32 + lane;
+    const float sl2 = p.scale * 1.4426950408889634f;
+    const float2 k2 = splat2(sl2);
+    const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+    bool ok = true;
+    uint32_t pv = 0, ig = 0;
+    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
+      const int qt = w / nzh, zh = w - qt * nzh;
+      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+      const int len = item_len(zo);
+      const int row0 = kPacked ? p.cu[zo] : zo * p.S;
+      const int rlim = kPacked ? len : p.S;  // rows of the sequence that exist
+      bf16* crow = p.C + (long long)(row0 + qt * 128 + r) * p.c_ld + zi * p.c_bi + half * 32;
+      const bool row_ok = qt * 128 + r < rlim;
+      if (qt * 128 >= len) {
+        if (kPacked) continue;
+        // a query tile in the padding: zero context rows (finite, so that masked reads stay harmless)
+        if (row_ok)
+          for (int e = 0; e < 4; e++) *reinterpret_cast<uint4*>(crow + 8 * e) = make_uint4(0, 0, 0, 0);
+        continue;
+      }
+      const int n = (len + 127) >> 7;
+      if (!mbar_wait(sfull, ig & 1, abort_flag, p.status)) { ok = false; break; }
+      tc_fence_after();
+      uint32_t s0[32], s1[32];
+      auto load = [&](int j) {  // this thread's 64 scores of block j, keys beyond the sequence at -inf
+        tc_ld32_issue(trow + j * 128 + half * 64, s0);
+        tc_ld32_issue(trow + j * 128 + half * 64 + 32, s1);
+        tc_ld32_wait(s0);
+        tc_ld32_wait(s1);
+        const int k0 = j * 128 + half * 64;
+        if (k0 + 64 > len) {
+#pragma unroll
+          for (int e = 0; e < 32; e++) {
+            if (k0 + e >= len) s0[e] = 0xff800000u;
+            if (k0 + 32 + e >= len) s1[e] = 0xff800000u;
+          }
+        }
+      };
+      // pass 1: the row's maximum
+      float mx = -INFINITY;
+      for (int j = 0; j < n; j++) {
+        load(j);
+        float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+          m0 = fmaxf(m0, __uint_as_float(s0[e]));
+          m1 = fmaxf(m1, __uint_as_float(s0[e + 1]));
+          m2 = fmaxf(m2, __uint_as_float(s1[e]));
+          m3 = fmaxf(m3, __uint_as_float(s1[e + 1]));
+        }
+        mx = fmaxf(mx, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)));
+      }
+      xch[me * 32 + lane] = mx;
+      if (!pair_sync(xflag, me, other, (int)ig * 2 + 1, lane, abort_flag, p.status)) { ok = false; break; }
+      mx = fmaxf(mx, xch[other * 32 + lane]);  // finite: at least one key is valid
+      // pass 2: exponentials, their sum, and P_j
+      const float2 nm2 = splat2(-mx * sl2);
+      float2 l0 = make_float2(0.f, 0.f), l1 = l0;
+      for (int j = 0; j < n; j++, pv++) {
+        load(j);
+#pragma unroll
+        for (int e = 0; e < 16; e++) {
+          const float2 a = __ffma2_rn(make_float2(__uint_as_float(s0[2 * e]), __uint_as_float(s0[2 * e + 1])), k2, nm2);
+          const float2 b = __ffma2_rn(make_float2(__uint_as_float(s1[2 * e]), __uint_as_float(s1[2 * e + 1])), k2, nm2);
+          const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y)), eb = make_float2(fast_exp2(b.x), fast_exp2(b.y));
+          l0 = __fadd2_rn(l0, ea);
+          l1 = __fadd2_rn(l1, eb);
+          const __nv_bfloat162 pa = __float22bfloat162_rn(ea), pb = __float22bfloat162_rn(eb);
+          s0[e] = *reinterpret_cast<const uint32_t*>(&pa);
+          s1[e] = *reinterpret_cast<const uint32_t*>(&pb);
+        }
+        const uint32_t b = pv & 1;
+        if (!mbar_wait(pfree0 + 8 * b, ((pv >> 1) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        uint8_t* prow = p_smem + b * 2 * AT_TILE_BYTES + half * AT_TILE_BYTES + r * 128;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          *reinterpret_cast<uint4*>(prow + ((c ^ (r & 7)) << 4)) = make_uint4(s0[4 * c], s0[4 * c + 1], s0[4 * c + 2], s0[4 * c + 3]);
+          *reinterpret_cast<uint4*>(prow + (((4 + c) ^ (r & 7)) << 4)) = make_uint4(s1[4 * c], s1[4 * c + 1], s1[4 * c + 2], s1[4 * c + 3]);
+        }
+        tc_fence_before();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(pready0 + 8 * b);
+      }
+      if (!ok) break;
+      float sum = (l0.x + l0.y) + (l1.x + l1.y);
+      float* xsum = xch + NUM_EPI_WARPS * 32;
+      xsum[me * 32 + lane] = sum;
+      if (!pair_sync(xflag, me, other, (int)ig * 2 + 2, lane, abort_flag, p.status)) { ok = false; break; }
+      sum = half ? xsum[other * 32 + lane] + sum : sum + xsum[other * 32 + lane];
+      if (p.lse && half == 0 && row_ok) p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = mx * sl2 + log2f(sum);
+      // the context: 32 of the row's 64 columns
+      if (!mbar_wait(ofull, ig & 1, abort_flag, p.status)) { ok = false; break; }
+      ig++;
+      tc_fence_after();
+      float2 v[16];
+      tc_ld32(trow + o_col(n) + half * 32, v);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(oempty);
+      if (row_ok) {
+        const float2 il = splat2(1.0f / sum);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          uint4 o;
+          __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+          for (int k = 0; k < 4; k++) h[k] = __float22bfloat162_rn(__fmul2_rn(v[4 * e + k], il));
+          *reinterpret_cast<uint4*>(crow + 8 * e) = o;
+        }
       }
     }
     if (kPacked) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
@@ -1430,7 +1696,7 @@ namespace {
 // per-device facts and one-time kernel attributes (a process may drive several GPUs)
 struct AttnDevice {
   int num_sms = 0, smem_optin = 0;
-  bool attr_fwd[2] = {false, false}, attr_long[2] = {false, false};
+  bool attr_fwd[2] = {false, false}, attr_rows[2] = {false, false}, attr_long = false;
   bool attr_bwd = false, attr_bwd_kv = false, attr_bwd_q = false;
 };
 constexpr int kMaxDevices = 64;
@@ -1481,7 +1747,7 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   p.S = S; p.heads = A; p.items = B * A * (long_rows ? (S + 127) / 128 : 1); p.scale = scale; p.seq_lens = seq_lens;
   p.cu = cu; p.rows = rows;
   p.lse = lse; p.lse_ld = (long long)B * S;
-  if ((cu && (!seq_lens || !rows)) || (cu && long_rows && probs) || (lse && !long_rows)) {
+  if ((cu && (!seq_lens || !rows)) || (cu && long_rows && probs) || (lse && (!long_rows || probs))) {
     snprintf(err, 256, "attention: packed rows need lengths and row counts; long packed rows store no probabilities");
     return MSLT_ERR_ARG;
   }
@@ -1515,15 +1781,26 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   else rc = get_map(base + 2 * H, d, mrows, 1, 3 * H, mbo, d, A, mseqs, 64, &mv, err);
   if (rc) return rc;
   for (int i = 0; i < 3; i++) { p.q_perm[i] = mq.perm[i]; p.k_perm[i] = mk.perm[i]; p.v_perm[i] = mv.perm[i]; }
+  if (long_rows && probs == nullptr) {
+    const size_t smem_rows = (size_t)(1 + AR_RING + 4) * AT_TILE_BYTES + 2 * NUM_EPI_WARPS * 32 * 4 + 1024 + 512;
+    if ((int)smem_rows > smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
+    const auto kernel = cu ? attn_fwd_rows_kernel<true> : attn_fwd_rows_kernel<false>;
+    rc = attn_opt_in(kernel, &adev->attr_rows[cu != nullptr], smem_optin, err);
+    if (rc) return rc;
+    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, NUM_THREADS, smem_rows, st, mq.map, mk.map, mv.map, p);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
+    g_attn_launches++;
+    return 0;
+  }
   if (long_rows) {
     const size_t smem_long = 2 * (size_t)AT_TILE_BYTES + 2 * (size_t)AL_RING * AT_TILE_BYTES + 2 * (size_t)AL_P_BYTES +
                              NUM_EPI_WARPS * AT_STAGING + 1024 + 512;
     if ((int)smem_long > smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
-    const auto kernel = cu ? attn_fwd_long_kernel<true> : attn_fwd_long_kernel<false>;
-    rc = attn_opt_in(kernel, &adev->attr_long[cu != nullptr], smem_optin, err);
+    rc = attn_opt_in(attn_fwd_long_kernel, &adev->attr_long, smem_optin, err);
     if (rc) return rc;
     const int grid_long = p.items < num_sms ? p.items : num_sms;
-    launch_pdl(kernel, grid_long, AL_THREADS, smem_long, st, mq.map, mk.map, mv.map, p);
+    launch_pdl(attn_fwd_long_kernel, grid_long, AL_THREADS, smem_long, st, mq.map, mk.map, mv.map, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
     g_attn_launches++;
