@@ -39,7 +39,8 @@ struct AttnParams {
   float scale;
   const int* seq_lens;
   const int* cu;      // packed rows: sequence b holds rows cu[b] .. cu[b] + len - 1 of qkv and C; null = b * S
-  const int* rows;    // packed: {rows in use, the same rounded up}; C's rows between the two are zeroed
+  const int* rows;    // packed: {rows in use, the same rounded up, query tiles}; C's rows between the first two are zeroed
+  const int* order;   // packed long rows: 8 * sequence + query tile of every tile that exists, longest sequences first
   float* lse;         // long rows: log2 of the row's sum of exponentials, [A][lse_ld] by row; or null
   long long lse_ld;
   bf16* P;            // [B, A, S, S] or null
@@ -762,11 +763,12 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
 // ---- forward for rows of 129..512 keys, no probabilities stored -----------------------------------
 // A work item is (sequence, head, tile of 128 queries).  Tensor memory holds the scores of a whole row
-// (four blocks of 128 keys), so they are formed once: all eight softmax warps read them twice, first for
+// (four blocks of 128 keys), so they are formed once: all sixteen softmax warps read them twice, first for
 // the row maximum, then for the exponentials, and the context accumulates over columns whose scores have
 // been used up (block 0 when there are four blocks, else the upper half of the unused block 3).
-// A thread owns one query row's half of every key block; the two halves of a row exchange maximum and
-// sum through shared memory.  P_j goes to one of two shared-memory blocks as the second product's operand.
+// A thread owns a quarter of one query row's scores in every key block; the quarters exchange maximum and
+// sum through shared memory.  (Eight warps with half a row each took 13.6 k cycles per item of four
+// blocks, two warps per scheduler being too few to cover the tensor-memory reads and the fences.)  P_j goes to one of two shared-memory blocks as the second product's operand.
 //   warp 0: TMA producer (Q tile, ring of K and V tiles: K_0 .. K_{n-1}, V_0 .. V_{n-1})
 //   warp 1: MMA issuer: the next item's scores are issued behind this item's last second product, so they
 //           are ready when the softmax warps have stored the context
@@ -775,18 +777,62 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 // per item of four blocks.
 constexpr int AR_RING = 8;
 constexpr int AR_BARS = 2 + 2 * AR_RING + 1 + 2 * 2 + 2;
+constexpr int AR_WARPS = 16;  // softmax warps: four per TMEM lane quarter
+constexpr int AR_THREADS = 64 + 32 * AR_WARPS;
+
+// 16 consecutive accumulator columns of this lane's row
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+// Hand-over between the four warps of a lane quarter (pair_sync for more partners).
+__device__ __forceinline__ bool quad_sync(volatile int* flags, int me, int seq, int lane, volatile int* abort_flag, int* status) {
+  __syncwarp();
+  int ok = 1;
+  if (lane == 0) {
+    __threadfence_block();
+    flags[me] = seq;
+    const long long t0 = now_cycles();
+    uint32_t spins = 0;
+    const int first = me & ~3;
+    while (flags[first] < seq || flags[first + 1] < seq || flags[first + 2] < seq || flags[first + 3] < seq) {
+      if ((++spins & 255u) == 0u) {
+        if (*abort_flag) { ok = 0; break; }
+        if (now_cycles() - t0 > *reinterpret_cast<volatile long long*>(abort_flag + 1)) {
+          *abort_flag = 1;
+          atomicOr(status, ST_WAIT_TIMEOUT);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    __threadfence_block();
+  }
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  return ok != 0;
+}
 
 template <bool kPacked>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(AR_THREADS, 1)
 attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* ring_smem = smem + AT_TILE_BYTES;                  // Q first
   uint8_t* p_smem = ring_smem + AR_RING * AT_TILE_BYTES;      // two blocks of P, 32 KB each
-  float* xch = (float*)(p_smem + 4 * AT_TILE_BYTES);          // [2][NUM_EPI_WARPS][32] maxima, sums
-  volatile int* xflag = (volatile int*)(xch + 2 * NUM_EPI_WARPS * 32);
-  uint64_t* bars = (uint64_t*)(xflag + NUM_EPI_WARPS);
+  float* xch = (float*)(p_smem + 4 * AT_TILE_BYTES);          // [2][AR_WARPS][32] maxima, sums
+  volatile int* xflag = (volatile int*)(xch + 2 * AR_WARPS * 32);
+  uint64_t* bars = (uint64_t*)(xflag + AR_WARPS);
   const uint32_t qfull = smem_u32(&bars[0]), qempty = smem_u32(&bars[1]);
   const uint32_t tfull0 = smem_u32(&bars[2]), tempty0 = smem_u32(&bars[2 + AR_RING]);
   const uint32_t sfull = smem_u32(&bars[2 + 2 * AR_RING]);
@@ -798,10 +844,10 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     mbar_init(qfull, 1); mbar_init(qempty, 1); mbar_init(sfull, 1); mbar_init(ofull, 1);
-    mbar_init(oempty, NUM_EPI_WARPS);
+    mbar_init(oempty, AR_WARPS);
     for (int s = 0; s < AR_RING; s++) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 1); }
-    for (int b = 0; b < 2; b++) { mbar_init(pready0 + 8 * b, NUM_EPI_WARPS); mbar_init(pfree0 + 8 * b, 1); }
-    for (int i = 0; i < NUM_EPI_WARPS; i++) xflag[i] = 0;
+    for (int b = 0; b < 2; b++) { mbar_init(pready0 + 8 * b, AR_WARPS); mbar_init(pfree0 + 8 * b, 1); }
+    for (int i = 0; i < AR_WARPS; i++) xflag[i] = 0;
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -817,7 +863,22 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
-  const int nzh = p.items / ((p.S + 127) >> 7);  // (sequence, head) pairs; the query tile is the slow index
+  // Items: packed batches list the query tiles that exist, those of the longest sequences first, so that
+  // dealing them out leaves the CTAs level; otherwise the query tile is the slow index.
+  const int nzh = p.items / ((p.S + 127) >> 7);
+  const int n_items = kPacked ? p.rows[2] * p.heads : p.items;
+  auto decode = [&](int w, int& zo, int& zi, int& qt) {
+    if (kPacked) {
+      const int e = w / p.heads;
+      zi = w - e * p.heads;
+      zo = p.order[e] >> 3;
+      qt = p.order[e] & 7;
+    } else {
+      qt = w / nzh;
+      zo = (w - qt * nzh) / p.heads;
+      zi = (w - qt * nzh) - zo * p.heads;
+    }
+  };
   auto item_len = [&](int zo) {
     int len = p.seq_lens ? p.seq_lens[zo] : p.S;
     return min(max(len, 1), p.S);
@@ -830,9 +891,9 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     // ------------------------------- TMA producer -------------------------------
     bool ok = true;
     uint32_t tt = 0, ig = 0;
-    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
-      const int qt = w / nzh, zh = w - qt * nzh;
-      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, qt;
+      decode(w, zo, zi, qt);
       const int len = item_len(zo);
       if (qt * 128 >= len) continue;
       const int n = (len + 127) >> 7;
@@ -865,9 +926,10 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     const uint32_t q_lo = (uint32_t)make_smem_desc(smem_u32(smem), 16);
     uint32_t tt = 0, pv = 0, ig = 0;  // ring tiles, second products, items
     int n_prev = 0;
-    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
-      const int qt = w / nzh, zh = w - qt * nzh;
-      const int len = item_len(zh / p.heads);
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, qt;
+      decode(w, zo, zi, qt);
+      const int len = item_len(zo);
       if (qt * 128 >= len) continue;
       const int n = (len + 127) >> 7;
       if (!mbar_wait(qfull, ig & 1, abort_flag, p.status)) { ok = false; break; }
@@ -925,45 +987,41 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     }
   } else if (warp >= 2) {
     // ------------------------------- softmax warps -------------------------------
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const int me = q * 2 + half, other = me ^ 1;
+    const int q = warp & 3, part = (warp - 2) >> 2;  // columns part * 32 .. of every key block
+    const int me = q * 4 + part;
     const int r = q * 32 + lane;
     const float sl2 = p.scale * 1.4426950408889634f;
     const float2 k2 = splat2(sl2);
     const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+    float* xsum = xch + AR_WARPS * 32;
     bool ok = true;
     uint32_t pv = 0, ig = 0;
-    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
-      const int qt = w / nzh, zh = w - qt * nzh;
-      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, qt;
+      decode(w, zo, zi, qt);
       const int len = item_len(zo);
       const int row0 = kPacked ? p.cu[zo] : zo * p.S;
       const int rlim = kPacked ? len : p.S;  // rows of the sequence that exist
-      bf16* crow = p.C + (long long)(row0 + qt * 128 + r) * p.c_ld + zi * p.c_bi + half * 32;
+      bf16* crow = p.C + (long long)(row0 + qt * 128 + r) * p.c_ld + zi * p.c_bi + part * 16;
       const bool row_ok = qt * 128 + r < rlim;
       if (qt * 128 >= len) {
-        if (kPacked) continue;
         // a query tile in the padding: zero context rows (finite, so that masked reads stay harmless)
         if (row_ok)
-          for (int e = 0; e < 4; e++) *reinterpret_cast<uint4*>(crow + 8 * e) = make_uint4(0, 0, 0, 0);
+          for (int e = 0; e < 2; e++) *reinterpret_cast<uint4*>(crow + 8 * e) = make_uint4(0, 0, 0, 0);
         continue;
       }
       const int n = (len + 127) >> 7;
       if (!mbar_wait(sfull, ig & 1, abort_flag, p.status)) { ok = false; break; }
       tc_fence_after();
-      uint32_t s0[32], s1[32];
-      auto load = [&](int j) {  // this thread's 64 scores of block j, keys beyond the sequence at -inf
-        tc_ld32_issue(trow + j * 128 + half * 64, s0);
-        tc_ld32_issue(trow + j * 128 + half * 64 + 32, s1);
-        tc_ld32_wait(s0);
-        tc_ld32_wait(s1);
-        const int k0 = j * 128 + half * 64;
-        if (k0 + 64 > len) {
+      uint32_t s[32];
+      auto load = [&](int j) {  // this thread's 32 scores of block j, keys beyond the sequence at -inf
+        tc_ld32_issue(trow + j * 128 + part * 32, s);
+        tc_ld32_wait(s);
+        const int k0 = j * 128 + part * 32;
+        if (k0 + 32 > len) {
 #pragma unroll
-          for (int e = 0; e < 32; e++) {
-            if (k0 + e >= len) s0[e] = 0xff800000u;
-            if (k0 + 32 + e >= len) s1[e] = 0xff800000u;
-          }
+          for (int e = 0; e < 32; e++)
+            if (k0 + e >= len) s[e] = 0xff800000u;
         }
       };
       // pass 1: the row's maximum
@@ -972,75 +1030,72 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         load(j);
         float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < 32; e += 2) {
-          m0 = fmaxf(m0, __uint_as_float(s0[e]));
-          m1 = fmaxf(m1, __uint_as_float(s0[e + 1]));
-          m2 = fmaxf(m2, __uint_as_float(s1[e]));
-          m3 = fmaxf(m3, __uint_as_float(s1[e + 1]));
+        for (int e = 0; e < 32; e += 4) {
+          m0 = fmaxf(m0, __uint_as_float(s[e]));
+          m1 = fmaxf(m1, __uint_as_float(s[e + 1]));
+          m2 = fmaxf(m2, __uint_as_float(s[e + 2]));
+          m3 = fmaxf(m3, __uint_as_float(s[e + 3]));
         }
         mx = fmaxf(mx, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)));
       }
       xch[me * 32 + lane] = mx;
-      if (!pair_sync(xflag, me, other, (int)ig * 2 + 1, lane, abort_flag, p.status)) { ok = false; break; }
-      mx = fmaxf(mx, xch[other * 32 + lane]);  // finite: at least one key is valid
+      if (!quad_sync(xflag, me, (int)ig * 2 + 1, lane, abort_flag, p.status)) { ok = false; break; }
+#pragma unroll
+      for (int o = 0; o < 4; o++) mx = fmaxf(mx, xch[(q * 4 + o) * 32 + lane]);  // finite: one key is valid
       // pass 2: exponentials, their sum, and P_j
       const float2 nm2 = splat2(-mx * sl2);
-      float2 l0 = make_float2(0.f, 0.f), l1 = l0;
+      float2 l0 = make_float2(0.f, 0.f);
       for (int j = 0; j < n; j++, pv++) {
         load(j);
 #pragma unroll
         for (int e = 0; e < 16; e++) {
-          const float2 a = __ffma2_rn(make_float2(__uint_as_float(s0[2 * e]), __uint_as_float(s0[2 * e + 1])), k2, nm2);
-          const float2 b = __ffma2_rn(make_float2(__uint_as_float(s1[2 * e]), __uint_as_float(s1[2 * e + 1])), k2, nm2);
-          const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y)), eb = make_float2(fast_exp2(b.x), fast_exp2(b.y));
+          const float2 a = __ffma2_rn(make_float2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), k2, nm2);
+          const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y));
           l0 = __fadd2_rn(l0, ea);
-          l1 = __fadd2_rn(l1, eb);
-          const __nv_bfloat162 pa = __float22bfloat162_rn(ea), pb = __float22bfloat162_rn(eb);
-          s0[e] = *reinterpret_cast<const uint32_t*>(&pa);
-          s1[e] = *reinterpret_cast<const uint32_t*>(&pb);
+          const __nv_bfloat162 pa = __float22bfloat162_rn(ea);
+          s[e] = *reinterpret_cast<const uint32_t*>(&pa);
         }
         const uint32_t b = pv & 1;
         if (!mbar_wait(pfree0 + 8 * b, ((pv >> 1) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
-        uint8_t* prow = p_smem + b * 2 * AT_TILE_BYTES + half * AT_TILE_BYTES + r * 128;
+        uint8_t* prow = p_smem + (b * 2 + (part >> 1)) * AT_TILE_BYTES + r * 128;
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-          *reinterpret_cast<uint4*>(prow + ((c ^ (r & 7)) << 4)) = make_uint4(s0[4 * c], s0[4 * c + 1], s0[4 * c + 2], s0[4 * c + 3]);
-          *reinterpret_cast<uint4*>(prow + (((4 + c) ^ (r & 7)) << 4)) = make_uint4(s1[4 * c], s1[4 * c + 1], s1[4 * c + 2], s1[4 * c + 3]);
-        }
+        for (int c = 0; c < 4; c++)
+          *reinterpret_cast<uint4*>(prow + ((((part & 1) * 4 + c) ^ (r & 7)) << 4)) = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
         tc_fence_before();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(pready0 + 8 * b);
       }
       if (!ok) break;
-      float sum = (l0.x + l0.y) + (l1.x + l1.y);
-      float* xsum = xch + NUM_EPI_WARPS * 32;
-      xsum[me * 32 + lane] = sum;
-      if (!pair_sync(xflag, me, other, (int)ig * 2 + 2, lane, abort_flag, p.status)) { ok = false; break; }
-      sum = half ? xsum[other * 32 + lane] + sum : sum + xsum[other * 32 + lane];
-      if (p.lse && half == 0 && row_ok) p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = mx * sl2 + log2f(sum);
-      // the context: 32 of the row's 64 columns
+      xsum[me * 32 + lane] = l0.x + l0.y;
+      if (!quad_sync(xflag, me, (int)ig * 2 + 2, lane, abort_flag, p.status)) { ok = false; break; }
+      float sum = 0.f;
+#pragma unroll
+      for (int o = 0; o < 4; o++) sum += xsum[(q * 4 + o) * 32 + lane];
+      if (p.lse && part == 0 && row_ok) p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = mx * sl2 + log2f(sum);
+      // the context: 16 of the row's 64 columns
       if (!mbar_wait(ofull, ig & 1, abort_flag, p.status)) { ok = false; break; }
       ig++;
       tc_fence_after();
-      float2 v[16];
-      tc_ld32(trow + o_col(n) + half * 32, v);
+      uint32_t v[16];
+      tc_ld16(trow + o_col(n) + part * 16, v);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(oempty);
       if (row_ok) {
         const float2 il = splat2(1.0f / sum);
 #pragma unroll
-        for (int e = 0; e < 4; e++) {
+        for (int e = 0; e < 2; e++) {
           uint4 o;
           __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
-          for (int k = 0; k < 4; k++) h[k] = __float22bfloat162_rn(__fmul2_rn(v[4 * e + k], il));
+          for (int t = 0; t < 4; t++)
+            h[t] = __float22bfloat162_rn(__fmul2_rn(make_float2(__uint_as_float(v[8 * e + 2 * t]), __uint_as_float(v[8 * e + 2 * t + 1])), il));
           *reinterpret_cast<uint4*>(crow + 8 * e) = o;
         }
       }
     }
-    if (kPacked) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
+    if (kPacked && warp < 2 + NUM_EPI_WARPS) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
   }
 
   tc_fence_before();
@@ -1368,6 +1423,7 @@ struct AttnBwdLongParams {
   const int* seq_lens;
   const int* cu;
   const int* rows;
+  const int* order;
   const float* lse;
   const float* delta;
   long long ld;       // rows of one head in lse and delta
@@ -1427,7 +1483,21 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
+  // items as in the forward kernel: packed batches list the tiles that exist, longest sequences first
   const int nt = (p.S + 127) >> 7, nzh = p.items / nt;
+  const int n_items = p.cu ? p.rows[2] * p.heads : p.items;
+  auto decode = [&](int w, int& zo, int& zi, int& tile) {
+    if (p.cu) {
+      const int e = w / p.heads;
+      zi = w - e * p.heads;
+      zo = p.order[e] >> 3;
+      tile = p.order[e] & 7;
+    } else {
+      tile = w / nzh;
+      zo = (w - tile * nzh) / p.heads;
+      zi = (w - tile * nzh) - zo * p.heads;
+    }
+  };
   auto item_len = [&](int zo) {
     int len = p.cu ? p.seq_lens[zo] : p.S;
     return min(max(len, 1), p.S);
@@ -1443,11 +1513,10 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       c[perm[0]] = row; c[perm[1]] = zi;
       tma_load_4d(dst, map, bar, c[0], c[1], c[2], c[3]);
     };
-    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
-      const int tile = w / nzh, zh = w - tile * nzh;  // tile slowest: those that may be padding come last
-      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, tile;
+      decode(w, zo, zi, tile);
       const int len = item_len(zo), row0 = row_base(zo);
-      if (tile * 128 >= len) continue;
       const int n = (len + 127) >> 7;
       if (!mbar_wait(fempty, (ni & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
       ni++;
@@ -1500,10 +1569,10 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     };
     const uint32_t f0 = smem_u32(smem), pa = addr16(smem_u32(p_smem)), da = addr16(smem_u32(ds_smem));
     uint32_t rt = 0, np = 0, ni = 0;  // score pairs (= ring tiles), accumulated pairs, items
-    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
-      const int tile = w / nzh, zh = w - tile * nzh;
-      const int len = item_len(zh / p.heads);
-      if (tile * 128 >= len) continue;
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, tile;
+      decode(w, zo, zi, tile);
+      const int len = item_len(zo);
       const int n = (len + 127) >> 7;
       if (!mbar_wait(ffull, ni & 1, abort_flag, p.status)) { ok = false; break; }
       auto accumulate = [&](int t) -> bool {  // the accumulating products of pair t of this item
@@ -1559,11 +1628,10 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     uint32_t sp = 0, ni = 0;
     uint8_t* prow = p_smem + half * AT_TILE_BYTES + r * 128;
     uint8_t* drow = ds_smem + half * AT_TILE_BYTES + r * 128;
-    for (int w = (int)blockIdx.x; w < p.items && ok; w += (int)gridDim.x) {
-      const int tile = w / nzh, zh = w - tile * nzh;
-      const int zo = zh / p.heads, zi = zh - zo * p.heads;
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, tile;
+      decode(w, zo, zi, tile);
       const int len = item_len(zo);
-      if (tile * 128 >= len) continue;
       const int n = (len + 127) >> 7;
       const long long row0 = row_base(zo);
       for (int t = 0; t < n && ok; t++) {
@@ -1730,7 +1798,8 @@ int attn_opt_in(K kernel, bool* done, int smem_optin, char* err) {
 }  // namespace
 
 int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens, int B, int S, int A, int d,
-                    float scale, int* status, cudaStream_t st, char* err, const int* cu, const int* rows, float* lse) {
+                    float scale, int* status, cudaStream_t st, char* err, const int* cu, const int* rows, float* lse,
+                    const int* order) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_attn_starve.exchange(0) != 0;
   AttnDevice* adev = attn_device(err);
@@ -1745,9 +1814,9 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   AttnParams p;
   memset(&p, 0, sizeof(p));
   p.S = S; p.heads = A; p.items = B * A * (long_rows ? (S + 127) / 128 : 1); p.scale = scale; p.seq_lens = seq_lens;
-  p.cu = cu; p.rows = rows;
+  p.cu = cu; p.rows = rows; p.order = order;
   p.lse = lse; p.lse_ld = (long long)B * S;
-  if ((cu && (!seq_lens || !rows)) || (cu && long_rows && probs) || (lse && (!long_rows || probs))) {
+  if ((cu && (!seq_lens || !rows || (long_rows && !order))) || (cu && long_rows && probs) || (lse && (!long_rows || probs))) {
     snprintf(err, 256, "attention: packed rows need lengths and row counts; long packed rows store no probabilities");
     return MSLT_ERR_ARG;
   }
@@ -1782,12 +1851,12 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   if (rc) return rc;
   for (int i = 0; i < 3; i++) { p.q_perm[i] = mq.perm[i]; p.k_perm[i] = mk.perm[i]; p.v_perm[i] = mv.perm[i]; }
   if (long_rows && probs == nullptr) {
-    const size_t smem_rows = (size_t)(1 + AR_RING + 4) * AT_TILE_BYTES + 2 * NUM_EPI_WARPS * 32 * 4 + 1024 + 512;
+    const size_t smem_rows = (size_t)(1 + AR_RING + 4) * AT_TILE_BYTES + 2 * AR_WARPS * 32 * 4 + 1024 + 512;
     if ((int)smem_rows > smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
     const auto kernel = cu ? attn_fwd_rows_kernel<true> : attn_fwd_rows_kernel<false>;
     rc = attn_opt_in(kernel, &adev->attr_rows[cu != nullptr], smem_optin, err);
     if (rc) return rc;
-    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, NUM_THREADS, smem_rows, st, mq.map, mk.map, mv.map, p);
+    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, AR_THREADS, smem_rows, st, mq.map, mk.map, mv.map, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
     g_attn_launches++;
@@ -1883,11 +1952,12 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
 
 int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, const float* lse, float* delta,
                          void* dqkv, int B, int S, int A, float scale, int* status, cudaStream_t st, char* err,
-                         const int* seq_lens, const int* cu, const int* rows) {
+                         const int* seq_lens, const int* cu, const int* rows, const int* order) {
   const bool starve = g_attn_starve.exchange(0) != 0;
   AttnDevice* adev = attn_device(err);
   if (!adev) return MSLT_ERR_CUDA;
-  if (S < 1 || S > 512 || B < 1 || A < 1 || !status || !lse || !delta || (cu && (!seq_lens || !rows))) {
+  if (S < 1 || S > 512 || B < 1 || A < 1 || !status || !lse || !delta || (seq_lens && !cu) ||
+      (cu && (!seq_lens || !rows || !order))) {
     snprintf(err, 256, "attention backward: bad arguments");
     return MSLT_ERR_ARG;
   }
@@ -1895,7 +1965,7 @@ int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, con
   AttnBwdLongParams p;
   memset(&p, 0, sizeof(p));
   p.S = S; p.heads = A; p.items = B * A * ((S + 127) / 128); p.scale = scale;
-  p.seq_lens = seq_lens; p.cu = cu; p.rows = rows; p.lse = lse; p.delta = delta; p.ld = T;
+  p.seq_lens = seq_lens; p.cu = cu; p.rows = rows; p.order = order; p.lse = lse; p.delta = delta; p.ld = T;
   p.dQKV = (bf16*)dqkv; p.g_ld = 3 * H; p.H = H;
   p.wait_limit = starve ? 40000000ll : WAIT_LIMIT_CYCLES;
   p.starve = starve ? 1 : 0;

@@ -45,12 +45,13 @@ void gemm_tc_set_variant(int variant);
 // probs ([B, A, S, S], may be null: not written) and ctx ([B*S, A*d]) are outputs.  `status` as for
 // gemm_launch.  Returns 0 or a negative mslt_status with a message in `err`.
 // cu (with rows, both device): the batch is packed, sequence b holds rows cu[b] .. cu[b] + len - 1 of
-// qkv and ctx (allocated for B*S rows); rows = {rows in use, rounded up}: ctx between the two is zeroed.
+// qkv and ctx (allocated for B*S rows); rows = {rows in use, rounded up, query tiles}: ctx between the
+// first two is zeroed.  order (more than 128 keys): 8 * sequence + tile of every query tile.
 // probs then still are [B, A, S, S], with zero rows where there is no query.
 // lse (more than 128 keys): [A, B*S] by row, log2 of the row's sum of exponentials, for the backward.
 int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens, int B, int S, int A, int d,
                     float scale, int* status, cudaStream_t st, char* err, const int* cu = nullptr,
-                    const int* rows = nullptr, float* lse = nullptr);
+                    const int* rows = nullptr, float* lse = nullptr, const int* order = nullptr);
 // Its backward: dqkv ([B*S, 3*A*d], queries | keys | values like qkv) from the saved probabilities
 // and the gradient of the context dctx ([B*S, A*d]); S a multiple of 8.
 //   dV = P^T dC,  dP = dC V^T,  dS = P o (dP - rowsum(dP o P)) * scale,  dQ = dS K,  dK = dS^T Q
@@ -62,7 +63,7 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
 // sequence has S rows.  Three launches.
 int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, const float* lse, float* delta,
                          void* dqkv, int B, int S, int A, float scale, int* status, cudaStream_t st, char* err,
-                         const int* seq_lens, const int* cu, const int* rows);
+                         const int* seq_lens, const int* cu, const int* rows, const int* order);
 long long attn_launches();
 // Test hook like gemm_tc_starve_next, for the next attention launch (forward or backward).
 void attn_starve_next(int on);

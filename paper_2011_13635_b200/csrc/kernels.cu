@@ -566,7 +566,7 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
                                      const int* __restrict__ seq_lens, int B, int S, int P, int V,
                                      int* __restrict__ rowsrc, int* __restrict__ rowlabel,
                                      int* __restrict__ n_valid, float* __restrict__ inv_n,
-                                     int* __restrict__ status, int* __restrict__ cu, int* __restrict__ rows) {
+                                     int* __restrict__ status, int* __restrict__ cu, int* __restrict__ rows, int* __restrict__ order) {
   pdl_begin();
   __shared__ int cnt;
   if (cu != nullptr) {
@@ -601,6 +601,30 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
       cu[B] = base;
       rows[0] = base;
       rows[1] = min((base + 127) / 128 * 128, B * S);
+    }
+    // the 128-row tiles of the sequences, those of the longest (in tiles: at most four) first
+    __shared__ int bucket[5];
+    if (threadIdx.x < 5) bucket[threadIdx.x] = 0;
+    __syncthreads();
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const int n = (min(max(seq_lens[b], 1), S) + 127) / 128;
+      atomicAdd(&bucket[n], n);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int at = 0;
+      for (int n = 4; n >= 1; n--) {
+        const int c = bucket[n];
+        bucket[n] = at;
+        at += c;
+      }
+      rows[2] = at;
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const int n = (min(max(seq_lens[b], 1), S) + 127) / 128;
+      const int at = atomicAdd(&bucket[n], n);  // the order inside a length changes nothing
+      for (int t = 0; t < n; t++) order[at + t] = 8 * b + t;
     }
     if (positions == nullptr) return;  // the layout was all that was asked for
     __syncthreads();
@@ -1564,9 +1588,9 @@ void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float
 
 void launch_slots_prepare(const int* positions, const int* labels, const int* seq_lens, int B,
                           int S, int P, int V, int* rowsrc, int* rowlabel, int* n_valid,
-                          float* inv_n, int* status, cudaStream_t st, int* cu, int* rows) {
+                          float* inv_n, int* status, cudaStream_t st, int* cu, int* rows, int* order) {
   launch_pdl(slots_prepare_kernel, 1, cu || B * P > 1024 ? 1024 : 256, 0, st, positions, labels, seq_lens, B, S, P, V,
-             rowsrc, rowlabel, n_valid, inv_n, status, cu, rows);
+             rowsrc, rowlabel, n_valid, inv_n, status, cu, rows, order);
 }
 
 void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, int R, int H,

@@ -39,10 +39,12 @@ void launch_softmax_fwd(bool bf, const void* sc, void* p, const int* seq_lens, i
                         int rows_per_seq, float scale, cudaStream_t st);
 void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float scale,
                         cudaStream_t st);
-// cu, rows (outputs, with seq_lens): the packed layout; positions null: only that
+// cu, rows, order (outputs, with seq_lens): the packed layout; rows[2] = number of 128-row tiles and order =
+// 8 * sequence + tile of each, longest sequences first (S <= 512); positions null: only that
 void launch_slots_prepare(const int* positions, const int* labels, const int* seq_lens, int B,
                           int S, int P, int V, int* rowsrc, int* rowlabel, int* n_valid,
-                          float* inv_n, int* status, cudaStream_t st, int* cu = nullptr, int* rows = nullptr);
+                          float* inv_n, int* status, cudaStream_t st, int* cu = nullptr, int* rows = nullptr,
+                          int* order = nullptr);
 // out [B, S, H] from packed rows; zero past a sequence's length
 void launch_unpack_rows(bool bf, const void* x, const int* cu, void* out, int B, int S, int H, cudaStream_t st);
 // fp32 rows of pitch ldi to dense rows of V (a strided device copy took 91 us for 720 x 30522, this 30)

@@ -84,7 +84,7 @@ struct Workspace {
   int *es_counts, *es_total, *es_start, *es_rank, *es_order, *es_blocksum, *es_hot;
   float* es_partial;  // embedding backward: rows sorted by token id
   char *x3a, *x3b, *x3e;                    // fp32: bf16 planes of a product's operands, of the word table
-  int *cu, *rows, *ptok, *pseg;             // packed batches: see kernels.h
+  int *cu, *rows, *order, *ptok, *pseg;             // packed batches: see kernels.h
   int* nsp_rowsrc;                          // NSP head: first-token row of every sequence
   char *cls, *up, *pooled, *dup, *dcls;     // [B,H] each
   float *hst, *logits, *nll, *dtm32;
@@ -247,7 +247,8 @@ void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char
     w.x3e = take((int64_t)a.vocab * H * 6);
   }
   w.cu = (int*)take(((int64_t)a.max_batch + 1) * 4);
-  w.rows = (int*)take(2 * 4);
+  w.rows = (int*)take(3 * 4);
+  w.order = (int*)take((int64_t)a.max_batch * ((a.max_seq + 127) / 128) * 4);
   w.ptok = (int*)take(T * 4);
   w.pseg = (int*)take(T * 4);
   w.rowsrc = (int*)take(R * 4);
@@ -397,7 +398,7 @@ int run_attention(mslt_ctx* c, const void* qkv, void* probs, float* lse, void* c
   char err[256] = "";
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
-  int rc = attn_fwd_launch(qkv, probs, ctx, seq_lens, B, S, A, d, scale, c->ws.scalars, c->st, err, c->cu, c->rows, lse);
+  int rc = attn_fwd_launch(qkv, probs, ctx, seq_lens, B, S, A, d, scale, c->ws.scalars, c->st, err, c->cu, c->rows, lse, c->ws.order);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({1, 4.0 * B * A * (double)S * S * d});
@@ -415,7 +416,7 @@ int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const voi
   // rows of more than 128 keys keep their sums of exponentials in the place of the probabilities
   int rc = S <= 128 ? attn_bwd_launch(qkv, probs, dctx, dqkv, B, S, A, d, scale, c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows)
                     : attn_bwd_long_launch(qkv, ctx, dctx, (const float*)probs, (float*)c->ws.dp, dqkv, B, S, A, scale,
-                                           c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows);
+                                           c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows, c->ws.order);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({1, 8.0 * B * A * (double)S * S * d});
@@ -963,7 +964,7 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
   mark(c, 0);
   pack_batch(c, d_seq_lens);
   KL(PC_OTHER, 16.0 * B * P, launch_slots_prepare(d_pos, d_lab, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel, w.scalars + 1,
-                          inv_n, status, c->st, c->cu ? w.cu : nullptr, w.rows));
+                          inv_n, status, c->st, c->cu ? w.cu : nullptr, w.rows, w.order));
   if (d_total_valid)  // the mean runs over the valid slots of every rank's batch
     KL(PC_OTHER, 8.0, launch_override_inv_n(d_total_valid, inv_n, c->st));
   // embeddings, then the frozen prefix: forward only, two buffers, nothing kept but the output
@@ -1154,7 +1155,7 @@ int mslt_forward(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens
   pack_batch(c, d_seq_lens);
   if (head || c->cu)
     KL(PC_OTHER, 8.0 * B * P, launch_slots_prepare(head ? d_pos : nullptr, nullptr, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel,
-                            w.scalars + 1, (float*)(w.scalars + 2), w.scalars, c->st, c->cu ? w.cu : nullptr, w.rows));
+                            w.scalars + 1, (float*)(w.scalars + 2), w.scalars, c->st, c->cu ? w.cu : nullptr, w.rows, w.order));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_embed_ln(c->bf, d_tokens, nullptr, Wc(c, toff(c, -1, "emb.word")), Wc(c, toff(c, -1, "emb.pos")),
                      c->a.nsp ? Wc(c, toff(c, -1, "emb.type")) : nullptr,
                      Wv(c, toff(c, -1, "emb.ln.gamma")), Wv(c, toff(c, -1, "emb.ln.beta")), w.xa,
