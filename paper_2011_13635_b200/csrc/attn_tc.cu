@@ -767,14 +767,15 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 // the row maximum, then for the exponentials, and the context accumulates over columns whose scores have
 // been used up (block 0 when there are four blocks, else the upper half of the unused block 3).
 // A thread owns a quarter of one query row's scores in every key block; the quarters exchange maximum and
-// sum through shared memory.  (Eight warps with half a row each took 13.6 k cycles per item of four
-// blocks, two warps per scheduler being too few to cover the tensor-memory reads and the fences.)  P_j goes to one of two shared-memory blocks as the second product's operand.
+// sum through shared memory.  P_j goes to one of two shared-memory blocks as the second product's operand.
 //   warp 0: TMA producer (Q tile, ring of K and V tiles: K_0 .. K_{n-1}, V_0 .. V_{n-1})
 //   warp 1: MMA issuer: the next item's scores are issued behind this item's last second product, so they
 //           are ready when the softmax warps have stored the context
-// Bound by the exponential unit (16 a clock: 1024 cycles per block) and the passes around it.  The form
-// before, with two groups of warps on items of their own and the scores formed twice, took 12.9 k cycles
-// per item of four blocks.
+// Bound by the exponential unit (16 a clock: 1024 cycles per block) and the passes around it.
+// 16 sequences x 16 heads x 512 keys: 59.5 us with two groups of warps on items of their own and the scores
+// formed twice; 49.5 us in this form with eight softmax warps (two per scheduler do not cover the
+// tensor-memory reads and the fences); 48.3 us with sixteen.  12 x 16 x 384 keys, uneven lengths: 27.5 us.
+// In steps of BERT-Large at 16 x (256..512) keys, packed tiles dealt out longest first: 56.8 -> 52.1 us a layer.
 constexpr int AR_RING = 8;
 constexpr int AR_BARS = 2 + 2 * AR_RING + 1 + 2 * 2 + 2;
 constexpr int AR_WARPS = 16;  // softmax warps: four per TMEM lane quarter
