@@ -71,4 +71,11 @@ void attn_starve_next(int on);
 // Kernels launched by the GEMM front end since the library was loaded (for launch accounting).
 int64_t gemm_launches();
 
+// The same in fp32 (attn_f32.cu), S a multiple of 8 up to 128, rows not packed.  probs may be null in the
+// forward; the backward needs it, and the context.
+int attn_f32_fwd_launch(const float* qkv, float* probs, float* ctx, const int* seq_lens, int B, int S, int A, float scale,
+                        cudaStream_t st, char* err);
+int attn_f32_bwd_launch(const float* qkv, const float* probs, const float* ctx, const float* dctx, float* dqkv,
+                        const int* seq_lens, int B, int S, int A, float scale, cudaStream_t st, char* err);
+
 }  // namespace mslt

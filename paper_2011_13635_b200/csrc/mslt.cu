@@ -390,6 +390,10 @@ bool getenv_unfused_attention() {
 
 // bf16 attention runs in the fused kernels (head width 64 and S <= 512 are checked at creation)
 bool fused_attention(const mslt_ctx* c) { return c->bf && !getenv_cuda_cores() && !getenv_unfused_attention(); }
+// fp32 attention of head width 64 does so for rows of at most 128 keys (see attn_f32.cu)
+bool fused_attention_f32(const mslt_ctx* c, int S) {
+  return !c->bf && c->a.hidden == 64 * c->a.heads && S <= 128 && !getenv_unfused_attention();
+}
 
 // scores, masked softmax and context of one layer in one kernel; for the backward pass either the
 // probabilities (S <= 128) or the rows' sums of exponentials (lse)
@@ -398,7 +402,9 @@ int run_attention(mslt_ctx* c, const void* qkv, void* probs, float* lse, void* c
   char err[256] = "";
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
-  int rc = attn_fwd_launch(qkv, probs, ctx, seq_lens, B, S, A, d, scale, c->ws.scalars, c->st, err, c->cu, c->rows, lse, c->ws.order);
+  int rc = c->bf ? attn_fwd_launch(qkv, probs, ctx, seq_lens, B, S, A, d, scale, c->ws.scalars, c->st, err, c->cu, c->rows, lse,
+                                   c->ws.order)
+                 : attn_f32_fwd_launch((const float*)qkv, (float*)probs, (float*)ctx, seq_lens, B, S, A, scale, c->st, err);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({1, 4.0 * B * A * (double)S * S * d});
@@ -414,7 +420,9 @@ int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const voi
   const bool prof = c->profile && c->prec.size() * 2 + 2 <= c->pev.size();
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
   // rows of more than 128 keys keep their sums of exponentials in the place of the probabilities
-  int rc = S <= 128 ? attn_bwd_launch(qkv, probs, dctx, dqkv, B, S, A, d, scale, c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows)
+  int rc = !c->bf ? attn_f32_bwd_launch((const float*)qkv, (const float*)probs, (const float*)ctx, (const float*)dctx,
+                                        (float*)dqkv, seq_lens, B, S, A, scale, c->st, err)
+         : S <= 128 ? attn_bwd_launch(qkv, probs, dctx, dqkv, B, S, A, d, scale, c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows)
                     : attn_bwd_long_launch(qkv, ctx, dctx, (const float*)probs, (float*)c->ws.dp, dqkv, B, S, A, scale,
                                            c->ws.scalars, c->st, err, seq_lens, c->cu, c->rows, c->ws.order);
   if (prof) {
@@ -422,7 +430,7 @@ int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const voi
     c->prec.push_back({1, 8.0 * B * A * (double)S * S * d});
   }
   if (rc) return fail(rc, "%s", err);
-  c->launches += S <= 128 ? 1 : 3;
+  c->launches += !c->bf || S <= 128 ? 1 : 3;
   return 0;
 }
 
@@ -548,6 +556,8 @@ int layer_forward(mslt_ctx* c, int l, const void* x, LayerBuf& b, void* out, boo
     // the probabilities go to memory only where the backward pass will read them
     TRY(run_attention(c, b.qkv, save && S <= 128 ? b.p : nullptr, save && S > 128 ? (float*)b.p : nullptr, b.c, seq_lens, B,
                       S, A, d, scale));
+  } else if (fused_attention_f32(c, S)) {
+    TRY(run_attention(c, b.qkv, save ? b.p : nullptr, nullptr, b.c, seq_lens, B, S, A, d, scale));
   } else {
     {  // scores[b,h,i,j] = q_i . k_j / sqrt(d)
       Lin g(c, S, S, d);
@@ -604,7 +614,7 @@ int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void
   TRY(linear_wgrad(c, w.dz1, T, H, H, b.c, H, toff(c, l, "out.weight"), c->rows));
   TRY(linear_dgrad(c, w.dz1, T, H, H, toff(c, l, "out.weight"), H, w.dc, 0, nullptr, nullptr, c->rows));
   const int64_t qs = (int64_t)S * 3 * H, ps = (int64_t)A * S * S, cs = (int64_t)S * H;
-  if (fused_attention(c)) {
+  if (fused_attention(c) || fused_attention_f32(c, S)) {
     // dV, dP, softmax backward, dQ and dK of the layer in one kernel
     TRY(run_attention_bwd(c, b.qkv, b.p, b.c, w.dc, w.dqkv, seq_lens, B, S, A, d, scale));
   } else {

@@ -225,3 +225,12 @@ def test_fp32_base_shapes_on_split_operands(layers, trainable, batch, seq):
     cfg = I.scaled(I.CONFIGS["base_stage"], layers=layers, trainable=trainable, batch=batch, seq=seq, pred=11,
                    dtype="fp32", varlen=(seq // 3, seq))
     _run(cfg, steps=2, lr=1e-3)
+
+
+@pytest.mark.parametrize("seq,varlen", [(8, (1, 8)), (40, None), (64, (1, 64)), (72, (5, 72)), (128, (30, 128)), (136, (1, 136))])
+def test_fp32_attention_row_lengths(seq, varlen):
+    """The fused fp32 attention at the edges of its 32-row blocks and 64-row buffers (and the batched
+    products just beyond its range), lengths that leave whole blocks without keys."""
+    cfg = I.StageConfig("attn32", hidden=128, heads=2, ffn=128, vocab=131, max_pos=136, layers=1, trainable=1, batch=4,
+                        seq=seq, pred=5, dtype="fp32", varlen=varlen, seed_index=37)
+    _run(cfg, steps=2, lr=1e-3)
