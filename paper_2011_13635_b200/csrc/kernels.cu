@@ -262,18 +262,18 @@ embed_ln_kernel(const int* __restrict__ tokens, const int* __restrict__ segments
 // LayerNorm backward: dz = rstd * (dxhat - mean(dxhat) - xhat * mean(dxhat * xhat)),
 // dgamma += sum_rows dy * xhat, dbeta += sum_rows dy and, when asked for, dbias += sum_rows dz
 // (the bias gradient of the linear layer whose output was normalised) - fp32 atomics, one per
-// column per block.
+// column per block.  kGelu: the normalised rows came out of a GELU of gelu_u, and dz is taken through it.
 // A row is split over NSLICE warps, each owning one 16-byte vector per lane, so that the column
 // accumulators cost a lane 3 x 8 registers instead of 3 x 24 and twice as many loads are in
 // flight per SM; a warp works on LN_BWD_ROWS rows at once and the NSLICE partial row sums meet in shared
 // memory (double-buffered: one block barrier per LR rows).
 // ---------------------------------------------------------------------------------------
-template <typename T, int NSLICE, int RG, int LN_BWD_ROWS>
+template <typename T, int NSLICE, int RG, int LN_BWD_ROWS, bool kGelu>
 __global__ void __launch_bounds__(NSLICE * RG * 32, 1)
 ln_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ z, const float* __restrict__ stats,
               const float* __restrict__ gamma, T* __restrict__ dz, float* __restrict__ dgamma,
               float* __restrict__ dbeta, float* __restrict__ dbias, int rows, int H,
-              const int* __restrict__ rows_dev) {
+              const int* __restrict__ rows_dev, const T* __restrict__ gelu_u) {
   pdl_begin();
   if (rows_dev != nullptr) rows = rows_dev[1];
   constexpr int VN = VecT<T>::N;
@@ -380,8 +380,17 @@ ln_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ z, const float* __
           const float2 gr = __fmul2_rn(make_float2(g[e], g[e + 1]), r2);
           const float2 o2 = __ffma2_rn(make_float2(a[e], a[e + 1]), gr,
                                        __ffma2_rn(make_float2(b[e], b[e + 1]), c22, c32));
-          const float2 za = __fadd2_rn(o2, make_float2(az[e], az[e + 1]));
           o[e] = o2.x; o[e + 1] = o2.y;
+        }
+        if (kGelu) {
+          float u[VN];
+          VecT<T>::load(gelu_u + (int64_t)(row0 + k) * H + c, u);
+#pragma unroll
+          for (int e = 0; e < VN; e++) o[e] = to_f<T>(from_f<T>(o[e])) * gelu_grad_f(u[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < VN; e += 2) {
+          const float2 za = __fadd2_rn(make_float2(o[e], o[e + 1]), make_float2(az[e], az[e + 1]));
           az[e] = za.x; az[e + 1] = za.y;
         }
         VecT<T>::store(dz + (int64_t)(row0 + k) * H + c, o);
@@ -561,13 +570,32 @@ softmax_bwd_kernel(T* __restrict__ dp, const T* __restrict__ p, int rows, int S,
 // ---------------------------------------------------------------------------------------
 // MLM slots: validity, source rows, labels, count; sequence-length check.
 // ---------------------------------------------------------------------------------------
-__global__ void slots_prepare_kernel(const int* __restrict__ positions,
+// The bias correction 1 / (1 - beta^t) of the step after the *t that have been taken, formed on the device so
+// that a captured step (CUDA graph) replays with the right values; second: that of the second moment.
+__device__ __forceinline__ void form_bias_correction(const int* t, float* bc, float beta1, float beta2, int on, bool second) {
+  bc[second] = on ? (float)(1.0 / (1.0 - pow((double)(second ? beta2 : beta1), (double)(*t + 1)))) : 1.f;
+}
+
+// One launch opens a call: block 0 clears the status words and prepares the slots (and the packed layout),
+// the others zero what the call adds into.  (A memset per range cost 1.5 us each and its gap, and broke the
+// chain of early launches.)
+__global__ void step_prepare_kernel(const ZeroRanges zr, int* __restrict__ scalars, const int* __restrict__ positions,
                                      const int* __restrict__ labels,
                                      const int* __restrict__ seq_lens, int B, int S, int P, int V,
                                      int* __restrict__ rowsrc, int* __restrict__ rowlabel,
-                                     int* __restrict__ n_valid, float* __restrict__ inv_n,
-                                     int* __restrict__ status, int* __restrict__ cu, int* __restrict__ rows, int* __restrict__ order) {
+                                     int* __restrict__ cu, int* __restrict__ rows, int* __restrict__ order) {
   pdl_begin();
+  if (blockIdx.x > 0) {
+    const int64_t first = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x, step = (int64_t)(gridDim.x - 1) * blockDim.x;
+    for (int k = 0; k < zr.n; k++)
+      for (int64_t i = first; i < zr.vecs[k]; i += step) reinterpret_cast<uint4*>(zr.p[k])[i] = make_uint4(0, 0, 0, 0);
+    return;
+  }
+  int* status = scalars;
+  int* n_valid = scalars + 1;
+  float* inv_n = (float*)(scalars + 2);
+  if (threadIdx.x < 4) scalars[threadIdx.x] = 0;
+  __syncthreads();
   __shared__ int cnt;
   if (cu != nullptr) {
     // packed batch: first row of every sequence, and {rows in use, the same rounded up to a tile}
@@ -626,9 +654,9 @@ __global__ void slots_prepare_kernel(const int* __restrict__ positions,
       const int at = atomicAdd(&bucket[n], n);  // the order inside a length changes nothing
       for (int t = 0; t < n; t++) order[at + t] = 8 * b + t;
     }
-    if (positions == nullptr) return;  // the layout was all that was asked for
     __syncthreads();
   }
+  if (positions == nullptr) return;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
   int local = 0, bad = 0;
@@ -720,6 +748,78 @@ copy_rows_kernel(const float* __restrict__ in, int64_t ldi, float* __restrict__ 
       if (c >= V) continue;
       if (VN == 2) __stcs(reinterpret_cast<float2*>(dst + c), v[u]);
       else __stcs(dst + c, v[u].x);
+    }
+  }
+}
+
+// The gradient that enters the layer stack: dx[row,:] = sum of d[r,:] over the slots r with rowsrc[r] = row,
+// zero for the rows without one, so that dx needs no clearing.  A block of 8 warps owns 32 rows of one
+// sequence, a warp four of them.  The last block zeroes the rows that pad a packed batch and does the
+// step's scalar work: the loss, and the bias corrections of the optimizer's next step count.
+// 8192 x 1024 bf16 with 1280 slots: 41 us as a memset and a walk over the slots, under 18 us in this form.
+template <typename T>
+__global__ void __launch_bounds__(256)
+head_dx_kernel(const T* __restrict__ d, const int* __restrict__ rowsrc, T* __restrict__ dx, int B, int P, int S, int H,
+               int chunks, const int* __restrict__ cu, const int* __restrict__ rows_dev, const HeadScalars hs) {
+  pdl_begin();
+  constexpr int VN = VecT<T>::N;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float zero[VN];
+#pragma unroll
+  for (int e = 0; e < VN; e++) zero[e] = 0.f;
+  if ((int)blockIdx.x == B * chunks) {
+    if (rows_dev != nullptr) {
+      T* tail = dx + (int64_t)rows_dev[0] * H;
+      for (int i = threadIdx.x * VN; i < (rows_dev[1] - rows_dev[0]) * H; i += 256 * VN) VecT<T>::store(tail + i, zero);
+    }
+    __shared__ float part[8];
+    float sum = 0.f;
+#pragma unroll 4
+    for (int r = threadIdx.x; r < hs.R; r += 256) sum += hs.nll[r];
+    sum = warp_sum(sum);
+    if (lane == 0) part[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float t = 0.f;
+      for (int w = 0; w < 8; w++) t += part[w];
+      *hs.loss = t * (*hs.inv_n);
+    }
+    if (threadIdx.x == 32 || threadIdx.x == 64) form_bias_correction(hs.t, hs.bc, hs.beta1, hs.beta2, hs.bias_correction, threadIdx.x == 64);
+    return;
+  }
+  const int b = blockIdx.x / chunks, s0 = (blockIdx.x - b * chunks) * 32 + warp;
+  const int row0 = cu ? cu[b] : b * S, len = cu ? cu[b + 1] - row0 : S;
+  int first[4], count[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) { first[i] = -1; count[i] = 0; }
+  for (int j0 = 0; j0 < P; j0 += 32) {
+    const int src = j0 + lane < P ? rowsrc[b * P + j0 + lane] : -1;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const unsigned hit = __ballot_sync(0xffffffffu, src == row0 + s0 + 8 * i);
+      if (hit && first[i] < 0) first[i] = j0 + __ffs(hit) - 1;
+      count[i] += __popc(hit);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    if (s0 + 8 * i >= len) break;
+    T* out = dx + (int64_t)(row0 + s0 + 8 * i) * H;
+    for (int c = lane * VN; c < H; c += 32 * VN) {
+      if (count[i] == 0) {
+        VecT<T>::store(out + c, zero);
+        continue;
+      }
+      float a[VN];
+      VecT<T>::load(d + (int64_t)(b * P + first[i]) * H + c, a);
+      for (int j = first[i] + 1; count[i] > 1 && j < P; j++) {  // slots that name a row again
+        if (rowsrc[b * P + j] != row0 + s0 + 8 * i) continue;
+        float t[VN];
+        VecT<T>::load(d + (int64_t)(b * P + j) * H + c, t);
+#pragma unroll
+        for (int e = 0; e < VN; e++) a[e] += t[e];
+      }
+      VecT<T>::store(out + c, a);
     }
   }
 }
@@ -1244,22 +1344,19 @@ embed_pos_grad_kernel(const T* __restrict__ dz, float* __restrict__ dpos, int B,
 // ---------------------------------------------------------------------------------------
 // Adam with decoupled weight decay over a table of chunks of the trainable slice.
 // ---------------------------------------------------------------------------------------
-// Advances the step count kept in device memory and forms the bias corrections 1 / (1 - beta^t)
-// there, so that a captured step (CUDA graph) replays with the right values.
-__global__ void adam_tick_kernel(int* __restrict__ t, float* __restrict__ bc, float beta1, float beta2,
-                                 int bias_correction) {
+// The corrections by themselves, for an update that is not part of a step call.
+__global__ void bias_correction_kernel(const int* __restrict__ t, float* __restrict__ bc, float beta1, float beta2,
+                                       int bias_correction) {
   pdl_begin();
-  const int n = *t + 1;
-  *t = n;
-  bc[0] = bias_correction ? (float)(1.0 / (1.0 - pow((double)beta1, (double)n))) : 1.f;
-  bc[1] = bias_correction ? (float)(1.0 / (1.0 - pow((double)beta2, (double)n))) : 1.f;
+  form_bias_correction(t, bc, beta1, beta2, bias_correction, threadIdx.x == 1);
 }
 
 __global__ void __launch_bounds__(256)
 adam_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w,
             const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-            bf16* __restrict__ wb, AdamHyper h, const float* __restrict__ bc) {
+            bf16* __restrict__ wb, AdamHyper h, const float* __restrict__ bc, int* __restrict__ t) {
   pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *t += 1;  // read by the next step only
   h.bc1 = bc[0];
   h.bc2 = bc[1];
   const AdamChunk ch = chunks[blockIdx.x];
@@ -1444,8 +1541,10 @@ lamb_moments_kernel(const AdamChunk* __restrict__ chunks, const float* __restric
 __global__ void __launch_bounds__(256)
 lamb_apply_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w, const float* __restrict__ m,
                   const float* __restrict__ v, bf16* __restrict__ wb, AdamHyper h,
-                  const float* __restrict__ bc, const float* __restrict__ norms) {
+                  const float* __restrict__ bc, const float* __restrict__ norms,
+                  int* __restrict__ t) {
   pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *t += 1;
   h.bc1 = bc[0];
   h.bc2 = bc[1];
   const AdamChunk ch = chunks[blockIdx.x];
@@ -1471,22 +1570,6 @@ lamb_apply_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ w, c
       pk.y = *reinterpret_cast<uint32_t*>(&hi);
       *reinterpret_cast<uint2*>(wb + o) = pk;
     }
-  }
-}
-
-// d[i] *= gelu'(u[i]) (MLM transform backward)
-template <typename T>
-__global__ void dgelu_kernel(T* __restrict__ d, const T* __restrict__ u, int64_t n) {
-  pdl_begin();
-  constexpr int VN = VecT<T>::N;
-  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * VN; i < n;
-       i += (int64_t)gridDim.x * blockDim.x * VN) {
-    float a[VN], b[VN];
-    VecT<T>::load(d + i, a);
-    VecT<T>::load(u + i, b);
-#pragma unroll
-    for (int e = 0; e < VN; e++) a[e] *= gelu_grad_f(b[e]);
-    VecT<T>::store(d + i, a);
   }
 }
 
@@ -1535,7 +1618,7 @@ void launch_embed_ln(bool bf, const int* tokens, const int* segments, const void
 
 void launch_ln_bwd(bool bf, const void* dy, const void* z, const float* stats, const float* gamma,
                    void* dz, float* dgamma, float* dbeta, float* dbias, int rows, int H, cudaStream_t st,
-                   const int* rows_dev) {
+                   const int* rows_dev, const void* gelu_u) {
   if (rows <= 0) return;
   // warps per row: one 16-byte vector per lane; row groups fill the block up to 12-16 warps
   const int vn = bf ? 8 : 4;
@@ -1545,8 +1628,9 @@ void launch_ln_bwd(bool bf, const void* dy, const void* z, const float* stats, c
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // one block per SM walks the rows: the column sums end in one atomic per column and block
 #define LN_BWD(NS, RG)                                                                                   \
-  DISPATCH_T(bf, (launch_pdl(ln_bwd_kernel<T, NS, RG, 4>, std::min(div_up(rows, RG * 4), sms), NS * RG * 32, 0, st,  \
-                     (const T*)dy, (const T*)z, stats, gamma, (T*)dz, dgamma, dbeta, dbias, rows, H, rows_dev)))
+  DISPATCH_T(bf, (launch_pdl(gelu_u ? ln_bwd_kernel<T, NS, RG, 4, true> : ln_bwd_kernel<T, NS, RG, 4, false>,            \
+                     std::min(div_up(rows, RG * 4), sms), NS * RG * 32, 0, st, (const T*)dy, (const T*)z, stats, gamma,  \
+                     (T*)dz, dgamma, dbeta, dbias, rows, H, rows_dev, (const T*)gelu_u)))
   if (nslice <= 1) LN_BWD(1, 8);
   else if (nslice <= 2) LN_BWD(2, 6);
   else if (nslice <= 3) LN_BWD(3, 4);
@@ -1586,11 +1670,15 @@ void launch_softmax_bwd(bool bf, void* dp, const void* p, int rows, int S, float
 #undef SM_BWD
 }
 
-void launch_slots_prepare(const int* positions, const int* labels, const int* seq_lens, int B,
-                          int S, int P, int V, int* rowsrc, int* rowlabel, int* n_valid,
-                          float* inv_n, int* status, cudaStream_t st, int* cu, int* rows, int* order) {
-  launch_pdl(slots_prepare_kernel, 1, cu || B * P > 1024 ? 1024 : 256, 0, st, positions, labels, seq_lens, B, S, P, V,
-             rowsrc, rowlabel, n_valid, inv_n, status, cu, rows, order);
+void launch_step_prepare(const ZeroRanges& zr, int* scalars, const int* positions, const int* labels, const int* seq_lens,
+                         int B, int S, int P, int V, int* rowsrc, int* rowlabel, cudaStream_t st, int* cu, int* rows,
+                         int* order) {
+  const int threads = cu || B * P > 1024 ? 1024 : 256;
+  int64_t vecs = 0;
+  for (int k = 0; k < zr.n; k++) vecs += zr.vecs[k];
+  const int blocks = 1 + (int)std::min<int64_t>((vecs + threads * 4 - 1) / (threads * 4), 148 * 2048 / threads);
+  launch_pdl(step_prepare_kernel, blocks, threads, 0, st, zr, scalars, positions, labels, seq_lens, B, S, P, V,
+             rowsrc, rowlabel, cu, rows, order);
 }
 
 void launch_gather_rows(bool bf, const void* x, const int* rowsrc, void* out, int R, int H,
@@ -1615,6 +1703,13 @@ void launch_scatter_rows(bool bf, const void* d, const int* rowsrc, void* dx, in
                          cudaStream_t st) {
   if (B <= 0 || P <= 0) return;
   DISPATCH_T(bf, (launch_pdl(scatter_rows_kernel<T>, B, 128, 0, st, (const T*)d, rowsrc, (T*)dx, P, H)));
+}
+
+void launch_head_dx(bool bf, const void* d, const int* rowsrc, void* dx, int B, int P, int S, int H, const int* cu,
+                    const int* rows_dev, const HeadScalars& hs, cudaStream_t st) {
+  const int chunks = div_up(S, 32);
+  DISPATCH_T(bf, (launch_pdl(head_dx_kernel<T>, B * chunks + 1, 256, 0, st, (const T*)d, rowsrc, (T*)dx, B, P, S, H, chunks, cu,
+                             rows_dev, hs)));
 }
 
 void launch_cross_entropy(bool bf, const float* logits, int64_t ldl, const int* rowlabel,
@@ -1655,8 +1750,6 @@ void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float*
   const int T = B * S;
   if (T <= 0) return;
   const int nb = div_up(T, ES_BLOCK), vb = div_up(V, 256);
-  cudaMemsetAsync(counts, 0, (size_t)nb * V * sizeof(int), st);
-  cudaMemsetAsync(hot, 0, 2 * sizeof(int), st);
   launch_pdl(embed_sort_count_kernel, nb, ES_BLOCK, 0, st, tokens, T, V, nb, counts, rank, rows_dev);
   launch_pdl(embed_sort_prefix_kernel, vb, 256, 0, st, counts, nb, V, total, start, blocksum, hot);
   launch_pdl(embed_sort_scan_kernel, 1, 1024, 0, st, blocksum, vb);
@@ -1676,21 +1769,18 @@ void launch_embed_grad_sorted(bool bf, const void* dz, const int* tokens, float*
 }
 
 void launch_adam(const AdamChunk* chunks, int n_chunks, float* w, const float* g, float* m, float* v,
-                 void* wb, const AdamHyper& h, int* t_dev, float* bc_dev, int bias_correction,
-                 cudaStream_t st) {
-  launch_pdl(adam_tick_kernel, 1, 1, 0, st, t_dev, bc_dev, h.beta1, h.beta2, bias_correction);
-  if (n_chunks <= 0) return;
-  launch_pdl(adam_kernel, n_chunks, 256, 0, st, chunks, w, g, m, v, (bf16*)wb, h, bc_dev);
+                 void* wb, const AdamHyper& h, int* t_dev, const float* bc_dev, cudaStream_t st) {
+  launch_pdl(adam_kernel, n_chunks, 256, 0, st, chunks, w, g, m, v, (bf16*)wb, h, bc_dev, t_dev);
 }
 
 void launch_lamb(const AdamChunk* chunks, int n_chunks, float* w, const float* g, float* m, float* v,
-                 void* wb, const AdamHyper& h, int* t_dev, float* bc_dev, int bias_correction,
-                 float* norms, int n_tensors, cudaStream_t st) {
-  launch_pdl(adam_tick_kernel, 1, 1, 0, st, t_dev, bc_dev, h.beta1, h.beta2, bias_correction);
-  if (n_chunks <= 0) return;
-  cudaMemsetAsync(norms, 0, (size_t)n_tensors * 2 * sizeof(float), st);
+                 void* wb, const AdamHyper& h, int* t_dev, const float* bc_dev, float* norms, cudaStream_t st) {
   launch_pdl(lamb_moments_kernel, n_chunks, 256, 0, st, chunks, w, g, m, v, h, bc_dev, norms);
-  launch_pdl(lamb_apply_kernel, n_chunks, 256, 0, st, chunks, w, m, v, (bf16*)wb, h, bc_dev, norms);
+  launch_pdl(lamb_apply_kernel, n_chunks, 256, 0, st, chunks, w, m, v, (bf16*)wb, h, bc_dev, norms, t_dev);
+}
+
+void launch_bias_correction(const int* t_dev, float* bc_dev, float beta1, float beta2, int bias_correction, cudaStream_t st) {
+  launch_pdl(bias_correction_kernel, 1, 2, 0, st, t_dev, bc_dev, beta1, beta2, bias_correction);
 }
 
 void launch_nsp_prepare(const int* labels, int B, int S, int* rowsrc, float* inv_n, const int* total_valid,
@@ -1718,13 +1808,6 @@ void launch_type_grad(bool bf, const void* dz, const int* segments, float* dtype
   const int rpb = 512;
   DISPATCH_T(bf, (launch_pdl(type_grad_kernel<T>, dim3(div_up(H, 128), div_up(rows, rpb)), 128, 0, st, 
                      (const T*)dz, segments, dtype, rows, H, rpb, rows_dev)));
-}
-
-void launch_dgelu(bool bf, void* d, const void* u, int64_t n, cudaStream_t st) {
-  if (n <= 0) return;
-  const int vn = bf ? 8 : 4;
-  int blocks = (int)std::min<int64_t>((n / vn + 255) / 256, 148 * 8);
-  DISPATCH_T(bf, (launch_pdl(dgelu_kernel<T>, blocks, 256, 0, st, (T*)d, (const T*)u, n)));
 }
 
 void launch_f32_to_bf16(const float* src, void* dst, int64_t n, cudaStream_t st) {

@@ -113,6 +113,7 @@ struct mslt_ctx {
   const int *cu, *rows;
   const void* a_split;  // fp32: left operand whose planes the last product left in x3a
   bool emb_split;       // fp32: x3e holds the planes of this call's word table
+  int* host_words;      // pinned copy of the status word, slot counts and loss
   int64_t launches;
   int Vp, num_sms;
   bool timing;
@@ -703,7 +704,6 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
     if (c->bf) {
       // few output tiles, a contraction over the whole vocabulary: split it across the machine
       // with fp32 partial sums, then round once to bf16
-      CUDA_TRY(cudaMemsetAsync(w.dtm32, 0, (size_t)R * H * 4, c->st));
       g.d.D = w.dtm32; g.d.ldd = H; g.d.d_fp32 = 1; g.d.accumulate = 1;
       g.d.split_k = dtm_splits(c, R);
       TRY(run_gemm(c, g.d));
@@ -721,24 +721,34 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
     TRY(run_gemm(c, g.d, nullptr, 0, true));
   }
   KL(PC_LN_BWD, 3.0 * R * H * c->esz, launch_ln_bwd(c->bf, w.dtm, w.gt, w.hst, Wv(c, toff(c, -1, "head.ln.gamma")), w.dgt,
-                   G(c, toff(c, -1, "head.ln.gamma")), G(c, toff(c, -1, "head.ln.beta")), nullptr, R, H, c->st));
-  KL(PC_OTHER, 3.0 * R * H * c->esz, launch_dgelu(c->bf, w.dgt, w.ut, (int64_t)R * H, c->st));
+                   G(c, toff(c, -1, "head.ln.gamma")), G(c, toff(c, -1, "head.ln.beta")), G(c, toff(c, -1, "head.transform.bias")), R, H, c->st,
+                   nullptr, w.ut));
   TRY(linear_wgrad(c, w.dgt, R, H, H, w.hm, H, toff(c, -1, "head.transform.weight")));
-  KL(PC_COLSUM, 1.0 * R * H * c->esz, launch_colsum(c->bf, w.dgt, H, R, H, G(c, toff(c, -1, "head.transform.bias")), c->st));
   TRY(linear_dgrad(c, w.dgt, R, H, H, toff(c, -1, "head.transform.weight"), H, w.dhm, 0, nullptr, nullptr));
-  CUDA_TRY(cudaMemsetAsync(w.dxa, 0, (size_t)B * S * H * c->esz, c->st));
-  KL(PC_OTHER, 2.0 * B * P * H * c->esz, launch_scatter_rows(c->bf, w.dhm, w.rowsrc, w.dxa, B, P, H, c->st));
+  HeadScalars hs = {w.nll, (const float*)(w.scalars + 2), (float*)(w.scalars + 3), R, w.scalars + 4, (float*)(w.scalars + 5),
+                    c->opt.beta1, c->opt.beta2, c->opt.bias_correction};
+  KL(PC_OTHER, 1.0 * B * S * H * c->esz, launch_head_dx(c->bf, w.dhm, w.rowsrc, w.dxa, B, P, S, H, c->cu, c->rows, hs, c->st));
   return 0;
 }
 
-int zero_trainable_grads(mslt_ctx* c) {
+// everything a step adds into
+ZeroRanges step_zero_ranges(mslt_ctx* c, int T, int R) {
   const int first = c->L - c->top_k;
-  if (c->top_k == c->L) CUDA_TRY(cudaMemsetAsync(c->grad + c->emb_off, 0, c->emb_cnt * 4, c->st));
+  const int64_t H = c->a.hidden;
+  Workspace& w = c->ws;
+  ZeroRanges z = {};
+  if (c->top_k == c->L) {
+    z.add(c->grad + c->emb_off, c->emb_cnt * 4);
+    z.add(w.es_counts, ((int64_t)T + 255) / 256 * c->a.vocab * 4);
+    z.add(w.es_hot, 2 * 4);
+  }
   if (c->top_k > 0)
-    CUDA_TRY(cudaMemsetAsync(c->grad + c->layer0_off + (int64_t)(first / group_of(c->a)) * c->layer_cnt, 0,
-                             (size_t)(c->top_k / group_of(c->a)) * c->layer_cnt * 4, c->st));
-  CUDA_TRY(cudaMemsetAsync(c->grad + c->head_off, 0, c->head_cnt * 4, c->st));
-  return 0;
+    z.add(c->grad + c->layer0_off + (int64_t)(first / group_of(c->a)) * c->layer_cnt,
+          (int64_t)(c->top_k / group_of(c->a)) * c->layer_cnt * 4);
+  z.add(c->grad + c->head_off, c->head_cnt * 4);
+  if (c->bf) z.add(w.dtm32, R * H * 4);
+  z.add(w.norms, (int64_t)c->tensors.size() * 2 * 4);
+  return z;
 }
 
 // Gradient buckets in the order in which a step completes them: the output layer, the trainable
@@ -789,9 +799,8 @@ void pack_batch(mslt_ctx* c, const int* seq_lens) {
 int finish(mslt_ctx* c, float* loss_out) {
   CUDA_TRY(cudaGetLastError());
   if (!loss_out) return 0;
-  int h[4];
-  CUDA_TRY(cudaStreamSynchronize(c->st));
-  CUDA_TRY(cudaMemcpyAsync(h, c->ws.scalars, 16, cudaMemcpyDeviceToHost, c->st));
+  const int* h = c->host_words;  // pinned, so that the copy is one more entry of the stream and one wait is enough
+  CUDA_TRY(cudaMemcpyAsync(c->host_words, c->ws.scalars, 16, cudaMemcpyDeviceToHost, c->st));
   CUDA_TRY(cudaStreamSynchronize(c->st));
   memcpy(loss_out, &h[3], 4);
   if (h[0] != 0)
@@ -889,6 +898,10 @@ int mslt_create(const mslt_arch* arch, void* dev_params, size_t param_bytes, voi
   }
   int rc = rebuild_chunks(c);
   if (rc) { delete c; return rc; }
+  if (cudaHostAlloc((void**)&c->host_words, 16, cudaHostAllocDefault) != cudaSuccess) {
+    delete c;
+    return fail(MSLT_ERR_CUDA, "no pinned host memory");
+  }
   *out = c;
   return 0;
 }
@@ -900,6 +913,7 @@ int mslt_destroy(mslt_ctx* c) {
   for (cudaEvent_t e : c->pev) cudaEventDestroy(e);
   for (cudaEvent_t e : c->bev) cudaEventDestroy(e);
   if (c->comm_done) cudaEventDestroy(c->comm_done);
+  cudaFreeHost(c->host_words);
   delete c;
   return 0;
 }
@@ -944,7 +958,7 @@ int mslt_set_optimizer(mslt_ctx* c, const mslt_opt* o) {
   return 0;
 }
 
-static int apply_update(mslt_ctx* c);
+static int apply_update(mslt_ctx* c, bool separate);
 
 // forward, loss and backward of one step; the optimizer runs too unless `defer_update`
 static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens,
@@ -969,12 +983,12 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
     for (int i = 0; i < 6; i++) CUDA_TRY(cudaEventCreate(&c->ev[i]));
     c->have_events = true;
   }
-  CUDA_TRY(cudaMemsetAsync(w.scalars, 0, 16, c->st));
   c->prec.clear();
   mark(c, 0);
   pack_batch(c, d_seq_lens);
-  KL(PC_OTHER, 16.0 * B * P, launch_slots_prepare(d_pos, d_lab, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel, w.scalars + 1,
-                          inv_n, status, c->st, c->cu ? w.cu : nullptr, w.rows, w.order));
+  const ZeroRanges zr = step_zero_ranges(c, T, R);
+  KL(PC_OTHER, 16.0 * B * P, launch_step_prepare(zr, w.scalars, d_pos, d_lab, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel, c->st,
+                                                 c->cu ? w.cu : nullptr, w.rows, w.order));
   if (d_total_valid)  // the mean runs over the valid slots of every rank's batch
     KL(PC_OTHER, 8.0, launch_override_inv_n(d_total_valid, inv_n, c->st));
   // embeddings, then the frozen prefix: forward only, two buffers, nothing kept but the output
@@ -999,7 +1013,6 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
   mark(c, 2);
   TRY(head_forward(c, cur, R, true));
   KL(PC_CROSS_ENTROPY, (double)R * c->Vp * (4 + c->esz), launch_cross_entropy(c->bf, w.logits, c->Vp, w.rowlabel, inv_n, w.dlogits, c->Vp, w.nll, R, V, c->st));
-  KL(PC_OTHER, 4.0 * R, launch_loss_reduce(w.nll, R, inv_n, loss, c->st));
   const bool nsp = c->a.nsp && d_nsp_lab != nullptr;
   float* nsp_inv_n = (float*)(w.scalars + 7);
   if (nsp) {
@@ -1011,7 +1024,6 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
                    nullptr, nullptr));
     KL(PC_OTHER, 2.0 * B * H * c->esz, launch_tanh(c->bf, w.up, w.pooled, (int64_t)B * H, c->st));
   }
-  TRY(zero_trainable_grads(c));
   TRY(head_backward(c, B, S, P, full));
   if (nsp) {
     // classifier, its loss (added to the MLM loss) and its gradients; then back through the pooler
@@ -1044,7 +1056,7 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
     KL(PC_OTHER, 2.0 * T * H * c->esz, launch_embed_grad_sorted(c->bf, w.dz2, c->cu ? w.ptok : d_tokens, G(c, toff(c, -1, "emb.word")),
                             G(c, toff(c, -1, "emb.pos")), B, S, H, V, w.es_counts, w.es_total, w.es_start,
                             w.es_rank, w.es_order, w.es_blocksum, w.es_hot, w.es_partial, c->st, c->cu, c->rows));
-    c->launches += 8;
+    c->launches += 7;
     if (c->a.nsp)
       KL(PC_OTHER, 1.0 * T * H * c->esz, launch_type_grad(c->bf, w.dz2, c->cu ? w.pseg : d_seg, G(c, toff(c, -1, "emb.type")), T, H, c->st, c->rows));
     TRY(bucket_done(c, c->top_k / group_of(c->a) + 1));
@@ -1054,7 +1066,7 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
     c->pending_update = true;
     return finish(c, loss_out);
   }
-  TRY(apply_update(c));
+  TRY(apply_update(c, false));
   mark(c, 5);
   if (c->timing && c->have_events) {
     CUDA_TRY(cudaEventSynchronize(c->ev[5]));
@@ -1073,7 +1085,8 @@ static int step_impl(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_
 }
 
 // the optimizer on the trainable slice (Adam or LAMB), after any gradient exchange
-static int apply_update(mslt_ctx* c) {
+// separate: not inside a step call, which has formed the bias corrections on its way
+static int apply_update(mslt_ctx* c, bool separate) {
   Workspace& w = c->ws;
   if (c->bucket_fn && c->comm) {  // the reductions enqueued on the communication stream come first
     if (!c->comm_done) CUDA_TRY(cudaEventCreateWithFlags(&c->comm_done, cudaEventDisableTiming));
@@ -1087,14 +1100,15 @@ static int apply_update(mslt_ctx* c) {
   h.omb1 = (float)(1.0 - (double)c->opt.beta1);
   h.omb2 = (float)(1.0 - (double)c->opt.beta2);
   h.bc1 = h.bc2 = 1.f;  // formed on the device from the step count kept there
+  float* bc = (float*)(w.scalars + 5);
+  if (separate) KL(PC_OTHER, 8.0, launch_bias_correction(w.scalars + 4, bc, h.beta1, h.beta2, c->opt.bias_correction, c->st));
   if (c->opt.lamb) {
     KL(PC_ADAM, 42.0 * c->n_chunks * kAdamChunk, launch_lamb(w.chunks, c->n_chunks, c->master, c->grad, c->m, c->v, c->wb, h,
-                   w.scalars + 4, (float*)(w.scalars + 5), c->opt.bias_correction, w.norms, (int)c->tensors.size(), c->st));
-    c->launches += 2;  // step-count kernel, moments kernel, update kernel
+                   w.scalars + 4, bc, w.norms, c->st));
+    c->launches++;  // moments kernel and update kernel
   } else {
     KL(PC_ADAM, 30.0 * c->n_chunks * kAdamChunk, launch_adam(w.chunks, c->n_chunks, c->master, c->grad, c->m, c->v, c->wb, h, w.scalars + 4,
-                   (float*)(w.scalars + 5), c->opt.bias_correction, c->st));
-    c->launches++;  // step-count kernel and update kernel
+                   bc, c->st));
   }
   return 0;
 }
@@ -1122,7 +1136,7 @@ int mslt_step_apply(mslt_ctx* c) {
   if (!c) return fail(MSLT_ERR_ARG, "null context");
   if (!c->pending_update) return fail(MSLT_ERR_STATE, "mslt_step_apply without a preceding mslt_step_backward");
   c->pending_update = false;
-  TRY(apply_update(c));
+  TRY(apply_update(c, true));
   CUDA_TRY(cudaGetLastError());
   return 0;
 }
@@ -1161,11 +1175,9 @@ int mslt_forward(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens
   if (head && P < 1) return fail(MSLT_ERR_ARG, "P must be >= 1");
   Workspace& w = c->ws;
   const int H = c->a.hidden, V = c->a.vocab, T = B * S;
-  CUDA_TRY(cudaMemsetAsync(w.scalars, 0, 16, c->st));
   pack_batch(c, d_seq_lens);
-  if (head || c->cu)
-    KL(PC_OTHER, 8.0 * B * P, launch_slots_prepare(head ? d_pos : nullptr, nullptr, d_seq_lens, B, S, P, V, w.rowsrc, w.rowlabel,
-                            w.scalars + 1, (float*)(w.scalars + 2), w.scalars, c->st, c->cu ? w.cu : nullptr, w.rows, w.order));
+  KL(PC_OTHER, 8.0 * B * P, launch_step_prepare(ZeroRanges{}, w.scalars, head ? d_pos : nullptr, nullptr, d_seq_lens, B, S, P, V,
+                                                w.rowsrc, w.rowlabel, c->st, c->cu ? w.cu : nullptr, w.rows, w.order));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_embed_ln(c->bf, d_tokens, nullptr, Wc(c, toff(c, -1, "emb.word")), Wc(c, toff(c, -1, "emb.pos")),
                      c->a.nsp ? Wc(c, toff(c, -1, "emb.type")) : nullptr,
                      Wv(c, toff(c, -1, "emb.ln.gamma")), Wv(c, toff(c, -1, "emb.ln.beta")), w.xa,
@@ -1173,12 +1185,14 @@ int mslt_forward(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens
   char* cur = w.xa;
   for (int l = 0; l < c->L; l++) {
     char* out = cur == w.xa ? w.xb : w.xa;
+    // the last layer writes its rows where the caller wants them
+    if (l == c->L - 1 && d_hidden_out && !c->cu && ((uintptr_t)d_hidden_out & 15) == 0) out = (char*)d_hidden_out;
     TRY(layer_forward(c, l, cur, w.scratch, out, false, B, S, d_seq_lens));
     cur = out;
   }
   if (d_hidden_out && c->cu)
     KL(PC_OTHER, 2.0 * T * H * c->esz, launch_unpack_rows(c->bf, cur, c->cu, d_hidden_out, B, S, H, c->st));
-  else if (d_hidden_out)
+  else if (d_hidden_out && cur != d_hidden_out)
     CUDA_TRY(cudaMemcpyAsync(d_hidden_out, cur, (size_t)T * H * c->esz, cudaMemcpyDeviceToDevice, c->st));
   if (head) {
     TRY(head_forward(c, cur, B * P, false));

@@ -234,3 +234,21 @@ def test_fp32_attention_row_lengths(seq, varlen):
     cfg = I.StageConfig("attn32", hidden=128, heads=2, ffn=128, vocab=131, max_pos=136, layers=1, trainable=1, batch=4,
                         seq=seq, pred=5, dtype="fp32", varlen=varlen, seed_index=37)
     _run(cfg, steps=2, lr=1e-3)
+
+
+@pytest.mark.parametrize("dtype,seq,varlen,pred", [("fp32", 40, None, 5), ("fp32", 72, (20, 72), 33), ("bf16", 136, (40, 136), 9),
+                                                   ("bf16", 64, None, 40)])
+def test_slots_that_name_a_position_twice(dtype, seq, varlen, pred):
+    """The slots' gradients are gathered by row: rows with no slot, one, several (some in another group
+    of 32 slots), empty slots, and the rows that pad a packed batch."""
+    cfg = I.StageConfig("twice", hidden=128, heads=2, ffn=128, vocab=131, max_pos=136, layers=1, trainable=1, batch=3,
+                        seq=seq, pred=pred, dtype=dtype, varlen=varlen, seed_index=41)
+    m, oracle = PT.build_pair(cfg, lr=1e-4)
+    tok, lens, pos, lab = I.make_batch(cfg)
+    pos, lab = pos.copy(), lab.copy()
+    pos[:, -1] = pos[:, 0]
+    pos[:, 2] = pos[:, 1]
+    lab[:, -1], lab[:, 2] = lab[:, 0], lab[:, 1]
+    lab[0, 3] = -1
+    PT.compare_step(m, oracle, cfg, (tok, lens, pos, lab), PT.TOL[dtype], [])
+    m.close()
