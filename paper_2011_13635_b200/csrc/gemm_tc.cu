@@ -49,6 +49,7 @@ struct TcParams {
   char* D;
   long long ldd, d_bo, d_bi;
   int d_fp32, accumulate, vec_ok;
+  int x32;              // rows of the extra operand start on 32 bytes
   int direct;           // rows of D (and aux) may be stored straight from registers, 32 bytes at a time
   int tma_store;        // bf16 D leaves through shared memory and tile stores of 32 rows x 64 columns
   int d_perm[3];        // slots of D's (row, inner-batch, outer-batch) coordinates in its tensor map
@@ -134,6 +135,33 @@ __device__ __forceinline__ void row32_store_f32(float* dst, const float2 (&w)[16
   }
 }
 
+// GELU of a lane's 32 columns, eight at a time
+__device__ __forceinline__ void gelu_row(float2 (&v)[16]) {
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    float2 g[4] = {v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]};
+    gelu_fast2(g);
+#pragma unroll
+    for (int e = 0; e < 4; e++) v[4 * j + e] = g[e];
+  }
+}
+
+// 32 bf16 columns of a lane's row, two 32-byte loads
+__device__ __forceinline__ void row32_load_bf16(const bf16* src, uint4 (&x)[4]) {
+#pragma unroll
+  for (int c = 0; c < 2; c++)
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(x[2 * c].x), "=r"(x[2 * c].y), "=r"(x[2 * c].z), "=r"(x[2 * c].w), "=r"(x[2 * c + 1].x),
+                   "=r"(x[2 * c + 1].y), "=r"(x[2 * c + 1].z), "=r"(x[2 * c + 1].w)
+                 : "l"(src + 16 * c)
+                 : "memory");
+}
+
+// brings `bytes` (a multiple of 16) of 16-byte aligned global memory to L2
+__device__ __forceinline__ void prefetch_l2(const void* g, int bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g), "r"(bytes) : "memory");
+}
+
 // One 32 x 32 chunk of a specialised flavour: a = this lane's 32 accumulator columns, bias_c = the
 // chunk's bias values in shared memory (zeros without a bias), x = this lane's 32 bf16 values of
 // the row-shaped extra operand (EPI_RESIDUAL, EPI_DGELU).
@@ -142,10 +170,12 @@ __device__ __forceinline__ void row32_store_f32(float* dst, const float2 (&w)[16
 // edges element by element (every lane of the warp takes the same branch).
 // `tile` != 0: the bf16 result goes into that staging tile (shared-memory address) as half `half`
 // of its 64 columns instead, for a tile store by the caller.
-template <int kMode>
+// `loaded` runs once the accumulator columns have been used up, so that their registers can take the next
+// chunk's read while this chunk is worked on; `x_used` likewise for x.
+template <int kMode, typename F, typename G>
 __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)[32], const uint4 (&x)[4],
                                           const float* bias_c, uint8_t* stg, int lane, long long zoff,
-                                          int m_warp, int n0, bool direct, uint32_t tile = 0, int half = 0) {
+                                          int m_warp, int n0, bool direct, uint32_t tile, int half, F loaded, G x_used) {
   float2 v[16];
   const float2 al = splat2(p.alpha);
   const float4* b4 = reinterpret_cast<const float4*>(bias_c);
@@ -157,6 +187,7 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
     v[2 * j + 1] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j + 2]), __uint_as_float(a[4 * j + 3])), al,
                               make_float2(t.z, t.w));
   }
+  loaded();
   const bool row_ok = m_warp + lane < p.M;
   const long long off = zoff + (long long)(m_warp + lane) * p.ldd + n0;
   if constexpr (kMode == EPI_GELU_AUX) {
@@ -164,16 +195,16 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
     else stage_store_bf16(stg, lane, v, p.aux + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
   }
   if constexpr (kMode == EPI_GELU || kMode == EPI_GELU_AUX) {
-#pragma unroll
-    for (int j = 0; j < 16; j++) v[j] = gelu_fast2(v[j]);
+    gelu_row(v);
   }
   if constexpr (kMode == EPI_DGELU) {
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-      v[4 * j] = __fmul2_rn(v[4 * j], gelu_grad_fast2(bf162_to_f2(x[j].x)));
-      v[4 * j + 1] = __fmul2_rn(v[4 * j + 1], gelu_grad_fast2(bf162_to_f2(x[j].y)));
-      v[4 * j + 2] = __fmul2_rn(v[4 * j + 2], gelu_grad_fast2(bf162_to_f2(x[j].z)));
-      v[4 * j + 3] = __fmul2_rn(v[4 * j + 3], gelu_grad_fast2(bf162_to_f2(x[j].w)));
+      float2 g[4] = {bf162_to_f2(x[j].x), bf162_to_f2(x[j].y), bf162_to_f2(x[j].z), bf162_to_f2(x[j].w)};
+      if (j == 3) x_used();
+      gelu_grad_fast2(g);
+#pragma unroll
+      for (int e = 0; e < 4; e++) v[4 * j + e] = __fmul2_rn(v[4 * j + e], g[e]);
     }
   }
   if constexpr (kMode == EPI_RESIDUAL) {
@@ -190,7 +221,13 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
     else stage_store_f32(stg, lane, v, reinterpret_cast<float*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok,
                          p.accumulate);
   } else {
-    if (tile) row32_stage_bf16(tile, lane, half, v);
+    if (tile) {
+      if (half == 0) {  // the tile store of the previous group must have read the staging tile
+        if (lane == 0) tma_store_wait_read();
+        __syncwarp();
+      }
+      row32_stage_bf16(tile, lane, half, v);
+    }
     else if (direct) { if (row_ok) row32_store_bf16(reinterpret_cast<bf16*>(p.D) + off, v); }
     else stage_store_bf16(stg, lane, v, reinterpret_cast<bf16*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
   }
@@ -528,14 +565,32 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         auto chunk_ok = [&](int i) { return ccol(i) * 32 < p.bn && chunk_n0(i) < p.N; };
         auto prefetch_x = [&](int i, uint4 (&x)[4]) {
           if (kHasXf && row_ok) {
-            const uint4* src = reinterpret_cast<const uint4*>(xsrc + off0 + chunk_n0(i));
+            const bf16* row = xsrc + off0 + chunk_n0(i);
+            if (p.x32) {
+              row32_load_bf16(row, x);
+            } else {
+              const uint4* src = reinterpret_cast<const uint4*>(row);
 #pragma unroll
-            for (int j = 0; j < 4; j++) x[j] = src[j];
+              for (int j = 0; j < 4; j++) x[j] = src[j];
+            }
           }
         };
         // the next work item and its bias (the loads travel while this tile is worked on)
         int nt2 = nt, mt2 = mt, z2 = z, sp2 = sp;
         advance(nt2, mt2, z2, sp2);
+        if constexpr (kHasXf) {
+          // the next tile's rows of the extra operand start on their way to L2: they come from memory where
+          // the operand is as large as the output (with this, chunk reads issued early and the polynomials
+          // interleaved: 16384 x 768 x 768 + residual 39.4 -> 35.3 us, 16384 x 3072 x 768 . GELU' 106 -> 102,
+          // with both outputs of a GELU 93 -> 89)
+          if (hsel == 0 && w + w_step < total_work && mt2 * mt_rows + (int)cta_rank * BM + q * 32 + lane < p.M && p.direct) {
+            const int zo2 = p.hdiv == 1 ? z2 : z2 / p.hdiv, zi2 = p.hdiv == 1 ? 0 : z2 - zo2 * p.hdiv;
+            const int cols = min(p.bn, p.N - nt2 * p.bn) & ~7;
+            if (cols > 0)
+              prefetch_l2(xsrc + zo2 * p.d_bo + zi2 * p.d_bi + (long long)(mt2 * mt_rows + (int)cta_rank * BM + q * 32 + lane) * p.ldd +
+                              nt2 * p.bn, cols * 2);
+          }
+        }
         const bool more = w + w_step < total_work && !tma_out;  // (of interest to the bias hand-over only)
         if (more) fetch_bias(nt2, bnext);
         uint4 x[4];
@@ -551,21 +606,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             else mbar_arrive(smem_u32(&tempty_bar[acc]));
           }
         };
-        auto work = [&](const uint32_t (&a)[32], int i, bool has_next) {
+        auto work = [&](const uint32_t (&a)[32], int i, bool has_next, auto loaded) {
+          // the next chunk of the extra operand: a chunk ahead, or, where the derivative of the GELU leaves
+          // no registers for that, as soon as this chunk's has been used
           uint4 xc[4];
-          if constexpr (kHasXf) {
+          if constexpr (kMode == EPI_RESIDUAL) {
 #pragma unroll
             for (int j = 0; j < 4; j++) xc[j] = x[j];
             if (has_next) prefetch_x(i + 1, x);
           }
+          const uint4(&xu)[4] = kMode == EPI_DGELU ? x : xc;
+          auto x_used = [&]() { if (has_next) prefetch_x(i + 1, x); };
           const int n0 = chunk_n0(i);
           if (tma_out) {
-            // an even chunk opens a 64-column group: the tile store of the previous group must
-            // have read the staging tile; an odd chunk, or the last one, closes it
-            if (!(i & 1)) {
-              if (lane == 0) tma_store_wait_read();
-              __syncwarp();
-            }
+            // an even chunk opens a 64-column group, an odd chunk, or the last one, closes it
             // The staging buffer holds the output tile, so the chunk's bias comes straight from
             // global memory (32 floats that every lane reads alike: one L1 line), or, for a
             // ragged chunk or no bias at all, from 32 floats of scratch.
@@ -576,7 +630,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               __syncwarp();
               bias_c = bias_r;
             }
-            epi_chunk<kMode>(p, a, xc, bias_c, stg, lane, zoff, m_warp, n0, p.direct != 0, stg_tile, i & 1);
+            epi_chunk<kMode>(p, a, xu, bias_c, stg, lane, zoff, m_warp, n0, p.direct != 0, stg_tile, i & 1,
+                             loaded, x_used);
             if ((i & 1) || !has_next) {
               fence_proxy_async_smem();
               __syncwarp();
@@ -586,19 +641,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               }
             }
           } else {
-            epi_chunk<kMode>(p, a, xc, bias_t + i * 32, stg, lane, zoff, m_warp, n0, p.direct && n0 + 32 <= p.N);  // warp-uniform
+            epi_chunk<kMode>(p, a, xu, bias_t + i * 32, stg, lane, zoff, m_warp, n0, p.direct && n0 + 32 <= p.N, 0, 0,
+                             loaded, x_used);  // warp-uniform
           }
         };
-        if (c0ok && kHasXf) {
-          // the flavours with a row-shaped extra operand have no registers to spare for a second
-          // chunk in flight
+        if (c0ok && (kHasXf || kMode == EPI_GELU_AUX)) {
+          // the flavours with a row-shaped extra operand or output have no registers to spare for a second
+          // chunk in flight beside the first: its read starts when the first has left its registers
           uint32_t ra[32];
+          tc_ld32_issue(trow + ccol(0) * 32, ra);
           for (int i = 0;; i++) {
             const bool v1 = chunk_ok(i + 1);
-            tc_ld32_issue(trow + ccol(i) * 32, ra);
             tc_ld32_wait(ra);
             if (!v1) release_acc();
-            work(ra, i, v1);
+            work(ra, i, v1, [&]() { if (v1) tc_ld32_issue(trow + ccol(i + 1) * 32, ra); });
             if (!v1) break;
           }
         } else if (c0ok) {
@@ -608,12 +664,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const bool v1 = chunk_ok(i + 1);
             tc_ld32_wait(ra);
             if (v1) tc_ld32_issue(trow + ccol(i + 1) * 32, rb); else release_acc();
-            work(ra, i, v1);
+            work(ra, i, v1, []() {});
             if (!v1) break;
             const bool v2 = chunk_ok(i + 2);
             tc_ld32_wait(rb);
             if (v2) tc_ld32_issue(trow + ccol(i + 2) * 32, ra); else release_acc();
-            work(rb, i + 1, v2);
+            work(rb, i + 1, v2, []() {});
             if (!v2) break;
           }
         } else {
@@ -756,7 +812,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             // the extra operand of the next chunk travels while this chunk is worked on
             if (has_next) prefetch_x(i + 1, x);
           }
-          epi_chunk<kMode>(p, a, xc, bias_s + i * 32, stg, lane, zoff, m_warp, n0, false);
+          epi_chunk<kMode>(p, a, xc, bias_s + i * 32, stg, lane, zoff, m_warp, n0, false, 0, 0, []() {}, []() {});
           return;
         }
         const long long off = off0 + n0;
@@ -780,16 +836,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         if (p.act == 1) {
           if (p.aux) stage_store_bf16(stg, lane, v, p.aux + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
-#pragma unroll
-          for (int j = 0; j < 16; j++) v[j] = gelu_fast2(v[j]);
+          gelu_row(v);
         } else if (p.act == 2 && row_ok) {
           if (fullv) {
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-              v[4 * j] = __fmul2_rn(v[4 * j], gelu_grad_fast2(bf162_to_f2(x[j].x)));
-              v[4 * j + 1] = __fmul2_rn(v[4 * j + 1], gelu_grad_fast2(bf162_to_f2(x[j].y)));
-              v[4 * j + 2] = __fmul2_rn(v[4 * j + 2], gelu_grad_fast2(bf162_to_f2(x[j].z)));
-              v[4 * j + 3] = __fmul2_rn(v[4 * j + 3], gelu_grad_fast2(bf162_to_f2(x[j].w)));
+              float2 g[4] = {bf162_to_f2(x[j].x), bf162_to_f2(x[j].y), bf162_to_f2(x[j].z), bf162_to_f2(x[j].w)};
+              gelu_grad_fast2(g);
+#pragma unroll
+              for (int e = 0; e < 4; e++) v[4 * j + e] = __fmul2_rn(v[4 * j + e], g[e]);
             }
           } else {
 #pragma unroll
@@ -797,7 +852,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               float2 u = make_float2(0.f, 0.f);
               if (n0 + 2 * j < p.N) u.x = __bfloat162float(p.aux[off + 2 * j]);
               if (n0 + 2 * j + 1 < p.N) u.y = __bfloat162float(p.aux[off + 2 * j + 1]);
-              v[j] = __fmul2_rn(v[j], gelu_grad_fast2(u));
+              float2 g[1] = {u};
+              gelu_grad_fast2(g);
+              v[j] = __fmul2_rn(v[j], g[0]);
             }
           }
         }
@@ -1039,6 +1096,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   // straight-from-register row stores write 32 bytes at a time
   auto al32 = [](const void* q) { return ((uintptr_t)q & 31) == 0; };
   const long long esz = d.d_fp32 ? 4 : 2;
+  p.x32 = al32(d.act == 2 ? d.aux : d.residual) && d.ldd % 16 == 0 && d.d_bo % 16 == 0 && d.d_bi % 16 == 0;
   p.direct = (p.vec_ok && al32(d.D) && (d.ldd * esz) % 32 == 0 && (d.d_bo * esz) % 32 == 0 && (d.d_bi * esz) % 32 == 0 &&
               !(d.d_fp32 && d.accumulate) &&  // vector reductions do better as whole row segments
               (!d.aux || d.act != 1 || (al32(d.aux) && (d.ldd * 2) % 32 == 0 && (d.d_bo * 2) % 32 == 0 && (d.d_bi * 2) % 32 == 0)))

@@ -219,12 +219,13 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         pack(u);
         *reinterpret_cast<uint4*>((bf16*)d.aux + o) = u;
       }
-#pragma unroll
-      for (int e = 0; e < 4; e++) v[e] = gelu_fast2(v[e]);
+      gelu_fast2(v);
     } else if (d.act == 2) {
       const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+      float2 g[4] = {bf162_to_f2(xw[0]), bf162_to_f2(xw[1]), bf162_to_f2(xw[2]), bf162_to_f2(xw[3])};
+      gelu_grad_fast2(g);
 #pragma unroll
-      for (int e = 0; e < 4; e++) v[e] = __fmul2_rn(v[e], gelu_grad_fast2(bf162_to_f2(xw[e])));
+      for (int e = 0; e < 4; e++) v[e] = __fmul2_rn(v[e], g[e]);
     }
     if (d.residual) {
       const uint32_t rw[4] = {res.x, res.y, res.z, res.w};

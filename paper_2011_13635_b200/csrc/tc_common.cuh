@@ -232,43 +232,57 @@ __device__ __forceinline__ float2 bf162_to_f2(uint32_t h) {
 // least-maximum-error fit on |u| <= 4 (gelu is off by less than 3e-5 in fp32 there, far inside bf16
 // resolution).  Outside, u^2 is clamped to 16 and Phi saturates to [0, 1], which gives gelu(u) = u
 // above and 0 below (the exact values differ from those by less than 2e-4).
-__device__ __forceinline__ float2 gelu_fast2(float2 u) {
-  float2 t = __fmul2_rn(u, u);
-  t.x = fminf(t.x, 16.0f);
-  t.y = fminf(t.y, 16.0f);
-  float2 q = splat2(8.093845117e-11f);
-  q = __ffma2_rn(q, t, splat2(-7.032516570e-09f));
-  q = __ffma2_rn(q, t, splat2(2.727248615e-07f));
-  q = __ffma2_rn(q, t, splat2(-6.317188128e-06f));
-  q = __ffma2_rn(q, t, splat2(9.916073864e-05f));
-  q = __ffma2_rn(q, t, splat2(-1.135572678e-03f));
-  q = __ffma2_rn(q, t, splat2(9.883344319e-03f));
-  q = __ffma2_rn(q, t, splat2(-6.642043264e-02f));
-  q = __ffma2_rn(q, t, splat2(3.989280708e-01f));
-  float2 phi;
-  phi.x = __saturatef(fmaf(q.x, u.x, 0.5f));
-  phi.y = __saturatef(fmaf(q.y, u.y, 0.5f));
-  return __fmul2_rn(u, phi);
+// N pairs side by side: one pair's polynomial is a chain of nine dependent instructions, and the two or three
+// warps of a scheduler do not cover it.
+template <int N>
+__device__ __forceinline__ void gelu_fast2(float2 (&u)[N]) {
+  constexpr float kQ[9] = {8.093845117e-11f, -7.032516570e-09f, 2.727248615e-07f, -6.317188128e-06f, 9.916073864e-05f,
+                           -1.135572678e-03f, 9.883344319e-03f, -6.642043264e-02f, 3.989280708e-01f};
+  float2 t[N], q[N];
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    t[i] = __fmul2_rn(u[i], u[i]);
+    t[i].x = fminf(t[i].x, 16.0f);
+    t[i].y = fminf(t[i].y, 16.0f);
+    q[i] = splat2(kQ[0]);
+  }
+#pragma unroll
+  for (int k = 1; k < 9; k++)
+#pragma unroll
+    for (int i = 0; i < N; i++) q[i] = __ffma2_rn(q[i], t[i], splat2(kQ[k]));
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    float2 phi;
+    phi.x = __saturatef(fmaf(q[i].x, u[i].x, 0.5f));
+    phi.y = __saturatef(fmaf(q[i].y, u[i].y, 0.5f));
+    u[i] = __fmul2_rn(u[i], phi);
+  }
 }
 // GELU'(u) = Phi(u) + u phi(u), also on the FMA pipe: 0.5 + u * P(u^2) with a degree-17 odd
 // least-maximum-error fit on |u| <= 4 (absolute error below 1e-4); beyond that the derivative is
 // 0 or 1 to within 5e-4.  The result multiplies a gradient that is then rounded to bf16.
-__device__ __forceinline__ float2 gelu_grad_fast2(float2 u) {
-  const float2 t = __fmul2_rn(u, u);
-  float2 p = splat2(9.837601957e-10f);
-  p = __ffma2_rn(p, t, splat2(-8.257008028e-08f));
-  p = __ffma2_rn(p, t, splat2(3.042579986e-06f));
-  p = __ffma2_rn(p, t, splat2(-6.523749948e-05f));
-  p = __ffma2_rn(p, t, splat2(9.104776309e-04f));
-  p = __ffma2_rn(p, t, splat2(-8.736754371e-03f));
-  p = __ffma2_rn(p, t, splat2(5.852845753e-02f));
-  p = __ffma2_rn(p, t, splat2(-2.649477277e-01f));
-  p = __ffma2_rn(p, t, splat2(7.976755055e-01f));
-  p = __ffma2_rn(p, u, splat2(0.5f));
-  // step(u) without a second comparison: u * 2^100 saturated to [0, 1]
-  p.x = fabsf(u.x) >= 4.0f ? __saturatef(u.x * 1.2676506e30f) : p.x;
-  p.y = fabsf(u.y) >= 4.0f ? __saturatef(u.y * 1.2676506e30f) : p.y;
-  return p;
+template <int N>
+__device__ __forceinline__ void gelu_grad_fast2(float2 (&u)[N]) {
+  constexpr float kP[9] = {9.837601957e-10f, -8.257008028e-08f, 3.042579986e-06f, -6.523749948e-05f, 9.104776309e-04f,
+                           -8.736754371e-03f, 5.852845753e-02f, -2.649477277e-01f, 7.976755055e-01f};
+  float2 t[N], p[N];
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    t[i] = __fmul2_rn(u[i], u[i]);
+    p[i] = splat2(kP[0]);
+  }
+#pragma unroll
+  for (int k = 1; k < 9; k++)
+#pragma unroll
+    for (int i = 0; i < N; i++) p[i] = __ffma2_rn(p[i], t[i], splat2(kP[k]));
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    p[i] = __ffma2_rn(p[i], u[i], splat2(0.5f));
+    // step(u) without a second comparison: u * 2^100 saturated to [0, 1]
+    p[i].x = fabsf(u[i].x) >= 4.0f ? __saturatef(u[i].x * 1.2676506e30f) : p[i].x;
+    p[i].y = fabsf(u[i].y) >= 4.0f ? __saturatef(u[i].y * 1.2676506e30f) : p[i].y;
+    u[i] = p[i];
+  }
 }
 // Staging buffer of one epilogue warp: 32 rows of 64 bytes (2 KB).  Lane r writes its row as four
 // 16-byte pieces; the slot function permutes the pieces so that both this
