@@ -1409,6 +1409,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // runs over query tiles and accumulates dV += P^T dC and dK += dS^T Q.  kQ = true: an item is a tile of
 // 128 queries, the loop runs over key tiles and accumulates dQ += dS K.  The second forms S and dP once
 // more (2 of 7 products) and in return needs no sums across CTAs: same bits on every run.
+// The rows of dS sum to zero, and the key bias' gradient is nothing but such sums: with delta from the
+// context, which was rounded to bf16 (and so were the probabilities it was formed from), it is noise (the first
+// update of a BERT-Large layer's projection bias was off by 0.165 of its mean, 0.15 allowed).  So kQ = true runs
+// first and leaves what each half row of P o (dP - delta) sums to, and kQ = false adds that to delta.
 //   warp 0: TMA producer (the item's two fixed tiles, a ring of three pairs of loop tiles)
 //   warp 1: one thread issues S and dP of a pair, then the accumulating products of the pair before
 //   warps 2-9: two warps per TMEM lane quarter, 64 columns each; a thread owns half a query row.
@@ -1426,7 +1430,7 @@ struct AttnBwdLongParams {
   const int* rows;
   const int* order;
   const float* lse;
-  const float* delta;
+  float* delta;       // [3][heads][ld]: delta, then the two halves' corrections
   long long ld;       // rows of one head in lse and delta
   bf16* dQKV;
   long long g_ld, H;
@@ -1635,13 +1639,15 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const int len = item_len(zo);
       const int n = (len + 127) >> 7;
       const long long row0 = row_base(zo);
+      float2 rest = make_float2(0.f, 0.f);
       for (int t = 0; t < n && ok; t++) {
         const int qrow = (kQ ? tile : t) * 128 + r, key0 = (kQ ? t : tile) * 128 + half * 64;
         // a row beyond the sequence gets probability 2^-inf = 0 everywhere
         float nl = -INFINITY, nd = 0.f;
         if (qrow < len) {
           nl = -p.lse[zi * p.ld + row0 + qrow];
-          nd = -p.delta[zi * p.ld + row0 + qrow];
+          const float* dl = p.delta + zi * p.ld + row0 + qrow;
+          nd = kQ ? -dl[0] : -(dl[0] + (dl[p.heads * p.ld] + dl[2 * p.heads * p.ld]));
         }
         const float2 nl2 = splat2(nl), nd2 = splat2(nd);
         if (!mbar_wait(sfull, sp & 1, abort_flag, p.status)) { ok = false; break; }
@@ -1670,7 +1676,9 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
               if (k0 + 2 * j + 1 >= len) pr.y = 0.f;
             }
             const float2 dp = __fadd2_rn(make_float2(__uint_as_float(d[2 * j]), __uint_as_float(d[2 * j + 1])), nd2);
-            const __nv_bfloat162 ds = __float22bfloat162_rn(__fmul2_rn(__fmul2_rn(dp, sc2), pr));
+            const float2 pd = __fmul2_rn(dp, pr);
+            if (kQ) rest = __fadd2_rn(rest, pd);
+            const __nv_bfloat162 ds = __float22bfloat162_rn(__fmul2_rn(pd, sc2));
             const __nv_bfloat162 pb = __float22bfloat162_rn(pr);
             s[j] = *reinterpret_cast<const uint32_t*>(&pb);
             d[j] = *reinterpret_cast<const uint32_t*>(&ds);
@@ -1696,6 +1704,7 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         if (lane == 0) mbar_arrive(pready);
       }
       if (!ok) break;
+      if (kQ && tile * 128 + r < len) p.delta[(1 + half) * p.heads * p.ld + zi * p.ld + row0 + tile * 128 + r] = rest.x + rest.y;
       // the item's gradients: row r of its tile
       if (!mbar_wait(accfull, ni & 1, abort_flag, p.status)) { ok = false; break; }
       ni++;
@@ -1994,8 +2003,8 @@ int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, con
   const int grid = p.items < adev->num_sms ? p.items : adev->num_sms;
   launch_pdl(attn_delta_kernel, (unsigned)((T * A * 8 + 255) / 256), 256, 0, st, (const bf16*)ctx, (const bf16*)dctx,
              delta, (int)T, A, T, rows);
-  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS, smem_kv, st, mq.map, mk.map, mv.map, mc.map, p);
   launch_pdl(attn_bwd_long_kernel<true>, grid, NUM_THREADS, smem_q, st, mq.map, mk.map, mv.map, mc.map, p);
+  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS, smem_kv, st, mq.map, mk.map, mv.map, mc.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches += 3;

@@ -59,7 +59,7 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
                     float scale, int* status, cudaStream_t st, char* err, const int* seq_lens = nullptr,
                     const int* cu = nullptr, const int* rows = nullptr);
 // The backward for 129 to 512 keys: no stored probabilities, they are formed again from lse.  ctx is the
-// forward's output, delta [A, B*S] scratch (per row and head: sum of dctx o ctx).  Without cu every
+// forward's output, delta [3, A, B*S] scratch (per row and head: sum of dctx o ctx).  Without cu every
 // sequence has S rows.  Three launches.
 int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, const float* lse, float* delta,
                          void* dqkv, int B, int S, int A, float scale, int* status, cudaStream_t st, char* err,
