@@ -87,6 +87,25 @@ __device__ __forceinline__ void zero_tail_rows(bf16* base, long long ld, long lo
     *reinterpret_cast<uint4*>(base + (r0 + i / vecs) * ld + (i % vecs) * 8) = make_uint4(0, 0, 0, 0);
 }
 
+// A 128-row tile that starts inside a sequence shorter than the tile goes on into the next sequence's rows, or into
+// rows that this call has not written.  Their probabilities are zero, but zero times a NaN or an infinity that lies
+// there is NaN, so every such row that is an operand along a contraction is cleared in shared memory first, by warps
+// of their own, so that no other role waits for it on a tile without such rows.  These warps see every round of a
+// ring (the producer waits for their arrival on the slot's empty barrier too); on a tile with rows to clear
+// they also complete the slot's clean barrier, which the thread that issues the products then waits for instead of
+// the full barrier.  (Cleared by the softmax warps: evaluation of 12 x (200..384) keys 2.79 -> 2.83 ms.)
+constexpr int CLEAR_WARPS = 2;  // a thread's registers stay the same: four schedulers, three or five warps each
+// rows from r0 on of a tile (128 bytes each; the swizzle permutes inside a row), shared out over the clearing warps
+__device__ __forceinline__ void clear_tile_rows(uint8_t* tile, int r0, int idx) {
+  for (int v = r0 * 8 + idx; v < 128 * 8; v += 32 * CLEAR_WARPS) reinterpret_cast<uint4*>(tile)[v] = make_uint4(0, 0, 0, 0);
+}
+// Every thread of a clearing warp: the tile's writes are visible to the tensor core once this has returned.
+__device__ __forceinline__ void clear_done(uint32_t clean, int lane) {
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(clean);
+}
+
 // Four 32-column reads of a row in flight together, one wait for all.
 __device__ __forceinline__ void tc_ld128(uint32_t taddr, float2 (&v)[4][16]) {
   uint32_t r0[32], r1[32], r2[32], r3[32];
@@ -114,7 +133,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 template <bool kPacked>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(NUM_THREADS + (kPacked ? 32 * CLEAR_WARPS : 0), 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -127,14 +146,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* sempty_bar = bars + 2 * AT_STAGES + 2; // [2] scores read by every epilogue warp
   uint64_t* pready_bar = bars + 2 * AT_STAGES + 4; // [2] probabilities of a group's item in shared memory
   uint64_t* ofull_bar = bars + 2 * AT_STAGES + 6;  // [2] context of a group's item complete
-  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * AT_STAGES + 8);
+  uint64_t* clean_bar = bars + 2 * AT_STAGES + 8;  // [AT_STAGES] packed: V's rows beyond the sequence are zero
+  uint32_t* tmem_slot = (uint32_t*)(bars + 3 * AT_STAGES + 8);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < AT_STAGES; s++) {
       mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), 1 + (kPacked ? CLEAR_WARPS : 0));
+      mbar_init(smem_u32(&clean_bar[s]), CLEAR_WARPS);
     }
     for (int a = 0; a < 2; a++) {
       mbar_init(smem_u32(&sfull_bar[a]), 1);
@@ -158,6 +179,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
   const int n_my = ((int)blockIdx.x < p.items) ? (p.items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  auto item_len = [&](int i) {  // valid keys of this block's item i
+    return p.seq_lens ? min(max(p.seq_lens[((int)blockIdx.x + i * (int)gridDim.x) / p.heads], 1), p.S) : p.S;
+  };
 
   if (warp == 0 && lane == 0 && !p.starve) {
     // ------------------------------- TMA producer -------------------------------
@@ -200,8 +224,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);           // same for both operand forms
     const uint32_t lbo_mn_lo = (uint32_t)make_smem_desc(0, 64 * BK * 2);   // low word carries the LBO field
-    auto issue_pv = [&](int j) {  // C = P V of item j; P lies over the item's Q and K tiles
+    uint32_t cleaned = 0;  // parity of every stage's clean barrier
+    auto issue_pv = [&](int j) -> bool {  // C = P V of item j; P lies over the item's Q and K tiles
       const uint32_t s = (uint32_t)(j % AT_STAGES), g = (uint32_t)j & 1;
+      if (kPacked && item_len(j) < 128) {
+        if (!mbar_wait(smem_u32(&clean_bar[s]), (cleaned >> s) & 1, abort_flag, p.status)) return false;
+        cleaned ^= 1u << s;
+        tc_fence_after();
+      }
       const uint32_t sq = smem_u32(smem + (size_t)s * AT_STAGE_BYTES);
       const uint32_t p_lo = (uint32_t)make_smem_desc(sq, 16);
       const uint32_t v_lo = lbo_mn_lo | (((sq + 2 * AT_TILE_BYTES) & 0x3FFFFu) >> 4);
@@ -217,6 +247,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
       tc_commit(smem_u32(&ofull_bar[g]));
       tc_commit(smem_u32(&empty_bar[s]));  // the item's tiles are no longer needed
+      return true;
     };
     for (int i = 0; i < n_my && ok; i++) {
       const uint32_t s = (uint32_t)(i % AT_STAGES), round = (uint32_t)(i / AT_STAGES);
@@ -237,14 +268,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const uint32_t g = (uint32_t)(i - 1) & 1, guse = (uint32_t)(i - 1) >> 1;
         if (!mbar_wait(smem_u32(&pready_bar[g]), guse & 1, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
-        issue_pv(i - 1);
+        if (!issue_pv(i - 1)) { ok = false; break; }
       }
     }
     if (ok && n_my > 0) {
       const uint32_t g = (uint32_t)(n_my - 1) & 1, guse = (uint32_t)(n_my - 1) >> 1;
       if (mbar_wait(smem_u32(&pready_bar[g]), guse & 1, abort_flag, p.status)) {
         tc_fence_after();
-        issue_pv(n_my - 1);
+        ok = issue_pv(n_my - 1);
       } else {
         ok = false;
       }
@@ -254,6 +285,18 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_commit(smem_u32(&sfull_bar[0]));
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 2000000ll) {}
+    }
+  } else if (kPacked && warp >= 2 + NUM_EPI_WARPS) {
+    // ------------------------------- clearing of rows beyond the sequence -------------------------------
+    for (int i = 0; i < n_my; i++) {
+      const int len = item_len(i);
+      const uint32_t s = (uint32_t)(i % AT_STAGES);
+      if (!mbar_wait(smem_u32(&full_bar[s]), (i / AT_STAGES) & 1, abort_flag, p.status)) break;
+      if (len < 128) {
+        clear_tile_rows(smem + (size_t)s * AT_STAGE_BYTES + 2 * AT_TILE_BYTES, len, threadIdx.x - NUM_THREADS);
+        clear_done(smem_u32(&clean_bar[s]), lane);
+      }
+      if (lane == 0) mbar_arrive(smem_u32(&empty_bar[s]));
     }
   } else if (warp >= 2) {
     // ------------------------------- softmax groups -------------------------------
@@ -266,8 +309,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const int w = (int)blockIdx.x + i * (int)gridDim.x;
       const int zo = w / p.heads, zi = w - zo * p.heads;
       const uint32_t s = (uint32_t)(i % AT_STAGES), use = (uint32_t)i >> 1;
-      int len = p.seq_lens ? p.seq_lens[zo] : p.S;
-      len = min(max(len, 1), p.S);
+      const int len = item_len(i);
       if (!mbar_wait(smem_u32(&sfull_bar[g]), use & 1, abort_flag, p.status)) { ok = false; break; }
       tc_fence_after();
       float2 v[4][16];  // the row's 128 scores, then its probabilities
@@ -771,13 +813,13 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 //   warp 0: TMA producer (Q tile, ring of K and V tiles: K_0 .. K_{n-1}, V_0 .. V_{n-1})
 //   warp 1: MMA issuer: the next item's scores are issued behind this item's last second product, so they
 //           are ready when the softmax warps have stored the context
+//   warps 2-17: softmax; packed batches: warps 18, 19 clear the last V tile's rows beyond the sequence
 // Bound by the exponential unit (16 a clock: 1024 cycles per block) and the passes around it.
 // 16 sequences x 16 heads x 512 keys: 59.5 us with two groups of warps on items of their own and the scores
 // formed twice; 49.5 us in this form with eight softmax warps (two per scheduler do not cover the
 // tensor-memory reads and the fences); 48.3 us with sixteen.  12 x 16 x 384 keys, uneven lengths: 27.5 us.
 // In steps of BERT-Large at 16 x (256..512) keys, packed tiles dealt out longest first: 56.8 -> 52.1 us a layer.
 constexpr int AR_RING = 8;
-constexpr int AR_BARS = 2 + 2 * AR_RING + 1 + 2 * 2 + 2;
 constexpr int AR_WARPS = 16;  // softmax warps: four per TMEM lane quarter
 constexpr int AR_THREADS = 64 + 32 * AR_WARPS;
 
@@ -824,7 +866,7 @@ __device__ __forceinline__ bool quad_sync(volatile int* flags, int me, int seq, 
 }
 
 template <bool kPacked>
-__global__ void __launch_bounds__(AR_THREADS, 1)
+__global__ void __launch_bounds__(AR_THREADS + (kPacked ? 32 * CLEAR_WARPS : 0), 1)
 attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -839,14 +881,19 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const uint32_t sfull = smem_u32(&bars[2 + 2 * AR_RING]);
   const uint32_t pready0 = smem_u32(&bars[3 + 2 * AR_RING]), pfree0 = smem_u32(&bars[5 + 2 * AR_RING]);  // [2] each
   const uint32_t ofull = smem_u32(&bars[7 + 2 * AR_RING]), oempty = smem_u32(&bars[8 + 2 * AR_RING]);
-  uint32_t* tmem_slot = (uint32_t*)(bars + 9 + 2 * AR_RING);
+  const uint32_t clean0 = smem_u32(&bars[9 + 2 * AR_RING]);  // [AR_RING]
+  uint32_t* tmem_slot = (uint32_t*)(bars + 9 + 3 * AR_RING);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     mbar_init(qfull, 1); mbar_init(qempty, 1); mbar_init(sfull, 1); mbar_init(ofull, 1);
     mbar_init(oempty, AR_WARPS);
-    for (int s = 0; s < AR_RING; s++) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 1); }
+    for (int s = 0; s < AR_RING; s++) {
+      mbar_init(tfull0 + 8 * s, 1);
+      mbar_init(tempty0 + 8 * s, 1 + (kPacked ? CLEAR_WARPS : 0));
+      mbar_init(clean0 + 8 * s, CLEAR_WARPS);
+    }
     for (int b = 0; b < 2; b++) { mbar_init(pready0 + 8 * b, AR_WARPS); mbar_init(pfree0 + 8 * b, 1); }
     for (int i = 0; i < AR_WARPS; i++) xflag[i] = 0;
     *abort_flag = 0;
@@ -926,6 +973,7 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     const uint32_t lbo_mn_lo = (uint32_t)make_smem_desc(0, 64 * BK * 2);
     const uint32_t q_lo = (uint32_t)make_smem_desc(smem_u32(smem), 16);
     uint32_t tt = 0, pv = 0, ig = 0;  // ring tiles, second products, items
+    uint32_t cleaned = 0;             // parity of every slot's clean barrier
     int n_prev = 0;
     for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
       int zo, zi, qt;
@@ -961,8 +1009,11 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       tt += n;
       for (int j = 0; j < n; j++, pv++, tt++) {  // C (+)= P_j V_j
         const uint32_t slot = tt % AR_RING, b = pv & 1;
+        const bool edge = kPacked && (j + 1) * 128 > len;
         if (!mbar_wait(pready0 + 8 * b, (pv >> 1) & 1, abort_flag, p.status) ||
-            !mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status)) { ok = false; break; }
+            !mbar_wait(edge ? clean0 + 8 * slot : tfull0 + 8 * slot, edge ? (cleaned >> slot) & 1 : (tt / AR_RING) & 1, abort_flag,
+                       p.status)) { ok = false; break; }
+        if (edge) cleaned ^= 1u << slot;
         tc_fence_after();
         const uint32_t p_lo = (uint32_t)make_smem_desc(smem_u32(p_smem + b * 2 * AT_TILE_BYTES), 16);
         const uint32_t v_lo = lbo_mn_lo | ((smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES) & 0x3FFFFu) >> 4);
@@ -985,6 +1036,24 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       tc_commit(sfull);
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 2000000ll) {}
+    }
+  } else if (kPacked && warp >= 2 + AR_WARPS) {
+    // ------------------------------- clearing of rows beyond the sequence -------------------------------
+    bool ok = true;
+    uint32_t tt = 0;
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, qt;
+      decode(w, zo, zi, qt);
+      const int len = item_len(zo), n = (len + 127) >> 7;
+      for (int i = 0; i < 2 * n; i++, tt++) {
+        const uint32_t slot = tt % AR_RING;
+        if (!mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status)) { ok = false; break; }
+        if (i == 2 * n - 1 && len < n * 128) {
+          clear_tile_rows(ring_smem + (size_t)slot * AT_TILE_BYTES, len - (n - 1) * 128, threadIdx.x - AR_THREADS);
+          clear_done(clean0 + 8 * slot, lane);
+        }
+        if (lane == 0) mbar_arrive(tempty0 + 8 * slot);
+      }
     }
   } else if (warp >= 2) {
     // ------------------------------- softmax warps -------------------------------
@@ -1137,7 +1206,7 @@ struct AttnBwdParams {
   uint32_t idesc_dv, idesc_dp, idesc_dq, idesc_dk;
 };
 
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(NUM_THREADS + 32 * CLEAR_WARPS, 1)
 attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmC,
                 const __grid_constant__ CUtensorMap tmP, const AttnBwdParams p) {
@@ -1151,18 +1220,20 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* dsready_bar = bars + 6;    // [2] dS in shared memory, dP read by the whole group
   uint64_t* gfull_bar = bars + 8;      // [2] dQ and dK complete
   uint64_t* accfree_bar = bars + 10;   // [2] the group has read dQ, dK, dV of its item
-  uint32_t* tmem_slot = (uint32_t*)(bars + 12);
+  uint64_t* clean_bar = bars + 12;     // [2] packed: the rows of the item's tiles beyond the sequence are zero
+  uint32_t* tmem_slot = (uint32_t*)(bars + 14);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int a = 0; a < 2; a++) {
       mbar_init(smem_u32(&full_bar[a]), 1);
-      mbar_init(smem_u32(&empty_bar[a]), 1);
+      mbar_init(smem_u32(&empty_bar[a]), 1 + (p.cu ? CLEAR_WARPS : 0));
       mbar_init(smem_u32(&dpfull_bar[a]), 1);
       mbar_init(smem_u32(&dsready_bar[a]), AT_GROUP_WARPS);
       mbar_init(smem_u32(&gfull_bar[a]), 1);
       mbar_init(smem_u32(&accfree_bar[a]), AT_GROUP_WARPS);
+      mbar_init(smem_u32(&clean_bar[a]), CLEAR_WARPS);
     }
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
@@ -1180,6 +1251,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
   const int n_my = ((int)blockIdx.x < p.items) ? (p.items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  auto item_len = [&](int i) {  // valid keys of this block's item i
+    return p.seq_lens ? min(max(p.seq_lens[((int)blockIdx.x + i * (int)gridDim.x) / p.heads], 1), p.S) : p.S;
+  };
 
   if (warp == 0 && lane == 0 && !p.starve) {
     // ------------------------------- TMA producer -------------------------------
@@ -1255,9 +1329,15 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_commit(smem_u32(&gfull_bar[g]));
       tc_commit(smem_u32(&empty_bar[g]));
     };
+    uint32_t cleaned = 0;  // parity of every stage's clean barrier
     for (int i = 0; i < n_my && ok; i++) {
       const uint32_t g = (uint32_t)i & 1, use = (uint32_t)i >> 1;
-      if (!mbar_wait(smem_u32(&full_bar[g]), use & 1, abort_flag, p.status)) { ok = false; break; }
+      const bool edge = p.cu && item_len(i) < 128;
+      if (!mbar_wait(smem_u32(edge ? &clean_bar[g] : &full_bar[g]), edge ? (cleaned >> g) & 1 : use & 1, abort_flag, p.status)) {
+        ok = false;
+        break;
+      }
+      if (edge) cleaned ^= 1u << g;
       if (!mbar_wait(smem_u32(&accfree_bar[g]), (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
       tc_fence_after();
       const uint32_t base = smem_u32(smem + (size_t)g * AB_STAGE_BYTES);
@@ -1294,6 +1374,19 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_commit(smem_u32(&dpfull_bar[0]));
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 2000000ll) {}
+    }
+  } else if (warp >= 2 + NUM_EPI_WARPS) {
+    // ------------------------------- clearing of rows beyond the sequence -------------------------------
+    for (int i = 0; i < n_my && p.cu; i++) {
+      const int len = item_len(i);
+      const uint32_t s = (uint32_t)i & 1;
+      if (!mbar_wait(smem_u32(&full_bar[s]), (i >> 1) & 1, abort_flag, p.status)) break;
+      if (len < 128) {
+        for (int t = 0; t < 4; t++)  // Q, K, V, dC
+          clear_tile_rows(smem + (size_t)s * AB_STAGE_BYTES + t * AT_TILE_BYTES, len, threadIdx.x - NUM_THREADS);
+        clear_done(smem_u32(&clean_bar[s]), lane);
+      }
+      if (lane == 0) mbar_arrive(smem_u32(&empty_bar[s]));
     }
   } else if (warp >= 2) {
     // ------------------------------- softmax-backward groups -------------------------------
@@ -1351,7 +1444,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&dsready_bar[g]));
-      const int rlim = p.cu ? min(max(p.seq_lens[zo], 1), p.S) : p.S;  // rows of the item that exist
+      const int rlim = p.cu ? item_len(i) : p.S;  // rows of the item that exist
       bf16* gq = p.dQKV + (p.cu ? p.cu[zo] * p.g_ld : zo * p.g_bo) + zi * 64;
       // dV (complete since dP was): key r, 64 columns
       tc_ld32(trow + 128, v[0]);
@@ -1416,6 +1509,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 //   warp 0: TMA producer (the item's two fixed tiles, a ring of three pairs of loop tiles)
 //   warp 1: one thread issues S and dP of a pair, then the accumulating products of the pair before
 //   warps 2-9: two warps per TMEM lane quarter, 64 columns each; a thread owns half a query row.
+//   warps 10, 11: clear the rows of the tiles that lie beyond the sequence
 // Tensor memory: S 128 columns, dP 128, accumulators 2 x 64.  Bound by the serial chain of a pair
 // (products, tensor-memory reads, exponentials, P and dS to shared memory): the products of the next
 // pair run while this one is worked on.
@@ -1442,7 +1536,7 @@ struct AttnBwdLongParams {
 };
 
 template <bool kQ>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(NUM_THREADS + 32 * CLEAR_WARPS, 1)
 attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmC,
                      const AttnBwdLongParams p) {
@@ -1460,16 +1554,19 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const uint32_t sfull = smem_u32(&misc[2]), sempty = smem_u32(&misc[3]);    // S and dP of a pair
   const uint32_t pready = smem_u32(&misc[4]), pfree = smem_u32(&misc[5]);    // P and dS in shared memory
   const uint32_t accfull = smem_u32(&misc[6]), accempty = smem_u32(&misc[7]);
-  uint32_t* tmem_slot = (uint32_t*)(misc + 8);
+  // the rows of these tiles beyond the sequence are zero: fixed tiles, [BL_RING]
+  const uint32_t fclean = smem_u32(&misc[8]), rclean0 = smem_u32(&misc[9]);
+  uint32_t* tmem_slot = (uint32_t*)(misc + 9 + BL_RING);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < BL_RING; s++) {
       mbar_init(smem_u32(&rfull_bar[s]), 1);
-      mbar_init(smem_u32(&rempty_bar[s]), 1);
+      mbar_init(smem_u32(&rempty_bar[s]), 1 + CLEAR_WARPS);
+      mbar_init(rclean0 + 8 * s, CLEAR_WARPS);
     }
-    mbar_init(ffull, 1); mbar_init(fempty, 1);
+    mbar_init(ffull, 1); mbar_init(fempty, 1 + CLEAR_WARPS); mbar_init(fclean, CLEAR_WARPS);
     mbar_init(sfull, 1); mbar_init(sempty, NUM_EPI_WARPS);
     mbar_init(pready, NUM_EPI_WARPS); mbar_init(pfree, 1);
     mbar_init(accfull, 1); mbar_init(accempty, NUM_EPI_WARPS);
@@ -1574,12 +1671,18 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     };
     const uint32_t f0 = smem_u32(smem), pa = addr16(smem_u32(p_smem)), da = addr16(smem_u32(ds_smem));
     uint32_t rt = 0, np = 0, ni = 0;  // score pairs (= ring tiles), accumulated pairs, items
+    uint32_t cleaned = 0;             // parity of every slot's clean barrier, the fixed tiles' behind them
     for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
       int zo, zi, tile;
       decode(w, zo, zi, tile);
       const int len = item_len(zo);
       const int n = (len + 127) >> 7;
-      if (!mbar_wait(ffull, ni & 1, abort_flag, p.status)) { ok = false; break; }
+      auto landed = [&](uint32_t full, uint32_t parity, uint32_t clean, uint32_t bit, bool edge) -> bool {
+        if (!mbar_wait(edge ? clean : full, edge ? (cleaned >> bit) & 1 : parity, abort_flag, p.status)) return false;
+        if (edge) cleaned ^= 1u << bit;
+        return true;
+      };
+      if (!landed(ffull, ni & 1, fclean, BL_RING, (tile + 1) * 128 > len)) { ok = false; break; }
       auto accumulate = [&](int t) -> bool {  // the accumulating products of pair t of this item
         if (!mbar_wait(pready, np & 1, abort_flag, p.status)) return false;
         if (t == 0 && !mbar_wait(accempty, (ni & 1) ^ 1, abort_flag, p.status)) return false;
@@ -1600,7 +1703,7 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       };
       for (int t = 0; t < n && ok; t++, rt++) {
         const uint32_t slot = rt % BL_RING, round = rt / BL_RING;
-        if (!mbar_wait(smem_u32(&rfull_bar[slot]), round & 1, abort_flag, p.status)) { ok = false; break; }
+        if (!landed(smem_u32(&rfull_bar[slot]), round & 1, rclean0 + 8 * slot, slot, (t + 1) * 128 > len)) { ok = false; break; }
         if (!mbar_wait(sempty, (rt & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t r0 = smem_u32(ring_smem + (size_t)slot * 2 * AT_TILE_BYTES);
@@ -1621,6 +1724,32 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       tc_commit(sfull);
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 2000000ll) {}
+    }
+  } else if (warp >= 2 + NUM_EPI_WARPS) {
+    // ------------------------------- clearing of rows beyond the sequence -------------------------------
+    bool ok = true;
+    uint32_t rt = 0, ni = 0;
+    auto clear = [&](uint32_t full, uint32_t parity, uint32_t clean, uint32_t empty, uint8_t* tiles, int r0) -> bool {
+      if (!mbar_wait(full, parity, abort_flag, p.status)) return false;
+      if (r0 < 128) {
+        for (int t = 0; t < 2; t++) clear_tile_rows(tiles + t * AT_TILE_BYTES, r0, threadIdx.x - NUM_THREADS);
+        clear_done(clean, lane);
+      }
+      if (lane == 0) mbar_arrive(empty);
+      return true;
+    };
+    for (int w = (int)blockIdx.x; w < n_items && ok; w += (int)gridDim.x) {
+      int zo, zi, tile;
+      decode(w, zo, zi, tile);
+      const int len = item_len(zo);
+      const int n = (len + 127) >> 7;
+      ok = clear(ffull, ni & 1, fclean, fempty, smem, len - tile * 128);
+      ni++;
+      for (int t = 0; t < n && ok; t++, rt++) {
+        const uint32_t slot = rt % BL_RING;
+        ok = clear(smem_u32(&rfull_bar[slot]), (rt / BL_RING) & 1, rclean0 + 8 * slot, smem_u32(&rempty_bar[slot]),
+                   ring_smem + (size_t)slot * 2 * AT_TILE_BYTES, len - t * 128);
+      }
     }
   } else if (warp >= 2) {
     // ------------------------------- softmax-backward warps -------------------------------
@@ -1866,7 +1995,7 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
     const auto kernel = cu ? attn_fwd_rows_kernel<true> : attn_fwd_rows_kernel<false>;
     rc = attn_opt_in(kernel, &adev->attr_rows[cu != nullptr], smem_optin, err);
     if (rc) return rc;
-    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, AR_THREADS, smem_rows, st, mq.map, mk.map, mv.map, p);
+    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, AR_THREADS + (cu ? 32 * CLEAR_WARPS : 0), smem_rows, st, mq.map, mk.map, mv.map, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
     g_attn_launches++;
@@ -1891,7 +2020,7 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   rc = attn_opt_in(kernel, &adev->attr_fwd[cu != nullptr], smem_optin, err);
   if (rc) return rc;
   const int grid = p.items < num_sms ? p.items : num_sms;
-  launch_pdl(kernel, grid, NUM_THREADS, smem_bytes, st, mq.map, mk.map, mv.map, p);
+  launch_pdl(kernel, grid, NUM_THREADS + (cu ? 32 * CLEAR_WARPS : 0), smem_bytes, st, mq.map, mk.map, mv.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches++;
@@ -1953,7 +2082,7 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
   rc = attn_opt_in(attn_bwd_kernel, &adev->attr_bwd, smem_optin, err);
   if (rc) return rc;
   const int grid = p.items < num_sms ? p.items : num_sms;
-  launch_pdl(attn_bwd_kernel, grid, NUM_THREADS, smem_bytes, st, mq.map, mk.map, mv.map, mc.map, mp.map, p);
+  launch_pdl(attn_bwd_kernel, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem_bytes, st, mq.map, mk.map, mv.map, mc.map, mp.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches++;
@@ -2003,8 +2132,8 @@ int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, con
   const int grid = p.items < adev->num_sms ? p.items : adev->num_sms;
   launch_pdl(attn_delta_kernel, (unsigned)((T * A * 8 + 255) / 256), 256, 0, st, (const bf16*)ctx, (const bf16*)dctx,
              delta, (int)T, A, T, rows);
-  launch_pdl(attn_bwd_long_kernel<true>, grid, NUM_THREADS, smem_q, st, mq.map, mk.map, mv.map, mc.map, p);
-  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS, smem_kv, st, mq.map, mk.map, mv.map, mc.map, p);
+  launch_pdl(attn_bwd_long_kernel<true>, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem_q, st, mq.map, mk.map, mv.map, mc.map, p);
+  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem_kv, st, mq.map, mk.map, mv.map, mc.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches += 3;

@@ -252,3 +252,65 @@ def test_slots_that_name_a_position_twice(dtype, seq, varlen, pred):
     lab[0, 3] = -1
     PT.compare_step(m, oracle, cfg, (tok, lens, pos, lab), PT.TOL[dtype], [])
     m.close()
+
+
+def _batch_of_lengths(cfg, lens):
+    """tokens, lengths, positions and labels of a batch with the given lengths."""
+    rng = np.random.default_rng(5)
+    tok = rng.integers(1, cfg.vocab, size=(cfg.batch, cfg.seq)).astype(np.int32)
+    pos = np.full((cfg.batch, cfg.pred), -1, dtype=np.int32)
+    lab = np.full((cfg.batch, cfg.pred), -1, dtype=np.int32)
+    for b, n in enumerate(lens):
+        tok[b, n:] = 0
+        k = min(cfg.pred, n)
+        pos[b, :k] = np.sort(rng.choice(n, size=k, replace=False))
+        lab[b, :k] = rng.integers(0, cfg.vocab, size=k)
+    return tok, np.array(lens, dtype=np.int32), pos, lab
+
+
+PACKED_EDGES = [(128, (30, 28, 20, 20, 30)), (256, (130, 20, 70, 6, 30)), (512, (3, 300, 1, 129, 79))]
+
+
+@pytest.mark.parametrize("seq,lens", PACKED_EDGES)
+def test_packed_batch_does_not_see_the_rows_of_an_earlier_call(seq, lens):
+    """A full batch with a NaN weight fills every activation buffer with NaN; the weights are restored
+    and a short packed batch follows whose last sequence ends a tile of 128 rows exactly, so that its
+    own tile reaches into rows that only the first call wrote."""
+    import torch
+    cfg = I.StageConfig("stale", hidden=192, heads=3, ffn=320, vocab=1037, max_pos=512, layers=2, trainable=1,
+                        batch=5, seq=seq, pred=9, dtype="bf16", varlen=(1, seq), seed_index=43)
+    assert sum(lens) % 128 == 0
+    m, oracle = PT.build_pair(cfg, lr=1e-4)
+    weights = {n: m.mslt_get_param(n) for n in oracle.p}
+    bad = weights["emb.word"].copy()
+    bad[:] = np.nan
+    m.mslt_set_param("emb.word", bad)
+    tok, _, pos, lab = _batch_of_lengths(cfg, (seq,) * cfg.batch)
+    assert math.isnan(m.mslt_step(*PT.to_cuda(torch, tok, None, pos, lab)))
+    m.set_params(weights)
+    m.mslt_set_trainable(cfg.trainable)      # moments and step count start again
+    PT.compare_step(m, oracle, cfg, _batch_of_lengths(cfg, lens), PT.TOL["bf16"])
+    m.close()
+
+
+@pytest.mark.parametrize("seq,lens", PACKED_EDGES)
+def test_packed_sequence_does_not_see_its_neighbour(seq, lens):
+    """A token whose word vector is infinite makes its own sequence NaN and no other."""
+    import torch
+    cfg = I.StageConfig("neighbour", hidden=192, heads=3, ffn=320, vocab=1037, max_pos=512, layers=2, trainable=1,
+                        batch=5, seq=seq, pred=9, dtype="bf16", varlen=(1, seq), seed_index=43)
+    m, oracle = PT.build_pair(cfg, lr=1e-4)
+    tok, length, pos, _ = _batch_of_lengths(cfg, lens)
+    tok[tok == 7] = 8
+    h_ref, _ = oracle.forward(tok, length, pos)
+    word = m.mslt_get_param("emb.word")
+    word[7] = np.inf
+    m.mslt_set_param("emb.word", word)
+    tok[1, 0] = tok[3, 0] = 7
+    hidden = m.mslt_forward(*PT.to_cuda(torch, tok, length))[0].float().cpu().numpy()
+    for b, n in enumerate(lens):
+        if b in (1, 3):
+            assert np.isnan(hidden[b, :n]).all()
+        else:
+            assert PT.max_rel(hidden[b, :n], h_ref[b, :n]) < PT.TOL["bf16"]["hidden"]
+    m.close()
