@@ -412,6 +412,17 @@ int mslt_op_attention_bwd(const void* d_qkv, const void* d_probs, const void* d_
                           int32_t S, int32_t heads, float scale, int32_t* d_status, void* cuda_stream,
                           int32_t sync);
 
+/* The pair of calls behind rows of 129..512 keys that run backward: no probabilities are kept.  The forward
+ * writes d_ctx as above and d_lse (device, fp32 [heads, B*S]): per row log2 of its sum of
+ * 2^(log2(e) * scale * q . k).  The backward forms the probabilities again from it; d_ctx is the forward's output,
+ * d_scratch device memory of 12 * heads * B*S bytes (contents on entry do not matter), the other arguments as in
+ * mslt_op_attention_bwd.  All keys are valid.  All buffers 16-byte aligned (d_dqkv 32) and caller-owned. */
+int mslt_op_attention_lse(const void* d_qkv, void* d_ctx, float* d_lse, int32_t B, int32_t S, int32_t heads, float scale,
+                          int32_t* d_status, void* cuda_stream, int32_t sync);
+int mslt_op_attention_lse_bwd(const void* d_qkv, const void* d_ctx, const float* d_lse, const void* d_dctx, void* d_dqkv,
+                              float* d_scratch, int32_t B, int32_t S, int32_t heads, float scale, int32_t* d_status,
+                              void* cuda_stream, int32_t sync);
+
 /*
  * mslt_op_cross_entropy without any device allocation by anybody.  (The paper has no counterpart
  * of this call; it exists for the integration below.)

@@ -58,7 +58,7 @@ EXPORTS = ["mslt_query_bytes", "mslt_create", "mslt_destroy", "mslt_add_layers",
            "mslt_op_gemm", "mslt_op_gemm_enqueue", "mslt_op_cross_entropy",
            "mslt_op_cross_entropy_scratch_bytes", "mslt_op_cross_entropy_noalloc", "mslt_op_layernorm",
            "mslt_op_layernorm_bwd", "mslt_op_softmax", "mslt_op_softmax_bwd", "mslt_op_colsum",
-           "mslt_op_attention", "mslt_op_attention_bwd",
+           "mslt_op_attention", "mslt_op_attention_bwd", "mslt_op_attention_lse", "mslt_op_attention_lse_bwd",
            "mslt_debug_starve_next_gemm", "mslt_debug_starve_next_attention", "mslt_debug_check_guards",
            "mslt_debug_set_gemm_variant"]
 
@@ -125,6 +125,9 @@ lib.mslt_op_softmax.argtypes = [C.c_int32, _P, _P, _P, C.c_int32, C.c_int32, C.c
 lib.mslt_op_softmax_bwd.argtypes = [C.c_int32, _P, _P, C.c_int32, C.c_int32, C.c_float, _P, C.c_int32]
 lib.mslt_op_attention.argtypes = [_P, _P, _P, _P, C.c_int32, C.c_int32, C.c_int32, C.c_float, _P, _P, C.c_int32]
 lib.mslt_op_attention_bwd.argtypes = [_P, _P, _P, _P, C.c_int32, C.c_int32, C.c_int32, C.c_float, _P, _P, C.c_int32]
+lib.mslt_op_attention_lse.argtypes = [_P, _P, _P, C.c_int32, C.c_int32, C.c_int32, C.c_float, _P, _P, C.c_int32]
+lib.mslt_op_attention_lse_bwd.argtypes = [_P, _P, _P, _P, _P, _P, C.c_int32, C.c_int32, C.c_int32, C.c_float, _P, _P,
+                                          C.c_int32]
 lib.mslt_op_colsum.argtypes = [C.c_int32, _P, C.c_int64, C.c_int32, C.c_int32, _P, _P, C.c_int32]
 
 
@@ -214,6 +217,21 @@ def mslt_op_attention_bwd(qkv, probs, dctx, dqkv, B: int, S: int, heads: int, sc
     """qkv, dqkv bf16 [B*S, 3*heads*64]; probs bf16 [B, heads, S, S]; dctx bf16 [B*S, heads*64]."""
     _check(lib.mslt_op_attention_bwd(qkv.data_ptr(), probs.data_ptr(), dctx.data_ptr(), dqkv.data_ptr(), B, S,
                                      heads, scale, status.data_ptr(), C.c_void_p(stream), int(sync)))
+
+
+def mslt_op_attention_lse(qkv, ctx, lse, B: int, S: int, heads: int, scale: float, status, stream: int,
+                          sync: bool = True) -> None:
+    """Rows of 129..512 keys, all valid; lse fp32 [heads, B*S] receives log2 of the rows' sums of exponentials."""
+    _check(lib.mslt_op_attention_lse(qkv.data_ptr(), ctx.data_ptr(), lse.data_ptr(), B, S, heads, scale,
+                                     status.data_ptr(), C.c_void_p(stream), int(sync)))
+
+
+def mslt_op_attention_lse_bwd(qkv, ctx, lse, dctx, dqkv, scratch, B: int, S: int, heads: int, scale: float, status,
+                              stream: int, sync: bool = True) -> None:
+    """scratch fp32 [3, heads, B*S]; the others as in mslt_op_attention_lse and mslt_op_attention_bwd."""
+    _check(lib.mslt_op_attention_lse_bwd(qkv.data_ptr(), ctx.data_ptr(), lse.data_ptr(), dctx.data_ptr(),
+                                         dqkv.data_ptr(), scratch.data_ptr(), B, S, heads, scale, status.data_ptr(),
+                                         C.c_void_p(stream), int(sync)))
 
 
 def mslt_op_softmax_bwd(dp, probs, scale: float, stream: int, sync: bool = True) -> None:

@@ -1502,10 +1502,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // runs over query tiles and accumulates dV += P^T dC and dK += dS^T Q.  kQ = true: an item is a tile of
 // 128 queries, the loop runs over key tiles and accumulates dQ += dS K.  The second forms S and dP once
 // more (2 of 7 products) and in return needs no sums across CTAs: same bits on every run.
-// The rows of dS sum to zero, and the key bias' gradient is nothing but such sums: with delta from the
-// context, which was rounded to bf16 (and so were the probabilities it was formed from), it is noise (the first
-// update of a BERT-Large layer's projection bias was off by 0.165 of its mean, 0.15 allowed).  So kQ = true runs
-// first and leaves what each half row of P o (dP - delta) sums to, and kQ = false adds that to delta.
+// The rows of dS sum to zero: the key bias' gradient is nothing but such sums, and in dQ they multiply the keys'
+// common part.  With delta from the context, which was rounded to bf16 (and so were the probabilities it was formed
+// from), they do not (the first update of a BERT-Large layer's projection bias was off by 0.165 of its mean, 0.15
+// allowed).  So kQ = true runs first, adds up what is left, rest = rowsum(P o (dP - delta)), and beside dS K
+// accumulates P K: dQ = dS K - scale rest P K is the product with the corrected dS.  It leaves rest (by half rows)
+// for kQ = false, which adds it to delta.
 //   warp 0: TMA producer (the item's two fixed tiles, a ring of three pairs of loop tiles)
 //   warp 1: one thread issues S and dP of a pair, then the accumulating products of the pair before
 //   warps 2-9: two warps per TMEM lane quarter, 64 columns each; a thread owns half a query row.
@@ -1544,9 +1546,11 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   // fixed tiles: K, V of the item (kQ: Q, dC); ring stage: Q, dC of a query tile (kQ: K, V of a key tile)
   uint8_t* ring_smem = smem + 2 * AT_TILE_BYTES;
-  uint8_t* p_smem = ring_smem + BL_RING * 2 * AT_TILE_BYTES;   // P, not used by kQ
-  uint8_t* ds_smem = p_smem + (kQ ? 0 : 2 * AT_TILE_BYTES);    // dS
-  uint64_t* bars = (uint64_t*)(ds_smem + 2 * AT_TILE_BYTES);
+  uint8_t* p_smem = ring_smem + BL_RING * 2 * AT_TILE_BYTES;   // P
+  uint8_t* ds_smem = p_smem + 2 * AT_TILE_BYTES;               // dS
+  float* xch = (float*)(ds_smem + 2 * AT_TILE_BYTES);          // kQ: [2][NUM_EPI_WARPS][32] sums of half rows
+  volatile int* xflag = (volatile int*)(xch + 2 * NUM_EPI_WARPS * 32);
+  uint64_t* bars = (uint64_t*)(xflag + NUM_EPI_WARPS);
   uint64_t* rfull_bar = bars;                    // [BL_RING]
   uint64_t* rempty_bar = bars + BL_RING;         // [BL_RING]
   uint64_t* misc = bars + 2 * BL_RING;
@@ -1570,6 +1574,7 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     mbar_init(sfull, 1); mbar_init(sempty, NUM_EPI_WARPS);
     mbar_init(pready, NUM_EPI_WARPS); mbar_init(pfree, 1);
     mbar_init(accfull, 1); mbar_init(accempty, NUM_EPI_WARPS);
+    for (int i = 0; i < NUM_EPI_WARPS; i++) xflag[i] = 0;
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1691,7 +1696,8 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const uint32_t r0 = smem_u32(ring_smem + (size_t)slot * 2 * AT_TILE_BYTES);
         const uint32_t acc = tmem_base + BL_ACC_COL;
         if (kQ) {
-          mma_k128(acc, lbo_k | da, KB_K, KS_K, lbo_mn1 | addr16(r0), p.idesc_q, t == 0);  // dQ += dS K
+          mma_k128(acc, lbo_k | da, KB_K, KS_K, lbo_mn1 | addr16(r0), p.idesc_q, t == 0);       // dQ += dS K
+          mma_k128(acc + 64, lbo_k | pa, KB_K, KS_K, lbo_mn1 | addr16(r0), p.idesc_q, t == 0);  // and P K
         } else {
           mma_k128(acc, lbo_mn2 | pa, KB_MN, KS_MN, lbo_mn1 | addr16(r0 + AT_TILE_BYTES), p.idesc_kv, t == 0);  // dV += P^T dC
           mma_k128(acc + 64, lbo_mn2 | da, KB_MN, KS_MN, lbo_mn1 | addr16(r0), p.idesc_kv, t == 0);             // dK += dS^T Q
@@ -1821,10 +1827,8 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
         for (int c = 0; c < 4; c++) {
           const int u0 = (c ^ (r & 7)) << 4, u1 = ((4 + c) ^ (r & 7)) << 4;
-          if (!kQ) {
-            *reinterpret_cast<uint4*>(prow + u0) = make_uint4(s0[4 * c], s0[4 * c + 1], s0[4 * c + 2], s0[4 * c + 3]);
-            *reinterpret_cast<uint4*>(prow + u1) = make_uint4(s1[4 * c], s1[4 * c + 1], s1[4 * c + 2], s1[4 * c + 3]);
-          }
+          *reinterpret_cast<uint4*>(prow + u0) = make_uint4(s0[4 * c], s0[4 * c + 1], s0[4 * c + 2], s0[4 * c + 3]);
+          *reinterpret_cast<uint4*>(prow + u1) = make_uint4(s1[4 * c], s1[4 * c + 1], s1[4 * c + 2], s1[4 * c + 3]);
           *reinterpret_cast<uint4*>(drow + u0) = make_uint4(d0[4 * c], d0[4 * c + 1], d0[4 * c + 2], d0[4 * c + 3]);
           *reinterpret_cast<uint4*>(drow + u1) = make_uint4(d1[4 * c], d1[4 * c + 1], d1[4 * c + 2], d1[4 * c + 3]);
         }
@@ -1833,7 +1837,14 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         if (lane == 0) mbar_arrive(pready);
       }
       if (!ok) break;
-      if (kQ && tile * 128 + r < len) p.delta[(1 + half) * p.heads * p.ld + zi * p.ld + row0 + tile * 128 + r] = rest.x + rest.y;
+      float total = rest.x + rest.y;
+      if (kQ) {  // the row's other half
+        if (tile * 128 + r < len) p.delta[(1 + half) * p.heads * p.ld + zi * p.ld + row0 + tile * 128 + r] = total;
+        float* x = xch + (ni & 1) * NUM_EPI_WARPS * 32;  // a partner may still read the item before
+        x[(half * 4 + q) * 32 + lane] = total;
+        if (!pair_sync(xflag, half * 4 + q, (half ^ 1) * 4 + q, (int)ni + 1, lane, abort_flag, p.status)) { ok = false; break; }
+        total += x[((half ^ 1) * 4 + q) * 32 + lane];
+      }
       // the item's gradients: row r of its tile
       if (!mbar_wait(accfull, ni & 1, abort_flag, p.status)) { ok = false; break; }
       ni++;
@@ -1841,13 +1852,16 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       float2 v0[16], v1[16];
       const uint32_t acol = BL_ACC_COL + (kQ ? half * 32 : half * 64);
       tc_ld32(trow + acol, v0);
-      if (!kQ) tc_ld32(trow + acol + 32, v1);
+      tc_ld32(trow + acol + (kQ ? 64 : 32), v1);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(accempty);
       if (tile * 128 + r < len) {
         bf16* g = p.dQKV + (row0 + tile * 128 + r) * p.g_ld + zi * 64;
         if (kQ) {
+          const float2 off = splat2(-p.scale * total);
+#pragma unroll
+          for (int j = 0; j < 16; j++) v0[j] = __ffma2_rn(v1[j], off, v0[j]);
           store_row32_bf16(g + half * 32, v0);
         } else {
           g += half ? p.H : 2 * p.H;  // the first accumulator is dV, the second dK
@@ -2123,17 +2137,16 @@ int attn_bwd_long_launch(const void* qkv, const void* ctx, const void* dctx, con
   for (int i = 0; i < 3; i++) {
     p.q_perm[i] = mq.perm[i]; p.k_perm[i] = mk.perm[i]; p.v_perm[i] = mv.perm[i]; p.c_perm[i] = mc.perm[i];
   }
-  const size_t smem_kv = (size_t)(2 + 2 * BL_RING + 4) * AT_TILE_BYTES + 1024 + 256;
-  const size_t smem_q = (size_t)(2 + 2 * BL_RING + 2) * AT_TILE_BYTES + 1024 + 256;
-  if ((int)smem_kv > adev->smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
+  const size_t smem = (size_t)(2 + 2 * BL_RING + 4) * AT_TILE_BYTES + 2 * NUM_EPI_WARPS * 32 * 4 + 1024 + 512;
+  if ((int)smem > adev->smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
   rc = attn_opt_in(attn_bwd_long_kernel<false>, &adev->attr_bwd_kv, adev->smem_optin, err);
   if (!rc) rc = attn_opt_in(attn_bwd_long_kernel<true>, &adev->attr_bwd_q, adev->smem_optin, err);
   if (rc) return rc;
   const int grid = p.items < adev->num_sms ? p.items : adev->num_sms;
   launch_pdl(attn_delta_kernel, (unsigned)((T * A * 8 + 255) / 256), 256, 0, st, (const bf16*)ctx, (const bf16*)dctx,
              delta, (int)T, A, T, rows);
-  launch_pdl(attn_bwd_long_kernel<true>, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem_q, st, mq.map, mk.map, mv.map, mc.map, p);
-  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem_kv, st, mq.map, mk.map, mv.map, mc.map, p);
+  launch_pdl(attn_bwd_long_kernel<true>, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem, st, mq.map, mk.map, mv.map, mc.map, p);
+  launch_pdl(attn_bwd_long_kernel<false>, grid, NUM_THREADS + 32 * CLEAR_WARPS, smem, st, mq.map, mk.map, mv.map, mc.map, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   g_attn_launches += 3;

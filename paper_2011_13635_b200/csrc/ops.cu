@@ -91,6 +91,25 @@ int finish_op(const char* what, cudaStream_t st, int sync) {
   return 0;
 }
 
+int finish_attention(const char* what, const int32_t* d_status, cudaStream_t st, int sync) {
+  int rc = finish_op(what, st, sync);
+  if (rc || !sync) return rc;
+  int h = 0;
+  if (cudaMemcpy(&h, d_status, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+    return op_fail(MSLT_ERR_CUDA, "%s: reading the status word failed", what);
+  if (h & 1) return op_fail(MSLT_ERR_DEVICE, "%s: a bounded wait ran out on the device", what);
+  return 0;
+}
+
+int check_attention_lse(const char* what, uintptr_t aligned16, int B, int S, int heads) {
+  if (aligned16 & 15) return op_fail(MSLT_ERR_ARG, "%s: buffers must be 16-byte aligned", what);
+  if (B < 1 || heads < 1 || S <= 128 || S > 512) return op_fail(MSLT_ERR_ARG, "%s: needs 129 <= S <= 512", what);
+  int ndev = 0;
+  if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1)
+    return op_fail(MSLT_ERR_CUDA, "no CUDA device: this library has no CPU path");
+  return 0;
+}
+
 int check_rows(const char* what, int dtype, int rows, int width, int width_mult, int width_max) {
   if (dtype != 0 && dtype != 1) return op_fail(MSLT_ERR_ARG, "%s: dtype must be 0 or 1", what);
   if (rows < 1) return op_fail(MSLT_ERR_ARG, "%s: rows must be >= 1", what);
@@ -207,16 +226,7 @@ int mslt_op_attention(const void* d_qkv, void* d_probs, void* d_ctx, const int32
   char err[256] = "";
   int rc = attn_fwd_launch(d_qkv, d_probs, d_ctx, d_seq_lens, B, S, heads, 64, scale, d_status, st, err);
   if (rc) return op_fail(rc, "%s", err);
-  if (sync) {
-    rc = finish_op("attention", st, 1);
-    if (rc) return rc;
-    int h = 0;
-    if (cudaMemcpy(&h, d_status, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-      return op_fail(MSLT_ERR_CUDA, "attention: reading the status word failed");
-    if (h & 1) return op_fail(MSLT_ERR_DEVICE, "attention: a bounded wait ran out on the device");
-    return 0;
-  }
-  return finish_op("attention", st, 0);
+  return finish_attention("attention", d_status, st, sync);
 }
 
 int mslt_op_attention_bwd(const void* d_qkv, const void* d_probs, const void* d_dctx, void* d_dqkv, int32_t B,
@@ -233,16 +243,35 @@ int mslt_op_attention_bwd(const void* d_qkv, const void* d_probs, const void* d_
   char err[256] = "";
   int rc = attn_bwd_launch(d_qkv, d_probs, d_dctx, d_dqkv, B, S, heads, 64, scale, d_status, st, err);
   if (rc) return op_fail(rc, "%s", err);
-  if (sync) {
-    rc = finish_op("attention_bwd", st, 1);
-    if (rc) return rc;
-    int h = 0;
-    if (cudaMemcpy(&h, d_status, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-      return op_fail(MSLT_ERR_CUDA, "attention_bwd: reading the status word failed");
-    if (h & 1) return op_fail(MSLT_ERR_DEVICE, "attention_bwd: a bounded wait ran out on the device");
-    return 0;
-  }
-  return finish_op("attention_bwd", st, 0);
+  return finish_attention("attention_bwd", d_status, st, sync);
+}
+
+int mslt_op_attention_lse(const void* d_qkv, void* d_ctx, float* d_lse, int32_t B, int32_t S, int32_t heads, float scale,
+                          int32_t* d_status, void* cuda_stream, int32_t sync) {
+  if (!d_qkv || !d_ctx || !d_lse || !d_status) return op_fail(MSLT_ERR_ARG, "attention_lse: null pointer");
+  int rc = check_attention_lse("attention_lse", (uintptr_t)d_qkv | (uintptr_t)d_ctx | (uintptr_t)d_lse, B, S, heads);
+  if (rc) return rc;
+  char err[256] = "";
+  rc = attn_fwd_launch(d_qkv, nullptr, d_ctx, nullptr, B, S, heads, 64, scale, d_status, (cudaStream_t)cuda_stream, err, nullptr,
+                       nullptr, d_lse);
+  if (rc) return op_fail(rc, "%s", err);
+  return finish_attention("attention_lse", d_status, (cudaStream_t)cuda_stream, sync);
+}
+
+int mslt_op_attention_lse_bwd(const void* d_qkv, const void* d_ctx, const float* d_lse, const void* d_dctx, void* d_dqkv,
+                              float* d_scratch, int32_t B, int32_t S, int32_t heads, float scale, int32_t* d_status,
+                              void* cuda_stream, int32_t sync) {
+  if (!d_qkv || !d_ctx || !d_lse || !d_dctx || !d_dqkv || !d_scratch || !d_status)
+    return op_fail(MSLT_ERR_ARG, "attention_lse_bwd: null pointer");
+  if ((uintptr_t)d_dqkv & 31) return op_fail(MSLT_ERR_ARG, "attention_lse_bwd: d_dqkv must be 32-byte aligned");
+  int rc = check_attention_lse("attention_lse_bwd", (uintptr_t)d_qkv | (uintptr_t)d_ctx | (uintptr_t)d_lse | (uintptr_t)d_dctx |
+                               (uintptr_t)d_scratch, B, S, heads);
+  if (rc) return rc;
+  char err[256] = "";
+  rc = attn_bwd_long_launch(d_qkv, d_ctx, d_dctx, d_lse, d_scratch, d_dqkv, B, S, heads, scale, d_status, (cudaStream_t)cuda_stream,
+                            err, nullptr, nullptr, nullptr, nullptr);
+  if (rc) return op_fail(rc, "%s", err);
+  return finish_attention("attention_lse_bwd", d_status, (cudaStream_t)cuda_stream, sync);
 }
 
 int mslt_op_softmax(int32_t dtype, const void* d_scores, void* d_probs, const int32_t* d_seq_lens,

@@ -255,6 +255,67 @@ def test_fused_attention_backward_matches_oracle(B, S, A, masked):
         assert err < 1.5e-2, (name, err)
 
 
+@pytest.mark.parametrize("k_mean,v_mean", [(0.0, 0.0), (4.0, 16.0)])
+@pytest.mark.parametrize("B,S,A", [(2, 136, 2), (1, 200, 3), (2, 256, 2), (3, 384, 1), (2, 512, 2), (13, 264, 12)])
+def test_long_row_attention_backward_matches_oracle(B, S, A, k_mean, v_mean):
+    """Rows of more than 128 keys, whose probabilities are formed again in the backward, at the tolerance of
+    the shorter rows.  With a common part in the keys and values, whatever the rows of dS lack to a sum of
+    zero shows in dQ (times the keys' part) and dK: with the row term from the bf16 context alone dQ is off by
+    0.10 to 0.23 of its range here (formed in float64 with the same roundings), corrected by 0.004 to 0.006."""
+    import math
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    d, H = 64, A * 64
+    rng = np.random.default_rng(B * 977 + S + A)
+    bf = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda().bfloat16()
+    x = rng.standard_normal((B, S, 3, A, d)) * 1.5
+    x[:, :, 1] += k_mean * rng.standard_normal((1, 1, A, d))
+    x[:, :, 2] += v_mean * rng.standard_normal((1, 1, A, d))
+    qkv = bf(x.reshape(B * S, 3 * H))
+    dctx = bf(rng.standard_normal((B * S, H)))
+    scale = 1.0 / math.sqrt(d)
+    x = qkv.float().cpu().numpy().astype(np.float64).reshape(B, S, 3, A, d)
+    q, k, v = (x[:, :, i].transpose(0, 2, 1, 3) for i in range(3))            # [B, A, S, d]
+    s = np.einsum("bhid,bhjd->bhij", q, k) * scale
+    p = O.masked_softmax(s, np.full(B, S))
+    dc = dctx.float().cpu().numpy().astype(np.float64).reshape(B, S, A, d).transpose(0, 2, 1, 3)
+    ds = O.softmax_backward(np.einsum("bhid,bhjd->bhij", dc, v), p) * scale
+    want = [np.einsum("bhij,bhjd->bhid", ds, k), np.einsum("bhij,bhid->bhjd", ds, q), np.einsum("bhij,bhid->bhjd", p, dc)]
+    ctx = torch.full((B * S, H), 7.0, device="cuda", dtype=torch.bfloat16)
+    lse = torch.full((A, B * S), 7.0, device="cuda")
+    scratch = torch.full((3, A, B * S), float("nan"), device="cuda")
+    dqkv = torch.full((B * S, 3 * H), 7.0, device="cuda", dtype=torch.bfloat16)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        Bd.mslt_op_attention_lse(qkv, ctx, lse, B, S, A, scale, status, _stream())
+        Bd.mslt_op_attention_lse_bwd(qkv, ctx, lse, dctx, dqkv, scratch, B, S, A, scale, status, _stream())
+    assert int(status.item()) == 0
+    lse_ref = np.log2(np.exp(s - s.max(-1, keepdims=True)).sum(-1)) + s.max(-1) * math.log2(math.e)
+    got = lse.cpu().numpy().reshape(A, B, S).transpose(1, 0, 2)
+    # a score is four steps of 16 products, each truncated by less than 2^-22 of the sum of magnitudes; the
+    # exponentials (2^-22 each) and the logarithm of their sum add less than 2^-19
+    size = np.einsum("bhid,bhjd->bhij", np.abs(q), np.abs(k)).max() * scale * math.log2(math.e)
+    assert np.abs(got - lse_ref).max() < 2.0 ** -20 * size + 2.0 ** -19
+    got = dqkv.float().cpu().numpy().reshape(B, S, 3, A, d)
+    for which, name in enumerate(("dq", "dk", "dv")):
+        ref = want[which].transpose(0, 2, 1, 3)
+        err = np.abs(got[:, :, which] - ref).max() / np.abs(ref).max()
+        assert err < 1.5e-2, (name, err)
+
+
+@pytest.mark.parametrize("B,S,A", [(1, 128, 2), (1, 520, 1), (0, 256, 1)])
+def test_long_row_attention_backward_rejects_other_shapes(B, S, A):
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    x = torch.zeros((520, 3 * 128), device="cuda", dtype=torch.bfloat16)
+    f = torch.zeros((3, 2, 520), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    with pytest.raises(Bd.MsltError):
+        Bd.mslt_op_attention_lse(x, x, f, B, S, A, 0.125, status, _stream())
+    with pytest.raises(Bd.MsltError):
+        Bd.mslt_op_attention_lse_bwd(x, x, f, x, x, f, B, S, A, 0.125, status, _stream())
+
+
 @pytest.mark.parametrize("which", ["forward", "forward_long_rows", "backward"])
 def test_attention_wait_that_runs_out_is_reported_and_leaves_the_device_usable(which):
     """Every wait in the attention kernels is bounded.  With the test hook armed the next launch has
