@@ -438,6 +438,7 @@ int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const voi
 // fp32 products that are large enough run on the tensor cores (gemm_f32x3.cu) on operands split into bf16
 // planes.  reuse_a: A is, unchanged, the left operand of the product before this one, so its planes may
 // still be there.  b_is_emb: B is the word table, whose planes are kept for the rest of the call.
+// The plane buffers are sized for the operands of the linear layers and the head, each a buffer of its own.
 int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_emb, bool* done) {
   *done = false;
   const bool a_ready = reuse_a && c->a_split == d.A, b_ready = b_is_emb && c->emb_split;
@@ -460,7 +461,7 @@ int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_em
 }
 
 int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, int rows_are_k = 0, bool reuse_a = false,
-             bool b_is_emb = false, bool b_static = false) {
+             bool b_is_emb = false, bool b_static = false, bool views = false) {
   if (d.M <= 0 || d.N <= 0 || d.K <= 0 || d.batch <= 0) return 0;
   char err[256] = "";
   const int64_t before = gemm_launches();
@@ -468,7 +469,7 @@ int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, in
   if (prof) cudaEventRecord(c->pev[2 * c->prec.size()], c->st);
   int rc = 0;
   bool done = false;
-  if (!c->bf) rc = run_gemm_x3(c, d, reuse_a, b_is_emb, &done);
+  if (!c->bf && !views) rc = run_gemm_x3(c, d, reuse_a, b_is_emb, &done);
   if (rc) return rc;
   if (!done) rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k, b_static);
   if (prof) {
@@ -479,6 +480,10 @@ int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, in
   if (rc) return fail(rc, "%s", err);
   return 0;
 }
+
+// A product of the attention: its operands are views into wider buffers (a third of the fused projection, rows
+// 3H apart), also where one head of one sequence leaves no batch.
+int run_attention_gemm(mslt_ctx* c, const mslt_gemm_desc& d) { return run_gemm(c, d, nullptr, 0, false, false, false, true); }
 
 // Y[T,N] = X[T,K] * W[N,K]^T (+ bias) with optional GELU / residual
 int linear_fwd(mslt_ctx* c, const void* x, int T, int K, int64_t w_off, int64_t b_off, int N,
@@ -570,7 +575,7 @@ int layer_forward(mslt_ctx* c, int l, const void* x, LayerBuf& b, void* out, boo
       // in its epilogue and writes probabilities straight away
       const bool fused = c->bf && S <= 128 && !getenv_cuda_cores();
       if (fused) { g.d.act = 3; g.d.seq_lens = seq_lens; }
-      TRY(run_gemm(c, g.d));
+      TRY(run_attention_gemm(c, g.d));
       if (!fused)
         KL(PC_SOFTMAX_FWD, 2.0 * B * A * S * S * c->esz,
            launch_softmax_fwd(c->bf, b.p, b.p, seq_lens, B * A * S, S, A * S, 1.0f, c->st));
@@ -581,7 +586,7 @@ int layer_forward(mslt_ctx* c, int l, const void* x, LayerBuf& b, void* out, boo
       g.d.A = b.p; g.d.a_rs = S; g.d.a_ks = 1; g.d.a_bo = (int64_t)A * S * S; g.d.a_bi = (int64_t)S * S;
       g.d.B = b.qkv + (int64_t)2 * H * E; g.d.b_rs = 1; g.d.b_ks = 3 * H; g.d.b_bo = (int64_t)S * 3 * H; g.d.b_bi = d;
       g.d.D = b.c; g.d.ldd = H; g.d.d_bo = (int64_t)S * H; g.d.d_bi = d;
-      TRY(run_gemm(c, g.d));
+      TRY(run_attention_gemm(c, g.d));
     }
   }
   TRY(linear_fwd(c, b.c, T, H, toff(c, l, "out.weight"), toff(c, l, "out.bias"), H, b.z1, 0, nullptr, x, false, 0, c->rows));
@@ -625,7 +630,7 @@ int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void
       g.d.A = b.p; g.d.a_rs = 1; g.d.a_ks = S; g.d.a_bo = ps; g.d.a_bi = (int64_t)S * S;
       g.d.B = w.dc; g.d.b_rs = 1; g.d.b_ks = H; g.d.b_bo = cs; g.d.b_bi = d;
       g.d.D = w.dqkv + (int64_t)2 * H * E; g.d.ldd = 3 * H; g.d.d_bo = qs; g.d.d_bi = d;
-      TRY(run_gemm(c, g.d));
+      TRY(run_attention_gemm(c, g.d));
     }
     {  // dP[i,j] = dC[i,:] . v_j
       Lin g(c, S, S, d);
@@ -633,7 +638,7 @@ int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void
       g.d.A = w.dc; g.d.a_rs = H; g.d.a_ks = 1; g.d.a_bo = cs; g.d.a_bi = d;
       g.d.B = b.qkv + (int64_t)2 * H * E; g.d.b_rs = 3 * H; g.d.b_ks = 1; g.d.b_bo = qs; g.d.b_bi = d;
       g.d.D = w.dp; g.d.ldd = S; g.d.d_bo = ps; g.d.d_bi = (int64_t)S * S;
-      TRY(run_gemm(c, g.d));
+      TRY(run_attention_gemm(c, g.d));
     }
     KL(PC_SOFTMAX_BWD, 3.0 * B * A * S * S * c->esz, launch_softmax_bwd(c->bf, w.dp, b.p, B * A * S, S, scale, c->st));
     {  // dQ[i,:] = sum_j dS[i,j] k_j
@@ -642,7 +647,7 @@ int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void
       g.d.A = w.dp; g.d.a_rs = S; g.d.a_ks = 1; g.d.a_bo = ps; g.d.a_bi = (int64_t)S * S;
       g.d.B = b.qkv + (int64_t)H * E; g.d.b_rs = 1; g.d.b_ks = 3 * H; g.d.b_bo = qs; g.d.b_bi = d;
       g.d.D = w.dqkv; g.d.ldd = 3 * H; g.d.d_bo = qs; g.d.d_bi = d;
-      TRY(run_gemm(c, g.d));
+      TRY(run_attention_gemm(c, g.d));
     }
     {  // dK[j,:] = sum_i dS[i,j] q_i
       Lin g(c, S, d, S);
@@ -650,7 +655,7 @@ int layer_backward(mslt_ctx* c, int l, const void* x_in, LayerBuf& b, const void
       g.d.A = w.dp; g.d.a_rs = 1; g.d.a_ks = S; g.d.a_bo = ps; g.d.a_bi = (int64_t)S * S;
       g.d.B = b.qkv; g.d.b_rs = 1; g.d.b_ks = 3 * H; g.d.b_bo = qs; g.d.b_bi = d;
       g.d.D = w.dqkv + (int64_t)H * E; g.d.ldd = 3 * H; g.d.d_bo = qs; g.d.d_bi = d;
-      TRY(run_gemm(c, g.d));
+      TRY(run_attention_gemm(c, g.d));
     }
   }
   TRY(linear_wgrad(c, w.dqkv, T, 3 * H, 3 * H, x_in, H, toff(c, l, "qkv.weight"), c->rows));

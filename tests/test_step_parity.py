@@ -314,3 +314,12 @@ def test_packed_sequence_does_not_see_its_neighbour(seq, lens):
         else:
             assert PT.max_rel(hidden[b, :n], h_ref[b, :n]) < PT.TOL["bf16"]["hidden"]
     m.close()
+
+
+@pytest.mark.parametrize("hidden,ffn", [(384, 1088), (448, 1280)])
+def test_fp32_one_head_of_one_sequence(hidden, ffn):
+    """The attention products of a single (sequence, head) have no batch and are as large as the linear ones,
+    but read views of the fused projection; compare_step checks that no kernel wrote outside its buffer."""
+    cfg = I.StageConfig("onehead", hidden=hidden, heads=1, ffn=ffn, vocab=131, max_pos=512, layers=1, trainable=1, batch=1,
+                        seq=512, pred=5, dtype="fp32", varlen=None, seed_index=47)
+    _run(cfg, steps=2, lr=1e-3)
