@@ -1021,6 +1021,16 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   }
   const int num_sms = di.num_sms, smem_optin = di.smem_optin;
   if (!status) { snprintf(err, 256, "gemm: the tensor-core kernel needs a device status word"); return MSLT_ERR_ARG; }
+  // every argument check comes before a form is chosen: there is none for an epilogue that does not exist
+  if (d.split_k > 1 && !(d.d_fp32 && d.accumulate)) {
+    snprintf(err, 256, "gemm: split_k needs an fp32 accumulating output");
+    return MSLT_ERR_ARG;
+  }
+  if (d.act == 3 && (d.N > 128 || d.d_fp32)) {
+    snprintf(err, 256, "gemm: the softmax epilogue needs bf16 output rows of at most 128 columns");
+    return MSLT_ERR_ARG;
+  }
+  if (d.batch % d.hdiv) { snprintf(err, 256, "gemm: batch must be a multiple of hdiv"); return MSLT_ERR_ARG; }
   TcParams p;
   memset(&p, 0, sizeof(p));
   p.M = d.M; p.N = d.N; p.K = d.K; p.batch = d.batch; p.hdiv = d.hdiv;
@@ -1041,10 +1051,6 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.kb_total = (d.K + round_k - 1) / round_k;
   const long long tiles = (long long)p.m_tiles * p.n_tiles * d.batch;
   const int units = pair ? num_sms / 2 : num_sms;  // CTAs or CTA pairs that run concurrently
-  if (splits > 1 && !(d.d_fp32 && d.accumulate)) {
-    snprintf(err, 256, "gemm: split_k needs an fp32 accumulating output");
-    return MSLT_ERR_ARG;
-  }
   if (splits > p.kb_total) splits = p.kb_total;
   // a split is a whole number of 128-deep slices in every form, so that the partial sums of a given
   // split count do not depend on the tile form
@@ -1053,10 +1059,6 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const long long total = tiles * p.splits;
   if (total > 0x7fffffffll) { snprintf(err, 256, "gemm: too many tiles"); return MSLT_ERR_SIZE; }
   p.total_work = (int)total;
-  if (d.act == 3 && (d.N > 128 || d.d_fp32 || splits != 1)) {
-    snprintf(err, 256, "gemm: the softmax epilogue needs bf16 output rows of at most 128 columns");
-    return MSLT_ERR_ARG;
-  }
   const int stage_bytes = ksub * (A_STAGE_BYTES + (pair ? p.bn / 2 : p.bn) * BK * 2);  // per CTA
   // barriers, then the softmax epilogue's exchange area or the 32 floats per epilogue warp that
   // hold the bias of a ragged chunk when the staging buffers carry output tiles
@@ -1070,7 +1072,6 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
 
   MapVal ma, mb;
   const int nb = d.batch / d.hdiv;
-  if (d.batch % d.hdiv) { snprintf(err, 256, "gemm: batch must be a multiple of hdiv"); return MSLT_ERR_ARG; }
   int rc = get_map(d.A, d.M, d.K, d.a_rs, d.a_ks, d.a_bo, d.a_bi, d.hdiv, nb, BM, &ma, err);
   if (rc) return rc;
   rc = get_map(d.B, d.N, d.K, d.b_rs, d.b_ks, d.b_bo, d.b_bi, d.hdiv, nb, pair ? p.bn / 2 : p.bn, &mb, err);

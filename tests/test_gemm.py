@@ -294,3 +294,27 @@ def test_bf16_tile_forms_the_estimate_picks(shape, majors, kw):
 def test_bf16_few_tile_kernel(shape, majors, kw):
     """Outputs of few tiles: partial sums added inside a cluster, every epilogue."""
     _run(1, *shape, *majors, **kw)
+
+
+@pytest.mark.parametrize("N,kw", [(129, dict(act=3)), (200, dict(act=3)), (64, dict(act=3, d_fp32=1)), (64, dict(split_k=2)),
+                                  (64, dict(split_k=2, d_fp32=1)), (64, dict(hdiv=2))])
+def test_bf16_descriptors_without_a_kernel_are_refused(N, kw):
+    """A softmax over rows that no tile holds, a k split without an output to add into, a batch that its inner
+    index does not divide: refused before a tile form is looked for."""
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    A = torch.zeros((64, 256), device="cuda", dtype=torch.bfloat16)
+    B = torch.zeros((N, 256), device="cuda", dtype=torch.bfloat16)
+    D = torch.zeros((64, 256), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    d = Bd.GemmDesc()
+    d.dtype, d.M, d.N, d.K, d.batch, d.hdiv, d.alpha = 1, 64, N, 256, 1, 1, 1.0
+    d.A, d.a_rs, d.a_ks = A.data_ptr(), 256, 1
+    d.B, d.b_rs, d.b_ks = B.data_ptr(), 256, 1
+    d.D, d.ldd = D.data_ptr(), 256
+    for k, v in kw.items():
+        setattr(d, k, v)
+    for call in (Bd.mslt_op_gemm, Bd.mslt_op_gemm_enqueue):
+        with pytest.raises(Bd.MsltError) as ei:
+            call(d, torch.cuda.current_stream().cuda_stream, status)
+        assert ei.value.code == -1
