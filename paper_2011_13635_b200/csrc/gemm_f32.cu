@@ -255,7 +255,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   // for 64 x 64 (row-contiguous B only: 45 % otherwise); 32 x 32 is bound by its chain of slices.
   const bool amn = d.a_rs == 1 && d.a_ks != 1, bmn = d.b_rs == 1 && d.b_ks != 1;
   const int kb_total = (d.K + FK - 1) / FK;
-  int t = 2, s = 1;
+  int t = 0, s = 1;
   double best = 1e30;
   for (int ti = 0; ti < 4; ti++) {
     const long long tiles = (long long)((d.M + kTile[ti] - 1) / kTile[ti]) * ((d.N + kTile[ti] - 1) / kTile[ti]) * d.batch;
@@ -263,6 +263,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
     // products with a batch read short rows of wide matrices: 64 x 64 took 22.8 us on 96 x (128 x 128 x 64)
     // inside a step, 32 x 32 without shared k 11.2
     if (ti == 1 && d.batch > 1) continue;
+    if (ti != 0 && (d.M + kTile[ti] - 1) / kTile[ti] > 65535) continue;  // row tiles are the grid's second index
     const double alone = ti == 0 ? share : ti == 1 ? 130. : ti == 2 ? 23. : 34.;
     const double per_block = ti == 0 ? 3000. : ti == 1 ? 600. : ti == 2 ? 700. : 150.;
     for (int si = 1; si <= 8 && (si == 1 || kb_total >= si); si *= 2) {

@@ -318,3 +318,8 @@ def test_bf16_descriptors_without_a_kernel_are_refused(N, kw):
         with pytest.raises(Bd.MsltError) as ei:
             call(d, torch.cuda.current_stream().cuda_stream, status)
         assert ei.value.code == -1
+
+
+def test_fp32_more_rows_than_narrow_tiles_can_index():
+    """Over 65535 x 32 rows only the tiles of more rows fit the launch grid."""
+    _run(0, 65535 * 32 + 70, 8, 8, "k", "k", bias=True, d_fp32=True)
