@@ -1190,15 +1190,19 @@ int mslt_forward(mslt_ctx* c, const int32_t* d_tokens, const int32_t* d_seq_lens
   char* cur = w.xa;
   for (int l = 0; l < c->L; l++) {
     char* out = cur == w.xa ? w.xb : w.xa;
-    // the last layer writes its rows where the caller wants them
+    // the last layer writes its rows where the caller wants them, if they can be written 16 bytes at a time
     if (l == c->L - 1 && d_hidden_out && !c->cu && ((uintptr_t)d_hidden_out & 15) == 0) out = (char*)d_hidden_out;
     TRY(layer_forward(c, l, cur, w.scratch, out, false, B, S, d_seq_lens));
     cur = out;
   }
-  if (d_hidden_out && c->cu)
-    KL(PC_OTHER, 2.0 * T * H * c->esz, launch_unpack_rows(c->bf, cur, c->cu, d_hidden_out, B, S, H, c->st));
-  else if (d_hidden_out && cur != d_hidden_out)
-    CUDA_TRY(cudaMemcpyAsync(d_hidden_out, cur, (size_t)T * H * c->esz, cudaMemcpyDeviceToDevice, c->st));
+  const char* rows = cur;  // [B, S, H]
+  if (d_hidden_out && c->cu) {
+    char* out = ((uintptr_t)d_hidden_out & 15) == 0 ? (char*)d_hidden_out : cur == w.xa ? w.xb : w.xa;
+    KL(PC_OTHER, 2.0 * T * H * c->esz, launch_unpack_rows(c->bf, cur, c->cu, out, B, S, H, c->st));
+    rows = out;
+  }
+  if (d_hidden_out && rows != d_hidden_out)
+    CUDA_TRY(cudaMemcpyAsync(d_hidden_out, rows, (size_t)T * H * c->esz, cudaMemcpyDeviceToDevice, c->st));
   if (head) {
     TRY(head_forward(c, cur, B * P, false));
     KL(PC_OTHER, 8.0 * B * P * V, launch_copy_rows(w.logits, c->Vp, d_logits_out, B * P, V, c->st));

@@ -323,3 +323,26 @@ def test_fp32_one_head_of_one_sequence(hidden, ffn):
     cfg = I.StageConfig("onehead", hidden=hidden, heads=1, ffn=ffn, vocab=131, max_pos=512, layers=1, trainable=1, batch=1,
                         seq=512, pred=5, dtype="fp32", varlen=None, seed_index=47)
     _run(cfg, steps=2, lr=1e-3)
+
+
+@pytest.mark.parametrize("varlen", [None, (20, 72)])
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_forward_outputs_need_no_alignment(dtype, varlen):
+    """The hidden states and logits of the C call go to any address of their element type."""
+    import ctypes as C
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    cfg = I.StageConfig("align", hidden=128, heads=2, ffn=128, vocab=130, max_pos=72, layers=2, trainable=1, batch=3, seq=72,
+                        pred=5, dtype=dtype, varlen=varlen, seed_index=51)
+    m, _ = PT.build_pair(cfg, lr=1e-4)
+    tok, lens, pos, _ = I.make_batch(cfg)
+    d_tok, d_lens, d_pos = PT.to_cuda(torch, tok, lens if varlen else None, pos)
+    h_ref, l_ref = m.mslt_forward(d_tok, d_lens, d_pos)
+    buf = torch.zeros(h_ref.numel() + 2, dtype=h_ref.dtype, device="cuda")
+    lbuf = torch.zeros(l_ref.numel() + 2, device="cuda")
+    Bd._check(Bd.lib.mslt_forward(m.h, d_tok.data_ptr(), Bd._ptr(d_lens), cfg.batch, cfg.seq,
+                                  C.c_void_p(buf[1:].data_ptr()), d_pos.data_ptr(), cfg.pred,
+                                  C.c_void_p(lbuf[1:].data_ptr())))
+    assert torch.equal(buf[1:-1].view_as(h_ref), h_ref) and torch.equal(lbuf[1:-1].view_as(l_ref), l_ref)
+    assert not buf[0] and not buf[-1] and not lbuf[0] and not lbuf[-1]
+    m.close()
