@@ -307,6 +307,17 @@ int mslt_op_gemm(const mslt_gemm_desc* desc, void* cuda_stream, int32_t* d_statu
 int mslt_op_gemm_enqueue(const mslt_gemm_desc* desc, void* cuda_stream, int32_t* d_status);
 
 /*
+ * The same contraction in fp32 on the tensor cores, the form that the step uses for its larger fp32 products: both
+ * operands split into three bf16 planes each, six plane products, sums of 64 of k added in fp32.  dtype 0, batch 1,
+ * act 0 to 2; pitches (a_rs / a_ks, whichever is not 1) multiples of 8, operands 16-byte aligned, and the storage
+ * behind an operand covers whole rows of its pitch.  d_scratch: device memory of the size that the first call
+ * returns, 256-byte aligned; contents on entry do not matter.  Synchronises like mslt_op_gemm.
+ */
+size_t mslt_op_gemm_f32_split_scratch_bytes(const mslt_gemm_desc* desc);
+int mslt_op_gemm_f32_split(const mslt_gemm_desc* desc, void* d_scratch, size_t scratch_bytes, void* cuda_stream,
+                           int32_t* d_status);
+
+/*
  * Test hook for the failure path.  Every wait inside the tensor-core kernel is bounded; when one
  * runs out the CTA sets bit 0 of the status word, drains, frees its tensor memory and returns, and
  * the host call reports MSLT_ERR_DEVICE.  After mslt_debug_starve_next_gemm(1) the NEXT dtype-1

@@ -55,7 +55,8 @@ EXPORTS = ["mslt_query_bytes", "mslt_create", "mslt_destroy", "mslt_add_layers",
            "mslt_set_param", "mslt_get_param_raw", "mslt_get_grad", "mslt_get_opt_state",
            "mslt_launch_count", "mslt_set_timing", "mslt_get_timings", "mslt_get_kernel_profile",
            "mslt_last_error",
-           "mslt_op_gemm", "mslt_op_gemm_enqueue", "mslt_op_cross_entropy",
+           "mslt_op_gemm", "mslt_op_gemm_enqueue", "mslt_op_gemm_f32_split", "mslt_op_gemm_f32_split_scratch_bytes",
+           "mslt_op_cross_entropy",
            "mslt_op_cross_entropy_scratch_bytes", "mslt_op_cross_entropy_noalloc", "mslt_op_layernorm",
            "mslt_op_layernorm_bwd", "mslt_op_softmax", "mslt_op_softmax_bwd", "mslt_op_colsum",
            "mslt_op_attention", "mslt_op_attention_bwd", "mslt_op_attention_lse", "mslt_op_attention_lse_bwd",
@@ -102,6 +103,9 @@ lib.mslt_get_timings.argtypes = [C.c_void_p, C.c_void_p, C.c_int32]
 lib.mslt_get_kernel_profile.argtypes = [C.c_void_p, C.c_void_p, C.c_int32]
 lib.mslt_op_gemm.argtypes = [C.POINTER(GemmDesc), C.c_void_p, C.c_void_p]
 lib.mslt_op_gemm_enqueue.argtypes = [C.POINTER(GemmDesc), C.c_void_p, C.c_void_p]
+lib.mslt_op_gemm_f32_split_scratch_bytes.restype = C.c_size_t
+lib.mslt_op_gemm_f32_split_scratch_bytes.argtypes = [C.POINTER(GemmDesc)]
+lib.mslt_op_gemm_f32_split.argtypes = [C.POINTER(GemmDesc), C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p]
 
 
 lib.mslt_op_cross_entropy_scratch_bytes.restype = C.c_size_t
@@ -158,6 +162,16 @@ def mslt_op_gemm(desc: GemmDesc, stream: int, status) -> None:
 
 def mslt_op_gemm_enqueue(desc: GemmDesc, stream: int, status) -> None:
     _check(lib.mslt_op_gemm_enqueue(C.byref(desc), C.c_void_p(stream), C.c_void_p(_ptr(status))))
+
+
+def mslt_op_gemm_f32_split_scratch_bytes(desc: GemmDesc) -> int:
+    return lib.mslt_op_gemm_f32_split_scratch_bytes(C.byref(desc))
+
+
+def mslt_op_gemm_f32_split(desc: GemmDesc, scratch, stream: int, status) -> None:
+    """scratch: uint8 CUDA tensor of mslt_op_gemm_f32_split_scratch_bytes(desc) bytes."""
+    _check(lib.mslt_op_gemm_f32_split(C.byref(desc), scratch.data_ptr(), scratch.numel(), C.c_void_p(stream),
+                                      C.c_void_p(_ptr(status))))
 
 
 def mslt_op_cross_entropy(dtype: int, logits, labels, V: int, dlogits, loss, scratch, stream: int) -> None:

@@ -20,11 +20,15 @@ int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err
 int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 // The same on the tensor cores (gemm_f32x3.cu), for products without a batch: each operand has first been
 // split into three bf16 planes (launch_split3; n elements of the operand's storage, 6 n bytes of planes).
-// wins: whether that is estimated to be faster; planes_ready: bit 0 / 1 = the planes of A / B exist already.
-void launch_split3(const float* x, void* planes, long long n, cudaStream_t st);
+// wide: device word, zeroed beforehand, that a split raises for a value the planes cannot stand for; the products
+// that are given it then read the operands themselves.
+// accepts: layouts the kernel takes; wins: whether it is estimated to be faster as well; planes_ready: bit 0 / 1 =
+// the planes of A / B exist already.
+void launch_split3(const float* x, void* planes, long long n, int* wide, cudaStream_t st);
+bool gemm_f32x3_accepts(const mslt_gemm_desc& d);
 bool gemm_f32x3_wins(const mslt_gemm_desc& d, int planes_ready);
-int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void* planes_b, int* status, cudaStream_t st,
-                      char* err);
+int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void* planes_b, const int* wide, int* status,
+                      cudaStream_t st, char* err);
 int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
                    bool b_static);

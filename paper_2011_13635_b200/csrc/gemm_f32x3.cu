@@ -1,7 +1,12 @@
-// fp32 contraction on the tensor cores.  Every fp32 operand value is the exact sum of three bf16 values
-// (8 + 8 + 8 bits of its 24), so a product a * b is a sum of nine bf16 products, each exact in fp32; the
-// three smallest (below 2^-25 of the product) are left out and six remain:
+// fp32 contraction on the tensor cores.  An fp32 operand value is the exact sum of three bf16 values
+// (8 + 8 + 8 bits of its 24; the decomposition of Henry, Tang and Heinecke, "Leveraging the bfloat16 artificial
+// intelligence datatype for higher-precision computations", 2019), so a product a * b is a sum of nine bf16
+// products, each exact in fp32; the three smallest (below 2^-25 of the product) are left out and six remain:
 //   a1 b1 + (a1 b2 + a2 b1) + (a1 b3 + a2 b2 + a3 b1).
+// Range: the sum is exact from 2^-110 up; of a smaller value the parts below the bf16 range (2^-133) are lost, an
+// error of at most 2^-134 per value.  Infinities, and values from 2^62 on, whose plane products could overflow with
+// either sign, have no such sum (inf * 0 and inf - inf are NaN): the split reports them, and tiles are then formed
+// again by ordinary fp32 multiply-adds of the operands themselves.  NaNs pass through the first plane.
 // The tensor core adds with truncation, which would build up over a long k (relative error 3e-6 at k =
 // 3072 and 3.5e-5 at 30528 measured, against 1.5e-7 and 6e-7 for a chain of fp32 multiply-adds).  So a
 // tensor-memory accumulator only ever holds 64 of k, smallest terms first, and is then added to the
@@ -27,6 +32,7 @@ constexpr int X3_STAGES = 2;
 
 struct X3Params {
   F32Params f;
+  const int* wide;  // device: not 0 when an operand split in this call held a value the planes cannot stand for
   int a_mn, b_mn, kb_total;
   int a_perm[2], b_perm[2];  // slots of the strided matrix index and of the plane
   uint32_t idesc;
@@ -34,9 +40,54 @@ struct X3Params {
   int* status;
 };
 
+// The block's partial tile by fp32 multiply-adds over k0 .. k1, 32 of k through shared memory at a time.  Called by
+// all threads; not on the way of ordinary values, so kept out of the kernel's registers.
+template <int BN>
+__device__ __noinline__ void plain_tile(const X3Params& p, float* tile, int m0, int n0, int k0, int k1) {
+  constexpr int KC = 32, CP = KC + 1, RN = BN / 16, PITCH = BN + 4;
+  const mslt_gemm_desc& d = p.f.d;
+  const float *A = (const float*)d.A, *B = (const float*)d.B;
+  float *as = tile, *bs = tile + BM * CP;
+  const int t = (int)threadIdx.x - (X3_THREADS - 256), ty = t >> 4, tx = t & 15;  // 16 x 16 threads of 8 x RN outputs
+  float acc[8][RN];
+#pragma unroll
+  for (int i = 0; i < 8; i++)
+#pragma unroll
+    for (int j = 0; j < RN; j++) acc[i][j] = 0.f;
+  for (int kc = k0; kc < k1; kc += KC) {
+    for (int i = threadIdx.x; i < (BM + BN) * KC; i += X3_THREADS) {
+      const int r = i / KC, k = kc + i % KC;
+      const bool isa = r < BM;
+      const int row = isa ? m0 + r : n0 + r - BM;
+      float v = 0.f;
+      if (k < k1 && row < (isa ? d.M : d.N)) v = isa ? A[row * d.a_rs + k * d.a_ks] : B[row * d.b_rs + k * d.b_ks];
+      as[r * CP + i % KC] = v;  // bs follows as
+    }
+    __syncthreads();
+    if (t >= 0)
+      for (int k = 0; k < KC; k++) {
+        float a[8], b[RN];
+#pragma unroll
+        for (int i = 0; i < 8; i++) a[i] = as[(ty + 16 * i) * CP + k];
+#pragma unroll
+        for (int j = 0; j < RN; j++) b[j] = bs[(tx + 16 * j) * CP + k];
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+#pragma unroll
+          for (int j = 0; j < RN; j++) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      }
+    __syncthreads();
+  }
+  if (t >= 0)
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+#pragma unroll
+      for (int j = 0; j < RN; j++) tile[(ty + 16 * i) * PITCH + tx + 16 * j] = acc[i][j];
+}
+
 template <int BN>
 __global__ void __launch_bounds__(X3_THREADS, 1)
-gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3Params p) {
+gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ X3Params p) {
   constexpr int A_PLANE = BM * BK * 2, B_PLANE = BN * BK * 2;
   constexpr int STAGE = 3 * (A_PLANE + B_PLANE), PITCH = BN + 4;
   static_assert(BM * PITCH * 4 <= X3_STAGES * STAGE, "the finished tile reuses the ring");
@@ -73,6 +124,7 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
+  const int wide = *reinterpret_cast<const volatile int*>(p.wide);  // looked at when the tile is finished
   const int rank = blockIdx.x % p.f.splits, nt = blockIdx.x / p.f.splits;
   const int m0 = blockIdx.y * BM, n0 = nt * BN;
   const int kb0 = min(p.kb_total, rank * p.f.kb_per_split), kb1 = min(p.kb_total, kb0 + p.f.kb_per_split);
@@ -169,12 +221,15 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   tc_fence_before();
   __syncthreads();
   float* tile = reinterpret_cast<float*>(smem);
-  if (warp >= 4) {
+  if (wide) {
+    plain_tile<BN>(p, tile, m0, n0, kb0 * BK, min(p.f.d.K, kb1 * BK));
+  } else if (warp >= 4) {
     const int r = (warp & 3) * 32 + lane, c0 = ((warp - 4) >> 2) * (BN / 2);
 #pragma unroll
     for (int i = 0; i < BN / 2; i += 4)
       *reinterpret_cast<float4*>(tile + r * PITCH + c0 + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
-  } else if (warp == 1) {
+  }
+  if (warp == 1) {
     __syncwarp();
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * BN) : "memory");
@@ -182,11 +237,12 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   cluster_add_and_finish<BM, BN, X3_THREADS, PITCH>(p.f, rank, tile, 0, m0, n0);
 }
 
-// x = p1 + p2 + p3 exactly (bf16 each, rounded to nearest); n a multiple of 8.  Values that round to
-// infinity take the largest bf16 below instead; infinities and NaNs stay in the first plane.
+// x = p1 + p2 + p3 exactly (bf16 each, rounded to nearest); n a multiple of 8.  *wide is raised for values of 2^62
+// and more (see the top of the file).
 __global__ void __launch_bounds__(256)
-split3_kernel(const float* __restrict__ x, bf16* __restrict__ out, long long n) {
+split3_kernel(const float* __restrict__ x, bf16* __restrict__ out, long long n, int* __restrict__ wide) {
   pdl_begin();
+  float most = 0.f;
   for (long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * 8; i < n; i += (long long)gridDim.x * 2048) {
     float v[8];
     *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(x + i);
@@ -194,10 +250,9 @@ split3_kernel(const float* __restrict__ x, bf16* __restrict__ out, long long n) 
     __align__(16) bf16 o[3][8];
 #pragma unroll
     for (int e = 0; e < 8; e++) {
-      bf16 h = __float2bfloat16_rn(v[e]);
-      const bool finite = fabsf(v[e]) <= 3.402823466e38f;
-      if (finite && fabsf(__bfloat162float(h)) > 3.402823466e38f) h = __float2bfloat16_rz(v[e]);
-      const float r1 = finite ? v[e] - __bfloat162float(h) : 0.f;
+      const bf16 h = __float2bfloat16_rn(v[e]);
+      most = fmaxf(most, fabsf(v[e]));  // passes over NaN
+      const float r1 = v[e] - __bfloat162float(h);
       const bf16 m = __float2bfloat16_rn(r1);
       o[0][e] = h;
       o[1][e] = m;
@@ -206,6 +261,7 @@ split3_kernel(const float* __restrict__ x, bf16* __restrict__ out, long long n) 
 #pragma unroll
     for (int pl = 0; pl < 3; pl++) *reinterpret_cast<uint4*>(out + pl * n + i) = *reinterpret_cast<const uint4*>(o[pl]);
   }
+  if (most >= 4.611686018427387904e18f) atomicOr(wide, 1);
 }
 
 constexpr int kMaxDevices = 64;
@@ -216,16 +272,20 @@ size_t x3_smem(int bn) { return (size_t)X3_STAGES * 3 * (BM + bn) * BK * 2 + 102
 
 }  // namespace
 
-void launch_split3(const float* x, void* planes, long long n, cudaStream_t st) {
+void launch_split3(const float* x, void* planes, long long n, int* wide, cudaStream_t st) {
   const long long blocks = (n / 8 + 255) / 256;
-  launch_pdl(split3_kernel, (unsigned)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st, x, (bf16*)planes, n);
+  launch_pdl(split3_kernel, (unsigned)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st, x, (bf16*)planes, n, wide);
+}
+
+bool gemm_f32x3_accepts(const mslt_gemm_desc& d) {
+  if (d.dtype != 0 || d.batch != 1 || d.act == 3 || (d.a_rs != 1 && d.a_ks != 1) || (d.b_rs != 1 && d.b_ks != 1)) return false;
+  const long long a_ld = d.a_ks == 1 ? d.a_rs : d.a_ks, b_ld = d.b_ks == 1 ? d.b_rs : d.b_ks;
+  return a_ld % 8 == 0 && b_ld % 8 == 0 && (((uintptr_t)d.A | (uintptr_t)d.B) & 15) == 0;
 }
 
 bool gemm_f32x3_wins(const mslt_gemm_desc& d, int planes_ready) {
   auto dense = [](long long rows, long long K, long long rs, long long ks) { return ks == 1 ? rows * rs : K * ks; };
-  if (d.dtype != 0 || d.batch != 1 || d.act == 3 || (d.a_rs != 1 && d.a_ks != 1) || (d.b_rs != 1 && d.b_ks != 1)) return false;
-  const long long a_ld = d.a_ks == 1 ? d.a_rs : d.a_ks, b_ld = d.b_ks == 1 ? d.b_rs : d.b_ks;
-  if (a_ld % 8 || b_ld % 8 || ((uintptr_t)d.A & 15) || ((uintptr_t)d.B & 15)) return false;
+  if (!gemm_f32x3_accepts(d)) return false;
   const double flops = 2.0 * d.M * d.N * (double)d.K;
   const double split = 1e-3 * 10. * ((planes_ready & 1 ? 0. : dense(d.M, d.K, d.a_rs, d.a_ks)) + (planes_ready & 2 ? 0. : dense(d.N, d.K, d.b_rs, d.b_ks)));
   // microseconds.  Measured: 28-38 TFLOP/s on the CUDA cores against 90-200 here, splitting at 4.5 TB/s:
@@ -235,7 +295,8 @@ bool gemm_f32x3_wins(const mslt_gemm_desc& d, int planes_ready) {
   return 5. + flops / 28e6 > 5. + flops / 130e6 + split / 4.5e3 + 1.5 * to_split;
 }
 
-int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void* planes_b, int* status, cudaStream_t st, char* err) {
+int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void* planes_b, const int* wide, int* status,
+                      cudaStream_t st, char* err) {
   int dev = 0, sms;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
     snprintf(err, 256, "gemm: no CUDA device");
@@ -254,6 +315,7 @@ int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void*
   X3Params p;
   memset(&p, 0, sizeof(p));
   p.f.d = d;
+  p.wide = wide;
   p.a_mn = d.a_rs == 1 && d.a_ks != 1;
   p.b_mn = d.b_rs == 1 && d.b_ks != 1;
   p.kb_total = (d.K + BK - 1) / BK;

@@ -595,6 +595,7 @@ __global__ void step_prepare_kernel(const ZeroRanges zr, int* __restrict__ scala
   int* n_valid = scalars + 1;
   float* inv_n = (float*)(scalars + 2);
   if (threadIdx.x < 4) scalars[threadIdx.x] = 0;
+  if (threadIdx.x == 8) scalars[8] = 0;  // raised by a split of fp32 operands (gemm_f32x3.cu)
   __syncthreads();
   __shared__ int cnt;
   if (cu != nullptr) {

@@ -49,7 +49,7 @@ struct ZeroRanges {
     vecs[n++] = (bytes + 15) / 16;
   }
 };
-// Opens a call: zeroes the ranges and scalars[0 .. 3] = {status, filled slots, 1 / filled slots, loss}, then
+// Opens a call: zeroes the ranges, scalars[0 .. 3] = {status, filled slots, 1 / filled slots, loss} and scalars[8], then
 // checks the slots and forms rowsrc / rowlabel (positions null: not).  cu, rows, order (outputs, with
 // seq_lens): the packed layout; rows[2] = number of 128-row tiles and order = 8 * sequence + tile of each,
 // longest sequences first (S <= 512).

@@ -435,6 +435,9 @@ int run_attention_bwd(mslt_ctx* c, const void* qkv, const void* probs, const voi
   return 0;
 }
 
+// elements of an operand's storage, whole rows of its pitch
+int64_t operand_elems(int64_t rows, int64_t K, int64_t rs, int64_t ks) { return ks == 1 ? rows * rs : K * ks; }
+
 // fp32 products that are large enough run on the tensor cores (gemm_f32x3.cu) on operands split into bf16
 // planes.  reuse_a: A is, unchanged, the left operand of the product before this one, so its planes may
 // still be there.  b_is_emb: B is the word table, whose planes are kept for the rest of the call.
@@ -446,14 +449,13 @@ int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_em
   if (!gemm_f32x3_wins(d, (a_ready ? 1 : 0) | (b_ready ? 2 : 0))) return 0;
   Workspace& w = c->ws;
   char* pb = b_is_emb ? w.x3e : w.x3b;
-  // the operands' storage, pitch included
-  const int64_t na = d.a_ks == 1 ? d.M * d.a_rs : d.K * d.a_ks, nb = d.b_ks == 1 ? d.N * d.b_rs : d.K * d.b_ks;
-  if (!a_ready) { launch_split3((const float*)d.A, w.x3a, na, c->st); c->launches++; }
-  if (!b_ready) { launch_split3((const float*)d.B, pb, nb, c->st); c->launches++; }
+  const int64_t na = operand_elems(d.M, d.K, d.a_rs, d.a_ks), nb = operand_elems(d.N, d.K, d.b_rs, d.b_ks);
+  if (!a_ready) { launch_split3((const float*)d.A, w.x3a, na, w.scalars + 8, c->st); c->launches++; }
+  if (!b_ready) { launch_split3((const float*)d.B, pb, nb, w.scalars + 8, c->st); c->launches++; }
   c->a_split = d.A;
   if (b_is_emb) c->emb_split = true;
   char err[256] = "";
-  int rc = gemm_f32x3_launch(d, w.x3a, pb, w.scalars, c->st, err);
+  int rc = gemm_f32x3_launch(d, w.x3a, pb, w.scalars + 8, w.scalars, c->st, err);
   if (rc) return fail(rc, "%s", err);
   c->launches++;
   *done = true;
@@ -1386,6 +1388,17 @@ static int check_gemm_desc(const mslt_gemm_desc* d) {
   return 0;
 }
 
+static int read_gemm_status(const int32_t* d_status, cudaStream_t st) {
+  CUDA_TRY(cudaStreamSynchronize(st));
+  if (d_status) {
+    int h = 0;
+    CUDA_TRY(cudaMemcpyAsync(&h, d_status, 4, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    if (h) return fail(MSLT_ERR_DEVICE, "device status 0x%x: a kernel wait ran out", h);
+  }
+  return 0;
+}
+
 int mslt_op_gemm_enqueue(const mslt_gemm_desc* d, void* cuda_stream, int32_t* d_status) {
   TRY(check_gemm_desc(d));
   char err[256] = "";
@@ -1397,15 +1410,34 @@ int mslt_op_gemm_enqueue(const mslt_gemm_desc* d, void* cuda_stream, int32_t* d_
 
 int mslt_op_gemm(const mslt_gemm_desc* d, void* cuda_stream, int32_t* d_status) {
   TRY(mslt_op_gemm_enqueue(d, cuda_stream, d_status));
+  return read_gemm_status(d_status, (cudaStream_t)cuda_stream);
+}
+
+size_t mslt_op_gemm_f32_split_scratch_bytes(const mslt_gemm_desc* d) {
+  if (!d) return 0;
+  return 256 + 6 * (size_t)(pad_to(operand_elems(d->M, d->K, d->a_rs, d->a_ks), 64) + pad_to(operand_elems(d->N, d->K, d->b_rs, d->b_ks), 64));
+}
+
+int mslt_op_gemm_f32_split(const mslt_gemm_desc* d, void* d_scratch, size_t scratch_bytes, void* cuda_stream, int32_t* d_status) {
+  TRY(check_gemm_desc(d));
+  if (!d_status || !gemm_f32x3_accepts(*d))
+    return fail(MSLT_ERR_ARG, "gemm_f32_split: needs fp32 operands without a batch, pitches that are multiples of 8, "
+                "16-byte aligned bases and a status word");
+  if (!d_scratch || ((uintptr_t)d_scratch & 255) || scratch_bytes < mslt_op_gemm_f32_split_scratch_bytes(d))
+    return fail(MSLT_ERR_SIZE, "gemm_f32_split: scratch must be 256-byte aligned and hold %zu bytes",
+                mslt_op_gemm_f32_split_scratch_bytes(d));
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  CUDA_TRY(cudaStreamSynchronize(st));
-  if (d_status) {
-    int h = 0;
-    CUDA_TRY(cudaMemcpyAsync(&h, d_status, 4, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    if (h) return fail(MSLT_ERR_DEVICE, "device status 0x%x: a kernel wait ran out", h);
-  }
-  return 0;
+  const int64_t na = operand_elems(d->M, d->K, d->a_rs, d->a_ks), nb = operand_elems(d->N, d->K, d->b_rs, d->b_ks);
+  int* wide = (int*)d_scratch;
+  char *pa = (char*)d_scratch + 256, *pb = pa + 6 * pad_to(na, 64);
+  CUDA_TRY(cudaMemsetAsync(wide, 0, 4, st));
+  launch_split3((const float*)d->A, pa, na, wide, st);
+  launch_split3((const float*)d->B, pb, nb, wide, st);
+  char err[256] = "";
+  int rc = gemm_f32x3_launch(*d, pa, pb, wide, d_status, st, err);
+  if (rc) return fail(rc, "%s", err);
+  CUDA_TRY(cudaGetLastError());
+  return read_gemm_status(d_status, st);
 }
 
 }  // extern "C"

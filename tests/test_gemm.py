@@ -21,13 +21,16 @@ def _dgelu(u):
 
 
 def _run(dtype, M, N, K, a_major, b_major, *, bias=False, act=0, residual=False, aux_out=False,
-         d_fp32=False, accumulate=False, alpha=1.0, split_k=0, seed=0):
+         d_fp32=False, accumulate=False, alpha=1.0, split_k=0, seed=0, planes=False, spoil=None, tol=None):
+    """planes: the fp32 form on split operands; spoil(A, B) changes the operands before they are stored."""
     import torch
     from paper_2011_13635_b200 import binding as Bd
     tdt = torch.float32 if dtype == 0 else torch.bfloat16
     rng = np.random.default_rng(seed)
     A = rng.standard_normal((M, K)).astype(np.float32)
     B = rng.standard_normal((N, K)).astype(np.float32)
+    if spoil:
+        spoil(A, B)
     tA = torch.from_numpy(A).cuda().to(tdt)
     tB = torch.from_numpy(B).cuda().to(tdt)
     A64, B64 = tA.double().cpu().numpy(), tB.double().cpu().numpy()
@@ -44,7 +47,8 @@ def _run(dtype, M, N, K, a_major, b_major, *, bias=False, act=0, residual=False,
     ldd = (N + 7) // 8 * 8
     D0 = rng.standard_normal((M, ldd)).astype(np.float32)
     tD = torch.from_numpy(D0).cuda().to(torch.float32 if d_fp32 else tdt)
-    ref = alpha * (A64 @ B64.T)
+    with np.errstate(invalid="ignore"):
+        ref = alpha * (A64 @ B64.T)
     d = Bd.GemmDesc()
     d.dtype, d.M, d.N, d.K, d.batch, d.hdiv = dtype, M, N, K, 1, 1
     d.A, d.a_rs, d.a_ks = sA.data_ptr(), a_rs, a_ks
@@ -79,9 +83,15 @@ def _run(dtype, M, N, K, a_major, b_major, *, bias=False, act=0, residual=False,
     if accumulate:
         ref = ref + D0[:, :N].astype(np.float64)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    Bd.mslt_op_gemm(d, torch.cuda.current_stream().cuda_stream, status)
+    if planes:
+        scratch = torch.full((Bd.mslt_op_gemm_f32_split_scratch_bytes(d),), 255, dtype=torch.uint8, device="cuda")
+        Bd.mslt_op_gemm_f32_split(d, scratch, torch.cuda.current_stream().cuda_stream, status)
+    else:
+        Bd.mslt_op_gemm(d, torch.cuda.current_stream().cuda_stream, status)
     out = tD.double().cpu().numpy()
-    tol = 2e-5 if dtype == 0 else (1e-5 if d_fp32 else 6e-3)
+    if spoil:
+        return out[:, :N], ref
+    tol = tol or (2e-5 if dtype == 0 else (1e-5 if d_fp32 else 6e-3))
     scale = np.abs(ref).max()
     assert np.abs(out[:, :N] - ref).max() / scale < tol, (M, N, K, a_major, b_major)
     # columns past N (padding of the leading dimension) are never written
@@ -323,3 +333,61 @@ def test_bf16_descriptors_without_a_kernel_are_refused(N, kw):
 def test_fp32_more_rows_than_narrow_tiles_can_index():
     """Over 65535 x 32 rows only the tiles of more rows fit the launch grid."""
     _run(0, 65535 * 32 + 70, 8, 8, "k", "k", bias=True, d_fp32=True)
+
+
+# the tile width and the k split that the size rule gives each shape stand behind it
+PLANE_SHAPES = [((64, 72, 200), ("k", "k")),        # 64, 1
+                ((130, 328, 136), ("mn", "k")),     # 64, 1
+                ((704, 760, 520), ("k", "mn")),     # 64, 2
+                ((256, 768, 768), ("mn", "mn")),    # 64, 4
+                ((72, 136, 3072), ("k", "k")),      # 64, 8
+                ((1000, 3072, 520), ("k", "k")),    # 128, 1
+                ((600, 1160, 1160), ("k", "mn")),   # 128, 2
+                ((520, 760, 1160), ("mn", "k")),    # 128, 4
+                ((160, 768, 30520), ("k", "mn")),   # 128, 8
+                ((1, 8, 8), ("k", "k"))]
+
+
+@pytest.mark.parametrize("shape,majors", PLANE_SHAPES)
+def test_fp32_product_on_split_operands(shape, majors):
+    """A sum of 64 products leaves tensor memory within 2^-21 of its size, and K / 64 of them are added in fp32:
+    far below the 2e-5 of the plain kernel's chain."""
+    wgrad = majors == ("mn", "mn")
+    _run(0, *shape, *majors, bias=not wgrad, residual=not wgrad, d_fp32=True, accumulate=wgrad, planes=True, tol=1e-6)
+
+
+@pytest.mark.parametrize("kw", [dict(act=1, aux_out=True, bias=True), dict(act=2), dict(alpha=0.125, residual=True)])
+def test_fp32_split_operands_epilogues(kw):
+    _run(0, 200, 136, 264, "k", "mn", d_fp32=True, planes=True, tol=2e-6, **kw)
+
+
+@pytest.mark.parametrize("ea,eb", [(-100, 58), (58, -100), (-58, -40), (58, 57)])
+def test_fp32_split_operands_over_the_exponent_range(ea, eb):
+    def scale(A, B):
+        A *= np.float32(2.0 ** ea)
+        B *= np.float32(2.0 ** eb)
+    out, ref = _run(0, 130, 136, 520, "k", "k", d_fp32=True, planes=True, spoil=scale)
+    assert np.abs(out - ref).max() / np.abs(ref).max() < 1e-6
+
+
+@pytest.mark.parametrize("shape,majors", [((130, 136, 520), ("k", "k")), ((72, 136, 3072), ("mn", "k")), ((600, 1160, 1160), ("k", "mn"))])
+def test_fp32_split_operands_with_infinities_and_the_largest_values(shape, majors):
+    """What has no sum of three bf16 values: the product is what fp32 multiply-adds give, infinite or NaN in
+    exactly the same places, and as precise as ever everywhere else."""
+    M, N, K = shape
+    def spoil(A, B):
+        B[:, 3] = np.exp2(np.floor(np.log2(np.abs(B[:, 3]) + 0.1)))   # powers of two: their lower planes are zero
+        A[5, 3], A[6, 3] = np.inf, -np.inf
+        A[7, 3], B[:, 4], A[7, 4] = np.inf, 2.0, -np.inf              # inf - inf
+        A[8, :] = 0.0
+        A[8, 5], B[:, 5] = 3.4028235e38, 0.25                         # would round to infinity in bf16
+        A[9, 6], B[:, 6] = np.nan, 1.0
+        B[2, 7], A[:, 7] = np.inf, np.where(np.arange(M) % 2, 1.0, 0.0)
+    out, ref = _run(0, M, N, K, *majors, d_fp32=True, planes=True, spoil=spoil)
+    assert np.isinf(ref[5]).any() and np.isnan(ref[7]).all() and np.isnan(ref[9]).all() and np.isfinite(ref[8]).sum() >= N - 1
+    assert np.array_equal(np.isnan(out), np.isnan(ref))
+    assert np.array_equal(np.isinf(out), np.isinf(ref)) and np.array_equal(np.sign(out[np.isinf(ref)]), np.sign(ref[np.isinf(ref)]))
+    fin = np.isfinite(ref)
+    small = fin & (np.arange(M) != 8)[:, None]
+    assert np.abs(out - ref)[small].max() / np.abs(ref[small]).max() < 2e-5
+    assert (np.abs(out[8] - ref[8]) / np.abs(ref[8]))[fin[8]].max() < 1e-6
