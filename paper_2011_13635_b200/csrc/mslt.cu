@@ -221,6 +221,24 @@ constexpr int64_t kAdamChunk = 8192;
 // saved-activation slots: one per layer that may be trainable at the same time
 int trainable_slots(const mslt_arch& a) { return a.max_trainable > 0 ? a.max_trainable : a.max_layers; }
 
+// Whether any linear or head product of the configuration can be large enough for split operands (gemm_f32x3.cu).
+// The estimate behind that is linear in the rows and lost without any, so the largest batch decides.
+bool any_product_on_planes(const mslt_arch& a) {
+  const int64_t H = a.hidden, F = a.ffn, V = a.vocab, T = (int64_t)a.max_batch * a.max_seq, R = (int64_t)a.max_batch * a.max_pred;
+  auto wins = [](int64_t rows, int64_t n, int64_t k) {  // of a layer's three products: rows x n, rows x k, n x k
+    for (int i = 0; i < 3; i++) {
+      mslt_gemm_desc d = {};
+      d.batch = d.hdiv = 1;
+      d.M = (int)(i < 2 ? rows : n); d.N = (int)(i == 0 ? n : k); d.K = (int)(i == 0 ? k : i == 1 ? n : rows);
+      d.a_rs = d.b_rs = pad_to(d.K, 8);
+      d.a_ks = d.b_ks = 1;
+      if (gemm_f32x3_wins(d, 0)) return true;
+    }
+    return false;
+  };
+  return a.dtype == 0 && (wins(T, 3 * H, H) || wins(T, H, H) || wins(T, F, H) || wins(R, H, H) || wins(R, V, H));
+}
+
 // Lays out the workspace; with base == nullptr only the size is computed.
 void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char* base,
                     Workspace& w) {
@@ -241,7 +259,8 @@ void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char
   const int64_t Vp = pad_to(a.vocab, 8);
   const int64_t P2 = (int64_t)a.max_batch * A * a.max_seq * a.max_seq;
   w.scalars = (int*)take(256);
-  if (a.dtype == 0) {
+  w.x3a = w.x3b = w.x3e = nullptr;
+  if (any_product_on_planes(a)) {
     const int64_t wide = std::max(3 * H, F);
     w.x3a = take(std::max(T * wide, R * std::max(Vp, H)) * 6);
     w.x3b = take(std::max(std::max(wide * H, R * H), T * std::max(F, H)) * 6);
@@ -446,8 +465,8 @@ int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_em
   *done = false;
   const bool a_ready = reuse_a && c->a_split == d.A, b_ready = b_is_emb && c->emb_split;
   c->a_split = a_ready ? d.A : nullptr;
-  if (!gemm_f32x3_wins(d, (a_ready ? 1 : 0) | (b_ready ? 2 : 0))) return 0;
   Workspace& w = c->ws;
+  if (!w.x3a || !gemm_f32x3_wins(d, (a_ready ? 1 : 0) | (b_ready ? 2 : 0))) return 0;
   char* pb = b_is_emb ? w.x3e : w.x3b;
   const int64_t na = operand_elems(d.M, d.K, d.a_rs, d.a_ks), nb = operand_elems(d.N, d.K, d.b_rs, d.b_ks);
   if (!a_ready) { launch_split3((const float*)d.A, w.x3a, na, w.scalars + 8, c->st); c->launches++; }

@@ -75,3 +75,12 @@ def test_no_cpu_path(binding):
     with pytest.raises(binding.MsltError):
         binding.Mslt(hidden=128, heads=2, ffn=512, vocab=1024, max_pos=64, init_layers=2, max_layers=2,
                      max_batch=8, max_seq=64, max_pred=10, dtype="fp32")
+
+
+def test_fp32_workspace_holds_planes_only_where_a_product_uses_them(binding):
+    """Twice the bf16 workspace is every buffer at 4 bytes an element; the planes of split operands come on top."""
+    def bytes_of(dtype, hidden, heads, ffn, vocab, batch, seq, pred):
+        return binding.mslt_query_bytes(binding.Arch(hidden, heads, ffn, vocab, 512, 2, 2, batch, seq, pred, dtype, 1e-12))[1]
+    tiny, base = (128, 2, 512, 1024, 8, 64, 10), (768, 12, 3072, 30522, 8, 128, 20)
+    assert bytes_of(0, *tiny) < 2 * bytes_of(1, *tiny)
+    assert bytes_of(0, *base) > 2 * bytes_of(1, *base)
