@@ -265,3 +265,28 @@ def test_embedding_gradients_have_the_same_bits_on_every_run():
         assert np.abs(got[0][0]).max() > 0
         if cfg.dtype == "fp32":
             assert np.array_equal(got[0][1], got[1][1])
+
+
+def test_more_contexts_than_pinned_slots():
+    """Contexts come and go without pinning memory of their own; beyond the shared page the loss is read through
+    pageable memory."""
+    import torch
+    from paper_2011_13635_b200.binding import Mslt
+    cfg = I.StageConfig("many", hidden=64, heads=1, ffn=64, vocab=16, max_pos=8, layers=1, trainable=1, batch=1, seq=8, pred=2,
+                        dtype="fp32", seed_index=53)
+    w = I.make_weights(cfg)
+    tok, _, pos, lab = PT.to_cuda(torch, *I.make_batch(cfg))
+    def first_loss(m):
+        m.set_params(w)
+        m.mslt_set_optimizer(lr=0.0)
+        return m.mslt_step(tok, None, pos, lab)
+    ms = [Mslt.from_config(cfg) for _ in range(260)]
+    want = first_loss(ms[0])
+    assert np.isfinite(want) and want > 0.5
+    assert [first_loss(m) for m in ms[250:]] == [want] * 10
+    for m in ms[::2]:
+        m.close()
+    again = [Mslt.from_config(cfg) for _ in range(130)]
+    assert [first_loss(m) for m in again[::13]] == [want] * 10
+    for m in ms[1::2] + again:
+        m.close()
