@@ -348,6 +348,13 @@ int mslt_debug_starve_next_attention(int32_t on);
 int mslt_debug_set_gemm_variant(int32_t variant);
 
 /*
+ * Which kernel the last contraction launched by this thread ran in (host, 5 words), for tests of the rules that
+ * choose: {0 none yet; 1 bf16 persistent; 2 bf16, few tiles; 3 fp32, CUDA cores; 4 fp32, split operands},
+ * tile rows (256: a pair of CTAs), tile columns, k blocks per round (kernel 3: groups of warps that share k),
+ * splits of k. */
+int mslt_debug_last_gemm_form(int32_t out[5]);
+
+/*
  * Memory-safety check for tests: every buffer the library carves out of the workspace is followed
  * by a 256-byte guard band that no kernel may write and that is zero from mslt_create on.  Counts
  * the guard bands that are no longer zero (*bad_out, host; 0 = no stray write).  Synchronises. */

@@ -11,6 +11,7 @@ namespace mslt {
 
 static std::atomic<int64_t> g_launches{0};
 int64_t gemm_launches() { return g_launches.load(); }
+thread_local GemmForm g_gemm_form;
 
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
                 bool b_static) {

@@ -72,6 +72,10 @@ long long attn_launches();
 // Test hook like gemm_tc_starve_next, for the next attention launch (forward or backward).
 void attn_starve_next(int on);
 
+// The form of the last contraction that this thread launched, for tests (mslt_debug_last_gemm_form).
+struct GemmForm { int kernel, tile_m, tile_n, k_blocks, splits; };
+extern thread_local GemmForm g_gemm_form;
+
 // Kernels launched by the GEMM front end since the library was loaded (for launch accounting).
 int64_t gemm_launches();
 

@@ -280,6 +280,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   p.kb_per_split = (kb_total + s - 1) / s;
   const int tile = kTile[t];
   p.n_tiles = (d.N + tile - 1) / tile;
+  g_gemm_form = {3, tile, tile, t == 2 ? 4 : 1, s};
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
   auto m4 = [](int64_t v) { return v % 4 == 0; };
   const bool vec = al16(d.A) && al16(d.B) && m4(amn ? d.a_ks : d.a_rs) && m4(bmn ? d.b_ks : d.b_rs) &&

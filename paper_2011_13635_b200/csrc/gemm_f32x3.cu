@@ -333,6 +333,7 @@ int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void*
   p.f.splits = splits;
   p.f.kb_per_split = (p.kb_total + splits - 1) / splits;
   p.f.n_tiles = (d.N + bn - 1) / bn;
+  g_gemm_form = {4, BM, bn, 1, splits};
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
   p.f.vec_out = al16(d.D) && al16(d.aux) && al16(d.residual) && al16(d.bias) && d.ldd % 4 == 0;
   p.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)p.a_mn << 15) | ((uint32_t)p.b_mn << 16) |

@@ -1056,6 +1056,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   // split count do not depend on the tile form
   p.kb_per_split = ((d.K + 2 * BK - 1) / (2 * BK) + splits - 1) / splits * (2 / ksub);
   p.splits = (p.kb_total + p.kb_per_split - 1) / p.kb_per_split;
+  g_gemm_form = {1, tile_m, p.bn, ksub, p.splits};
   const long long total = tiles * p.splits;
   if (total > 0x7fffffffll) { snprintf(err, 256, "gemm: too many tiles"); return MSLT_ERR_SIZE; }
   p.total_work = (int)total;

@@ -301,6 +301,7 @@ int gemm_tc_small_launch(const mslt_gemm_desc& d, int splits, bool early, int* s
   p.status = status;
   p.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)p.a_mn << 15) | ((uint32_t)p.b_mn << 16) |
             ((uint32_t)(TS_BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+  g_gemm_form = {2, BM, TS_BN, 1, splits};
   MapVal ma, mb;
   int rc = get_map(d.A, d.M, d.K, d.a_rs, d.a_ks, 0, 0, 1, 1, BM, &ma, err);
   if (!rc) rc = get_map(d.B, d.N, d.K, d.b_rs, d.b_ks, 0, 0, 1, 1, TS_BN, &mb, err);

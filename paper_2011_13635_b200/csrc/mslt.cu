@@ -1462,6 +1462,13 @@ int mslt_op_gemm(const mslt_gemm_desc* d, void* cuda_stream, int32_t* d_status) 
   return read_gemm_status(d_status, (cudaStream_t)cuda_stream);
 }
 
+int mslt_debug_last_gemm_form(int32_t out[5]) {
+  if (!out) return fail(MSLT_ERR_ARG, "null pointer");
+  const GemmForm& f = g_gemm_form;
+  out[0] = f.kernel; out[1] = f.tile_m; out[2] = f.tile_n; out[3] = f.k_blocks; out[4] = f.splits;
+  return 0;
+}
+
 size_t mslt_op_gemm_f32_split_scratch_bytes(const mslt_gemm_desc* d) {
   if (!d) return 0;
   return 256 + 6 * (size_t)(pad_to(operand_elems(d->M, d->K, d->a_rs, d->a_ks), 64) + pad_to(operand_elems(d->N, d->K, d->b_rs, d->b_ks), 64));

@@ -21,8 +21,10 @@ def _dgelu(u):
 
 
 def _run(dtype, M, N, K, a_major, b_major, *, bias=False, act=0, residual=False, aux_out=False,
-         d_fp32=False, accumulate=False, alpha=1.0, split_k=0, seed=0, planes=False, spoil=None, tol=None):
-    """planes: the fp32 form on split operands; spoil(A, B) changes the operands before they are stored."""
+         d_fp32=False, accumulate=False, alpha=1.0, split_k=0, seed=0, planes=False, spoil=None, tol=None,
+         form=None):
+    """planes: the fp32 form on split operands; spoil(A, B) changes the operands before they are stored; form: what
+    mslt_debug_last_gemm_form has to report."""
     import torch
     from paper_2011_13635_b200 import binding as Bd
     tdt = torch.float32 if dtype == 0 else torch.bfloat16
@@ -88,6 +90,8 @@ def _run(dtype, M, N, K, a_major, b_major, *, bias=False, act=0, residual=False,
         Bd.mslt_op_gemm_f32_split(d, scratch, torch.cuda.current_stream().cuda_stream, status)
     else:
         Bd.mslt_op_gemm(d, torch.cuda.current_stream().cuda_stream, status)
+    if form:
+        assert Bd.mslt_debug_last_gemm_form() == form
     out = tD.double().cpu().numpy()
     if spoil:
         return out[:, :N], ref
@@ -249,18 +253,23 @@ def test_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
     assert int(status.item()) == 0
 
 
-@pytest.mark.parametrize("shape,majors", [
-    ((1024, 768, 768), ("k", "k")),      # 32 x 32 tiles
-    ((1024, 2304, 96), ("k", "k")),      # 128 x 128 tiles
-    ((160, 768, 2500), ("k", "mn")),     # k split over a cluster, last slice ragged
-    ((2304, 760, 1000), ("mn", "mn")),   # 64 x 64 tiles in clusters, ragged columns
-    ((3000, 760, 200), ("mn", "mn")),    # 128 x 128 tiles, ragged both ways
-    ((33, 31, 260), ("mn", "k")), ((1, 1, 1), ("k", "k"))])
-def test_fp32_tiles_and_cluster_splits(shape, majors):
+@pytest.mark.parametrize("shape,majors,form", [
+    ((1024, 768, 768), ("k", "k"), (32, 1, 1)),
+    ((1024, 2304, 96), ("k", "k"), (128, 1, 1)),
+    ((160, 768, 2500), ("k", "mn"), (64, 1, 8)),         # last slice ragged
+    ((2304, 760, 1000), ("mn", "mn"), (64, 1, 1)),       # ragged columns
+    ((1024, 760, 1000), ("mn", "mn"), (64, 1, 2)),
+    ((600, 600, 2000), ("k", "mn"), (64, 1, 4)),
+    ((3000, 760, 200), ("mn", "mn"), (128, 1, 1)),       # ragged both ways
+    ((1000, 1000, 500), ("k", "mn"), (128, 1, 2)),
+    ((512, 128, 512), ("k", "k"), (32, 4, 2)),           # warps of a block share k, and a cluster does
+    ((33, 31, 260), ("mn", "k"), (32, 4, 4)), ((1, 1, 1), ("k", "k"), (32, 4, 1))])
+def test_fp32_tiles_and_cluster_splits(shape, majors, form):
     """Every tile size and k split that the fp32 kernel's rule chooses, with remainders.  Sums of K
     products of unit normals: the error of a running fp32 sum grows as sqrt(K) * 2^-24 of its range."""
     wgrad = majors == ("mn", "mn")
-    _run(0, *shape, *majors, bias=not wgrad, d_fp32=True, accumulate=wgrad)
+    tile, groups, splits = form
+    _run(0, *shape, *majors, bias=not wgrad, d_fp32=True, accumulate=wgrad, form=(3, tile, tile, groups, splits))
 
 
 def test_fp32_unaligned_operands_take_the_element_wise_copies():
@@ -282,28 +291,65 @@ def test_fp32_unaligned_operands_take_the_element_wise_copies():
     assert ((D.double() - ref).abs().max() / ref.abs().max()).item() < 2e-5
 
 
-@pytest.mark.parametrize("shape,majors,kw", [
-    ((64, 768, 200), ("k", "k"), dict(bias=True, residual=True)),          # 64-wide tiles, two k blocks per round
-    ((130, 72, 136), ("k", "mn"), dict(act=2)),
-    ((1100, 2304, 136), ("k", "k"), dict(bias=True)),                       # 128-wide
-    ((4096, 760, 264), ("k", "k"), dict(bias=True, residual=True)),         # 192-wide, ragged last tile
-    ((4096, 768, 320), ("k", "mn"), dict(residual=True)),
-    ((4000, 768, 1160), ("k", "k"), dict(bias=True, act=1, aux_out=True)),  # pairs of 192 columns
-    ((2304, 768, 2408), ("mn", "mn"), dict(d_fp32=True, accumulate=True)),  # 192-wide, k split
-    ((24, 768, 4000), ("k", "mn"), dict(d_fp32=True, accumulate=True))])    # narrow tiles, k split many ways
-def test_bf16_tile_forms_the_estimate_picks(shape, majors, kw):
-    _run(1, *shape, *majors, **kw)
+@pytest.mark.parametrize("shape,majors,kw,form", [
+    # one CTA: rows, columns, k blocks per round, k splits
+    ((33, 72, 64), ("k", "k"), dict(bias=True), (128, 64, 1, 1)),
+    ((64, 768, 200), ("k", "k"), dict(bias=True, residual=True), (128, 64, 2, 1)),
+    ((130, 72, 136), ("k", "mn"), dict(act=2), (128, 64, 2, 1)),
+    ((160, 96, 136), ("k", "mn"), dict(act=2), (128, 64, 2, 1)),
+    ((24, 768, 4000), ("k", "mn"), dict(d_fp32=True, accumulate=True), (128, 64, 2, 11)),
+    ((2056, 544, 136), ("k", "k"), dict(bias=True, residual=True), (128, 128, 2, 1)),
+    ((2056, 544, 136), ("k", "mn"), dict(act=2), (128, 128, 2, 1)),
+    ((2100, 520, 136), ("k", "k"), dict(bias=True, act=1, aux_out=True), (128, 128, 2, 1)),
+    ((130, 3072, 1160), ("mn", "mn"), dict(d_fp32=True, accumulate=True), (128, 128, 2, 3)),
+    ((1100, 2304, 136), ("k", "k"), dict(bias=True), (128, 192, 1, 1)),
+    ((4096, 760, 264), ("k", "k"), dict(bias=True, residual=True), (128, 192, 1, 1)),     # general epilogue
+    ((4096, 768, 320), ("k", "mn"), dict(residual=True), (128, 192, 1, 1)),
+    ((4096, 736, 264), ("k", "k"), dict(residual=True), (128, 192, 1, 1)),                # ragged last tile
+    ((520, 4104, 136), ("k", "k"), dict(bias=True, act=1, aux_out=True), (128, 192, 1, 1)),
+    ((4000, 520, 136), ("k", "k"), dict(bias=True, act=1), (128, 192, 1, 1)),
+    ((4000, 768, 1160), ("k", "k"), dict(bias=True, act=1, aux_out=True), (128, 192, 1, 1)),
+    ((2304, 768, 2408), ("mn", "mn"), dict(d_fp32=True, accumulate=True), (128, 192, 1, 2)),
+    ((3000, 1160, 136), ("k", "k"), dict(bias=True, act=1), (128, 256, 1, 1)),
+    ((3000, 1184, 136), ("k", "k"), dict(residual=True), (128, 256, 1, 1)),
+    ((3000, 1184, 136), ("k", "k"), dict(act=2), (128, 256, 1, 1)),
+    ((3000, 1160, 136), ("k", "k"), dict(d_fp32=True, bias=True), (128, 256, 1, 1)),
+    ((1100, 1040, 2408), ("mn", "mn"), dict(d_fp32=True, accumulate=True), (128, 256, 1, 3)),
+    # a pair of CTAs
+    ((2056, 520, 2408), ("k", "k"), dict(bias=True, act=1, aux_out=True), (256, 128, 2, 1)),
+    ((2056, 544, 2408), ("k", "mn"), dict(residual=True), (256, 128, 2, 1)),
+    ((2056, 544, 2408), ("k", "k"), dict(act=2), (256, 128, 2, 1)),
+    ((4000, 520, 2408), ("k", "k"), dict(bias=True, act=1), (256, 192, 2, 1)),
+    ((520, 4104, 2408), ("k", "k"), dict(bias=True, act=1, aux_out=True), (256, 192, 2, 1)),
+    ((520, 4128, 2408), ("k", "k"), dict(bias=True, residual=True), (256, 192, 2, 1)),
+    ((520, 4128, 2408), ("k", "k"), dict(act=2), (256, 192, 2, 1)),
+    ((8200, 520, 2408), ("k", "k"), dict(d_fp32=True, accumulate=True), (256, 192, 2, 2)),
+    ((6000, 1160, 2408), ("k", "k"), dict(bias=True, act=1), (256, 256, 2, 1)),
+    ((6000, 1184, 2408), ("k", "mn"), dict(act=2), (256, 256, 2, 1)),
+    ((8200, 1160, 2408), ("mn", "mn"), dict(d_fp32=True, accumulate=True), (256, 256, 2, 2))])
+def test_bf16_tile_forms_the_estimate_picks(shape, majors, kw, form):
+    """Every form of the persistent kernel and epilogues on each; small shapes with the few-tile kernel off."""
+    from paper_2011_13635_b200 import binding as Bd
+    few = form[1] == 64 and not kw.get("d_fp32")
+    if few:
+        Bd._check(Bd.lib.mslt_debug_set_gemm_variant(1))
+    try:
+        _run(1, *shape, *majors, form=(1,) + form, **kw)
+    finally:
+        if few:
+            Bd._check(Bd.lib.mslt_debug_set_gemm_variant(0))
 
 
-@pytest.mark.parametrize("shape,majors,kw", [
-    ((1, 8, 64), ("k", "k"), dict(bias=True)),                              # one row, one round
-    ((64, 768, 3072), ("k", "k"), dict(bias=True, residual=True)),          # k over a cluster of eight
-    ((130, 776, 3080), ("k", "mn"), dict(residual=True, alpha=0.5)),        # second row tile of two rows, ragged k and columns
-    ((200, 768, 1160), ("mn", "k"), dict(bias=True, act=1, aux_out=True)),  # ring reused inside a block
-    ((33, 136, 72), ("mn", "mn"), dict(act=2)), ((129, 64, 640), ("k", "k"), dict(bias=True, act=1))])
-def test_bf16_few_tile_kernel(shape, majors, kw):
+@pytest.mark.parametrize("shape,majors,kw,splits", [
+    ((1, 8, 64), ("k", "k"), dict(bias=True), 1),                              # one row, one round
+    ((64, 768, 3072), ("k", "k"), dict(bias=True, residual=True), 8),          # k over a cluster of eight
+    ((130, 776, 3080), ("k", "mn"), dict(residual=True, alpha=0.5), 4),        # second row tile of two rows, ragged k and columns
+    ((200, 768, 1160), ("mn", "k"), dict(bias=True, act=1, aux_out=True), 4),  # ring reused inside a block
+    ((300, 776, 776), ("k", "k"), dict(bias=True, act=1), 2),
+    ((33, 136, 72), ("mn", "mn"), dict(act=2), 1), ((129, 64, 640), ("k", "k"), dict(bias=True, act=1), 4)])
+def test_bf16_few_tile_kernel(shape, majors, kw, splits):
     """Outputs of few tiles: partial sums added inside a cluster, every epilogue."""
-    _run(1, *shape, *majors, **kw)
+    _run(1, *shape, *majors, form=(2, 128, 64, 1, splits), **kw)
 
 
 @pytest.mark.parametrize("N,kw", [(129, dict(act=3)), (200, dict(act=3)), (64, dict(act=3, d_fp32=1)), (64, dict(split_k=2)),
@@ -332,28 +378,24 @@ def test_bf16_descriptors_without_a_kernel_are_refused(N, kw):
 
 def test_fp32_more_rows_than_narrow_tiles_can_index():
     """Over 65535 x 32 rows only the tiles of more rows fit the launch grid."""
-    _run(0, 65535 * 32 + 70, 8, 8, "k", "k", bias=True, d_fp32=True)
+    _run(0, 65535 * 32 + 70, 8, 8, "k", "k", bias=True, d_fp32=True, form=(3, 64, 64, 1, 1))
 
 
-# the tile width and the k split that the size rule gives each shape stand behind it
-PLANE_SHAPES = [((64, 72, 200), ("k", "k")),        # 64, 1
-                ((130, 328, 136), ("mn", "k")),     # 64, 1
-                ((704, 760, 520), ("k", "mn")),     # 64, 2
-                ((256, 768, 768), ("mn", "mn")),    # 64, 4
-                ((72, 136, 3072), ("k", "k")),      # 64, 8
-                ((1000, 3072, 520), ("k", "k")),    # 128, 1
-                ((600, 1160, 1160), ("k", "mn")),   # 128, 2
-                ((520, 760, 1160), ("mn", "k")),    # 128, 4
-                ((160, 768, 30520), ("k", "mn")),   # 128, 8
-                ((1, 8, 8), ("k", "k"))]
+# with the tile width and the k split
+PLANE_SHAPES = [((64, 72, 200), ("k", "k"), (64, 1)), ((130, 328, 136), ("mn", "k"), (64, 1)),
+                ((704, 760, 520), ("k", "mn"), (64, 2)), ((256, 768, 768), ("mn", "mn"), (64, 4)),
+                ((72, 136, 3072), ("k", "k"), (64, 8)), ((1000, 3072, 520), ("k", "k"), (128, 1)),
+                ((600, 1160, 1160), ("k", "mn"), (128, 2)), ((520, 760, 1160), ("mn", "k"), (128, 4)),
+                ((160, 768, 30520), ("k", "mn"), (128, 8)), ((1, 8, 8), ("k", "k"), (64, 1))]
 
 
-@pytest.mark.parametrize("shape,majors", PLANE_SHAPES)
-def test_fp32_product_on_split_operands(shape, majors):
+@pytest.mark.parametrize("shape,majors,form", PLANE_SHAPES)
+def test_fp32_product_on_split_operands(shape, majors, form):
     """A sum of 64 products leaves tensor memory within 2^-21 of its size, and K / 64 of them are added in fp32:
     far below the 2e-5 of the plain kernel's chain."""
     wgrad = majors == ("mn", "mn")
-    _run(0, *shape, *majors, bias=not wgrad, residual=not wgrad, d_fp32=True, accumulate=wgrad, planes=True, tol=1e-6)
+    _run(0, *shape, *majors, bias=not wgrad, residual=not wgrad, d_fp32=True, accumulate=wgrad, planes=True, tol=1e-6,
+         form=(4, 128, form[0], 1, form[1]))
 
 
 @pytest.mark.parametrize("kw", [dict(act=1, aux_out=True, bias=True), dict(act=2), dict(alpha=0.125, residual=True)])
