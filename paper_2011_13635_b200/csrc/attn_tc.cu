@@ -1198,7 +1198,7 @@ struct AttnBwdParams {
   const int* rows;
   bf16* dQKV;         // element (b, i, which, h, e) at dQKV + b * g_bo + i * g_ld + which * H + h * 64 + e
   long long g_ld, g_bo, H;
-  int vec_ok, fast;
+  int vec_ok;
   int q_perm[3], k_perm[3], v_perm[3], c_perm[3], p_perm[3];
   long long wait_limit;
   int starve;         // test hook, as in the forward kernels
@@ -1449,15 +1449,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // dV (complete since dP was): key r, 64 columns
       tc_ld32(trow + 128, v[0]);
       tc_ld32(trow + 160, v[1]);
-      if (p.fast) {
-        if (r < rlim) {
-          store_row32_bf16(gq + 2 * p.H + (long long)r * p.g_ld, v[0]);
-          store_row32_bf16(gq + 2 * p.H + (long long)r * p.g_ld + 32, v[1]);
-        }
-      } else {
-        stage_store_bf16(stg, lane, v[0], gq + 2 * p.H, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[1], gq + 2 * p.H, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
-      }
+      // (32-byte row stores straight from registers were slower here, 58 against 54 us: three 128-byte pieces per row)
+      stage_store_bf16(stg, lane, v[0], gq + 2 * p.H, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
+      stage_store_bf16(stg, lane, v[1], gq + 2 * p.H, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
       if (!mbar_wait(smem_u32(&gfull_bar[g]), use & 1, abort_flag, p.status)) { ok = false; break; }
       tc_fence_after();
 #pragma unroll
@@ -1465,20 +1459,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[g]));
-      if (p.fast) {
-        if (r < rlim) {
-          bf16* row = gq + (long long)r * p.g_ld;
-          store_row32_bf16(row, v[0]);
-          store_row32_bf16(row + 32, v[1]);
-          store_row32_bf16(row + p.H, v[2]);
-          store_row32_bf16(row + p.H + 32, v[3]);
-        }
-      } else {
-        stage_store_bf16(stg, lane, v[0], gq, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[1], gq, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[2], gq + p.H, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
-        stage_store_bf16(stg, lane, v[3], gq + p.H, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
-      }
+      stage_store_bf16(stg, lane, v[0], gq, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
+      stage_store_bf16(stg, lane, v[1], gq, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
+      stage_store_bf16(stg, lane, v[2], gq + p.H, p.g_ld, q * 32, 0, rlim, 64, p.vec_ok);
+      stage_store_bf16(stg, lane, v[3], gq + p.H, p.g_ld, q * 32, 32, rlim, 64, p.vec_ok);
     }
     if (p.cu) zero_tail_rows(p.dQKV, p.g_ld, p.g_ld, p.rows);
   }
@@ -2059,7 +2043,6 @@ int attn_bwd_launch(const void* qkv, const void* probs, const void* dctx, void* 
   p.S = S; p.heads = A; p.items = B * A; p.scale = scale;
   p.dQKV = (bf16*)dqkv; p.g_ld = 3 * H; p.g_bo = (long long)S * 3 * H; p.H = H;
   p.vec_ok = ((uintptr_t)dqkv & 15) == 0 ? 1 : 0;
-  p.fast = 0;  // direct 32-byte row stores measured slower here (58 vs 54 us): three 128-byte pieces per row
   p.wait_limit = WAIT_LIMIT_CYCLES;
   p.status = status;
   if (starve) {  // armed by mslt_debug_starve_next_attention

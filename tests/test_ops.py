@@ -303,6 +303,35 @@ def test_long_row_attention_backward_matches_oracle(B, S, A, k_mean, v_mean):
         assert err < 1.5e-2, (name, err)
 
 
+@pytest.mark.parametrize("which", ["forward", "backward"])
+def test_long_row_attention_wait_that_runs_out_is_reported(which):
+    """As for the other attention kernels below: an idle producer and a 20 ms limit leave the status bit set, and
+    the next call works again."""
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    B, S, A = 2, 200, 2
+    rng = np.random.default_rng(5)
+    bf = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda().bfloat16()
+    qkv, dctx = bf(B * S, 3 * 64 * A), bf(B * S, 64 * A)
+    ctx, dqkv = torch.zeros_like(dctx), torch.zeros_like(qkv)
+    lse, scratch = torch.zeros((A, B * S), device="cuda"), torch.zeros((3, A, B * S), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    calls = dict(forward=lambda: Bd.mslt_op_attention_lse(qkv, ctx, lse, B, S, A, 0.125, status, _stream()),
+                 backward=lambda: Bd.mslt_op_attention_lse_bwd(qkv, ctx, lse, dctx, dqkv, scratch, B, S, A, 0.125, status,
+                                                               _stream()))
+    calls["forward"]()
+    calls["backward"]()
+    want = dqkv.clone()
+    Bd.lib.mslt_debug_starve_next_attention(1)
+    with pytest.raises(Bd.MsltError) as ei:
+        calls[which]()
+    assert ei.value.code == -5 and int(status.item()) & 1
+    status.zero_()
+    calls["forward"]()
+    calls["backward"]()
+    assert int(status.item()) == 0 and torch.equal(dqkv, want)
+
+
 @pytest.mark.parametrize("B,S,A", [(1, 128, 2), (1, 520, 1), (0, 256, 1)])
 def test_long_row_attention_backward_rejects_other_shapes(B, S, A):
     import torch
