@@ -206,6 +206,35 @@ def test_fused_attention_matches_oracle(B, S, A, masked, want_probs):
         assert err / np.abs(ref[b, :lens[b]]).max() < 1.5e-2, (b, err)
 
 
+def test_fused_attention_of_more_items_than_a_block_keeps_a_list_of():
+    """Rows of more than 128 keys: a block describes its first 256 (sequence, head, query tile) items in shared
+    memory and reads the words of any further ones from global memory; with one block per SM those are the second
+    query tiles of the last sequences here."""
+    import math
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    S, A, d = 136, 10, 64
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = (sms * 256 + 1500) // (2 * A)
+    H = A * d
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    qkv = torch.empty((B * S, 3 * H), device="cuda", dtype=torch.bfloat16).normal_(generator=gen)
+    lens = torch.full((B,), S, device="cuda", dtype=torch.int32)
+    lens[-3:] = torch.tensor([129, 90, 133], dtype=torch.int32)
+    ctx = torch.full((B * S, H), 7.0, device="cuda", dtype=torch.bfloat16)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Bd.mslt_op_attention(qkv, None, ctx, lens, B, S, A, 1.0 / math.sqrt(d), status, _stream())
+    assert int(status.item()) == 0
+    for first in (0, B - 8):
+        x = qkv.view(B, S, 3, A, d)[first:first + 8].double()
+        q, k, v = (x[:, :, i].transpose(1, 2) for i in range(3))
+        mask = torch.arange(S, device="cuda")[None] < lens[first:first + 8, None]
+        p = torch.softmax((q @ k.transpose(-1, -2) / math.sqrt(d)).masked_fill(~mask[:, None, None], float("-inf")), -1)
+        ref = (p @ v).transpose(1, 2).reshape(8, S, H)
+        err = (ctx.view(B, S, H)[first:first + 8].double() - ref)[mask].abs().max() / ref.abs().max()
+        assert err < 1.5e-2
+
+
 def test_fused_attention_rejects_other_shapes():
     import torch
     from paper_2011_13635_b200 import binding as Bd
