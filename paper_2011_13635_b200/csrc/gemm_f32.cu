@@ -248,11 +248,21 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   }
   F32Params p;
   p.d = d;
+  auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
+  auto m4 = [](int64_t v) { return v % 4 == 0; };
+  p.vec_out = al16(d.D) && al16(d.aux) && al16(d.residual) && al16(d.bias) && m4(d.ldd) &&
+              (d.batch == 1 || (m4(d.d_bo) && m4(d.d_bi)));
   // Tile and split: the estimate below (SM cycles) reproduces the measured order of the choices on
   // every product of BERT-Base at 1024 tokens and of the small configurations.  A block alone on an
   // SM takes `alone` cycles per k, n blocks share the fp32 pipe at `share` cycles each: measured 58 %
   // of the pipe for 128 x 128 (k-contiguous B), 67 % (row-contiguous B, packed multiply-adds), 60 %
   // for 64 x 64 (row-contiguous B only: 45 % otherwise); 32 x 32 is bound by its chain of slices.
+  // The epilogue is a chain too: a thread takes its outputs four at a time, and the loads of one four wait for the
+  // stores of the last.  With a short k that is most of the time (664 x 1040 x 16 with GELU and its pre-activation
+  // 13.6 us in 64 x 64 tiles, 5.3 to 7.1 in 32 x 32; 592 x 1385 x 25 accumulated, rows of odd pitch, 20.8 and 6.8).
+  // The blocks of a cluster share out the tile's rows, and their constants have the epilogue in them.  Over 244 timed
+  // shapes of all layouts and epilogues the pick is 4.3 % slower than the best form on average and 1.5 times at
+  // worst; without the term 10 % and 3.7 times.  (Products with a batch were fitted without it.)
   const bool amn = d.a_rs == 1 && d.a_ks != 1, bmn = d.b_rs == 1 && d.b_ks != 1;
   const int kb_total = (d.K + FK - 1) / FK;
   int t = 0, s = 1;
@@ -265,6 +275,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
     if (ti == 1 && d.batch > 1) continue;
     if (ti != 0 && (d.M + kTile[ti] - 1) / kTile[ti] > 65535) continue;  // row tiles are the grid's second index
     const double alone = ti == 0 ? share : ti == 1 ? 130. : ti == 2 ? 23. : 34.;
+    const int fours = kTile[ti] * kTile[ti] / kThreads[ti] / 4;  // of a thread
     const double per_block = ti == 0 ? 3000. : ti == 1 ? 600. : ti == 2 ? 700. : 150.;
     for (int si = 1; si <= 8 && (si == 1 || kb_total >= si); si *= 2) {
       const double per_split = ti == 0 ? 6000. : ti == 1 ? 1500. : ti == 2 ? 1000. + 400. * si : 2000.;  // exchange of the partial tile
@@ -272,6 +283,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
       const int units = ti == 0 && si >= 4 ? sms * (si == 4 ? 8 : 7) / 9 : sms;
       const double n = (double)((tiles * si + units - 1) / units);
       const double c = (kb_total + si - 1) / si * FK * (n * share > alone ? n * share : alone) + n * (per_block + (si > 1 ? per_split : 0.)) +
+                       (si == 1 && d.batch == 1 ? (fours - 1) * (p.vec_out ? 350. : 525.) : 0.) +
                        (ti == 3 ? 3000. : 0.);  // its short rows of threads start and end slowly
       if (c < best) { best = c; t = ti; s = si; }
     }
@@ -281,12 +293,8 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   const int tile = kTile[t];
   p.n_tiles = (d.N + tile - 1) / tile;
   g_gemm_form = {3, tile, tile, t == 2 ? 4 : 1, s};
-  auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
-  auto m4 = [](int64_t v) { return v % 4 == 0; };
   const bool vec = al16(d.A) && al16(d.B) && m4(amn ? d.a_ks : d.a_rs) && m4(bmn ? d.b_ks : d.b_rs) &&
                    (d.batch == 1 || (m4(d.a_bo) && m4(d.a_bi) && m4(d.b_bo) && m4(d.b_bi)));
-  p.vec_out = al16(d.D) && al16(d.aux) && al16(d.residual) && al16(d.bias) && m4(d.ldd) &&
-              (d.batch == 1 || (m4(d.d_bo) && m4(d.d_bi)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.n_tiles * s, (d.M + tile - 1) / tile, d.batch);
   if (cfg.gridDim.y > 65535 || cfg.gridDim.z > 65535) {

@@ -272,6 +272,19 @@ def test_fp32_tiles_and_cluster_splits(shape, majors, form):
     _run(0, *shape, *majors, bias=not wgrad, d_fp32=True, accumulate=wgrad, form=(3, tile, tile, groups, splits))
 
 
+@pytest.mark.parametrize("shape,majors,kw,form", [
+    ((664, 1040, 16), ("k", "k"), dict(bias=True, act=1, aux_out=True), (32, 4, 1)),
+    ((976, 744, 24), ("k", "k"), dict(residual=True), (32, 1, 1)),
+    ((440, 3000, 48), ("k", "mn"), dict(act=2), (32, 1, 1)),
+    ((592, 1385, 25), ("mn", "mn"), dict(accumulate=True), (32, 4, 1)),
+    ((538, 1422, 17), ("k", "mn"), dict(bias=True, act=1), (32, 4, 1))])
+def test_fp32_short_k_takes_tiles_of_few_outputs_per_thread(shape, majors, kw, form):
+    """Where k is short the epilogue is the time, and a thread of a 64 x 64 tile has 64 outputs of it: two to
+    three times slower than these."""
+    tile, groups, splits = form
+    _run(0, *shape, *majors, d_fp32=True, form=(3, tile, tile, groups, splits), **kw)
+
+
 def test_fp32_unaligned_operands_take_the_element_wise_copies():
     import torch
     from paper_2011_13635_b200 import binding as Bd
