@@ -935,10 +935,14 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     return make_int4(kPacked ? p.cu[zo] : zo * p.S, min(max(len, 1), p.S), zo, qt << 24 | zi);
   };
   // Every role needs these words at the start of every item, and read from memory one after another they held up each
-  // item by 0.7 us (64 sequences x 12 heads x 256 keys: 50.0 us without lengths, 58.6 with).  So all are fetched once.
-  for (int i = threadIdx.x; i < min(n_my, AR_TABLE); i += blockDim.x) table[i] = describe(i);
-  __syncthreads();
-  auto item = [&](int i) -> int4 { return i < AR_TABLE ? table[i] : describe(i); };
+  // item by 0.7 us (64 sequences x 12 heads x 256 keys: 50.0 us without lengths, 58.6 with).  So all are fetched once;
+  // a block of a single item has nothing to gain (5 x 12 x 256: 8.5 us, 9.0 by way of the table).
+  const int listed = n_my > 1 ? min(n_my, AR_TABLE) : 0;
+  if (listed) {
+    for (int i = threadIdx.x; i < listed; i += blockDim.x) table[i] = describe(i);
+    __syncthreads();
+  }
+  auto item = [&](int i) -> int4 { return i < listed ? table[i] : describe(i); };
   // column of the context accumulator, and the key block it lies in
   auto o_block = [](int n) { return n == 4 ? 0 : 3; };
   auto o_col = [](int n) { return n == 4 ? 0u : 448u; };
