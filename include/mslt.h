@@ -220,7 +220,8 @@ int mslt_read_loss(mslt_ctx* ctx, float* loss_out);
  * Forward only, nothing saved at any layer, no update: the pass that the bottom layers of a stage
  * take part in (Section 3.2, "only participate in forward computation"), here through the whole
  * stack and optionally through the output layer, e.g. for evaluation between stages.
- *   d_hidden_out  device [B,S,H] in the compute dtype (float or bf16), or NULL
+ *   d_hidden_out  device [B,S,H] in the compute dtype (float or bf16), or NULL.  Rows at or beyond a sequence's
+ *   length: zero with dtype 1, unspecified with dtype 0
  *   d_mlm_positions device [B,P] or NULL; d_logits_out device [B*P, vocab] fp32 or NULL
  *   (rows of empty slots are computed from a zero feature row).
  * Synchronises the stream before returning.
@@ -409,9 +410,11 @@ int mslt_op_colsum(int32_t dtype, const void* d_x, int64_t ld, int32_t rows, int
 
 /* Attention of one encoder layer in a single kernel (the paper defers the encoder to BERT,
  * Section 4.1: scaled dot-product attention with a key-padding mask), bf16 only, head width 64,
- * 1 <= S <= 512 (rows of more than 128 keys run a two-pass form of the kernel):  probs[b,h,i,:] = softmax over the valid keys j < d_seq_lens[b] (NULL: all S) of
+ * 1 <= S <= 512 (rows of more than 128 keys run kernels of their own, one that stores the probabilities and one
+ * that does not):  probs[b,h,i,:] = softmax over the valid keys j < d_seq_lens[b] (NULL: all S) of
  * scale * q_i . k_j, masked probabilities exactly 0;  ctx[b,i,h,:] = sum_j probs[b,h,i,j] v_j with
- * probs rounded to bf16 first.  d_qkv: device, [B*S, 3*heads*64] row-major, columns = queries |
+ * the probabilities (beyond 128 keys without d_probs: the exponentials, before the division by their sum) rounded
+ * to bf16 first.  d_qkv: device, [B*S, 3*heads*64] row-major, columns = queries |
  * keys | values, head h in columns h*64.. of each; d_probs: device, [B, heads, S, S] or NULL (not
  * written); d_ctx: device, [B*S, heads*64].  All buffers 16-byte aligned and caller-owned.
  * d_status: device int32 that receives bit 0 if a bounded wait ran out (returned as

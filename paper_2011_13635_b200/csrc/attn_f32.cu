@@ -9,7 +9,9 @@
 // Bound by launches and the chain copy - product - softmax - product where sequences are few, by the
 // shared-memory reads of the products otherwise (2 x 4 outputs on twice the threads: backward 36.7 -> 51.6 us).
 // 16 heads x 64 keys: forward 8.3 -> 5.5 us and one launch in the place of three, backward 13.0 -> 7.8 us and
-// one for five; 96 x 128 keys: 17 and 37 us.  Rows of at most 128 keys only: steps of 2 to 3 layers with
+// one for five; 96 x 128 keys: 17 and 37 us.  A step of two layers is faster with it at every batch and head count
+// tried, 16 to 1536 items (8 x 64 keys x 2 heads 310 -> 296 us, 32 x 128 x 12 3276 -> 3157, 64 x 128 x 16 9445 -> 9376,
+// 128 x 128 x 12 11768 -> 11533), so the rule looks at the row length only.  Rows of at most 128 keys: steps of 2 to 3 layers with
 // 256 keys take the same time either way (476 and 477 us, 2 234 and 2 219 us), with 512 keys the batched
 // products and their larger tiles are ahead (517 against 551 us).
 #include <mutex>

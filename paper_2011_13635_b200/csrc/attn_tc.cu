@@ -429,7 +429,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   }
 }
 
-// ---- forward for rows of 129..512 keys that stores the probabilities (single-kernel entry point) -----------------------------------------------------------
+// ---- forward for rows of 129..512 keys that stores the probabilities (single-kernel entry point) ----
 // A work item is (sequence, head, tile of 128 queries); the keys come in blocks of 128.  The scores
 // of a row do not fit tensor memory next to two context accumulators, so an item runs two passes over
 // the key blocks: pass 1 forms the row maximum and the sum of exponentials (S = Q K_j^T only), pass 2

@@ -1,5 +1,6 @@
 // Front end of the dense contraction: validates the descriptor and picks the kernel.
-// dtype 0 runs on the CUDA cores in fp32; dtype 1 on the tcgen05 tensor cores.
+// dtype 0 runs on the CUDA cores in fp32 (the step's larger fp32 products take gemm_f32x3.cu before they get here);
+// dtype 1 on the tcgen05 tensor cores.
 #include <stdio.h>
 #include <stdlib.h>
 

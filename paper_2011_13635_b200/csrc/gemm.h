@@ -1,6 +1,7 @@
 // Dense contraction with the step's fused epilogue; see mslt_gemm_desc in mslt.h.
 //   D[z][m][n] = epilogue(alpha * sum_k A[z](m,k) * B[z](n,k))
-// dtype 0: fp32 CUDA-core kernel (gemm_f32.cu); dtype 1: bf16 tcgen05 kernel (gemm_tc.cu).
+// dtype 0: fp32 on the CUDA cores (gemm_f32.cu), or on the tensor cores after a split (gemm_f32x3.cu);
+// dtype 1: bf16 on tcgen05 (gemm_tc.cu; gemm_tc_small.cu where the output has few tiles).
 #pragma once
 #include <cuda_runtime.h>
 

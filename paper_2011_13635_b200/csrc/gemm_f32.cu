@@ -1,12 +1,11 @@
 // fp32 contraction on the CUDA cores:  D[z][m][n] = epilogue(alpha * sum_k A[z](m,k) * B[z](n,k)).
 // TF32 tensor cores are not used: the fp32 path is held to 1e-4 and every product stays a full
-// fp32 multiply-add.  Measured (back-to-back launches, 1024 tokens of BERT-Base widths): 1024 x 2304 x
-// 768 98.6 us, input gradient 1024 x 768 x 3072 120 us, weight gradients 3072 x 768 x 1024 92 us,
-// 160 x 768 x 30528 262 us; an average product of that step took 171 us in the 64 x 64 kernel with
-// unpipelined loads that this one replaces, one of the smallest configuration (512 x 128 x 512) 20 us,
-// then 6, and with four groups of warps sharing the k of a 32 x 32 tile 3.1 to 6.0.  The fp32 pipe is
-// 50-67 % busy at 128 x 128; 16 warps per SM with fragments of one k (128 registers), packed
-// multiply-adds along k and slices of 16 were no faster.
+// fp32 multiply-add.  What runs here: the products of small configurations, the attention products, and any
+// operands that the split form does not take.  Measured (back-to-back launches): a product of the smallest
+// configuration (512 x 128 x 512) 20 us in the 64 x 64 kernel with unpipelined loads that this one replaces, then 6,
+// and with four groups of warps sharing the k of a 32 x 32 tile 3.1 to 6.0; 128 x 768 x 768 16.7, 1024 x 2304 x 768
+// 97 (24 in gemm_f32x3.cu with both splits).  The fp32 pipe is 50-67 % busy at 128 x 128; 16 warps per SM with
+// fragments of one k (128 registers), packed multiply-adds along k and slices of 16 were no faster.
 //
 // Bound by the fp32 pipe (128 lanes per SM) where there is work for every SM, by the serial chain of
 // k slices where there is not.  A block owns an output tile (128 x 128, 64 x 64 or 32 x 32) and walks
@@ -279,7 +278,8 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
     const double per_block = ti == 0 ? 3000. : ti == 1 ? 600. : ti == 2 ? 700. : 150.;
     for (int si = 1; si <= 8 && (si == 1 || kb_total >= si); si *= 2) {
       const double per_split = ti == 0 ? 6000. : ti == 1 ? 1500. : ti == 2 ? 1000. + 400. * si : 2000.;  // exchange of the partial tile
-      // one 128 x 128 block fits an SM, so clusters of four and eight leave SMs of a GPC unused
+      // one 128 x 128 block fits an SM, so clusters of four and eight leave SMs of a GPC unused: 132 and 120 of
+      // 148 blocks run at once (cudaOccupancyMaxActiveClusters)
       const int units = ti == 0 && si >= 4 ? sms * (si == 4 ? 8 : 7) / 9 : sms;
       const double n = (double)((tiles * si + units - 1) / units);
       const double c = (kb_total + si - 1) / si * FK * (n * share > alone ? n * share : alone) + n * (per_block + (si > 1 ? per_split : 0.)) +

@@ -288,9 +288,11 @@ bool gemm_f32x3_wins(const mslt_gemm_desc& d, int planes_ready) {
   if (!gemm_f32x3_accepts(d)) return false;
   const double flops = 2.0 * d.M * d.N * (double)d.K;
   const double split = 1e-3 * 10. * ((planes_ready & 1 ? 0. : dense(d.M, d.K, d.a_rs, d.a_ks)) + (planes_ready & 2 ? 0. : dense(d.N, d.K, d.b_rs, d.b_ks)));
-  // microseconds.  Measured: 28-38 TFLOP/s on the CUDA cores against 90-200 here, splitting at 4.5 TB/s:
-  // 1024 x 2304 x 768 97 -> 18.7 us + 5.4 for both operands, 256 x 768 x 768 17.2 -> 8.0 + 3.4; products
-  // below about 0.15 GFLOP stay on the CUDA cores (512 x 384 x 128 5.9 us there).
+  // microseconds.  One rate stands for each side: measured 20-38 TFLOP/s on the CUDA cores from 0.6 GFLOP on, 60-200
+  // here, splitting at 4.5 TB/s.  Both sides (CUDA cores | product here, + split of one operand, + of both):
+  // 512 x 384 x 128 5.1 | 6.3 8.1 9.6, 64 x 768 x 768 8.4 | 8.4 9.9 11.7, 128 x 768 x 768 16.7 | 8.4 10.0 11.8,
+  // 192 x 768 x 768 17.0 | 8.7 10.3 12.3, 1024 x 2304 x 768 97 | 18.4 21.1 24.2, 160 x 30520 x 768 232 | 85 87 123.
+  // The line falls near 0.2 GFLOP; a split that is there already belongs to a product beyond it.
   const int to_split = (planes_ready & 1 ? 0 : 1) + (planes_ready & 2 ? 0 : 1);
   return 5. + flops / 28e6 > 5. + flops / 130e6 + split / 4.5e3 + 1.5 * to_split;
 }
@@ -325,7 +327,7 @@ int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void*
   for (int w = 64; w <= 128; w += 64)
     for (int s = 1; s <= 8 && (s == 1 || p.kb_total >= 2 * s); s *= 2) {
       const long long tiles = (long long)((d.M + BM - 1) / BM) * ((d.N + w - 1) / w);
-      const int units = s >= 4 ? sms * (s == 4 ? 8 : 7) / 9 : sms;  // one block per SM: clusters leave some unused
+      const int units = s >= 4 ? sms * (s == 4 ? 8 : 7) / 9 : sms;  // one block per SM: clusters of 4 and 8 run 132 and 120 at once
       const double n = (double)((tiles * s + units - 1) / units);
       const double c = n * ((p.kb_total + s - 1) / s * (w == 64 ? 1900. : 2500.) + 4000. + w * 20. + (s > 1 ? 4500. + w * 10. * (s > 2) : 0.));
       if (c < best) { best = c; bn = w; splits = s; }

@@ -580,9 +580,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         advance(nt2, mt2, z2, sp2);
         if constexpr (kHasXf) {
           // the next tile's rows of the extra operand start on their way to L2: they come from memory where
-          // the operand is as large as the output (with this, chunk reads issued early and the polynomials
-          // interleaved: 16384 x 768 x 768 + residual 39.4 -> 35.3 us, 16384 x 3072 x 768 . GELU' 106 -> 102,
-          // with both outputs of a GELU 93 -> 89)
+          // the operand is as large as the output.  This, the accumulator reads issued early and the interleaved
+          // polynomials came in together; apart (us at 16384 rows; all three | without this | without early reads |
+          // one pair of columns at a time): 768 x 768 + residual 29.7 | 30.5 | 31.7 | 29.7, 768 x 3072 + residual
+          // 66.8 | 70.2 | 67.0 | 67.5, 3072 x 768 . GELU' 95.5 | 91.9 | 94.0 | 91.1, both outputs of a GELU
+          // 87.1 | 87.2 | 85.8 | 87.2; before them 34.9, 69.7, 98.4 and 89.6.  The residual gains by the first
+          // two; for GELU' none of the three pays by itself.
           if (hsel == 0 && w + w_step < total_work && mt2 * mt_rows + (int)cta_rank * BM + q * 32 + lane < p.M && p.direct) {
             const int zo2 = p.hdiv == 1 ? z2 : z2 / p.hdiv, zi2 = p.hdiv == 1 ? 0 : z2 - zo2 * p.hdiv;
             const int cols = min(p.bn, p.N - nt2 * p.bn) & ~7;

@@ -259,7 +259,7 @@ int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, double* t) {
   for (int s = 1; s <= 8; s *= 2) {
     const int per = (kb + s - 1) / s;
     if (s > 1 && per < 2) continue;
-    if (tiles * s > (s >= 4 ? num_sms * (s == 4 ? 8 : 7) / 9 : num_sms)) continue;  // one wave
+    if (tiles * s > (s >= 4 ? num_sms * (s == 4 ? 8 : 7) / 9 : num_sms)) continue;  // one wave (200 KB blocks in clusters of 4 and 8: 132 and 120 of 148 at once)
     // fitted to the launches named at the top of the file: start and end, rounds, the exchange in the
     // cluster, rows of the epilogue, blocks that share L2
     const double c = 3.4 + 0.23 * per + (s > 1 ? 0.3 + 0.1 * s : 0.) + (d.M < BM ? d.M : BM) / 128. + 0.4 * tiles * s / num_sms;
