@@ -94,10 +94,14 @@ __device__ __forceinline__ void zero_tail_rows(bf16* base, long long ld, long lo
 // ring (the producer waits for their arrival on the slot's empty barrier too); on a tile with rows to clear
 // they also complete the slot's clean barrier, which the thread that issues the products then waits for instead of
 // the full barrier.  (Cleared by the softmax warps: evaluation of 12 x (200..384) keys 2.79 -> 2.83 ms.)
+// Where every tile has such rows the hand-over shows: training steps on 299 x (16..32) keys, 3 layers, 2449 -> 2507 us.
+// In the forward of up to 128 keys the contraction therefore ends with the 16 keys that hold the last one, only those
+// are cleared, and lengths are asked for one item early (evaluation of 75 x (16..32) keys 908 us without clearing, 914
+// with, 912 so); the same in the backward made no difference (2449 -> 2504 us).
 constexpr int CLEAR_WARPS = 2;  // a thread's registers stay the same: four schedulers, three or five warps each
-// rows from r0 on of a tile (128 bytes each; the swizzle permutes inside a row), shared out over the clearing warps
-__device__ __forceinline__ void clear_tile_rows(uint8_t* tile, int r0, int idx) {
-  for (int v = r0 * 8 + idx; v < 128 * 8; v += 32 * CLEAR_WARPS) reinterpret_cast<uint4*>(tile)[v] = make_uint4(0, 0, 0, 0);
+// rows r0 .. r1 of a tile (128 bytes each; the swizzle permutes inside a row), shared out over the clearing warps
+__device__ __forceinline__ void clear_tile_rows(uint8_t* tile, int r0, int r1, int idx) {
+  for (int v = r0 * 8 + idx; v < r1 * 8; v += 32 * CLEAR_WARPS) reinterpret_cast<uint4*>(tile)[v] = make_uint4(0, 0, 0, 0);
 }
 // Every thread of a clearing warp: the tile's writes are visible to the tensor core once this has returned.
 __device__ __forceinline__ void clear_done(uint32_t clean, int lane) {
@@ -225,9 +229,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);           // same for both operand forms
     const uint32_t lbo_mn_lo = (uint32_t)make_smem_desc(0, 64 * BK * 2);   // low word carries the LBO field
     uint32_t cleaned = 0;  // parity of every stage's clean barrier
-    auto issue_pv = [&](int j) -> bool {  // C = P V of item j; P lies over the item's Q and K tiles
+    auto issue_pv = [&](int j, int len) -> bool {  // C = P V of item j; P lies over the item's Q and K tiles
       const uint32_t s = (uint32_t)(j % AT_STAGES), g = (uint32_t)j & 1;
-      if (kPacked && item_len(j) < 128) {
+      if (kPacked && (len & 15)) {
         if (!mbar_wait(smem_u32(&clean_bar[s]), (cleaned >> s) & 1, abort_flag, p.status)) return false;
         cleaned ^= 1u << s;
         tc_fence_after();
@@ -240,6 +244,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (int kb = 0; kb < 2; kb++)
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; k++) {
+          if (kPacked && kb * BK + k * UMMA_K >= len) continue;  // keys beyond the sequence
           const uint64_t ad = ((uint64_t)hi << 32) | (p_lo + kb * (AT_TILE_BYTES / 16) + k * (UMMA_K * 2 / 16));
           const uint64_t bd = ((uint64_t)hi << 32) | (v_lo + kb * (AT_TILE_BYTES / 2 / 16) + k * (UMMA_K * 128 / 16));
           tc_mma(tmem_base + AT_O_COL + g * 64, ad, bd, p.idesc_o, accum);
@@ -249,7 +254,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       tc_commit(smem_u32(&empty_bar[s]));  // the item's tiles are no longer needed
       return true;
     };
+    int len_before = 0;  // a length is asked for one item before it is needed
     for (int i = 0; i < n_my && ok; i++) {
+      const int len = kPacked ? item_len(i) : 128;
       const uint32_t s = (uint32_t)(i % AT_STAGES), round = (uint32_t)(i / AT_STAGES);
       const uint32_t b = (uint32_t)i & 1, use = (uint32_t)i >> 1;
       if (!mbar_wait(smem_u32(&full_bar[s]), round & 1, abort_flag, p.status)) { ok = false; break; }
@@ -268,14 +275,15 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const uint32_t g = (uint32_t)(i - 1) & 1, guse = (uint32_t)(i - 1) >> 1;
         if (!mbar_wait(smem_u32(&pready_bar[g]), guse & 1, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
-        if (!issue_pv(i - 1)) { ok = false; break; }
+        if (!issue_pv(i - 1, len_before)) { ok = false; break; }
       }
+      len_before = len;
     }
     if (ok && n_my > 0) {
       const uint32_t g = (uint32_t)(n_my - 1) & 1, guse = (uint32_t)(n_my - 1) >> 1;
       if (mbar_wait(smem_u32(&pready_bar[g]), guse & 1, abort_flag, p.status)) {
         tc_fence_after();
-        ok = issue_pv(n_my - 1);
+        ok = issue_pv(n_my - 1, len_before);
       } else {
         ok = false;
       }
@@ -288,12 +296,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     }
   } else if (kPacked && warp >= 2 + NUM_EPI_WARPS) {
     // ------------------------------- clearing of rows beyond the sequence -------------------------------
+    int next = n_my ? item_len(0) : 0;
     for (int i = 0; i < n_my; i++) {
-      const int len = item_len(i);
+      const int len = next;
+      if (i + 1 < n_my) next = item_len(i + 1);
       const uint32_t s = (uint32_t)(i % AT_STAGES);
       if (!mbar_wait(smem_u32(&full_bar[s]), (i / AT_STAGES) & 1, abort_flag, p.status)) break;
-      if (len < 128) {
-        clear_tile_rows(smem + (size_t)s * AT_STAGE_BYTES + 2 * AT_TILE_BYTES, len, threadIdx.x - NUM_THREADS);
+      if (len & 15) {
+        clear_tile_rows(smem + (size_t)s * AT_STAGE_BYTES + 2 * AT_TILE_BYTES, len, (len + 15) & ~15, threadIdx.x - NUM_THREADS);
         clear_done(smem_u32(&clean_bar[s]), lane);
       }
       if (lane == 0) mbar_arrive(smem_u32(&empty_bar[s]));
@@ -1057,7 +1067,7 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const uint32_t slot = tt % AR_RING;
         if (!mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status)) { ok = false; break; }
         if (k == 2 * n - 1 && len < n * 128) {
-          clear_tile_rows(ring_smem + (size_t)slot * AT_TILE_BYTES, len - (n - 1) * 128, threadIdx.x - AR_THREADS);
+          clear_tile_rows(ring_smem + (size_t)slot * AT_TILE_BYTES, len - (n - 1) * 128, 128, threadIdx.x - AR_THREADS);
           clear_done(clean0 + 8 * slot, lane);
         }
         if (lane == 0) mbar_arrive(tempty0 + 8 * slot);
@@ -1389,7 +1399,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (!mbar_wait(smem_u32(&full_bar[s]), (i >> 1) & 1, abort_flag, p.status)) break;
       if (len < 128) {
         for (int t = 0; t < 4; t++)  // Q, K, V, dC
-          clear_tile_rows(smem + (size_t)s * AB_STAGE_BYTES + t * AT_TILE_BYTES, len, threadIdx.x - NUM_THREADS);
+          clear_tile_rows(smem + (size_t)s * AB_STAGE_BYTES + t * AT_TILE_BYTES, len, 128, threadIdx.x - NUM_THREADS);
         clear_done(smem_u32(&clean_bar[s]), lane);
       }
       if (lane == 0) mbar_arrive(smem_u32(&empty_bar[s]));
@@ -1728,7 +1738,7 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     auto clear = [&](uint32_t full, uint32_t parity, uint32_t clean, uint32_t empty, uint8_t* tiles, int r0) -> bool {
       if (!mbar_wait(full, parity, abort_flag, p.status)) return false;
       if (r0 < 128) {
-        for (int t = 0; t < 2; t++) clear_tile_rows(tiles + t * AT_TILE_BYTES, r0, threadIdx.x - NUM_THREADS);
+        for (int t = 0; t < 2; t++) clear_tile_rows(tiles + t * AT_TILE_BYTES, r0, 128, threadIdx.x - NUM_THREADS);
         clear_done(clean, lane);
       }
       if (lane == 0) mbar_arrive(empty);

@@ -316,6 +316,13 @@ def test_packed_sequence_does_not_see_its_neighbour(seq, lens):
     m.close()
 
 
+@pytest.mark.parametrize("lens", [(1, 15, 16, 17, 79), (31, 32, 33, 16, 16), (96, 97, 127, 128, 64)])
+def test_packed_sequences_around_the_ends_of_contraction_steps(lens):
+    """The context of rows of up to 128 keys is contracted 16 keys at a time, up to the last one of the sequence."""
+    test_packed_batch_does_not_see_the_rows_of_an_earlier_call(128, lens)
+    test_packed_sequence_does_not_see_its_neighbour(128, lens)
+
+
 @pytest.mark.parametrize("hidden,ffn", [(384, 1088), (448, 1280)])
 def test_fp32_one_head_of_one_sequence(hidden, ffn):
     """The attention products of a single (sequence, head) have no batch and are as large as the linear ones,
