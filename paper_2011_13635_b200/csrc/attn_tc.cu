@@ -187,7 +187,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     return p.seq_lens ? min(max(p.seq_lens[((int)blockIdx.x + i * (int)gridDim.x) / p.heads], 1), p.S) : p.S;
   };
 
-  if (warp == 0 && lane == 0 && !p.starve) {
+  if (warp == 0 && !p.starve && elect_one()) {
     // ------------------------------- TMA producer -------------------------------
     bool ok = true;
     int issued = 0;
@@ -223,7 +223,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         while (!mbar_try_wait(fb, (uint32_t)(j / AT_STAGES) & 1) && now_cycles() - t0 < 200000000ll) {}
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ------------------------------- MMA issuer -------------------------------
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);           // same for both operand forms
@@ -524,7 +524,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   // (K_j, V_{j-1}) for j = 1 .. n-1, then V_{n-1} (the scores of block j are issued before the second
   // product of block j - 1, which has to wait for that block's probabilities).
 
-  if ((warp == 0 || warp == 11) && lane == 0 && !p.starve) {
+  if ((warp == 0 || warp == 11) && !p.starve && elect_one()) {
     // ------------------------------- TMA producer of group g -------------------------------
     bool ok = true;
     uint32_t tt = 0, ig = 0;
@@ -566,7 +566,7 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 4000000ll) {}
     }
-  } else if ((warp == 1 || warp == 10) && lane == 0) {
+  } else if ((warp == 1 || warp == 10) && elect_one()) {
     // ------------------------------- MMA issuer of group g -------------------------------
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);
@@ -957,7 +957,7 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   auto o_block = [](int n) { return n == 4 ? 0 : 3; };
   auto o_col = [](int n) { return n == 4 ? 0u : 448u; };
 
-  if (warp == 0 && lane == 0 && !p.starve) {
+  if (warp == 0 && !p.starve && elect_one()) {
     // ------------------------------- TMA producer -------------------------------
     bool ok = true;
     uint32_t tt = 0, ig = 0;
@@ -987,7 +987,7 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 4000000ll) {}
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ------------------------------- MMA issuer -------------------------------
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);
@@ -1271,7 +1271,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     return p.seq_lens ? min(max(p.seq_lens[((int)blockIdx.x + i * (int)gridDim.x) / p.heads], 1), p.S) : p.S;
   };
 
-  if (warp == 0 && lane == 0 && !p.starve) {
+  if (warp == 0 && !p.starve && elect_one()) {
     // ------------------------------- TMA producer -------------------------------
     bool ok = true;
     int issued = 0;
@@ -1310,7 +1310,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         while (!mbar_try_wait(fb, (uint32_t)(j >> 1) & 1) && now_cycles() - t0 < 200000000ll) {}
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ------------------------------- MMA issuer -------------------------------
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);
@@ -1611,7 +1611,7 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   };
   auto row_base = [&](int zo) { return p.cu ? p.cu[zo] : zo * p.S; };
 
-  if (warp == 0 && lane == 0 && !p.starve) {
+  if (warp == 0 && !p.starve && elect_one()) {
     // ------------------------------- TMA producer -------------------------------
     bool ok = true;
     uint32_t rt = 0, ni = 0;
@@ -1645,7 +1645,7 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 4000000ll) {}
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ------------------------------- MMA issuer -------------------------------
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);

@@ -130,7 +130,7 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int kb0 = min(p.kb_total, rank * p.f.kb_per_split), kb1 = min(p.kb_total, kb0 + p.f.kb_per_split);
   float acc[BN / 2];
 
-  if ((warp == 0 || warp == 2) && lane == 0) {
+  if ((warp == 0 || warp == 2) && elect_one()) {
     // ------------------------------- TMA producers -------------------------------
     const bool isa = warp == 0;
     const CUtensorMap* map = isa ? &tmA : &tmB;
@@ -158,7 +158,7 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 4000000ll) {}
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ------------------------------- MMA issuer -------------------------------
     const uint64_t a0 = make_smem_desc(smem_u32(smem), p.a_mn ? 64 * BK * 2 : 16);
     const uint64_t b0 = make_smem_desc(smem_u32(smem) + 3 * A_PLANE, p.b_mn ? 64 * BK * 2 : 16);

@@ -328,7 +328,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int tiles_per_z = m_tiles * p.n_tiles;
   const int per_split = tiles_per_z * p.batch;
 
-  if ((warp == 0 || warp == 2 || warp == 3) && lane == 0 && !p.starve) {
+  if ((warp == 0 || warp == 2 || warp == 3) && !p.starve && elect_one()) {
     // ------------------------------- TMA producers -------------------------------
     // Producer j takes the k blocks whose running index is j modulo NUM_PRODUCERS.  Every producer
     // walks the whole work list (ring position as (stage, phase) counters, tile coordinates in
@@ -416,7 +416,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
     }
-  } else if (warp == 1 && lane == 0 && leader) {
+  } else if (warp == 1 && leader && elect_one()) {
     // ------------------------------- MMA issuer -------------------------------
     // One thread feeds the tensor core, so its loop is kept short: ring position as counters,
     // descriptors as a constant high word plus a low word that only gains the stage and k offsets.

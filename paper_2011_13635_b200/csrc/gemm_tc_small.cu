@@ -96,7 +96,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       if (p.b_mn) { c[0] = n0; c[p.b_perm] = (kb0 + r) * BK; } else { c[0] = (kb0 + r) * BK; c[p.b_perm] = n0; }
       tma_load_4d(smem_u32(smem) + slot * TS_STAGE + A_STAGE_BYTES, &tmB, fb, c[0], c[1], c[2], c[3]);
     };
-    const bool mine = lane == 0 && !p.starve;
+    const bool mine = !p.starve && elect_one();
     const int n_early = p.early ? min(n_kb, TS_ROUNDS) : 0;
     if (mine)
       for (int r = 0; r < n_early; r++) load_b(r);
@@ -125,7 +125,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     pdl_begin();
     if (p.rows) active = m0 < *p.rows;
     if (active) load_extra(threadIdx.x);
-    if (warp == 1 && lane == 0 && active) {
+    if (warp == 1 && active && elect_one()) {
       const uint64_t a0 = make_smem_desc(smem_u32(smem), p.a_mn ? 64 * BK * 2 : 16);
       const uint64_t bd0 = make_smem_desc(smem_u32(smem) + A_STAGE_BYTES, p.b_mn ? 64 * BK * 2 : 16);
       const uint32_t a_ks = (p.a_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4, b_ks = (p.b_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
