@@ -171,6 +171,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmQ);
+    prefetch_map(&tmK);
+    prefetch_map(&tmV);
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(AT_TMEM_COLS)
@@ -484,6 +489,11 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmQ);
+    prefetch_map(&tmK);
+    prefetch_map(&tmV);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -912,6 +922,11 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmQ);
+    prefetch_map(&tmK);
+    prefetch_map(&tmV);
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(AT_TMEM_COLS)
@@ -1255,6 +1270,13 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmQ);
+    prefetch_map(&tmK);
+    prefetch_map(&tmV);
+    prefetch_map(&tmC);
+    prefetch_map(&tmP);
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(AT_TMEM_COLS)
@@ -1578,6 +1600,12 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmQ);
+    prefetch_map(&tmK);
+    prefetch_map(&tmV);
+    prefetch_map(&tmC);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),

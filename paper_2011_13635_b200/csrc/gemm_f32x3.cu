@@ -101,6 +101,10 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   uint32_t* tmem_slot = (uint32_t*)(accfull_bar + 4);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmA);
+    prefetch_map(&tmB);
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < X3_STAGES; s++) {
       mbar_init(smem_u32(&full_bar[s]), 2);

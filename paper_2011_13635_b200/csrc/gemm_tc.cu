@@ -51,7 +51,8 @@ struct TcParams {
   int d_fp32, accumulate, vec_ok;
   int x32;              // rows of the extra operand start on 32 bytes
   int direct;           // rows of D (and aux) may be stored straight from registers, 32 bytes at a time
-  int tma_store;        // bf16 D leaves through shared memory and tile stores of 32 rows x 64 columns
+  int tma_store;        // D leaves through shared memory and tile stores of 32 rows x 128 bytes
+  int early;            // B and the bias are not written by the kernels before this one: read ahead of the wait for them
   int d_perm[3];        // slots of D's (row, inner-batch, outer-batch) coordinates in its tensor map
   float alpha;
   const float* bias;
@@ -118,6 +119,15 @@ __device__ __forceinline__ void row32_stage_bf16(uint32_t tile, int lane, int ha
                  : "memory");
   }
 }
+// 32 fp32 columns into such a tile, which they fill
+__device__ __forceinline__ void row32_stage_f32(uint32_t tile, int lane, const float2 (&w)[16]) {
+  const uint32_t row = tile + (uint32_t)lane * 128u;
+#pragma unroll
+  for (int c = 0; c < 8; c++)
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(row + (uint32_t)((c ^ (lane & 7)) * 16)), "f"(w[2 * c].x),
+                 "f"(w[2 * c].y), "f"(w[2 * c + 1].x), "f"(w[2 * c + 1].y)
+                 : "memory");
+}
 __device__ __forceinline__ void row32_store_f32(float* dst, const float2 (&w)[16], int accumulate) {
   if (accumulate) {
 #pragma unroll
@@ -163,13 +173,13 @@ __device__ __forceinline__ void prefetch_l2(const void* g, int bytes) {
 }
 
 // One 32 x 32 chunk of a specialised flavour: a = this lane's 32 accumulator columns, bias_c = the
-// chunk's bias values in shared memory (zeros without a bias), x = this lane's 32 bf16 values of
+// chunk's bias values in shared memory (null: no bias), x = this lane's 32 bf16 values of
 // the row-shaped extra operand (EPI_RESIDUAL, EPI_DGELU).
 // `direct`: this lane's row exists and the whole chunk lies inside the output, so the lane stores
 // its 32 columns itself; otherwise the chunk goes through the staging buffer, which handles ragged
 // edges element by element (every lane of the warp takes the same branch).
-// `tile` != 0: the bf16 result goes into that staging tile (shared-memory address) as half `half`
-// of its 64 columns instead, for a tile store by the caller.
+// `tile` != 0: the result goes into that staging tile (shared-memory address) instead, a bf16 one as half
+// `half` of its 64 columns, for a tile store by the caller.
 // `loaded` runs once the accumulator columns have been used up, so that their registers can take the next
 // chunk's read while this chunk is worked on; `x_used` likewise for x.
 template <int kMode, typename F, typename G>
@@ -181,7 +191,7 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
   const float4* b4 = reinterpret_cast<const float4*>(bias_c);
 #pragma unroll
   for (int j = 0; j < 8; j++) {
-    const float4 t = b4[j];
+    const float4 t = bias_c ? b4[j] : make_float4(0.f, 0.f, 0.f, 0.f);
     v[2 * j] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j]), __uint_as_float(a[4 * j + 1])), al,
                           make_float2(t.x, t.y));
     v[2 * j + 1] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j + 2]), __uint_as_float(a[4 * j + 3])), al,
@@ -217,13 +227,18 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
     }
   }
   if constexpr (kMode == EPI_F32) {
-    if (direct) { if (row_ok) row32_store_f32(reinterpret_cast<float*>(p.D) + off, v, p.accumulate); }
+    if (p.tma_store) {  // the chunk before must have left the staging buffer
+      if (elect_one()) tma_store_wait_read();
+      __syncwarp();
+    }
+    if (tile) row32_stage_f32(tile, lane, v);
+    else if (direct) { if (row_ok) row32_store_f32(reinterpret_cast<float*>(p.D) + off, v, p.accumulate); }
     else stage_store_f32(stg, lane, v, reinterpret_cast<float*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok,
                          p.accumulate);
   } else {
     if (tile) {
       if (half == 0) {  // the tile store of the previous group must have read the staging tile
-        if (lane == 0) tma_store_wait_read();
+        if (elect_one()) tma_store_wait_read();
         __syncwarp();
       }
       row32_stage_bf16(tile, lane, half, v);
@@ -232,6 +247,35 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
     else stage_store_bf16(stg, lane, v, reinterpret_cast<bf16*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
   }
 }
+
+// Coordinates of a work item: digits of its index (n tile fastest, then m tile, batch, split).  They advance
+// by mixed-radix addition, so that divisions are done once, ahead of the wait for the preceding kernel.
+struct Walk {
+  int nt, mt, z, sp, d_nt, d_mt, d_z, d_sp;
+  __device__ __forceinline__ void start(int w, int step, int n_tiles, int m_tiles, int batch) {
+    const int tiles = n_tiles * m_tiles, per_split = tiles * batch;
+    int r = w;
+    sp = r / per_split; r -= sp * per_split;
+    z = r / tiles; r -= z * tiles;
+    mt = r / n_tiles; nt = r - mt * n_tiles;
+    r = step;
+    d_sp = r / per_split; r -= d_sp * per_split;
+    d_z = r / tiles; r -= d_z * tiles;
+    d_mt = r / n_tiles; d_nt = r - d_mt * n_tiles;
+  }
+  __device__ __forceinline__ void advance(int n_tiles, int m_tiles, int batch) {
+    nt += d_nt;
+    int c = nt >= n_tiles ? 1 : 0;
+    nt -= c ? n_tiles : 0;
+    mt += d_mt + c;
+    c = mt >= m_tiles ? 1 : 0;
+    mt -= c ? m_tiles : 0;
+    z += d_z + c;
+    c = z >= batch ? 1 : 0;
+    z -= c ? batch : 0;
+    sp += d_sp + c;
+  }
+};
 
 // ---- the kernel ---------------------------------------------------------------------------------
 // 12 warps: a thread may use up to 168 registers
@@ -276,6 +320,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmA);
+    prefetch_map(&tmB);
+    if (p.tma_store) prefetch_map(&tmD);
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; s++) {
       mbar_init(smem_u32(&full_bar[s]), 1);
@@ -309,12 +358,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (kPair) cluster_sync_all();  // the peer's barriers must exist before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_begin();
 
+  // Every role works out its first item before it waits for the preceding kernel, and reads what that kernel
+  // cannot write (1 us and more of every launch that its first product waited for otherwise: divisions,
+  // instruction fetches, the weights' first tiles).
   // The number of rows that hold anything may be known on the device only (batches with padding are
   // kept packed): the tile list is then cut to it.  Rows between that count and M stay unwritten.
   int m_tiles = p.m_tiles, kb_total = p.kb_total, kb_per_split = p.kb_per_split, total_work = p.total_work;
-  if (p.rows != nullptr) {
+  Walk at;
+  at.start(w_first, w_step, p.n_tiles, m_tiles, p.batch);
+  auto begin = [&]() {
+    pdl_begin();
+    if (p.rows == nullptr) return;
     const int rows = *p.rows;
     if (p.rows_are_k) {
       kb_total = (rows + KSUB * BK - 1) / (KSUB * BK);
@@ -323,10 +378,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else {
       m_tiles = (rows + mt_rows - 1) / mt_rows;
       total_work = m_tiles * p.n_tiles * p.batch * p.splits;
+      // with one batch and one split the digits do not depend on the count of m tiles
+      if (p.batch * p.splits > 1 && total_work > 0) at.start(w_first, w_step, p.n_tiles, m_tiles, p.batch);
     }
-  }
-  const int tiles_per_z = m_tiles * p.n_tiles;
-  const int per_split = tiles_per_z * p.batch;
+  };
 
   if ((warp == 0 || warp == 2 || warp == 3) && !p.starve && elect_one()) {
     // ------------------------------- TMA producers -------------------------------
@@ -345,18 +400,28 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t smem0 = smem_u32(smem);
     const uint32_t full0 = smem_u32(&full_bar[0]), empty0 = smem_u32(&empty_bar[0]);
     const uint32_t tx_bytes = kPair ? 2 * stage_bytes : stage_bytes;
+    const uint32_t tx_b = (kPair ? 2 : 1) * KSUB * b_stage_bytes;
     const int a_boxes = p.a_mn ? BM / 64 : 1, b_boxes = p.b_mn ? bn_cta / 64 : 1;
-    for (int w = w_first; w < total_work && ok; w += w_step) {
-      const int split = w / per_split;
-      int r = w - split * per_split;
-      const int z = r / tiles_per_z;
-      r -= z * tiles_per_z;
-      const int mt = r / p.n_tiles, nt = r - mt * p.n_tiles;
-      const int zo = z / p.hdiv, zi = z - zo * p.hdiv;
-      const int kb0 = split * kb_per_split;
-      const int kb1 = min(kb_total, kb0 + kb_per_split);
-      const int row0 = mt * mt_rows + (int)cta_rank * BM;
-      const int col0 = nt * p.bn + (int)cta_rank * bn_cta;
+    // k-contiguous operand: one box {64 k, rows} per k block; row-contiguous: boxes {64 rows,
+    // 64 k}.  A k block that starts at or beyond K is filled with zeros by the copy engine.
+    auto copy = [&](const CUtensorMap* map, uint32_t dst, uint32_t fb, int mn, int kslot, int boxes, int c0, int c1, int c2, int c3) {
+#pragma unroll
+      for (int sub = 0; sub < KSUB; sub++) {
+        const int ko = sub * BK;
+        const int x0 = c0 + (kslot == 0 ? ko : 0), x1 = c1 + (kslot == 1 ? ko : 0), x2 = c2 + (kslot == 2 ? ko : 0),
+                  x3 = c3 + (kslot == 3 ? ko : 0);
+        for (int h = 0; h < boxes; h++) {
+          const uint32_t to = dst + sub * (uint32_t)sub_bytes + h * (64 * BK * 2);
+          if (kPair) tma_load_4d_pair(to, map, fb, x0 + (mn ? h * 64 : 0), x1, x2, x3);
+          else tma_load_4d(to, map, fb, x0 + (mn ? h * 64 : 0), x1, x2, x3);
+        }
+      }
+    };
+    int a0, a1, a2, a3, b0, b1, b2, b3;
+    auto coords = [&](int kb0) {
+      const int zo = at.z / p.hdiv, zi = at.z - zo * p.hdiv;
+      const int row0 = at.mt * mt_rows + (int)cta_rank * BM;
+      const int col0 = at.nt * p.bn + (int)cta_rank * bn_cta;
       int ca[4], cb[4];
       if (!p.a_mn) { ca[0] = kb0 * RK; ca[p.a_perm[0]] = row0; }
       else         { ca[0] = row0; ca[p.a_perm[0]] = kb0 * RK; }
@@ -364,34 +429,46 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (!p.b_mn) { cb[0] = kb0 * RK; cb[p.b_perm[0]] = col0; }
       else         { cb[0] = col0; cb[p.b_perm[0]] = kb0 * RK; }
       cb[p.b_perm[1]] = zi; cb[p.b_perm[2]] = zo;
-      int a0 = ca[0], a1 = ca[1], a2 = ca[2], a3 = ca[3];
-      int b0 = cb[0], b1 = cb[1], b2 = cb[2], b3 = cb[3];
+      a0 = ca[0]; a1 = ca[1]; a2 = ca[2]; a3 = ca[3];
+      b0 = cb[0]; b1 = cb[1]; b2 = cb[2]; b3 = cb[3];
+    };
+    // pair mode: both CTAs' copies are counted on the leader's barrier
+    auto barrier_of = [&](uint32_t slot) { return kPair ? mapa_u32(full0 + slot * 8, 0) : full0 + slot * 8; };
+    coords(at.sp * kb_per_split);
+    uint32_t n_early = 0;
+    if (p.early && w_first < total_work) {
+      n_early = (uint32_t)min(p.stages, min(kb_total, (at.sp + 1) * kb_per_split) - at.sp * kb_per_split);
+      for (uint32_t r = me; r < n_early; r += NUM_PRODUCERS) {
+        if (leader) mbar_expect_more(full0 + r * 8, tx_b);
+        const int k = (int)r;
+        copy(&tmB, smem0 + r * (uint32_t)stage_bytes + A_STAGE_BYTES, barrier_of(r), p.b_mn, bk, b_boxes, b0 + k * db0, b1 + k * db1,
+             b2 + k * db2, b3 + k * db3);
+      }
+    }
+    begin();
+    if (w_first >= total_work && leader) {
+      // fewer rows than the launch had to reckon with: nothing will use the early tiles, but they land before the CTA leaves
+      for (uint32_t r = me; r < n_early; r += NUM_PRODUCERS) {
+        mbar_arrive(full0 + r * 8);
+        if (!mbar_wait(full0 + r * 8, 0, abort_flag, p.status)) break;
+      }
+    }
+    for (int w = w_first; w < total_work && ok; w += w_step) {
+      const int kb0 = at.sp * kb_per_split;
+      const int kb1 = min(kb_total, kb0 + kb_per_split);
+      coords(kb0);
       for (int kb = kb0; kb < kb1; kb++, it++) {
         if (turn == me) {
-          if (!mbar_wait(empty0 + s * 8, ph ^ 1, abort_flag, p.status)) { ok = false; break; }
-          const uint32_t fb_own = full0 + s * 8;
-          // pair mode: both CTAs' copies are counted on the leader's barrier
-          const uint32_t fb = kPair ? mapa_u32(fb_own, 0) : fb_own;
-          if (leader) mbar_expect_tx(fb_own, tx_bytes);
-          // k-contiguous operand: one box {64 k, rows} per k block; row-contiguous: boxes {64 rows,
-          // 64 k}.  A k block that starts at or beyond K is filled with zeros by the copy engine.
-#pragma unroll
-          for (int sub = 0; sub < KSUB; sub++) {
-            const uint32_t sa = smem0 + s * (uint32_t)stage_bytes + sub * (uint32_t)sub_bytes;
-            const uint32_t sb = sa + A_STAGE_BYTES;
-            const int ko = sub * BK;
-            const int x0 = a0 + (ak == 0 ? ko : 0), x1 = a1 + (ak == 1 ? ko : 0), x2 = a2 + (ak == 2 ? ko : 0),
-                      x3 = a3 + (ak == 3 ? ko : 0);
-            const int y0 = b0 + (bk == 0 ? ko : 0), y1 = b1 + (bk == 1 ? ko : 0), y2 = b2 + (bk == 2 ? ko : 0),
-                      y3 = b3 + (bk == 3 ? ko : 0);
-            for (int h = 0; h < a_boxes; h++) {
-              if (kPair) tma_load_4d_pair(sa + h * (64 * BK * 2), &tmA, fb, x0 + (p.a_mn ? h * 64 : 0), x1, x2, x3);
-              else tma_load_4d(sa + h * (64 * BK * 2), &tmA, fb, x0 + (p.a_mn ? h * 64 : 0), x1, x2, x3);
-            }
-            for (int h = 0; h < b_boxes; h++) {
-              if (kPair) tma_load_4d_pair(sb + h * (64 * BK * 2), &tmB, fb, y0 + (p.b_mn ? h * 64 : 0), y1, y2, y3);
-              else tma_load_4d(sb + h * (64 * BK * 2), &tmB, fb, y0 + (p.b_mn ? h * 64 : 0), y1, y2, y3);
-            }
+          const uint32_t fb_own = full0 + s * 8, fb = barrier_of(s);
+          const uint32_t dst = smem0 + s * (uint32_t)stage_bytes;
+          if (it < n_early) {
+            if (leader) mbar_expect_tx(fb_own, tx_bytes - tx_b);
+            copy(&tmA, dst, fb, p.a_mn, ak, a_boxes, a0, a1, a2, a3);
+          } else {
+            if (!mbar_wait(empty0 + s * 8, ph ^ 1, abort_flag, p.status)) { ok = false; break; }
+            if (leader) mbar_expect_tx(fb_own, tx_bytes);
+            copy(&tmA, dst, fb, p.a_mn, ak, a_boxes, a0, a1, a2, a3);
+            copy(&tmB, dst + A_STAGE_BYTES, fb, p.b_mn, bk, b_boxes, b0, b1, b2, b3);
           }
           last_it = it;
           mine++;
@@ -401,6 +478,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         if (++turn == (uint32_t)NUM_PRODUCERS) turn = 0;
       }
+      at.advance(p.n_tiles, m_tiles, p.batch);
     }
     if (!ok || *abort_flag) {
       // give up: let this thread's copies that may still be in flight land before the CTA leaves
@@ -438,9 +516,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // of the current block, and its answer is only read afterwards: `ready` for the next ring
     // slot, `acc_free` for the next work item's accumulator.
     uint32_t ready = 0, acc_free = 0;
+    begin();
     for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
-      const int split = w / per_split;
-      const int kb0 = split * kb_per_split;
+      const int kb0 = at.sp * kb_per_split;
       const int kb1 = min(kb_total, kb0 + kb_per_split);
       const uint32_t acc = tile & 1, use = tile >> 1;
       if (!acc_free && !mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
@@ -478,6 +556,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (ok) {  // accumulator complete
         if (kPair) tc_commit_pair(smem_u32(&tfull_bar[acc])); else tc_commit(smem_u32(&tfull_bar[acc]));
       }
+      at.advance(p.n_tiles, m_tiles, p.batch);
     }
     if (!ok || *abort_flag) {
       // make sure no MMA is still writing tensor memory before it is freed
@@ -505,35 +584,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // and a lane stores its row segment straight from registers.
       constexpr bool kHasXf = kMode == EPI_RESIDUAL || kMode == EPI_DGELU;
       const bf16* xsrc = kMode == EPI_DGELU ? p.aux : kMode == EPI_RESIDUAL ? p.residual : nullptr;
-      // digits of the work index (n tile fastest, then m tile, batch, split) and of the step
-      int nt, mt, z, sp, d_nt, d_mt, d_z, d_sp;
-      {
-        int r = w_first;
-        sp = r / per_split; r -= sp * per_split;
-        z = r / tiles_per_z; r -= z * tiles_per_z;
-        mt = r / p.n_tiles; nt = r - mt * p.n_tiles;
-        r = w_step;
-        d_sp = r / per_split; r -= d_sp * per_split;
-        d_z = r / tiles_per_z; r -= d_z * tiles_per_z;
-        d_mt = r / p.n_tiles; d_nt = r - d_mt * p.n_tiles;
-      }
-      auto advance = [&](int& nt_, int& mt_, int& z_, int& sp_) {
-        nt_ += d_nt;
-        int c = nt_ >= p.n_tiles ? 1 : 0;
-        nt_ -= c ? p.n_tiles : 0;
-        mt_ += d_mt + c;
-        c = mt_ >= m_tiles ? 1 : 0;
-        mt_ -= c ? m_tiles : 0;
-        z_ += d_z + c;
-        c = z_ >= p.batch ? 1 : 0;
-        z_ -= c ? p.batch : 0;
-        sp_ += d_sp + c;
-      };
       // This warp's i-th chunk, in units of 32 columns.  The two warps of a quarter interleave
-      // their chunks; with tile stores they interleave pairs of chunks, so that a warp owns whole
+      // their chunks; with tile stores of bf16 they interleave pairs of chunks, so that a warp owns whole
       // 64-column (128-byte) groups.
-      const bool tma_out = p.tma_store != 0;
-      auto ccol = [&](int i) { return tma_out ? 2 * (hsel + 2 * (i >> 1)) + (i & 1) : hsel + 2 * i; };
+      const bool tma_out = p.tma_store != 0, tma_pairs = tma_out && kMode != EPI_F32;
+      auto ccol = [&](int i) { return tma_pairs ? 2 * (hsel + 2 * (i >> 1)) + (i & 1) : hsel + 2 * i; };
       const uint32_t stg_tile = smem_u32(stg);
       // bias values of this warp's columns of tile `nt_`, one value per lane and chunk
       auto fetch_bias = [&](int nt_, float (&b)[4]) {
@@ -543,23 +598,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           b[i] = (ccol(i) * 32 < p.bn && p.bias && n < p.N) ? p.bias[n] : 0.f;
         }
       };
-      float bnext[4];
-      if (w_first < total_work && !tma_out) {
-        fetch_bias(nt, bnext);
-#pragma unroll
-        for (int i = 0; i < 4; i++) bias_s[i * 32 + lane] = bnext[i];
-        __syncwarp();
-      }
+      // Every lane holds one column's value of each chunk, fetched while the tile is still multiplied; a chunk's 32 values go through
+      // shared memory when its turn comes (read from memory there they cost a chunk 300 to 600 cycles).
+      float bcur[4] = {0.f, 0.f, 0.f, 0.f};
+      if (p.early && w_first < total_work) fetch_bias(at.nt, bcur);
+      begin();
+      if (!p.early && w_first < total_work) fetch_bias(at.nt, bcur);
       for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
-        const int zo = p.hdiv == 1 ? z : z / p.hdiv, zi = p.hdiv == 1 ? 0 : z - zo * p.hdiv;
+        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
         const uint32_t acc = tile & 1, use = tile >> 1;
-        const int m_warp = mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
+        const int m_warp = at.mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
         const int m = m_warp + lane;
         const bool row_ok = m < p.M;
         const long long zoff = zo * p.d_bo + zi * p.d_bi;
         const long long off0 = zoff + (long long)m * p.ldd;
-        const int n_base = nt * p.bn;
-        const float* bias_t = bias_s + (tile & 1) * 128;
+        const int n_base = at.nt * p.bn;
         const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 256;
         auto chunk_n0 = [&](int i) { return n_base + ccol(i) * 32; };
         auto chunk_ok = [&](int i) { return ccol(i) * 32 < p.bn && chunk_n0(i) < p.N; };
@@ -576,8 +629,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         };
         // the next work item and its bias (the loads travel while this tile is worked on)
-        int nt2 = nt, mt2 = mt, z2 = z, sp2 = sp;
-        advance(nt2, mt2, z2, sp2);
+        at.advance(p.n_tiles, m_tiles, p.batch);
+        const int nt2 = at.nt, mt2 = at.mt, z2 = at.z;
         if constexpr (kHasXf) {
           // the next tile's rows of the extra operand start on their way to L2: they come from memory where
           // the operand is as large as the output.  This, the accumulator reads issued early and the interleaved
@@ -594,8 +647,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                               nt2 * p.bn, cols * 2);
           }
         }
-        const bool more = w + w_step < total_work && !tma_out;  // (of interest to the bias hand-over only)
-        if (more) fetch_bias(nt2, bnext);
         uint4 x[4];
         const bool c0ok = chunk_ok(0);
         if (c0ok) prefetch_x(0, x);
@@ -604,7 +655,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         auto release_acc = [&]() {  // every TMEM read of this tile has returned
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) {
+          // nobody waits for the last use of an accumulator, and no arrival may be under way when a CTA leaves
+          if (lane == 0 && w + 2 * w_step < total_work) {
             if (kPair && !leader) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty_bar[acc]), 0));
             else mbar_arrive(smem_u32(&tempty_bar[acc]));
           }
@@ -621,31 +673,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const uint4(&xu)[4] = kMode == EPI_DGELU ? x : xc;
           auto x_used = [&]() { if (has_next) prefetch_x(i + 1, x); };
           const int n0 = chunk_n0(i);
-          if (tma_out) {
-            // an even chunk opens a 64-column group, an odd chunk, or the last one, closes it
-            // The staging buffer holds the output tile, so the chunk's bias comes straight from
-            // global memory (32 floats that every lane reads alike: one L1 line), or, for a
-            // ragged chunk or no bias at all, from 32 floats of scratch.
-            const float* bias_c = p.bias + n0;
-            if (!p.bias || n0 + 32 > p.N) {
-              __syncwarp();
-              bias_r[lane] = (p.bias && n0 + lane < p.N) ? p.bias[n0 + lane] : 0.f;
-              __syncwarp();
-              bias_c = bias_r;
+          const float* bias_c = nullptr;
+          if (p.bias) {
+            __syncwarp();
+            bias_r[lane] = i == 0 ? bcur[0] : i == 1 ? bcur[1] : i == 2 ? bcur[2] : bcur[3];
+            __syncwarp();
+            bias_c = bias_r;
+          }
+          // a chunk of fp32 whose last 16-byte piece would reach beyond the row goes the other way
+          const bool through_tile = tma_out && (kMode != EPI_F32 || n0 + 32 <= p.N || p.N % 4 == 0);
+          epi_chunk<kMode>(p, a, xu, bias_c, stg, lane, zoff, m_warp, n0, p.direct && (tma_pairs || n0 + 32 <= p.N),
+                           through_tile ? stg_tile : 0, i & 1, loaded, x_used);  // warp-uniform
+          // an even chunk of bf16 opens a 64-column group, an odd chunk, or the last one, closes it
+          if (through_tile && (kMode == EPI_F32 || (i & 1) || !has_next)) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (m_warp < p.M && elect_one()) {
+              auto slot = [&](int sl) { return p.d_perm[0] == sl ? m_warp : (p.d_perm[1] == sl ? zi : zo); };
+              if (kMode != EPI_F32) tma_store_4d(&tmD, stg_tile, n0 - (i & 1) * 32, slot(1), slot(2), slot(3));
+              else if (p.accumulate) tma_add_4d(&tmD, stg_tile, n0, slot(1), slot(2), slot(3));
+              else tma_store_4d(&tmD, stg_tile, n0, slot(1), slot(2), slot(3));
             }
-            epi_chunk<kMode>(p, a, xu, bias_c, stg, lane, zoff, m_warp, n0, p.direct != 0, stg_tile, i & 1,
-                             loaded, x_used);
-            if ((i & 1) || !has_next) {
-              fence_proxy_async_smem();
-              __syncwarp();
-              if (lane == 0 && m_warp < p.M) {
-                auto slot = [&](int sl) { return p.d_perm[0] == sl ? m_warp : (p.d_perm[1] == sl ? zi : zo); };
-                tma_store_4d(&tmD, stg_tile, n0 - (i & 1) * 32, slot(1), slot(2), slot(3));
-              }
-            }
-          } else {
-            epi_chunk<kMode>(p, a, xu, bias_t + i * 32, stg, lane, zoff, m_warp, n0, p.direct && n0 + 32 <= p.N, 0, 0,
-                             loaded, x_used);  // warp-uniform
           }
         };
         if (c0ok && (kHasXf || kMode == EPI_GELU_AUX)) {
@@ -678,21 +726,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         } else {
           release_acc();
         }
-        if (more) {
-          float* bias_n = bias_s + ((tile + 1) & 1) * 128;
-#pragma unroll
-          for (int i = 0; i < 4; i++) bias_n[i * 32 + lane] = bnext[i];
-          __syncwarp();
-        }
-        nt = nt2; mt = mt2; z = z2; sp = sp2;
+        if (w + w_step < total_work) fetch_bias(nt2, bcur);
       }
-    } else
+    } else {
+    begin();
     for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
-      const int split = w / per_split;
-      int r = w - split * per_split;
-      const int z = r / tiles_per_z;
-      r -= z * tiles_per_z;
-      const int mt = r / p.n_tiles, nt = r - mt * p.n_tiles;
+      const int z = at.z, mt = at.mt, nt = at.nt;
+      at.advance(p.n_tiles, m_tiles, p.batch);
       const int zo = z / p.hdiv, zi = z - zo * p.hdiv;
       const uint32_t acc = tile & 1, use = tile >> 1;
       const int m_warp = mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
@@ -800,7 +840,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       auto release_acc = [&]() {  // every TMEM read of this tile has returned
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) {
+        if (lane == 0 && w + 2 * w_step < total_work) {
           if (kPair && !leader) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty_bar[acc]), 0));
           else mbar_arrive(smem_u32(&tempty_bar[acc]));
         }
@@ -916,13 +956,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       }
     }
-    // tile stores read this CTA's shared memory: they end before the CTA does
-    if (p.tma_store && lane == 0) tma_store_wait_all();
+    }
+    // tile stores have read this CTA's shared memory before it leaves
+    if (p.tma_store && elect_one()) tma_store_wait_read();
   }
 
   tc_fence_before();
   __syncthreads();
-  if (kPair) cluster_sync_all();  // neither CTA frees tensor memory while the other may still use it
+  if (kPair) cluster_sync_exit();  // neither CTA frees tensor memory while the other may still use it
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
@@ -1088,6 +1129,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.seq_lens = d.seq_lens;
   p.rows = rows;
   p.rows_are_k = rows_are_k;
+  p.early = b_static && !starve ? 1 : 0;
   p.wait_limit = WAIT_LIMIT_CYCLES;
   if (starve) {  // armed by mslt_debug_starve_next_gemm
     p.starve = 1;
@@ -1128,12 +1170,13 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   MapVal md;
   md.map = ma.map;
   p.tma_store = 0;
-  if ((mode == EPI_STORE || mode == EPI_RESIDUAL || mode == EPI_GELU || mode == EPI_DGELU ||
-       (mode == EPI_GELU_AUX && p.direct && d.N % 32 == 0)) &&
-      p.bn >= 128 && p.vec_ok && d.N % 8 == 0 &&  // a tile store was seen to write whole 16-byte pieces
-      g_store_variant.load() != 1) {
+  if ((((mode == EPI_STORE || mode == EPI_RESIDUAL || mode == EPI_GELU || mode == EPI_DGELU ||
+         (mode == EPI_GELU_AUX && p.direct && d.N % 32 == 0)) &&
+        p.bn >= 128 && d.N % 8 == 0) ||  // a tile store was seen to write whole 16-byte pieces
+       (mode == EPI_F32 && d.N >= 32)) &&
+      p.vec_ok && g_store_variant.load() != 1) {
     char ignored[256];
-    if (get_map(d.D, d.M, d.N, d.ldd, 1, d.d_bo, d.d_bi, d.hdiv, nb, 32, &md, ignored) == 0) {
+    if (get_map(d.D, d.M, d.N, d.ldd, 1, d.d_bo, d.d_bi, d.hdiv, nb, 32, &md, ignored, mode == EPI_F32) == 0) {
       p.tma_store = 1;
       for (int i = 0; i < 3; i++) p.d_perm[i] = md.perm[i];
     } else {

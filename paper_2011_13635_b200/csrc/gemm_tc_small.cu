@@ -47,6 +47,10 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const int rank = blockIdx.x % SPLITS, nt = blockIdx.x / SPLITS;
   const int m0 = blockIdx.y * BM, n0 = nt * TS_BN;
   const int kb0 = min(p.kb_total, rank * p.kb_per_split), n_kb = min(p.kb_total, kb0 + p.kb_per_split) - kb0;
+  if (warp == 2 && elect_one()) {
+    prefetch_map(&tmA);
+    prefetch_map(&tmB);
+  }
   if (threadIdx.x == 0) {
     for (int r = 0; r < TS_ROUNDS; r++) {
       mbar_init(smem_u32(&full_bar[r]), 1);
@@ -91,7 +95,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     auto load_b = [&](int r) {
       const int slot = r % TS_ROUNDS;
       const uint32_t fb = smem_u32(&full_bar[slot]);
-      mbar_expect_tx(fb, TS_STAGE);
+      mbar_expect_more(fb, TS_STAGE - A_STAGE_BYTES);
       int c[4] = {0, 0, 0, 0};
       if (p.b_mn) { c[0] = n0; c[p.b_perm] = (kb0 + r) * BK; } else { c[0] = (kb0 + r) * BK; c[p.b_perm] = n0; }
       tma_load_4d(smem_u32(smem) + slot * TS_STAGE + A_STAGE_BYTES, &tmB, fb, c[0], c[1], c[2], c[3]);
@@ -108,6 +112,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int slot = r % TS_ROUNDS;
         if (r >= TS_ROUNDS && !mbar_wait(smem_u32(&empty_bar[slot]), (r / TS_ROUNDS - 1) & 1, abort_flag, p.status)) { ok = false; break; }
         if (r >= n_early) load_b(r);
+        mbar_expect_tx(smem_u32(&full_bar[slot]), A_STAGE_BYTES);
         for (int h = 0; h < (p.a_mn ? 2 : 1); h++) {
           int c[4] = {0, 0, 0, 0};
           if (p.a_mn) { c[0] = m0 + h * 64; c[p.a_perm] = (kb0 + r) * BK; } else { c[0] = (kb0 + r) * BK; c[p.a_perm] = m0; }
@@ -119,6 +124,11 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         while (now_cycles() - t0 < 4000000ll) {}
       }
     }
+    if (mine && !active)  // beyond the rows that exist: the early tiles land before the block leaves
+      for (int r = 0; r < n_early; r++) {
+        mbar_arrive(smem_u32(&full_bar[r]));
+        if (!mbar_wait(smem_u32(&full_bar[r]), 0, abort_flag, p.status)) break;
+      }
     __syncwarp();
     if (active) load_extra(threadIdx.x);
   } else {
@@ -236,7 +246,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     pack(out);
     *reinterpret_cast<uint4*>((bf16*)d.D + o) = out;
   }
-  if (SPLITS > 1) cluster_sync_all();  // no block leaves while its tile is read
+  if (SPLITS > 1) cluster_sync_exit();  // no block leaves while its tile is read
 }
 
 typedef void (*TcSmallFn)(const CUtensorMap, const CUtensorMap, const TcSmallParams);
@@ -294,7 +304,7 @@ int gemm_tc_small_launch(const mslt_gemm_desc& d, int splits, bool early, int* s
   p.splits = splits;
   p.kb_total = (d.K + BK - 1) / BK;
   p.kb_per_split = (p.kb_total + splits - 1) / splits;
-  p.early = early && !rows && !starve ? 1 : 0;
+  p.early = early && !starve ? 1 : 0;
   p.rows = rows;
   p.starve = starve ? 1 : 0;
   p.wait_limit = starve ? 40000000ll : WAIT_LIMIT_CYCLES;

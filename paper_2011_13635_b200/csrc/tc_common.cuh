@@ -55,6 +55,10 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+// more bytes for the barrier's phase to wait for, without an arrival
+__device__ __forceinline__ void mbar_expect_more(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -87,6 +91,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
   }
 }
+// Brings a tensor map to the copy engine, which would fetch it at the first copy through it otherwise.  Called
+// before pdl_begin (a map is a kernel parameter, nobody writes it), the fetch hides behind the preceding kernel.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
                                             int c1, int c2, int c3) {
   asm volatile(
@@ -104,9 +113,15 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t sr
                : "memory");
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
+// the same, added to what is there (fp32)
+__device__ __forceinline__ void tma_add_4d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.reduce.async.bulk.tensor.4d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+               ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
 // the issuing thread's tile stores have all read their shared memory / have all completed
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // makes this thread's shared-memory writes visible to the copy engine
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // ---- CTA-pair (cta_group::2) forms: the two CTAs of a cluster work on one 256-row tile ----
@@ -123,6 +138,11 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank) {
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// The last meeting of a cluster, before its blocks leave: it orders no memory, so it need not wait for the stores
+// and reductions on their way (the releasing form took 1.2 us at the end of every launch).
+__device__ __forceinline__ void cluster_sync_exit() {
+  asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait;" ::: "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -431,7 +451,7 @@ EncodeTiledFn get_encode() {
 struct MapKey {
   const void* ptr;
   long long rows, K, rs, ks, bo, bi;
-  int hdiv, nb, box_rows;
+  int hdiv, nb, box_rows, f32;
   bool operator==(const MapKey& o) const { return memcmp(this, &o, sizeof(MapKey)) == 0; }
 };
 struct MapKeyHash {
@@ -449,15 +469,16 @@ struct MapVal {
 
 // Builds (or fetches) the rank-4 tensor map of one operand: dim 0 is the contiguous index (k for a
 // K-major operand, the row index otherwise); the other matrix index and the two batch indices
-// follow in order of increasing stride.
+// follow in order of increasing stride.  Boxes are 128 bytes of dim 0 wide: 64 bf16, or 32 fp32 with f32.
 int get_map(const void* ptr, long long rows, long long K, long long rs, long long ks, long long bo,
-            long long bi, int hdiv, int nb, int box_rows, MapVal* out, char* err) {
+            long long bi, int hdiv, int nb, int box_rows, MapVal* out, char* err, bool f32 = false) {
   static std::unordered_map<MapKey, MapVal, MapKeyHash> cache;
   static std::mutex mu;
   MapKey key;
   memset(&key, 0, sizeof(key));
   key.ptr = ptr; key.rows = rows; key.K = K; key.rs = rs; key.ks = ks; key.bo = bo; key.bi = bi;
   key.hdiv = hdiv; key.nb = nb; key.box_rows = box_rows;
+  key.f32 = f32;
   std::lock_guard<std::mutex> lock(mu);
   auto itf = cache.find(key);
   if (itf != cache.end()) { *out = itf->second; return 0; }
@@ -481,13 +502,13 @@ int get_map(const void* ptr, long long rows, long long K, long long rs, long lon
   cuuint64_t gdim[4], gstr[3];
   cuuint32_t bdim[4], estr[4] = {1, 1, 1, 1};
   gdim[0] = (cuuint64_t)ext0;
-  bdim[0] = 64;
+  bdim[0] = f32 ? 32 : 64;
   long long last = 16;
   for (int sl = 0; sl < 3; sl++) {
     const int li = order[sl];
     gdim[sl + 1] = (cuuint64_t)ext[li];
     bdim[sl + 1] = box[li];
-    long long sb = eff(li) == big ? last : str[li] * 2;
+    long long sb = eff(li) == big ? last : str[li] * (f32 ? 4 : 2);
     if (sb <= 0 || sb % 16) {
       snprintf(err, 256, "gemm: operand stride %lld bytes is not a positive multiple of 16", sb);
       return MSLT_ERR_ARG;
@@ -497,7 +518,7 @@ int get_map(const void* ptr, long long rows, long long K, long long rs, long lon
     out->perm[li] = sl + 1;
   }
   if ((uintptr_t)ptr & 15) { snprintf(err, 256, "gemm: operand base is not 16-byte aligned"); return MSLT_ERR_ARG; }
-  CUresult r = enc(&out->map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), gdim, gstr, bdim,
+  CUresult r = enc(&out->map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), gdim, gstr, bdim,
                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {

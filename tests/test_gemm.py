@@ -148,6 +148,21 @@ def test_bf16_epilogues_over_several_wide_tiles(variant):
         Bd.lib.mslt_debug_set_gemm_variant(0)
 
 
+@pytest.mark.parametrize("variant", [0, 1, 2, 4], ids=["auto", "single", "pair", "auto-rowstores"])
+@pytest.mark.parametrize("shape", [(33, 36, 64), (1, 32, 72), (257, 60, 136), (300, 1037, 192), (130, 1022, 200), (520, 768, 392)])
+def test_bf16_operands_with_fp32_output(shape, variant):
+    """fp32 outputs, stored and added to what is there, at row and column counts where the 32 x 32 tiles that leave
+    through the copy engine end inside the output, or inside a 16-byte piece of it."""
+    from paper_2011_13635_b200 import binding as Bd
+    assert Bd.lib.mslt_debug_set_gemm_variant(variant) == 0
+    try:
+        _run(1, *shape, "k", "k", bias=True, d_fp32=True)
+        _run(1, *shape, "mn", "mn", d_fp32=True, accumulate=True)
+        _run(1, *shape, "k", "mn", d_fp32=True, accumulate=True, split_k=2, alpha=0.5)
+    finally:
+        Bd.lib.mslt_debug_set_gemm_variant(0)
+
+
 def test_bf16_long_contraction_split_k():
     """Weight-gradient shape: small output, long contraction, partial sums added in fp32."""
     _run(1, 768, 256, 4096, "mn", "mn", d_fp32=True, accumulate=True)

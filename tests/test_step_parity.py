@@ -236,6 +236,16 @@ def test_fp32_attention_row_lengths(seq, varlen):
     _run(cfg, steps=2, lr=1e-3)
 
 
+@pytest.mark.parametrize("batch,rest", [(32, 1), (32, 9), (4, 8)])
+def test_packed_batch_of_few_rows(batch, rest):
+    """Sequences far shorter than the batch is wide: most blocks of a launch find no rows left for them, after they
+    have asked for their first weights."""
+    cfg = I.scaled(I.CONFIGS["base_stage"], layers=2, trainable=1, batch=batch, varlen=(1, 128))
+    m, oracle = PT.build_pair(cfg, lr=1e-4)
+    PT.compare_step(m, oracle, cfg, _batch_of_lengths(cfg, (40,) + (rest,) * (batch - 1)), PT.TOL["bf16"])
+    m.close()
+
+
 @pytest.mark.parametrize("dtype,seq,varlen,pred", [("fp32", 40, None, 5), ("fp32", 72, (20, 72), 33), ("bf16", 136, (40, 136), 9),
                                                    ("bf16", 64, None, 40)])
 def test_slots_that_name_a_position_twice(dtype, seq, varlen, pred):
