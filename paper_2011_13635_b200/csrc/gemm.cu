@@ -15,17 +15,18 @@ int64_t gemm_launches() { return g_launches.load(); }
 thread_local GemmForm g_gemm_form;
 
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
-                bool b_static) {
+                bool b_static, int* parts) {
   if ((d.a_rs != 1 && d.a_ks != 1) || (d.b_rs != 1 && d.b_ks != 1)) {
     snprintf(err, 256, "gemm: each operand needs one unit stride");
     return MSLT_ERR_ARG;
   }
   int rc;
+  if (parts) *parts = 1;
   if (d.dtype == 1) {
     // MSLT_BF16_CUDA_CORES=1 routes bf16 products to the CUDA-core kernel: a debugging aid for
     // telling a tensor-core kernel fault from an orchestration fault, never a silent fallback.
     static const bool cuda_cores = getenv("MSLT_BF16_CUDA_CORES") && atoi(getenv("MSLT_BF16_CUDA_CORES")) == 1;
-    rc = cuda_cores ? gemm_simt_launch(d, st, err) : gemm_tc_launch(d, status, st, err, rows, rows_are_k, b_static);
+    rc = cuda_cores ? gemm_simt_launch(d, st, err) : gemm_tc_launch(d, status, st, err, rows, rows_are_k, b_static, parts);
   } else if (d.dtype == 0) {
     rc = gemm_f32_launch(d, st, err);
   } else {

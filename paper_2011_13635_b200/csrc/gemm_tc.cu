@@ -48,6 +48,7 @@ struct TcParams {
   int a_perm[3], b_perm[3];  // slot (1..3) of the (outer, inner-batch, outer-batch) coordinates
   char* D;
   long long ldd, d_bo, d_bi;
+  long long part;       // distance of the results of two splits, 0 where they add to one
   int d_fp32, accumulate, vec_ok;
   int x32;              // rows of the extra operand start on 32 bytes
   int direct;           // rows of D (and aux) may be stored straight from registers, 32 bytes at a time
@@ -605,12 +606,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       begin();
       if (!p.early && w_first < total_work) fetch_bias(at.nt, bcur);
       for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
-        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
+        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = p.part ? at.sp : p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
         const uint32_t acc = tile & 1, use = tile >> 1;
         const int m_warp = at.mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
         const int m = m_warp + lane;
         const bool row_ok = m < p.M;
-        const long long zoff = zo * p.d_bo + zi * p.d_bi;
+        const long long zoff = zo * p.d_bo + zi * (p.part ? p.part : p.d_bi);
         const long long off0 = zoff + (long long)m * p.ldd;
         const int n_base = at.nt * p.bn;
         const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 256;
@@ -1009,7 +1010,7 @@ std::mutex g_dev_mu;
 //   an epilogue that overlaps the next tile's loop, one more at the end;
 //   start-up (pairs have a cluster to set up); singles slow down a little when many waves of them
 //   contend for L2, where a pair fetches a third less per flop.
-static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, bool can_split, bool* pair, int* bn,
+static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, int max_splits, bool* pair, int* bn,
                           int* ksub, int* splits) {
   struct Form { bool pair; int bn, ksub; double per_k; };
   static const Form forms[] = {{false, 64, 2, 0.202}, {false, 128, 2, 0.280}, {false, 192, 1, 0.362}, {false, 256, 1, 0.413},
@@ -1033,7 +1034,7 @@ static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, b
     const int rows = f.pair ? 2 * BM : BM, units = f.pair ? num_sms / 2 : num_sms;
     const long long tiles = (long long)((d.M + rows - 1) / rows) * ((d.N + f.bn - 1) / f.bn) * d.batch;
     const double epi = e0 + e1 * f.bn / 256.;
-    for (int sp = fixed_splits; sp == fixed_splits || (can_split && sp <= 16 && sp * 4 <= kblocks); sp++) {
+    for (int sp = fixed_splits; sp == fixed_splits || (sp <= max_splits && sp * 4 <= kblocks); sp++) {
       const double waves = (double)((tiles * sp + units - 1) / units);
       const int kb = ((kblocks + sp - 1) / sp + ks - 1) / ks * ks;
       const double loop = kb * f.per_k + 0.66;
@@ -1046,7 +1047,7 @@ static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, b
 }
 
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
-                   bool b_static) {
+                   bool b_static, int* parts) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_starve_next.exchange(0) != 0;
   int dev = 0;
@@ -1066,7 +1067,11 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const int num_sms = di.num_sms, smem_optin = di.smem_optin;
   if (!status) { snprintf(err, 256, "gemm: the tensor-core kernel needs a device status word"); return MSLT_ERR_ARG; }
   // every argument check comes before a form is chosen: there is none for an epilogue that does not exist
-  if (d.split_k > 1 && !(d.d_fp32 && d.accumulate)) {
+  if (parts && (!d.d_fp32 || d.accumulate || d.batch != 1 || d.split_k > kMaxParts)) {
+    snprintf(err, 256, "gemm: results by split need one fp32 output that is not accumulated");
+    return MSLT_ERR_ARG;
+  }
+  if (d.split_k > 1 && !(d.d_fp32 && (d.accumulate || parts))) {
     snprintf(err, 256, "gemm: split_k needs an fp32 accumulating output");
     return MSLT_ERR_ARG;
   }
@@ -1081,10 +1086,10 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.a_mn = (d.a_rs == 1 && d.a_ks != 1) ? 1 : 0;
   p.b_mn = (d.b_rs == 1 && d.b_ks != 1) ? 1 : 0;
   const int variant = g_tile_variant.load();
-  const bool can_split = d.split_k == 0 && d.d_fp32 && d.accumulate;
+  const int max_splits = d.split_k != 0 || !d.d_fp32 ? 0 : d.accumulate ? 16 : parts ? kMaxParts : 0;
   bool pair = false;
   int splits = d.split_k > 1 ? d.split_k : 1, ksub = 1;
-  const double estimate = choose_tiling(d, num_sms, variant, can_split, &pair, &p.bn, &ksub, &splits);
+  const double estimate = choose_tiling(d, num_sms, variant, max_splits, &pair, &p.bn, &ksub, &splits);
   double t_small = 0.;
   const int s_small = variant == 0 && g_store_variant.load() == 0 && !rows_are_k ? gemm_tc_small_plan(d, num_sms, &t_small) : 0;
   if (s_small && t_small < estimate) return gemm_tc_small_launch(d, s_small, b_static, status, st, err, rows, starve);
@@ -1101,6 +1106,10 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.kb_per_split = ((d.K + 2 * BK - 1) / (2 * BK) + splits - 1) / splits * (2 / ksub);
   p.splits = (p.kb_total + p.kb_per_split - 1) / p.kb_per_split;
   g_gemm_form = {1, tile_m, p.bn, ksub, p.splits};
+  if (parts) {
+    *parts = p.splits;
+    p.part = (long long)d.M * d.ldd;
+  }
   const long long total = tiles * p.splits;
   if (total > 0x7fffffffll) { snprintf(err, 256, "gemm: too many tiles"); return MSLT_ERR_SIZE; }
   p.total_work = (int)total;
@@ -1176,7 +1185,9 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
        (mode == EPI_F32 && d.N >= 32)) &&
       p.vec_ok && g_store_variant.load() != 1) {
     char ignored[256];
-    if (get_map(d.D, d.M, d.N, d.ldd, 1, d.d_bo, d.d_bi, d.hdiv, nb, 32, &md, ignored, mode == EPI_F32) == 0) {
+    // the results of the splits are addressed like a batch
+    if (get_map(d.D, d.M, d.N, d.ldd, 1, d.d_bo, parts ? p.part : d.d_bi, parts ? p.splits : d.hdiv, nb, 32, &md, ignored,
+                mode == EPI_F32) == 0) {
       p.tma_store = 1;
       for (int i = 0; i < 3; i++) p.d_perm[i] = md.perm[i];
     } else {

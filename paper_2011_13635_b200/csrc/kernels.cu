@@ -1604,6 +1604,27 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ src, bf16* __restri
     dst[i] = __float2bfloat16_rn(src[i]);
 }
 
+// out = the sum of `parts` fp32 arrays of n elements (`stride` apart), added in their order and rounded once.
+// The gradient of the head's transform is a sum over the whole vocabulary, split over the machine; added by atomics
+// its rounding, and with it every gradient below, differed from run to run.  2560 x 768 in seven parts: 10.9 us.
+__global__ void __launch_bounds__(256)
+sum_parts_kernel(const float* __restrict__ src, int64_t stride, int parts, bf16* __restrict__ dst, int64_t n) {
+  pdl_begin();
+  const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
+  if (i >= n) return;  // n is a multiple of 4
+  float4 s = *reinterpret_cast<const float4*>(src + i);
+#pragma unroll 4
+  for (int k = 1; k < parts; k++) {
+    const float4 t = *reinterpret_cast<const float4*>(src + k * stride + i);
+    s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+  }
+  uint2 o;
+  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
+  h[0] = __floats2bfloat162_rn(s.x, s.y);
+  h[1] = __floats2bfloat162_rn(s.z, s.w);
+  *reinterpret_cast<uint2*>(dst + i) = o;
+}
+
 // ---------------------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------------------
@@ -1841,6 +1862,10 @@ void launch_type_grad(bool bf, const void* dz, const int* segments, float* dtype
                      (const T*)dz, segments, dtype, rows, H, rpb, rows_dev)));
 }
 
+void launch_sum_parts(const float* src, int64_t stride, int parts, void* dst, int64_t n, cudaStream_t st) {
+  if (n <= 0) return;
+  launch_pdl(sum_parts_kernel, div_up(n, 1024), 256, 0, st, src, stride, parts, (bf16*)dst, n);
+}
 void launch_f32_to_bf16(const float* src, void* dst, int64_t n, cudaStream_t st) {
   if (n <= 0) return;
   int blocks = (int)std::min<int64_t>((n + 255) / 256, 148 * 8);

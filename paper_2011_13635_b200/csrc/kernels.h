@@ -120,6 +120,7 @@ void launch_type_grad(bool bf, const void* dz, const int* segments, float* dtype
                       cudaStream_t st, const int* rows_dev = nullptr);
 // data-parallel steps: the loss normaliser becomes 1 / *total_valid (0 when that count is 0)
 void launch_override_inv_n(const int* total_valid, float* inv_n, cudaStream_t st);
+void launch_sum_parts(const float* src, int64_t stride, int parts, void* dst, int64_t n, cudaStream_t st);
 void launch_f32_to_bf16(const float* src, void* dst, int64_t n, cudaStream_t st);
 
 }  // namespace mslt

@@ -309,7 +309,7 @@ void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char
   w.dlogits = take(R * Vp * E);
   w.nll = (float*)take(R * 4);
   w.dtm = take(R * H * E); w.dgt = take(R * H * E); w.dhm = take(R * H * E);
-  w.dtm32 = (float*)take(R * H * 4);
+  w.dtm32 = (float*)take(R * H * 4 * (a.dtype == 1 ? kMaxParts : 1));
   if (a.nsp) {
     const int64_t Bm = a.max_batch;
     w.nsp_rowsrc = (int*)take(Bm * 4);
@@ -485,7 +485,7 @@ int run_gemm_x3(mslt_ctx* c, const mslt_gemm_desc& d, bool reuse_a, bool b_is_em
 }
 
 int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, int rows_are_k = 0, bool reuse_a = false,
-             bool b_is_emb = false, bool b_static = false, bool views = false) {
+             bool b_is_emb = false, bool b_static = false, bool views = false, int* parts = nullptr) {
   if (d.M <= 0 || d.N <= 0 || d.K <= 0 || d.batch <= 0) return 0;
   char err[256] = "";
   const int64_t before = gemm_launches();
@@ -495,7 +495,7 @@ int run_gemm(mslt_ctx* c, const mslt_gemm_desc& d, const int* rows = nullptr, in
   bool done = false;
   if (!c->bf && !views) rc = run_gemm_x3(c, d, reuse_a, b_is_emb, &done);
   if (rc) return rc;
-  if (!done) rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k, b_static);
+  if (!done) rc = gemm_launch(d, c->ws.scalars, c->st, err, rows ? rows + 1 : nullptr, rows_are_k, b_static, parts);
   if (prof) {
     cudaEventRecord(c->pev[2 * c->prec.size() + 1], c->st);
     c->prec.push_back({d.batch > 1 ? 1 : 0, 2.0 * d.M * d.N * (double)d.K * d.batch});
@@ -713,7 +713,7 @@ int dtm_splits(const mslt_ctx* c, int R) {
   const long long tiles = (long long)((R + 255) / 256) * ((H + 255) / 256), units = c->num_sms / 2;
   int splits = 1;
   double best = 0.;
-  for (int sp = 1; sp <= 16 && sp * 256 <= V; sp++) {
+  for (int sp = 1; sp <= kMaxParts && sp * 256 <= V; sp++) {
     if (sp > 1 && tiles >= 2 * units) break;
     const long long waves = (tiles * sp + units - 1) / units;
     const double e = (double)(tiles * sp) / (double)(waves * units);
@@ -732,11 +732,12 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
     g.d.B = Wc(c, toff(c, -1, "emb.word")); g.d.b_rs = 1; g.d.b_ks = H;
     if (c->bf) {
       // few output tiles, a contraction over the whole vocabulary: split it across the machine
-      // with fp32 partial sums, then round once to bf16
-      g.d.D = w.dtm32; g.d.ldd = H; g.d.d_fp32 = 1; g.d.accumulate = 1;
+      // with fp32 partial sums, added in their order, then round once to bf16
+      g.d.D = w.dtm32; g.d.ldd = H; g.d.d_fp32 = 1;
       g.d.split_k = dtm_splits(c, R);
-      TRY(run_gemm(c, g.d));
-      KL(PC_OTHER, 6.0 * R * H, launch_f32_to_bf16(w.dtm32, w.dtm, (int64_t)R * H, c->st));
+      int parts = 1;
+      TRY(run_gemm(c, g.d, nullptr, 0, false, false, false, false, &parts));
+      KL(PC_OTHER, (4.0 * parts + 2.0) * R * H, launch_sum_parts(w.dtm32, (int64_t)R * H, parts, w.dtm, (int64_t)R * H, c->st));
     } else {
       g.d.D = w.dtm; g.d.ldd = H;
       TRY(run_gemm(c, g.d, nullptr, 0, false, true));
@@ -775,7 +776,6 @@ ZeroRanges step_zero_ranges(mslt_ctx* c, int T, int R) {
     z.add(c->grad + c->layer0_off + (int64_t)(first / group_of(c->a)) * c->layer_cnt,
           (int64_t)(c->top_k / group_of(c->a)) * c->layer_cnt * 4);
   z.add(c->grad + c->head_off, c->head_cnt * 4);
-  if (c->bf) z.add(w.dtm32, R * H * 4);
   z.add(w.norms, (int64_t)c->tensors.size() * 2 * 4);
   return z;
 }
