@@ -25,6 +25,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <string>
@@ -1089,9 +1090,16 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const int max_splits = d.split_k != 0 || !d.d_fp32 ? 0 : d.accumulate ? 16 : parts ? kMaxParts : 0;
   bool pair = false;
   int splits = d.split_k > 1 ? d.split_k : 1, ksub = 1;
-  const double estimate = choose_tiling(d, num_sms, variant, max_splits, &pair, &p.bn, &ksub, &splits);
+  // Where the row count is known on the device only, the form is chosen for part of what the launch has to reckon with:
+  // lengths between a quarter or a half of the longest and the longest leave 0.62 to 0.75 of a batch.
+  mslt_gemm_desc likely = d;
+  if (rows) {
+    int& n = rows_are_k ? likely.K : likely.M;
+    n = std::max(1, (int)(0.7 * n));
+  }
+  const double estimate = choose_tiling(likely, num_sms, variant, max_splits, &pair, &p.bn, &ksub, &splits);
   double t_small = 0.;
-  const int s_small = variant == 0 && g_store_variant.load() == 0 && !rows_are_k ? gemm_tc_small_plan(d, num_sms, &t_small) : 0;
+  const int s_small = variant == 0 && g_store_variant.load() == 0 && !rows_are_k ? gemm_tc_small_plan(likely, num_sms, &t_small) : 0;
   if (s_small && t_small < estimate) return gemm_tc_small_launch(d, s_small, b_static, status, st, err, rows, starve);
   const int tile_m = pair ? 2 * BM : BM;
   p.m_tiles = (d.M + tile_m - 1) / tile_m;
