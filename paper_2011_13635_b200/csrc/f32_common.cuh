@@ -10,12 +10,30 @@ namespace {
 struct F32Params {
   mslt_gemm_desc d;
   int splits, kb_per_split, n_tiles;
+  int early;    // B is not written by the kernels before this one: read ahead of the wait for them
   int vec_out;  // D, aux, residual and bias rows allow 16-byte access
 };
 
 __device__ __forceinline__ uint32_t f32_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int m, int n, float4 v4) {
+// What the epilogue reads beside the sums, for four columns of a row.  Where a thread has one piece of a small tile
+// (kLoaded) it asks for them ahead of the main loop; asked for at the end they add a trip to L2 to every launch.  Larger
+// tiles read them piece by piece (1 % of the split-operand kernel).
+struct Extra4 { float4 bias, aux, residual; };
+__device__ __forceinline__ Extra4 load_extra4(const F32Params& p, int64_t zoff, int m, int n) {
+  const mslt_gemm_desc& d = p.d;
+  Extra4 x;
+  x.bias = x.aux = x.residual = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!p.vec_out || m >= d.M || n + 4 > d.N) return x;
+  const int64_t o = zoff + (int64_t)m * d.ldd + n;
+  if (d.bias) x.bias = *reinterpret_cast<const float4*>(d.bias + n);
+  if (d.act == 2) x.aux = *reinterpret_cast<const float4*>((const float*)d.aux + o);
+  if (d.residual) x.residual = *reinterpret_cast<const float4*>((const float*)d.residual + o);
+  return x;
+}
+
+template <bool kLoaded>
+__device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int m, int n, float4 v4, const Extra4& x4) {
   const mslt_gemm_desc& d = p.d;
   if (m >= d.M || n >= d.N) return;
   const int64_t o = zoff + (int64_t)m * d.ldd + n;
@@ -23,7 +41,7 @@ __device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int 
   float* D = (float*)d.D;
   if (p.vec_out && n + 4 <= d.N) {
     if (d.bias) {
-      const float4 b = *reinterpret_cast<const float4*>(d.bias + n);
+      const float4 b = kLoaded ? x4.bias : *reinterpret_cast<const float4*>(d.bias + n);
       v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
     }
     if (d.act == 1) {
@@ -31,11 +49,11 @@ __device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int 
 #pragma unroll
       for (int e = 0; e < 4; e++) v[e] = gelu_f(v[e]);
     } else if (d.act == 2) {
-      const float4 u = *reinterpret_cast<const float4*>((const float*)d.aux + o);
+      const float4 u = kLoaded ? x4.aux : *reinterpret_cast<const float4*>((const float*)d.aux + o);
       v[0] *= gelu_grad_f(u.x); v[1] *= gelu_grad_f(u.y); v[2] *= gelu_grad_f(u.z); v[3] *= gelu_grad_f(u.w);
     }
     if (d.residual) {
-      const float4 r = *reinterpret_cast<const float4*>((const float*)d.residual + o);
+      const float4 r = kLoaded ? x4.residual : *reinterpret_cast<const float4*>((const float*)d.residual + o);
       v[0] += r.x; v[1] += r.y; v[2] += r.z; v[3] += r.w;
     }
     if (d.accumulate)
@@ -61,9 +79,14 @@ __device__ __forceinline__ void epilogue4(const F32Params& p, int64_t zoff, int 
 
 // Partial tiles [BMT][BNT] (rows PITCH floats apart) of the blocks of a cluster are added in rank order;
 // each block finishes its share of the rows.  A block may itself hold KG partial tiles, one after the
-// other.  Without a split the tile just leaves through the epilogue.
+// other.  Without a split the tile just leaves through the epilogue.  mine: load_extra4 of the thread's first piece (KG > 1).
+template <int BNT>
+__device__ __forceinline__ void first_piece(const F32Params& p, int rank, int share, int* r, int* c) {
+  *r = rank * share + (int)threadIdx.x / (BNT / 4);
+  *c = ((int)threadIdx.x % (BNT / 4)) * 4;
+}
 template <int BMT, int BNT, int NT, int PITCH = BNT, int KG = 1>
-__device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int rank, float* tile, int64_t zoff, int m0, int n0) {
+__device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int rank, float* tile, int64_t zoff, int m0, int n0, const Extra4& mine) {
   const uint32_t base = f32_smem(tile);
   if (p.splits == 1) __syncthreads();
   else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -71,6 +94,8 @@ __device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int r
   for (int idx = threadIdx.x; idx < share * (BNT / 4); idx += NT) {
     const int r = rank * share + idx / (BNT / 4), c = (idx % (BNT / 4)) * 4;
     const uint32_t at = base + (uint32_t)(r * PITCH + c) * 4u;
+    Extra4 x;
+    if (KG > 1) x = idx == (int)threadIdx.x ? mine : load_extra4(p, zoff, m0 + r, n0 + c);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (p.splits == 1) {
 #pragma unroll
@@ -90,10 +115,10 @@ __device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int r
         s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
       }
     }
-    epilogue4(p, zoff, m0 + r, n0 + c, s);
+    epilogue4<(KG > 1)>(p, zoff, m0 + r, n0 + c, s, x);
   }
-  // no block leaves while its tile is read
-  if (p.splits > 1) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  // no block leaves while its tile is read (nothing is ordered by this, so stores on their way do not hold it up)
+  if (p.splits > 1) asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait;" ::: "memory");
 }
 
 }  // namespace

@@ -28,7 +28,7 @@ int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err
     static const bool cuda_cores = getenv("MSLT_BF16_CUDA_CORES") && atoi(getenv("MSLT_BF16_CUDA_CORES")) == 1;
     rc = cuda_cores ? gemm_simt_launch(d, st, err) : gemm_tc_launch(d, status, st, err, rows, rows_are_k, b_static, parts);
   } else if (d.dtype == 0) {
-    rc = gemm_f32_launch(d, st, err);
+    rc = gemm_f32_launch(d, st, err, b_static);
   } else {
     snprintf(err, 256, "gemm: unknown dtype %d", d.dtype);
     return MSLT_ERR_ARG;

@@ -21,7 +21,7 @@ constexpr int kMaxParts = 8;
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows = nullptr,
                 int rows_are_k = 0, bool b_static = false, int* parts = nullptr);
 
-int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
+int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err, bool b_static);
 // The same on the tensor cores (gemm_f32x3.cu), for products without a batch: each operand has first been
 // split into three bf16 planes (launch_split3; n elements of the operand's storage, 6 n bytes of planes).
 // wide: device word, zeroed beforehand, that a split raises for a value the planes cannot stand for; the products

@@ -97,7 +97,6 @@ gemm_f32_kernel(const F32Params p) {
   constexpr int STAGE = (BMT + BNT) * FK;  // floats
   static_assert(KG * BMT * BNT <= STAGE * STAGES, "the partial tile reuses the ring");
   extern __shared__ __align__(128) float f32_ring[];
-  pdl_begin();
   const mslt_gemm_desc& d = p.d;
   const int rank = blockIdx.x % p.splits, nt = blockIdx.x / p.splits;
   const int z = blockIdx.z, zo = z / d.hdiv, zi = z - zo * d.hdiv;
@@ -116,17 +115,31 @@ gemm_f32_kernel(const F32Params p) {
   SliceLoader<BNT, NT, BMN, VEC> lb;
   la.init(A, d.a_rs, d.a_ks, m0, d.M, kb0 * FK, d.K);
   lb.init(B, d.b_rs, d.b_ks, n0, d.N, kb0 * FK, d.K);
+  // Weights are asked for ahead of the wait for the preceding kernel; they join the first slices' groups.
+  if (p.early) {
+#pragma unroll
+    for (int s = 0; s < STAGES - 1; s++)
+      if (kb0 + s < kb1) lb.load(ring + (uint32_t)s * STAGE * 4u + BMT * FK * 4u);
+  }
+  pdl_begin();
   auto issue = [&](int kb) {  // called once for every kb, in order
     if (kb < kb1) {
       const uint32_t st = ring + (uint32_t)((kb - kb0) % STAGES) * STAGE * 4u;
       la.load(st);
-      lb.load(st + BMT * FK * 4u);
+      if (!p.early || kb - kb0 >= STAGES - 1) lb.load(st + BMT * FK * 4u);
     }
     cp_commit();  // an empty group keeps the count of groups in step
   };
 #pragma unroll
   for (int s = 0; s < STAGES - 1; s++) issue(kb0 + s);
 
+  Extra4 mine = {};
+  if (KG > 1) {
+    int r, c;
+    const int share = BMT / p.splits;
+    first_piece<BNT>(p, rank, share, &r, &c);
+    if ((int)threadIdx.x < share * (BNT / 4)) mine = load_extra4(p, zoff, m0 + r, n0 + c);
+  }
   float2 acc[TM][TN / 2];  // pairs of neighbouring columns
 #pragma unroll
   for (int i = 0; i < TM; i++)
@@ -191,7 +204,7 @@ gemm_f32_kernel(const F32Params p) {
     for (int i = 0; i < TM; i++)
 #pragma unroll
       for (int h = 0; h < TN / 4; h++)
-        epilogue4(p, zoff, m0 + row_t + (i >> 2) * 16 + (i & 3), n0 + col_t + h * 32, out4(i, h));
+        epilogue4<false>(p, zoff, m0 + row_t + (i >> 2) * 16 + (i & 3), n0 + col_t + h * 32, out4(i, h), mine);
     return;
   }
   __syncthreads();
@@ -200,7 +213,7 @@ gemm_f32_kernel(const F32Params p) {
 #pragma unroll
     for (int h = 0; h < TN / 4; h++)
       *reinterpret_cast<float4*>(f32_ring + kg * BMT * BNT + (row_t + (i >> 2) * 16 + (i & 3)) * BNT + col_t + h * 32) = out4(i, h);
-  cluster_add_and_finish<BMT, BNT, NT, BNT, KG>(p, rank, f32_ring, zoff, m0, n0);
+  cluster_add_and_finish<BMT, BNT, NT, BNT, KG>(p, rank, f32_ring, zoff, m0, n0, mine);
 }
 
 typedef void (*F32Fn)(const F32Params);
@@ -221,7 +234,7 @@ std::mutex g_dev_mu;
 
 }  // namespace
 
-int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
+int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err, bool b_static) {
   if (d.act == 3) {
     snprintf(err, 256, "gemm: the softmax epilogue exists only in the tensor-core kernel");
     return MSLT_ERR_ARG;
@@ -249,6 +262,7 @@ int gemm_f32_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err) {
   p.d = d;
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
   auto m4 = [](int64_t v) { return v % 4 == 0; };
+  p.early = b_static ? 1 : 0;
   p.vec_out = al16(d.D) && al16(d.aux) && al16(d.residual) && al16(d.bias) && m4(d.ldd) &&
               (d.batch == 1 || (m4(d.d_bo) && m4(d.d_bi)));
   // Tile and split: the estimate below (SM cycles) reproduces the measured order of the choices on

@@ -238,7 +238,7 @@ gemm_f32x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * BN) : "memory");
   }
-  cluster_add_and_finish<BM, BN, X3_THREADS, PITCH>(p.f, rank, tile, 0, m0, n0);
+  cluster_add_and_finish<BM, BN, X3_THREADS, PITCH>(p.f, rank, tile, 0, m0, n0, Extra4{});
 }
 
 // x = p1 + p2 + p3 exactly (bf16 each, rounded to nearest); n a multiple of 8.  *wide is raised for values of 2^62

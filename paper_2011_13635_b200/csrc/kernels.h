@@ -25,7 +25,7 @@ struct AdamHyper {
 // to a tile of 128}.  The launchers below then get the allocated row count for their grid and work on the
 // rows in use only; null = every row.
 void launch_ln_fwd(bool bf, const void* z, const float* gamma, const float* beta, void* y,
-                   float* stats, int rows, int H, float eps, cudaStream_t st, const int* rows_dev = nullptr);
+                   float* stats, int rows, int H, float eps, cudaStream_t st, const int* rows_dev = nullptr, bool early = false);
 // segments / type: segment ids and the two-row segment table, or null (no segment term).  rows = B * S.
 // Packed: ptok (and pseg) receive the token id (segment) of every packed row, -1 past the last.
 void launch_embed_ln(bool bf, const int* tokens, const int* segments, const void* word, const void* pos,

@@ -615,12 +615,12 @@ int layer_forward(mslt_ctx* c, int l, const void* x, LayerBuf& b, void* out, boo
   }
   TRY(linear_fwd(c, b.c, T, H, toff(c, l, "out.weight"), toff(c, l, "out.bias"), H, b.z1, 0, nullptr, x, false, 0, c->rows));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_ln_fwd(c->bf, b.z1, Wv(c, toff(c, l, "ln1.gamma")), Wv(c, toff(c, l, "ln1.beta")), b.y,
-                   save ? b.st1 : nullptr, T, H, c->a.ln_eps, c->st, c->rows));
+                   save ? b.st1 : nullptr, T, H, c->a.ln_eps, c->st, c->rows, true));
   TRY(linear_fwd(c, b.y, T, H, toff(c, l, "ffn1.weight"), toff(c, l, "ffn1.bias"), F, b.g, 1,
                  save ? b.u : nullptr, nullptr, false, 0, c->rows));
   TRY(linear_fwd(c, b.g, T, F, toff(c, l, "ffn2.weight"), toff(c, l, "ffn2.bias"), H, b.z2, 0, nullptr, b.y, false, 0, c->rows));
   KL(PC_LN_FWD, 2.0 * T * H * c->esz, launch_ln_fwd(c->bf, b.z2, Wv(c, toff(c, l, "ln2.gamma")), Wv(c, toff(c, l, "ln2.beta")), out,
-                   save ? b.st2 : nullptr, T, H, c->a.ln_eps, c->st, c->rows));
+                   save ? b.st2 : nullptr, T, H, c->a.ln_eps, c->st, c->rows, true));
   return 0;
 }
 
@@ -696,7 +696,7 @@ int head_forward(mslt_ctx* c, const void* x, int R, bool save) {
   TRY(linear_fwd(c, w.hm, R, H, toff(c, -1, "head.transform.weight"), toff(c, -1, "head.transform.bias"),
                  H, w.gt, 1, save ? w.ut : nullptr, nullptr));
   KL(PC_LN_FWD, 2.0 * R * H * c->esz, launch_ln_fwd(c->bf, w.gt, Wv(c, toff(c, -1, "head.ln.gamma")), Wv(c, toff(c, -1, "head.ln.beta")),
-                   w.tm, save ? w.hst : nullptr, R, H, c->a.ln_eps, c->st));
+                   w.tm, save ? w.hst : nullptr, R, H, c->a.ln_eps, c->st, nullptr, true));
   // tied decoder: logits = tm * E^T + bv, fp32, rows padded to Vp columns
   TRY(linear_fwd(c, w.tm, R, H, toff(c, -1, "emb.word"), toff(c, -1, "head.decoder.bias"), V, w.logits,
                  0, nullptr, nullptr, true, c->Vp));
