@@ -361,6 +361,37 @@ def test_long_row_attention_wait_that_runs_out_is_reported(which):
     assert int(status.item()) == 0 and torch.equal(dqkv, want)
 
 
+@pytest.mark.parametrize("S", [136, 200, 264, 512])
+def test_long_row_attention_with_scores_far_above_the_first(S):
+    """The exponentials are formed relative to the largest of a row's first 32 scores.  Keys whose scores lie 2^64 and
+    more above it, in the first block and in later ones, move the sum and the context to a new reference, for some
+    rows of a warp and not for others.  Probabilities are rounded to bf16 as in the other attention tests; the sums'
+    logarithms reach a few thousand and are held to 2^-17 of that."""
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    B, A, d = 2, 2, 64
+    rng = np.random.default_rng(S)
+    x = rng.standard_normal((B, S, 3, A, d))
+    for at, much in ((20, 3.0), (40, 40.0), (100, 100.0), (130, 300.0), (260, 600.0), (S - 1, 900.0)):
+        if at < S:
+            x[:, at, 1] *= much
+    qkv = torch.from_numpy(x.reshape(B * S, 3 * A * d).astype(np.float32)).cuda().bfloat16()
+    x = qkv.float().cpu().numpy().astype(np.float64).reshape(B, S, 3, A, d)
+    q, k, v = (x[:, :, i].transpose(0, 2, 1, 3) for i in range(3))
+    s = np.einsum("bhid,bhjd->bhij", q, k) * 0.125
+    top = s.max(-1, keepdims=True)
+    e = np.exp(s - top)
+    want = np.einsum("bhij,bhjd->bhid", e / e.sum(-1, keepdims=True), v).transpose(0, 2, 1, 3).reshape(B * S, A * d)
+    want_lse = ((top + np.log(e.sum(-1, keepdims=True)))[..., 0] / np.log(2)).transpose(1, 0, 2).reshape(A, B * S)
+    ctx = torch.full((B * S, A * d), 7.0, device="cuda", dtype=torch.bfloat16)
+    lse = torch.full((A, B * S), 7.0, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Bd.mslt_op_attention_lse(qkv, ctx, lse, B, S, A, 0.125, status, _stream())
+    assert int(status.item()) == 0
+    assert np.abs(ctx.double().cpu().numpy() - want).max() / np.abs(want).max() < 1.5e-2
+    assert np.abs(lse.double().cpu().numpy() - want_lse).max() / np.abs(want_lse).max() < 2.0 ** -17
+
+
 @pytest.mark.parametrize("B,S,A", [(1, 128, 2), (1, 520, 1), (0, 256, 1)])
 def test_long_row_attention_backward_rejects_other_shapes(B, S, A):
     import torch
