@@ -828,10 +828,14 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 // warps own every second item of the block, whole: their own Q tile, ring of K and V tiles, score and context
 // accumulators, P block, copying thread and issuing thread; while one group waits (for a product, for the hand-over
 // of P, for its context) the other computes.
-// A thread owns a query row and reads its 128 scores of a block from tensor memory once.  The exponentials are taken
-// relative to the largest score so far; where a block raises it, the row's sum and context move to the new one.  (A
-// reference that stays unless a score lies 2^64 above it is as fast, but the largest probability is then no longer
-// exactly 1 and is rounded like the others: the context's error grew from 0.16 to 0.23 % where one key dominates.)
+// A thread owns a query row and reads its scores from tensor memory once, 32 at a time, the next 32 on their way.
+// The exponentials are taken relative to a reference that need not be the row's maximum: bf16 and fp32 numbers are
+// as precise at any scale, so the largest of the row's first 32 scores serves, and only a score more than 2^64 times
+// above it makes the row's sum and context move to a new reference and the block of keys start over.  The context is
+// divided by the sum of the rounded exponentials that it is made of, so that the weights add up to one: with the sum
+// of the unrounded ones a key that dominates its row leaves its own rounding behind, which it does not where the
+// maximum is the reference and its weight exactly 1 (error of the context at scores of 9 rms: 0.165 % with the
+// maximum, 0.226 % with this reference and the unrounded sum).  The unrounded sum is kept for the backward.
 //   warps 0, 10: TMA producers of the groups (ring order K_0, K_1, V_0, K_2, V_1, .. on through the items)
 //   warps 1, 11: MMA issuers: the scores of a block are issued ahead of the second product of the block before
 //   warps 2-5, 6-9: softmax groups
@@ -850,27 +854,15 @@ constexpr int AR_THREADS = 12 * 32;
 constexpr int AR_GROUP_TILES = 1 + AR_RING + 2;  // Q, ring, P
 constexpr int AR_BARS = 8 + 2 * AR_RING;         // per group
 
-// 16 consecutive accumulator columns of this lane's row, read and written
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};"
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
       ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+        "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+        "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
       : "memory");
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
@@ -1104,76 +1096,86 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       }
       const int n = (len + 127) >> 7;
       float ref = 0.f;                          // the exponentials' reference
-      float2 sum = make_float2(0.f, 0.f);
+      float2 sum = make_float2(0.f, 0.f), sumr = make_float2(0.f, 0.f);  // of the exponentials, and rounded
       for (int j = 0; j < n && ok; j++, nb++) {
         if (!mbar_wait(sfull, nb & 1, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
-        uint32_t s[4][32];
+        bool waited = false, again;
+        float2 part, partr;
+        do {
+          again = false;
+          part = partr = make_float2(0.f, 0.f);
+          float top = -INFINITY;                // largest score of the block
+          uint32_t s[2][32];
+          tc_ld32_issue(srow, s[0]);
 #pragma unroll
-        for (int c = 0; c < 4; c++) tc_ld32_issue(srow + c * 32, s[c]);
+          for (int c = 0; c < 4; c++) {
+            uint32_t(&x)[32] = s[c & 1];
+            tc_ld32_wait(x);
+            if (c < 3) tc_ld32_issue(srow + (c + 1) * 32, s[(c + 1) & 1]);
+            const int k0 = j * 128 + c * 32;
+            if (k0 + 32 > len) {                // keys beyond the sequence
 #pragma unroll
-        for (int c = 0; c < 4; c++) tc_ld32_wait(s[c]);
-        tc_fence_before();                      // the scores have been read
-        __syncwarp();
-        if (lane == 0) mbar_arrive(sempty);
-        float m0 = -INFINITY, m1 = -INFINITY;   // three-input maxima
+              for (int e = 0; e < 32; e++)
+                if (k0 + e >= len) x[e] = 0xff800000u;
+            }
+            float m0 = -INFINITY, m1 = top;     // three-input maxima
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-          const int k0 = j * 128 + c * 32;
-          if (k0 + 32 > len) {                  // keys beyond the sequence
+            for (int e = 0; e < 32; e += 4) {
+              m0 = fmaxf(fmaxf(m0, __uint_as_float(x[e])), __uint_as_float(x[e + 1]));
+              m1 = fmaxf(fmaxf(m1, __uint_as_float(x[e + 2])), __uint_as_float(x[e + 3]));
+            }
+            top = fmaxf(m0, m1);
+            if (j == 0 && c == 0 && !waited) ref = fmaxf(top, -1e30f);
+            if (c == 3) {
+              const bool over = (top - ref) * sl2 > 64.f;
+              if (__any_sync(0xffffffffu, over)) {
+                // a new reference for this warp's rows that need one; P of this block has not been handed over
+                const float to = over ? top : ref, f = fast_exp2((ref - to) * sl2);
+                ref = to;
+                sum = __fmul2_rn(sum, splat2(f));
+                sumr = __fmul2_rn(sumr, splat2(f));
+                if (j > 0) {                    // the products of the blocks before have completed: P was free
 #pragma unroll
-            for (int e = 0; e < 32; e++)
-              if (k0 + e >= len) s[c][e] = 0xff800000u;
+                  for (int h = 0; h < 2; h++) {
+                    tc_ld32_issue(orow + h * 32, s[0]);
+                    tc_ld32_wait(s[0]);
+#pragma unroll
+                    for (int e = 0; e < 32; e++) s[0][e] = __float_as_uint(__uint_as_float(s[0][e]) * f);
+                    tc_st32(orow + h * 32, s[0]);
+                  }
+                }
+                again = true;
+                break;
+              }
+              tc_fence_before();                // the scores have been read
+              __syncwarp();
+              if (lane == 0) mbar_arrive(sempty);
+            }
+            const float2 nm2 = splat2(-ref * sl2);
+            uint32_t h[16];
+#pragma unroll
+            for (int e = 0; e < 16; e++) {
+              const float2 a = __ffma2_rn(make_float2(__uint_as_float(x[2 * e]), __uint_as_float(x[2 * e + 1])), k2, nm2);
+              const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y));
+              part = __fadd2_rn(part, ea);
+              const __nv_bfloat162 pa = __float22bfloat162_rn(ea);
+              h[e] = *reinterpret_cast<const uint32_t*>(&pa);
+              partr = __fadd2_rn(partr, bf162_to_f2(h[e]));
+            }
+            if (!waited) {                      // the block before has been multiplied: P may be written
+              waited = true;
+              ok = __all_sync(0xffffffffu, mbar_wait(pfree, (nb & 1) ^ 1, abort_flag, p.status));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+              *reinterpret_cast<uint4*>(prow + (c >> 1) * AT_TILE_BYTES + ((((c & 1) * 4 + u) ^ (r & 7)) << 4)) =
+                  make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
           }
-#pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            m0 = fmaxf(fmaxf(m0, __uint_as_float(s[c][e])), __uint_as_float(s[c][e + 1]));
-            m1 = fmaxf(fmaxf(m1, __uint_as_float(s[c][e + 2])), __uint_as_float(s[c][e + 3]));
-          }
-        }
-        const float top = fmaxf(m0, m1);
-        bool waited = false;
-        if (j == 0) {
-          ref = fmaxf(top, -1e30f);
-        } else if (__any_sync(0xffffffffu, top > ref)) {
-          // the products of the blocks before have to be complete
-          waited = true;
-          ok = __all_sync(0xffffffffu, mbar_wait(pfree, (nb & 1) ^ 1, abort_flag, p.status));
-          if (!ok) break;
-          tc_fence_after();
-          const float to = fmaxf(ref, top), f = fast_exp2((ref - to) * sl2);
-          ref = to;
-          sum = __fmul2_rn(sum, splat2(f));
-#pragma unroll
-          for (int h = 0; h < 4; h++) {
-            uint32_t o[16];
-            tc_ld16(orow + h * 16, o);
-#pragma unroll
-            for (int e = 0; e < 16; e++) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
-            tc_st16(orow + h * 16, o);
-          }
-        }
-        const float2 nm2 = splat2(-ref * sl2);
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-#pragma unroll
-          for (int e = 0; e < 16; e++) {
-            const float2 a = __ffma2_rn(make_float2(__uint_as_float(s[c][2 * e]), __uint_as_float(s[c][2 * e + 1])), k2, nm2);
-            const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y));
-            sum = __fadd2_rn(sum, ea);
-            const __nv_bfloat162 pa = __float22bfloat162_rn(ea);
-            s[c][e] = *reinterpret_cast<const uint32_t*>(&pa);
-          }
-          if (c == 0 && !waited) {              // the block before has been multiplied: P may be written
-            ok = __all_sync(0xffffffffu, mbar_wait(pfree, (nb & 1) ^ 1, abort_flag, p.status));
-            if (!ok) break;
-          }
-#pragma unroll
-          for (int u = 0; u < 4; u++)
-            *reinterpret_cast<uint4*>(prow + (c >> 1) * AT_TILE_BYTES + ((((c & 1) * 4 + u) ^ (r & 7)) << 4)) =
-                make_uint4(s[c][4 * u], s[c][4 * u + 1], s[c][4 * u + 2], s[c][4 * u + 3]);
-        }
+        } while (again && ok);
         if (!ok) break;
+        sum = __fadd2_rn(sum, part);
+        sumr = __fadd2_rn(sumr, partr);
         if (kPacked && q == 0 && j == n - 1 && (len & 15)) {
           // position of the block's V tile in the ring: after the next block's K tile, if there is one
           const uint32_t pos = 2 * nb + (i == n_my - 1 ? 1 : 2), slot = pos % AR_RING;
@@ -1203,7 +1205,7 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       __syncwarp();
       if (lane == 0) mbar_arrive(oempty);
       if (row_ok) {
-        const float2 il = splat2(1.0f / total);
+        const float2 il = splat2(1.0f / (sumr.x + sumr.y));
 #pragma unroll
         for (int h = 0; h < 2; h++) {
           float2 w[16];

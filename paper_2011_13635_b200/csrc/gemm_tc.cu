@@ -84,10 +84,15 @@ enum : int {
   EPI_SOFTMAX,     // masked row softmax (its own epilogue)
   EPI_COUNT
 };
-// Epilogue warps of a flavour: four per TMEM lane quarter, two in the general and the softmax one.  A chunk of 32
-// columns is a chain (accumulator read, arithmetic, shared memory, tile store); two warps per scheduler left each unit
-// idle most of it, and a tile's epilogue of GELU or GELU' took 8.5 k cycles beside 6.1 k of its main loop (K = 768).
-template <int kMode> constexpr int kEpiWarps = kMode == EPI_GENERIC || kMode == EPI_SOFTMAX ? NUM_EPI_WARPS : 2 * NUM_EPI_WARPS;
+// Flavours with four epilogue warps per TMEM lane quarter instead of two (96 registers a thread instead of 168).  A
+// chunk of 32 columns is a chain: accumulator read, arithmetic, shared memory, tile store; two warps per scheduler
+// leave each unit idle most of it, and a tile's epilogue of GELU took 8.5 k cycles beside 6.1 k of its main loop at
+// K = 768.  us with two | four: 2400 x 2304 x 768 + bias 13.8 | 13.0, 4096 x 2304 x 768 16.3 | 15.4, 2400 x 3072 x 768 +
+// GELU 18.1 | 16.4, with its pre-activation 19.6 | 17.7, 16384 rows 84 | 79.  The flavours that read a second row or
+// write fp32 lose by it (2400 x 768 x 3072 + residual 16.1 | 16.9, 16384 x 3072 x 768 . GELU' 101 | 127, weight gradient
+// 3072 x 768 x 2400 14.5 | 15.7): their loads and reductions do not overlap better, and they need the registers.
+template <int kMode> constexpr bool kWide = kMode == EPI_STORE || kMode == EPI_GELU || kMode == EPI_GELU_AUX;
+template <int kMode> constexpr int kEpiWarps = kWide<kMode> ? 2 * NUM_EPI_WARPS : NUM_EPI_WARPS;
 
 // A lane that owns a row stores 32 of its columns without a trip through shared memory: two
 // 32-byte stores for bf16 (every store fills a whole sector), four for fp32, or eight 16-byte
@@ -106,9 +111,27 @@ __device__ __forceinline__ void row32_store_bf16(bf16* dst, const float2 (&w)[16
                  "r"(h[8 * c + 6]), "r"(h[8 * c + 7])
                  : "memory");
 }
-// A lane's row of 64 bytes in a 32-row staging tile, in the 64-byte swizzle of the output's tensor map (slot_b16):
-// 32 columns of bf16, or 16 of fp32.
-__device__ __forceinline__ void row_stage_bf16(uint32_t tile, int lane, const float2 (&w)[16]) {
+// The same 32 columns into a 32-row x 128-byte staging tile in the 128-byte swizzle layout of the
+// output's tensor map: row `lane`, 16-byte units 4 * half .. 4 * half + 3, unit u stored at
+// position u ^ (row & 7).  Eight neighbouring lanes hit eight different bank groups.
+__device__ __forceinline__ void row32_stage_bf16(uint32_t tile, int lane, int half, const float2 (&w)[16]) {
+  uint32_t h[16];
+#pragma unroll
+  for (int e = 0; e < 16; e++) {
+    const __nv_bfloat162 t = __float22bfloat162_rn(w[e]);
+    h[e] = *reinterpret_cast<const uint32_t*>(&t);
+  }
+  const uint32_t row = tile + (uint32_t)lane * 128u;
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const uint32_t u = (uint32_t)((4 * half + c) ^ (lane & 7));
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + u * 16u), "r"(h[4 * c]), "r"(h[4 * c + 1]),
+                 "r"(h[4 * c + 2]), "r"(h[4 * c + 3])
+                 : "memory");
+  }
+}
+// A lane's 32 columns into a 32-row x 64-byte staging tile in the 64-byte swizzle of the output's tensor map (slot_b16)
+__device__ __forceinline__ void row32_stage_half(uint32_t tile, int lane, const float2 (&w)[16]) {
 #pragma unroll
   for (int c = 0; c < 4; c++) {
     uint32_t h[4];
@@ -121,11 +144,13 @@ __device__ __forceinline__ void row_stage_bf16(uint32_t tile, int lane, const fl
                  : "memory");
   }
 }
-__device__ __forceinline__ void row_stage_f32(uint32_t tile, int lane, int half, const float2 (&w)[16]) {
+// 32 fp32 columns into a tile of 128-byte rows, which they fill
+__device__ __forceinline__ void row32_stage_f32(uint32_t tile, int lane, const float2 (&w)[16]) {
+  const uint32_t row = tile + (uint32_t)lane * 128u;
 #pragma unroll
-  for (int c = 0; c < 4; c++)
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(tile + slot_b16(lane, c)), "f"(w[8 * half + 2 * c].x),
-                 "f"(w[8 * half + 2 * c].y), "f"(w[8 * half + 2 * c + 1].x), "f"(w[8 * half + 2 * c + 1].y)
+  for (int c = 0; c < 8; c++)
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(row + (uint32_t)((c ^ (lane & 7)) * 16)), "f"(w[2 * c].x),
+                 "f"(w[2 * c].y), "f"(w[2 * c + 1].x), "f"(w[2 * c + 1].y)
                  : "memory");
 }
 __device__ __forceinline__ void row32_store_f32(float* dst, const float2 (&w)[16], int accumulate) {
@@ -173,45 +198,33 @@ __device__ __forceinline__ void prefetch_l2(const void* g, int bytes) {
 }
 
 // One 32 x 32 chunk of a specialised flavour: a = this lane's 32 accumulator columns, bias_c = the
-// chunk's bias values (null: none, or columns that end inside the chunk: then every lane holds one in bias_l), x = this lane's 32 bf16 values of
+// chunk's bias values in shared memory (null: no bias), x = this lane's 32 bf16 values of
 // the row-shaped extra operand (EPI_RESIDUAL, EPI_DGELU).
 // `direct`: this lane's row exists and the whole chunk lies inside the output, so the lane stores
 // its 32 columns itself; otherwise the chunk goes through the staging buffer, which handles ragged
 // edges element by element (every lane of the warp takes the same branch).
-// through_tile: results leave through tile_store(values, 0 = D, 1 = aux).
-// `x_used` runs once x has been used up, so that its registers can take the next chunk's values.
-template <int kMode, typename G, typename S>
+// `tile` != 0: the result goes into that staging tile (shared-memory address) instead, a bf16 one as half
+// `half` of its 64 columns, for a tile store by the caller.
+// `loaded` runs once the accumulator columns have been used up, so that their registers can take the next
+// chunk's read while this chunk is worked on; `x_used` likewise for x.
+template <int kMode, typename F, typename G>
 __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)[32], const uint4 (&x)[4],
-                                          const float* bias_c, float bias_l, uint8_t* stg, int lane, long long zoff,
-                                          int m_warp, int n0, bool direct, bool through_tile, G x_used, S tile_store) {
+                                          const float* bias_c, uint8_t* stg, int lane, long long zoff,
+                                          int m_warp, int n0, bool direct, uint32_t tile, int half, F loaded, G x_used) {
   float2 v[16];
   const float2 al = splat2(p.alpha);
-  if (bias_c) {
-    const float4* b4 = reinterpret_cast<const float4*>(bias_c);
+  const float4* b4 = reinterpret_cast<const float4*>(bias_c);
 #pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const float4 t = b4[j];
-      v[2 * j] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j]), __uint_as_float(a[4 * j + 1])), al, make_float2(t.x, t.y));
-      v[2 * j + 1] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j + 2]), __uint_as_float(a[4 * j + 3])), al, make_float2(t.z, t.w));
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 16; j++) {
-      float2 b = make_float2(0.f, 0.f);
-      if (p.bias) b = make_float2(__shfl_sync(0xffffffffu, bias_l, 2 * j), __shfl_sync(0xffffffffu, bias_l, 2 * j + 1));
-      v[j] = __ffma2_rn(make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])), al, b);
-    }
+  for (int j = 0; j < 8; j++) {
+    const float4 t = bias_c ? b4[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[2 * j] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j]), __uint_as_float(a[4 * j + 1])), al,
+                          make_float2(t.x, t.y));
+    v[2 * j + 1] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j + 2]), __uint_as_float(a[4 * j + 3])), al,
+                              make_float2(t.z, t.w));
   }
+  loaded();
   const bool row_ok = m_warp + lane < p.M;
   const long long off = zoff + (long long)(m_warp + lane) * p.ldd + n0;
-  if constexpr (kMode == EPI_GELU_AUX) {
-    if (through_tile) tile_store(v, 1);
-    else if (direct) { if (row_ok) row32_store_bf16(p.aux + off, v); }
-    else stage_store_bf16(stg, lane, v, p.aux + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
-  }
-  if constexpr (kMode == EPI_GELU || kMode == EPI_GELU_AUX) {
-    gelu_row(v);
-  }
   if constexpr (kMode == EPI_DGELU) {
 #pragma unroll
     for (int j = 0; j < 4; j++) {
@@ -230,21 +243,24 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
       v[4 * j + 2] = __fadd2_rn(v[4 * j + 2], bf162_to_f2(x[j].z));
       v[4 * j + 3] = __fadd2_rn(v[4 * j + 3], bf162_to_f2(x[j].w));
     }
-    x_used();
   }
   if constexpr (kMode == EPI_F32) {
-    if (through_tile) {
-      tile_store(v, 0);
-    } else {
-      if (p.tma_store) {  // the chunk before must have left the staging buffer
+    if (p.tma_store) {  // the chunk before must have left the staging buffer
+      if (elect_one()) tma_store_wait_read();
+      __syncwarp();
+    }
+    if (tile) row32_stage_f32(tile, lane, v);
+    else if (direct) { if (row_ok) row32_store_f32(reinterpret_cast<float*>(p.D) + off, v, p.accumulate); }
+    else stage_store_f32(stg, lane, v, reinterpret_cast<float*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok,
+                         p.accumulate);
+  } else {
+    if (tile) {
+      if (half == 0) {  // the tile store of the previous group must have read the staging tile
         if (elect_one()) tma_store_wait_read();
         __syncwarp();
       }
-      if (direct) { if (row_ok) row32_store_f32(reinterpret_cast<float*>(p.D) + off, v, p.accumulate); }
-      else stage_store_f32(stg, lane, v, reinterpret_cast<float*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok, p.accumulate);
+      row32_stage_bf16(tile, lane, half, v);
     }
-  } else {
-    if (through_tile) tile_store(v, 0);
     else if (direct) { if (row_ok) row32_store_bf16(reinterpret_cast<bf16*>(p.D) + off, v); }
     else stage_store_bf16(stg, lane, v, reinterpret_cast<bf16*>(p.D) + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
   }
@@ -280,7 +296,7 @@ struct Walk {
 };
 
 // ---- the kernel ---------------------------------------------------------------------------------
-// 20 warps: a thread may use up to 96 registers (12 warps and 168 in the general and the softmax flavour)
+// 12 warps: a thread may use up to 168 registers; 20 warps (kWide): 96
 template <int kMode, bool kPair, int KSUB>
 __global__ void __launch_bounds__(32 * (FIRST_EPI_WARP + kEpiWarps<kMode>), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -570,16 +586,105 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   } else if (warp >= FIRST_EPI_WARP) {
     // ------------------------------- epilogue -------------------------------
-    // EW / 4 warps share each TMEM lane quarter and take 32-column chunks in turn.  A warp reads
+    // Two warps share each TMEM lane quarter and take alternate 32-column chunks.  A warp reads
     // its 32 x 32 chunk (one row per lane), applies the epilogue, then turns the chunk through a
     // swizzled staging buffer so that global stores cover whole row segments.
     const int q = warp & 3;              // TMEM lane quarter this warp may read
     const int hsel = (warp - FIRST_EPI_WARP) >> 2;    // which of the warps of the quarter
     uint8_t* stg = staging + (size_t)(warp - FIRST_EPI_WARP) * (STAGING_TOTAL / EW);
     float* bias_s = reinterpret_cast<float*>(stg + 2048);  // bias of this warp's columns, chunk by chunk
+    float* bias_r = reinterpret_cast<float*>((uint8_t*)bars + 256) + (warp - FIRST_EPI_WARP) * 32;
     uint32_t tile = 0;
     bool ok = true;
-    if constexpr (kMode != EPI_GENERIC && !kSoftmax) {
+    if constexpr (kWide<kMode>) {
+      // One bf16 result, or two, from the accumulator and the bias alone.  A warp owns chunks hsel and hsel + 4 of a
+      // tile; a chunk's bias values are asked for while the tile is still multiplied and come from L1 when it is their
+      // turn (columns that end inside a chunk: one value per lane, handed round).
+      const uint32_t tile_s = smem_u32(stg);
+      auto fetch_bias = [&](int nt_, float (&b)[2]) {
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+          const int c = hsel + 4 * i, n = nt_ * p.bn + c * 32 + lane;
+          b[i] = 0.f;
+          if (p.bias && c * 32 < p.bn && n < p.N) asm volatile("ld.global.f32 %0, [%1];" : "=f"(b[i]) : "l"(p.bias + n));
+        }
+      };
+      float bcur[2] = {0.f, 0.f};
+      if (p.early && w_first < total_work) fetch_bias(at.nt, bcur);
+      begin();
+      if (!p.early && w_first < total_work) fetch_bias(at.nt, bcur);
+      for (int w = w_first; w < total_work; w += w_step, tile++) {
+        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
+        const uint32_t acc = tile & 1, use = tile >> 1;
+        const int m_warp = at.mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
+        const long long zoff = zo * p.d_bo + zi * p.d_bi;
+        const int n_base = at.nt * p.bn;
+        const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 256;
+        at.advance(p.n_tiles, m_tiles, p.batch);
+        if (!mbar_wait(smem_u32(&tfull_bar[acc]), use & 1, abort_flag, p.status)) break;
+        tc_fence_after();
+        // the chunk into the staging buffer, once the tile store before has read it, and out
+        auto put = [&](const float2 (&v)[16], int n0, const CUtensorMap* map, bf16* base) {
+          if (p.tma_store) {
+            if (elect_one()) tma_store_wait_read();
+            __syncwarp();
+            row32_stage_half(tile_s, lane, v);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (m_warp < p.M && elect_one()) {
+              auto slot = [&](int sl) { return p.d_perm[0] == sl ? m_warp : (p.d_perm[1] == sl ? zi : zo); };
+              tma_store_4d(map, tile_s, n0, slot(1), slot(2), slot(3));
+            }
+          } else if (p.direct && n0 + 32 <= p.N) {
+            if (m_warp + lane < p.M) row32_store_bf16(base + zoff + (long long)(m_warp + lane) * p.ldd + n0, v);
+          } else {
+            stage_store_bf16(stg, lane, v, base + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
+          }
+        };
+        auto has = [&](int i) { const int c = hsel + 4 * i; return i < 2 && c * 32 < p.bn && n_base + c * 32 < p.N; };
+        bool more = has(0);
+        for (int i = 0; more; i++) {
+          const int n0 = n_base + (hsel + 4 * i) * 32;
+          uint32_t a[32];
+          tc_ld32_issue(trow + (hsel + 4 * i) * 32, a);
+          tc_ld32_wait(a);
+          more = has(i + 1);
+          tc_fence_before();
+          __syncwarp();
+          if (!more && lane == 0 && w + 2 * w_step < total_work) {
+            if (kPair && !leader) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty_bar[acc]), 0));
+            else mbar_arrive(smem_u32(&tempty_bar[acc]));
+          }
+          float2 v[16];
+          const float2 al = splat2(p.alpha);
+          if (p.bias && p.vec_ok && n0 + 32 <= p.N) {
+            const float4* b4 = reinterpret_cast<const float4*>(p.bias + n0);
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+              const float4 t = b4[j];
+              v[2 * j] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j]), __uint_as_float(a[4 * j + 1])), al, make_float2(t.x, t.y));
+              v[2 * j + 1] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j + 2]), __uint_as_float(a[4 * j + 3])), al, make_float2(t.z, t.w));
+            }
+          } else {
+            const float bl = i ? bcur[1] : bcur[0];
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+              float2 b = make_float2(0.f, 0.f);
+              if (p.bias) b = make_float2(__shfl_sync(0xffffffffu, bl, 2 * j), __shfl_sync(0xffffffffu, bl, 2 * j + 1));
+              v[j] = __ffma2_rn(make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])), al, b);
+            }
+          }
+          if (kMode == EPI_GELU_AUX) put(v, n0, &tmX, p.aux);
+          if (kMode != EPI_STORE) gelu_row(v);
+          put(v, n0, &tmD, reinterpret_cast<bf16*>(p.D));
+        }
+        if (!has(0) && lane == 0 && w + 2 * w_step < total_work) {
+          if (kPair && !leader) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty_bar[acc]), 0));
+          else mbar_arrive(smem_u32(&tempty_bar[acc]));
+        }
+        if (w + w_step < total_work) fetch_bias(at.nt, bcur);
+      }
+    } else if constexpr (kMode != EPI_GENERIC && !kSoftmax) {
       // The specialised flavours.  What keeps a tile's epilogue short enough to hide behind the
       // next tile's main loop: the work-item coordinates advance by mixed-radix addition (no
       // division per tile); the bias of the NEXT tile is fetched while this tile is worked on; the
@@ -587,22 +692,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // and a lane stores its row segment straight from registers.
       constexpr bool kHasXf = kMode == EPI_RESIDUAL || kMode == EPI_DGELU;
       const bf16* xsrc = kMode == EPI_DGELU ? p.aux : kMode == EPI_RESIDUAL ? p.residual : nullptr;
-      // This warp's i-th chunk, in units of 32 columns
-      const bool tma_out = p.tma_store != 0;
-      constexpr int WQ = EW / 4, MAXC = 8 / WQ;  // warps of a quarter, chunks of a warp
-      auto ccol = [&](int i) { return hsel + WQ * i; };
+      // This warp's i-th chunk, in units of 32 columns.  The two warps of a quarter interleave
+      // their chunks; with tile stores of bf16 they interleave pairs of chunks, so that a warp owns whole
+      // 64-column (128-byte) groups.
+      const bool tma_out = p.tma_store != 0, tma_pairs = tma_out && kMode != EPI_F32;
+      auto ccol = [&](int i) { return tma_pairs ? 2 * (hsel + 2 * (i >> 1)) + (i & 1) : hsel + 2 * i; };
       const uint32_t stg_tile = smem_u32(stg);
-      // Bias values of this warp's columns of tile `nt_`, one value per lane and chunk, asked for while the tile is
-      // still multiplied.  A whole chunk reads its 32 again, from L1 by then (from L2 that cost it 300 to 600 cycles).
-      auto fetch_bias = [&](int nt_, float (&b)[MAXC]) {
+      // bias values of this warp's columns of tile `nt_`, one value per lane and chunk
+      auto fetch_bias = [&](int nt_, float (&b)[4]) {
 #pragma unroll
-        for (int i = 0; i < MAXC; i++) {
+        for (int i = 0; i < 4; i++) {
           const int n = nt_ * p.bn + ccol(i) * 32 + lane;
-          b[i] = 0.f;
-          if (ccol(i) * 32 < p.bn && p.bias && n < p.N) asm volatile("ld.global.f32 %0, [%1];" : "=f"(b[i]) : "l"(p.bias + n));
+          b[i] = (ccol(i) * 32 < p.bn && p.bias && n < p.N) ? p.bias[n] : 0.f;
         }
       };
-      float bcur[MAXC] = {};
+      // Every lane holds one column's value of each chunk, fetched while the tile is still multiplied; a chunk's 32 values go through
+      // shared memory when its turn comes (read from memory there they cost a chunk 300 to 600 cycles).
+      float bcur[4] = {0.f, 0.f, 0.f, 0.f};
       if (p.early && w_first < total_work) fetch_bias(at.nt, bcur);
       begin();
       if (!p.early && w_first < total_work) fetch_bias(at.nt, bcur);
@@ -663,44 +769,67 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             else mbar_arrive(smem_u32(&tempty_bar[acc]));
           }
         };
-        auto work = [&](const uint32_t (&a)[32], int i, bool has_next) {
-          const int n0 = chunk_n0(i);
-          const bool whole = n0 + 32 <= p.N;
-          const float* bias_c = p.bias && whole && p.vec_ok ? p.bias + n0 : nullptr;
-          float bias_l = bcur[0];
+        auto work = [&](const uint32_t (&a)[32], int i, bool has_next, auto loaded) {
+          // the next chunk of the extra operand: a chunk ahead, or, where the derivative of the GELU leaves
+          // no registers for that, as soon as this chunk's has been used
+          uint4 xc[4];
+          if constexpr (kMode == EPI_RESIDUAL) {
 #pragma unroll
-          for (int c = 1; c < MAXC; c++) bias_l = i == c ? bcur[c] : bias_l;
-          // a chunk of fp32 whose last 16-byte piece would reach beyond the row goes the other way
-          const bool through_tile = tma_out && (kMode != EPI_F32 || whole || p.N % 4 == 0);
-          // the chunk into the staging buffer, once the tile store before has read it, and out
-          auto tile_store = [&](const float2 (&v)[16], int which) {
-#pragma unroll
-            for (int h = 0; h < (kMode == EPI_F32 ? 2 : 1); h++) {
-              if (elect_one()) tma_store_wait_read();
-              __syncwarp();
-              if (kMode == EPI_F32) row_stage_f32(stg_tile, lane, h, v); else row_stage_bf16(stg_tile, lane, v);
-              fence_proxy_async_smem();
-              __syncwarp();
-              const int c0 = n0 + 16 * h;
-              if (m_warp < p.M && c0 < p.N && elect_one()) {
-                auto slot = [&](int sl) { return p.d_perm[0] == sl ? m_warp : (p.d_perm[1] == sl ? zi : zo); };
-                if (kMode == EPI_F32 && p.accumulate) tma_add_4d(&tmD, stg_tile, c0, slot(1), slot(2), slot(3));
-                else tma_store_4d(kMode == EPI_GELU_AUX && which ? &tmX : &tmD, stg_tile, c0, slot(1), slot(2), slot(3));
-              }
-            }
-          };
+            for (int j = 0; j < 4; j++) xc[j] = x[j];
+            if (has_next) prefetch_x(i + 1, x);
+          }
+          const uint4(&xu)[4] = kMode == EPI_DGELU ? x : xc;
           auto x_used = [&]() { if (has_next) prefetch_x(i + 1, x); };
-          epi_chunk<kMode>(p, a, x, bias_c, bias_l, stg, lane, zoff, m_warp, n0, p.direct && whole, through_tile, x_used, tile_store);
+          const int n0 = chunk_n0(i);
+          const float* bias_c = nullptr;
+          if (p.bias) {
+            __syncwarp();
+            bias_r[lane] = i == 0 ? bcur[0] : i == 1 ? bcur[1] : i == 2 ? bcur[2] : bcur[3];
+            __syncwarp();
+            bias_c = bias_r;
+          }
+          // a chunk of fp32 whose last 16-byte piece would reach beyond the row goes the other way
+          const bool through_tile = tma_out && (kMode != EPI_F32 || n0 + 32 <= p.N || p.N % 4 == 0);
+          epi_chunk<kMode>(p, a, xu, bias_c, stg, lane, zoff, m_warp, n0, p.direct && (tma_pairs || n0 + 32 <= p.N),
+                           through_tile ? stg_tile : 0, i & 1, loaded, x_used);  // warp-uniform
+          // an even chunk of bf16 opens a 64-column group, an odd chunk, or the last one, closes it
+          if (through_tile && (kMode == EPI_F32 || (i & 1) || !has_next)) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (m_warp < p.M && elect_one()) {
+              auto slot = [&](int sl) { return p.d_perm[0] == sl ? m_warp : (p.d_perm[1] == sl ? zi : zo); };
+              if (kMode != EPI_F32) tma_store_4d(&tmD, stg_tile, n0 - (i & 1) * 32, slot(1), slot(2), slot(3));
+              else if (p.accumulate) tma_add_4d(&tmD, stg_tile, n0, slot(1), slot(2), slot(3));
+              else tma_store_4d(&tmD, stg_tile, n0, slot(1), slot(2), slot(3));
+            }
+          }
         };
-        if (c0ok) {
+        if (c0ok && kHasXf) {
+          // the flavours with a row-shaped extra operand have no registers to spare for a second
+          // chunk in flight beside the first: its read starts when the first has left its registers
+          uint32_t ra[32];
+          tc_ld32_issue(trow + ccol(0) * 32, ra);
           for (int i = 0;; i++) {
             const bool v1 = chunk_ok(i + 1);
-            uint32_t ra[32];
-            tc_ld32_issue(trow + ccol(i) * 32, ra);
             tc_ld32_wait(ra);
             if (!v1) release_acc();
-            work(ra, i, v1);
+            work(ra, i, v1, [&]() { if (v1) tc_ld32_issue(trow + ccol(i + 1) * 32, ra); });
             if (!v1) break;
+          }
+        } else if (c0ok) {
+          uint32_t ra[32], rb[32];
+          tc_ld32_issue(trow + ccol(0) * 32, ra);
+          for (int i = 0;; i += 2) {
+            const bool v1 = chunk_ok(i + 1);
+            tc_ld32_wait(ra);
+            if (v1) tc_ld32_issue(trow + ccol(i + 1) * 32, rb); else release_acc();
+            work(ra, i, v1, []() {});
+            if (!v1) break;
+            const bool v2 = chunk_ok(i + 2);
+            tc_ld32_wait(rb);
+            if (v2) tc_ld32_issue(trow + ccol(i + 2) * 32, ra); else release_acc();
+            work(rb, i + 1, v2, []() {});
+            if (!v2) break;
           }
         } else {
           release_acc();
@@ -834,6 +963,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             // the extra operand of the next chunk travels while this chunk is worked on
             if (has_next) prefetch_x(i + 1, x);
           }
+          epi_chunk<kMode>(p, a, xc, bias_s + i * 32, stg, lane, zoff, m_warp, n0, false, 0, 0, []() {}, []() {});
           return;
         }
         const long long off = off0 + n0;
@@ -1100,7 +1230,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const int stage_bytes = ksub * (A_STAGE_BYTES + (pair ? p.bn / 2 : p.bn) * BK * 2);  // per CTA
   // barriers, then the softmax epilogue's exchange area or the 32 floats per epilogue warp that
   // hold the bias of a ragged chunk when the staging buffers carry output tiles
-  const int book_bytes = 256 + (d.act == 3 ? 64 + 2 * NUM_EPI_WARPS * 32 * 4 : 0);
+  const int book_bytes = 256 + (d.act == 3 ? 64 + 2 * NUM_EPI_WARPS * 32 * 4 : NUM_EPI_WARPS * 32 * 4);
   int stages = (smem_optin - STAGING_TOTAL - 1024 - book_bytes) / stage_bytes;
   if (stages > MAX_STAGES) stages = MAX_STAGES;
   if (stages < 2) { snprintf(err, 256, "gemm: not enough shared memory"); return MSLT_ERR_CUDA; }
@@ -1164,15 +1294,15 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   md.map = mx.map = ma.map;
   p.tma_store = 0;
   if ((((mode == EPI_STORE || mode == EPI_RESIDUAL || mode == EPI_GELU || mode == EPI_DGELU ||
-         (mode == EPI_GELU_AUX && p.direct && d.N % 32 == 0)) &&
-        d.N % 8 == 0) ||  // a tile store was seen to write whole 16-byte pieces
+         mode == EPI_GELU_AUX) &&
+        p.bn >= 128 && d.N % 8 == 0) ||  // a tile store was seen to write whole 16-byte pieces
        (mode == EPI_F32 && d.N >= 32)) &&
       p.vec_ok && g_store_variant.load() != 1) {
     char ignored[256];
     // the results of the splits are addressed like a batch
     if (get_map(d.D, d.M, d.N, d.ldd, 1, d.d_bo, parts ? p.part : d.d_bi, parts ? p.splits : d.hdiv, nb, 32, &md, ignored,
-                mode == EPI_F32 ? MAP_F32_OUT : MAP_BF16_OUT) == 0 &&
-        (mode != EPI_GELU_AUX || get_map(d.aux, d.M, d.N, d.ldd, 1, d.d_bo, d.d_bi, d.hdiv, nb, 32, &mx, ignored, MAP_BF16_OUT) == 0)) {
+                mode == EPI_F32 ? MAP_F32 : mode == EPI_RESIDUAL || mode == EPI_DGELU ? MAP_BF16 : MAP_HALF) == 0 &&
+        (mode != EPI_GELU_AUX || get_map(d.aux, d.M, d.N, d.ldd, 1, d.d_bo, d.d_bi, d.hdiv, nb, 32, &mx, ignored, MAP_HALF) == 0)) {
       p.tma_store = 1;
       for (int i = 0; i < 3; i++) p.d_perm[i] = md.perm[i];
     } else {
@@ -1201,8 +1331,8 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const KernelFn fn = kernels[mode][pair ? 2 : ksub - 1];
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  const int epi = mode == EPI_GENERIC || mode == EPI_SOFTMAX ? kEpiWarps<EPI_GENERIC> : kEpiWarps<EPI_STORE>;
-  cfg.blockDim = dim3(32 * (FIRST_EPI_WARP + epi));
+  const bool wide = mode == EPI_STORE || mode == EPI_GELU || mode == EPI_GELU_AUX;
+  cfg.blockDim = dim3(32 * (FIRST_EPI_WARP + (wide ? kEpiWarps<EPI_STORE> : kEpiWarps<EPI_F32>)));
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];

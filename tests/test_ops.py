@@ -363,9 +363,9 @@ def test_long_row_attention_wait_that_runs_out_is_reported(which):
 
 @pytest.mark.parametrize("S", [136, 200, 264, 512])
 def test_long_row_attention_with_scores_far_above_the_first(S):
-    """The exponentials are formed relative to the largest score so far.  Blocks of keys that raise it, by little and by
-    more than exponentials can bridge, move the sum and the context to a new reference, for some rows of a warp and
-    not for others.  Probabilities are rounded to bf16 as in the other attention tests; the sums'
+    """The exponentials are formed relative to the largest of a row's first 32 scores.  Keys whose scores lie 2^64 and
+    more above it, in the first block and in later ones, move the sum and the context to a new reference, for some
+    rows of a warp and not for others.  Probabilities are rounded to bf16 as in the other attention tests; the sums'
     logarithms reach a few thousand and are held to 2^-17 of that."""
     import torch
     from paper_2011_13635_b200 import binding as Bd
