@@ -40,7 +40,7 @@ namespace {
 
 constexpr int NUM_PRODUCERS = 3;                              // warps 0, 2, 3
 constexpr int FIRST_EPI_WARP = 4;                             // warps 4..11 (warp & 3 = TMEM lane quarter)
-constexpr int STAGING_TOTAL = NUM_EPI_WARPS * STAGING_BYTES;  // shared out over the epilogue warps
+constexpr int GEMM_THREADS = 32 * (FIRST_EPI_WARP + NUM_EPI_WARPS);
 
 struct TcParams {
   int M, N, K, batch, hdiv;
@@ -84,15 +84,6 @@ enum : int {
   EPI_SOFTMAX,     // masked row softmax (its own epilogue)
   EPI_COUNT
 };
-// Flavours with four epilogue warps per TMEM lane quarter instead of two (96 registers a thread instead of 168).  A
-// chunk of 32 columns is a chain: accumulator read, arithmetic, shared memory, tile store; two warps per scheduler
-// leave each unit idle most of it, and a tile's epilogue of GELU took 8.5 k cycles beside 6.1 k of its main loop at
-// K = 768.  us with two | four: 2400 x 2304 x 768 + bias 13.8 | 13.0, 4096 x 2304 x 768 16.3 | 15.4, 2400 x 3072 x 768 +
-// GELU 18.1 | 16.4, with its pre-activation 19.6 | 17.7, 16384 rows 84 | 79.  The flavours that read a second row or
-// write fp32 lose by it (2400 x 768 x 3072 + residual 16.1 | 16.9, 16384 x 3072 x 768 . GELU' 101 | 127, weight gradient
-// 3072 x 768 x 2400 14.5 | 15.7): their loads and reductions do not overlap better, and they need the registers.
-template <int kMode> constexpr bool kWide = kMode == EPI_STORE || kMode == EPI_GELU || kMode == EPI_GELU_AUX;
-template <int kMode> constexpr int kEpiWarps = kWide<kMode> ? 2 * NUM_EPI_WARPS : NUM_EPI_WARPS;
 
 // A lane that owns a row stores 32 of its columns without a trip through shared memory: two
 // 32-byte stores for bf16 (every store fills a whole sector), four for fp32, or eight 16-byte
@@ -130,21 +121,7 @@ __device__ __forceinline__ void row32_stage_bf16(uint32_t tile, int lane, int ha
                  : "memory");
   }
 }
-// A lane's 32 columns into a 32-row x 64-byte staging tile in the 64-byte swizzle of the output's tensor map (slot_b16)
-__device__ __forceinline__ void row32_stage_half(uint32_t tile, int lane, const float2 (&w)[16]) {
-#pragma unroll
-  for (int c = 0; c < 4; c++) {
-    uint32_t h[4];
-#pragma unroll
-    for (int e = 0; e < 4; e++) {
-      const __nv_bfloat162 t = __float22bfloat162_rn(w[4 * c + e]);
-      h[e] = *reinterpret_cast<const uint32_t*>(&t);
-    }
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + slot_b16(lane, c)), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3])
-                 : "memory");
-  }
-}
-// 32 fp32 columns into a tile of 128-byte rows, which they fill
+// 32 fp32 columns into such a tile, which they fill
 __device__ __forceinline__ void row32_stage_f32(uint32_t tile, int lane, const float2 (&w)[16]) {
   const uint32_t row = tile + (uint32_t)lane * 128u;
 #pragma unroll
@@ -225,6 +202,13 @@ __device__ __forceinline__ void epi_chunk(const TcParams& p, const uint32_t (&a)
   loaded();
   const bool row_ok = m_warp + lane < p.M;
   const long long off = zoff + (long long)(m_warp + lane) * p.ldd + n0;
+  if constexpr (kMode == EPI_GELU_AUX) {
+    if (direct) { if (row_ok) row32_store_bf16(p.aux + off, v); }
+    else stage_store_bf16(stg, lane, v, p.aux + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
+  }
+  if constexpr (kMode == EPI_GELU || kMode == EPI_GELU_AUX) {
+    gelu_row(v);
+  }
   if constexpr (kMode == EPI_DGELU) {
 #pragma unroll
     for (int j = 0; j < 4; j++) {
@@ -296,12 +280,11 @@ struct Walk {
 };
 
 // ---- the kernel ---------------------------------------------------------------------------------
-// 12 warps: a thread may use up to 168 registers; 20 warps (kWide): 96
+// 12 warps: a thread may use up to 168 registers
 template <int kMode, bool kPair, int KSUB>
-__global__ void __launch_bounds__(32 * (FIRST_EPI_WARP + kEpiWarps<kMode>), 1)
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmX, const TcParams p) {
-  constexpr int EW = kEpiWarps<kMode>;
+               const __grid_constant__ CUtensorMap tmD, const TcParams p) {
   constexpr bool kSoftmax = kMode == EPI_SOFTMAX;
   constexpr bool kHasX = kMode == EPI_RESIDUAL || kMode == EPI_DGELU;
   extern __shared__ uint8_t smem_raw[];
@@ -325,7 +308,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int sub_bytes = A_STAGE_BYTES + b_stage_bytes;
   const int stage_bytes = KSUB * sub_bytes;
   uint8_t* staging = smem + (size_t)p.stages * stage_bytes;
-  uint64_t* bars = (uint64_t*)(staging + STAGING_TOTAL);
+  uint64_t* bars = (uint64_t*)(staging + NUM_EPI_WARPS * STAGING_BYTES);
   uint64_t* full_bar = bars;
   uint64_t* empty_bar = bars + MAX_STAGES;
   uint64_t* tfull_bar = bars + 2 * MAX_STAGES;
@@ -343,7 +326,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     prefetch_map(&tmA);
     prefetch_map(&tmB);
     if (p.tma_store) prefetch_map(&tmD);
-    if (p.tma_store && kMode == EPI_GELU_AUX) prefetch_map(&tmX);
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; s++) {
@@ -352,7 +334,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
     for (int a = 0; a < 2; a++) {
       mbar_init(smem_u32(&tfull_bar[a]), 1);
-      mbar_init(smem_u32(&tempty_bar[a]), kPair ? 2 * EW : EW);
+      mbar_init(smem_u32(&tempty_bar[a]), kPair ? 2 * NUM_EPI_WARPS : NUM_EPI_WARPS);
     }
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;  // read by every bounded wait
@@ -590,101 +572,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // its 32 x 32 chunk (one row per lane), applies the epilogue, then turns the chunk through a
     // swizzled staging buffer so that global stores cover whole row segments.
     const int q = warp & 3;              // TMEM lane quarter this warp may read
-    const int hsel = (warp - FIRST_EPI_WARP) >> 2;    // which of the warps of the quarter
-    uint8_t* stg = staging + (size_t)(warp - FIRST_EPI_WARP) * (STAGING_TOTAL / EW);
+    const int hsel = (warp - FIRST_EPI_WARP) >> 2;    // which of the two warps of the quarter
+    uint8_t* stg = staging + (size_t)(warp - FIRST_EPI_WARP) * STAGING_BYTES;
     float* bias_s = reinterpret_cast<float*>(stg + 2048);  // bias of this warp's columns, chunk by chunk
     float* bias_r = reinterpret_cast<float*>((uint8_t*)bars + 256) + (warp - FIRST_EPI_WARP) * 32;
     uint32_t tile = 0;
     bool ok = true;
-    if constexpr (kWide<kMode>) {
-      // One bf16 result, or two, from the accumulator and the bias alone.  A warp owns chunks hsel and hsel + 4 of a
-      // tile; a chunk's bias values are asked for while the tile is still multiplied and come from L1 when it is their
-      // turn (columns that end inside a chunk: one value per lane, handed round).
-      const uint32_t tile_s = smem_u32(stg);
-      auto fetch_bias = [&](int nt_, float (&b)[2]) {
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-          const int c = hsel + 4 * i, n = nt_ * p.bn + c * 32 + lane;
-          b[i] = 0.f;
-          if (p.bias && c * 32 < p.bn && n < p.N) asm volatile("ld.global.f32 %0, [%1];" : "=f"(b[i]) : "l"(p.bias + n));
-        }
-      };
-      float bcur[2] = {0.f, 0.f};
-      if (p.early && w_first < total_work) fetch_bias(at.nt, bcur);
-      begin();
-      if (!p.early && w_first < total_work) fetch_bias(at.nt, bcur);
-      for (int w = w_first; w < total_work; w += w_step, tile++) {
-        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
-        const uint32_t acc = tile & 1, use = tile >> 1;
-        const int m_warp = at.mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
-        const long long zoff = zo * p.d_bo + zi * p.d_bi;
-        const int n_base = at.nt * p.bn;
-        const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 256;
-        at.advance(p.n_tiles, m_tiles, p.batch);
-        if (!mbar_wait(smem_u32(&tfull_bar[acc]), use & 1, abort_flag, p.status)) break;
-        tc_fence_after();
-        // the chunk into the staging buffer, once the tile store before has read it, and out
-        auto put = [&](const float2 (&v)[16], int n0, const CUtensorMap* map, bf16* base) {
-          if (p.tma_store) {
-            if (elect_one()) tma_store_wait_read();
-            __syncwarp();
-            row32_stage_half(tile_s, lane, v);
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (m_warp < p.M && elect_one()) {
-              auto slot = [&](int sl) { return p.d_perm[0] == sl ? m_warp : (p.d_perm[1] == sl ? zi : zo); };
-              tma_store_4d(map, tile_s, n0, slot(1), slot(2), slot(3));
-            }
-          } else if (p.direct && n0 + 32 <= p.N) {
-            if (m_warp + lane < p.M) row32_store_bf16(base + zoff + (long long)(m_warp + lane) * p.ldd + n0, v);
-          } else {
-            stage_store_bf16(stg, lane, v, base + zoff, p.ldd, m_warp, n0, p.M, p.N, p.vec_ok);
-          }
-        };
-        auto has = [&](int i) { const int c = hsel + 4 * i; return i < 2 && c * 32 < p.bn && n_base + c * 32 < p.N; };
-        bool more = has(0);
-        for (int i = 0; more; i++) {
-          const int n0 = n_base + (hsel + 4 * i) * 32;
-          uint32_t a[32];
-          tc_ld32_issue(trow + (hsel + 4 * i) * 32, a);
-          tc_ld32_wait(a);
-          more = has(i + 1);
-          tc_fence_before();
-          __syncwarp();
-          if (!more && lane == 0 && w + 2 * w_step < total_work) {
-            if (kPair && !leader) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty_bar[acc]), 0));
-            else mbar_arrive(smem_u32(&tempty_bar[acc]));
-          }
-          float2 v[16];
-          const float2 al = splat2(p.alpha);
-          if (p.bias && p.vec_ok && n0 + 32 <= p.N) {
-            const float4* b4 = reinterpret_cast<const float4*>(p.bias + n0);
-#pragma unroll
-            for (int j = 0; j < 8; j++) {
-              const float4 t = b4[j];
-              v[2 * j] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j]), __uint_as_float(a[4 * j + 1])), al, make_float2(t.x, t.y));
-              v[2 * j + 1] = __ffma2_rn(make_float2(__uint_as_float(a[4 * j + 2]), __uint_as_float(a[4 * j + 3])), al, make_float2(t.z, t.w));
-            }
-          } else {
-            const float bl = i ? bcur[1] : bcur[0];
-#pragma unroll
-            for (int j = 0; j < 16; j++) {
-              float2 b = make_float2(0.f, 0.f);
-              if (p.bias) b = make_float2(__shfl_sync(0xffffffffu, bl, 2 * j), __shfl_sync(0xffffffffu, bl, 2 * j + 1));
-              v[j] = __ffma2_rn(make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])), al, b);
-            }
-          }
-          if (kMode == EPI_GELU_AUX) put(v, n0, &tmX, p.aux);
-          if (kMode != EPI_STORE) gelu_row(v);
-          put(v, n0, &tmD, reinterpret_cast<bf16*>(p.D));
-        }
-        if (!has(0) && lane == 0 && w + 2 * w_step < total_work) {
-          if (kPair && !leader) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty_bar[acc]), 0));
-          else mbar_arrive(smem_u32(&tempty_bar[acc]));
-        }
-        if (w + w_step < total_work) fetch_bias(at.nt, bcur);
-      }
-    } else if constexpr (kMode != EPI_GENERIC && !kSoftmax) {
+    if constexpr (kMode != EPI_GENERIC && !kSoftmax) {
       // The specialised flavours.  What keeps a tile's epilogue short enough to hide behind the
       // next tile's main loop: the work-item coordinates advance by mixed-radix addition (no
       // division per tile); the bias of the NEXT tile is fetched while this tile is worked on; the
@@ -804,8 +698,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
           }
         };
-        if (c0ok && kHasXf) {
-          // the flavours with a row-shaped extra operand have no registers to spare for a second
+        if (c0ok && (kHasXf || kMode == EPI_GELU_AUX)) {
+          // the flavours with a row-shaped extra operand or output have no registers to spare for a second
           // chunk in flight beside the first: its read starts when the first has left its registers
           uint32_t ra[32];
           tc_ld32_issue(trow + ccol(0) * 32, ra);
@@ -1231,11 +1125,11 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   // barriers, then the softmax epilogue's exchange area or the 32 floats per epilogue warp that
   // hold the bias of a ragged chunk when the staging buffers carry output tiles
   const int book_bytes = 256 + (d.act == 3 ? 64 + 2 * NUM_EPI_WARPS * 32 * 4 : NUM_EPI_WARPS * 32 * 4);
-  int stages = (smem_optin - STAGING_TOTAL - 1024 - book_bytes) / stage_bytes;
+  int stages = (smem_optin - NUM_EPI_WARPS * STAGING_BYTES - 1024 - book_bytes) / stage_bytes;
   if (stages > MAX_STAGES) stages = MAX_STAGES;
   if (stages < 2) { snprintf(err, 256, "gemm: not enough shared memory"); return MSLT_ERR_CUDA; }
   p.stages = stages;
-  const size_t smem_bytes = (size_t)stages * stage_bytes + STAGING_TOTAL + 1024 + book_bytes;
+  const size_t smem_bytes = (size_t)stages * stage_bytes + NUM_EPI_WARPS * STAGING_BYTES + 1024 + book_bytes;
   if ((int)smem_bytes > smem_optin) { snprintf(err, 256, "gemm: not enough shared memory"); return MSLT_ERR_CUDA; }
 
   MapVal ma, mb;
@@ -1290,27 +1184,26 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   // hold up the operand loads that share the SM's path to L2: 16384 x 2304 x 768 took 51.7 us with
   // them, 41.3 us with the stores left out, and a load stream beside such stores fell from 68 to
   // 12 bytes per clock per SM while beside copy-engine stores it kept 68.
-  MapVal md, mx;
-  md.map = mx.map = ma.map;
+  MapVal md;
+  md.map = ma.map;
   p.tma_store = 0;
   if ((((mode == EPI_STORE || mode == EPI_RESIDUAL || mode == EPI_GELU || mode == EPI_DGELU ||
-         mode == EPI_GELU_AUX) &&
+         (mode == EPI_GELU_AUX && p.direct && d.N % 32 == 0)) &&
         p.bn >= 128 && d.N % 8 == 0) ||  // a tile store was seen to write whole 16-byte pieces
        (mode == EPI_F32 && d.N >= 32)) &&
       p.vec_ok && g_store_variant.load() != 1) {
     char ignored[256];
     // the results of the splits are addressed like a batch
     if (get_map(d.D, d.M, d.N, d.ldd, 1, d.d_bo, parts ? p.part : d.d_bi, parts ? p.splits : d.hdiv, nb, 32, &md, ignored,
-                mode == EPI_F32 ? MAP_F32 : mode == EPI_RESIDUAL || mode == EPI_DGELU ? MAP_BF16 : MAP_HALF) == 0 &&
-        (mode != EPI_GELU_AUX || get_map(d.aux, d.M, d.N, d.ldd, 1, d.d_bo, d.d_bi, d.hdiv, nb, 32, &mx, ignored, MAP_HALF) == 0)) {
+                mode == EPI_F32) == 0) {
       p.tma_store = 1;
       for (int i = 0; i < 3; i++) p.d_perm[i] = md.perm[i];
     } else {
-      md.map = mx.map = ma.map;
+      md.map = ma.map;
     }
   }
 
-  typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams);
+  typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcParams);
   // [one CTA, one k block per round | one CTA, two | pair, two]
 #define FORMS(mode) {gemm_tc_kernel<mode, false, 1>, gemm_tc_kernel<mode, false, 2>, gemm_tc_kernel<mode, true, 2>}
   static const KernelFn kernels[EPI_COUNT][3] = {
@@ -1331,8 +1224,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const KernelFn fn = kernels[mode][pair ? 2 : ksub - 1];
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  const bool wide = mode == EPI_STORE || mode == EPI_GELU || mode == EPI_GELU_AUX;
-  cfg.blockDim = dim3(32 * (FIRST_EPI_WARP + (wide ? kEpiWarps<EPI_STORE> : kEpiWarps<EPI_F32>)));
+  cfg.blockDim = dim3(GEMM_THREADS);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -1351,7 +1243,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   } else {
     cfg.gridDim = dim3(p.total_work < num_sms ? p.total_work : num_sms);
   }
-  cudaError_t e = cudaLaunchKernelEx(&cfg, fn, ma.map, mb.map, md.map, mx.map, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, fn, ma.map, mb.map, md.map, p);
   if (e != cudaSuccess) { snprintf(err, 256, "gemm: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
   return 0;
 }

@@ -451,7 +451,7 @@ EncodeTiledFn get_encode() {
 struct MapKey {
   const void* ptr;
   long long rows, K, rs, ks, bo, bi;
-  int hdiv, nb, box_rows, kind;
+  int hdiv, nb, box_rows, f32;
   bool operator==(const MapKey& o) const { return memcmp(this, &o, sizeof(MapKey)) == 0; }
 };
 struct MapKeyHash {
@@ -467,21 +467,18 @@ struct MapVal {
   int perm[3];
 };
 
-enum { MAP_BF16 = 0, MAP_F32, MAP_HALF };
 // Builds (or fetches) the rank-4 tensor map of one operand: dim 0 is the contiguous index (k for a
 // K-major operand, the row index otherwise); the other matrix index and the two batch indices
-// follow in order of increasing stride.  Boxes are 128 bytes of dim 0 wide, 64 bf16 or (MAP_F32)
-// 32 fp32; with MAP_HALF 64 bytes, 32 bf16, with the swizzle to match.
+// follow in order of increasing stride.  Boxes are 128 bytes of dim 0 wide: 64 bf16, or 32 fp32 with f32.
 int get_map(const void* ptr, long long rows, long long K, long long rs, long long ks, long long bo,
-            long long bi, int hdiv, int nb, int box_rows, MapVal* out, char* err, int kind = MAP_BF16) {
-  const bool f32 = kind == MAP_F32;
+            long long bi, int hdiv, int nb, int box_rows, MapVal* out, char* err, bool f32 = false) {
   static std::unordered_map<MapKey, MapVal, MapKeyHash> cache;
   static std::mutex mu;
   MapKey key;
   memset(&key, 0, sizeof(key));
   key.ptr = ptr; key.rows = rows; key.K = K; key.rs = rs; key.ks = ks; key.bo = bo; key.bi = bi;
   key.hdiv = hdiv; key.nb = nb; key.box_rows = box_rows;
-  key.kind = kind;
+  key.f32 = f32;
   std::lock_guard<std::mutex> lock(mu);
   auto itf = cache.find(key);
   if (itf != cache.end()) { *out = itf->second; return 0; }
@@ -505,7 +502,7 @@ int get_map(const void* ptr, long long rows, long long K, long long rs, long lon
   cuuint64_t gdim[4], gstr[3];
   cuuint32_t bdim[4], estr[4] = {1, 1, 1, 1};
   gdim[0] = (cuuint64_t)ext0;
-  bdim[0] = kind == MAP_BF16 ? 64 : 32;
+  bdim[0] = f32 ? 32 : 64;
   long long last = 16;
   for (int sl = 0; sl < 3; sl++) {
     const int li = order[sl];
@@ -522,7 +519,7 @@ int get_map(const void* ptr, long long rows, long long K, long long rs, long lon
   }
   if ((uintptr_t)ptr & 15) { snprintf(err, 256, "gemm: operand base is not 16-byte aligned"); return MSLT_ERR_ARG; }
   CUresult r = enc(&out->map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), gdim, gstr, bdim,
-                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE, kind == MAP_HALF ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     snprintf(err, 256, "gemm: cuTensorMapEncodeTiled failed with code %d (dims %llu,%llu,%llu,%llu)", (int)r,
