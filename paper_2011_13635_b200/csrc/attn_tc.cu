@@ -824,78 +824,105 @@ attn_fwd_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 }
 
 // ---- forward for rows of 129..512 keys, no probabilities stored -----------------------------------
-// A work item is (sequence, head, tile of 128 queries), walked in blocks of 128 keys.  Two groups of four softmax
-// warps own every second item of the block, whole: their own Q tile, ring of K and V tiles, score and context
-// accumulators, P block, copying thread and issuing thread; while one group waits (for a product, for the hand-over
-// of P, for its context) the other computes.
-// A thread owns a query row and reads its scores from tensor memory once, 32 at a time, the next 32 on their way.
-// The exponentials are taken relative to a reference that need not be the row's maximum: bf16 and fp32 numbers are
-// as precise at any scale, so the largest of the row's first 32 scores serves, and only a score more than 2^64 times
-// above it makes the row's sum and context move to a new reference and the block of keys start over.  The context is
-// divided by the sum of the rounded exponentials that it is made of, so that the weights add up to one: with the sum
-// of the unrounded ones a key that dominates its row leaves its own rounding behind, which it does not where the
-// maximum is the reference and its weight exactly 1 (error of the context at scores of 9 rms: 0.165 % with the
-// maximum, 0.226 % with this reference and the unrounded sum).  The unrounded sum is kept for the backward.
-//   warps 0, 10: TMA producers of the groups (ring order K_0, K_1, V_0, K_2, V_1, .. on through the items)
-//   warps 1, 11: MMA issuers: the scores of a block are issued ahead of the second product of the block before
-//   warps 2-5, 6-9: softmax groups
-// The last V tile of a packed sequence goes on into rows that are not its own (see above): the second product ends
-// with the 16 keys that hold the sequence's last one, and the first warp of the group clears the others of them
-// before it hands P over.  (Clearing warps of their own, which see every tile, made the block fourteen warps of 128
-// registers: 16 x 16 heads x (256..512) keys 41.2 us in a step; one producer and one such warp for both groups 45.3.)
-// Bound by the exponential unit (16 a clock: 1024 cycles per block of an item; two groups together take 1750, the
-// rest is the hand-over of P at the end of a block and the start and end of an item).  The form before held the scores
-// of a whole row in tensor memory, one item at a time, and read them twice, with sixteen warps that met twice an
-// item: 16 x 16 heads x 512 keys 46.4 -> 40.4 us, 64 x 12 x 256 49.0 -> 39.0, 21 x 12 x 232 20.8 -> 16.7, in steps
-// 16 x 16 x (256..512) 46.6 -> 38.6 and 12 x 16 x (200..384) 24.9 -> 22.4.
-constexpr int AR_RING = 4;           // 16 KB tiles per group
-constexpr int AR_TABLE = 32;         // items of a group described in shared memory; any beyond are read from memory
-constexpr int AR_THREADS = 12 * 32;
-constexpr int AR_GROUP_TILES = 1 + AR_RING + 2;  // Q, ring, P
-constexpr int AR_BARS = 8 + 2 * AR_RING;         // per group
+// A work item is (sequence, head, tile of 128 queries).  Tensor memory holds the scores of a whole row
+// (four blocks of 128 keys), so they are formed once: all sixteen softmax warps read them twice, first for
+// the row maximum, then for the exponentials, and the context accumulates over columns whose scores have
+// been used up (block 0 when there are four blocks, else the upper half of the unused block 3).
+// A thread owns a quarter of one query row's scores in every key block; the quarters exchange maximum and
+// sum through shared memory.  P_j goes to one of two shared-memory blocks as the second product's operand.
+//   warp 0: TMA producer (Q tile, ring of K and V tiles: K_0 .. K_{n-1}, V_0 .. V_{n-1})
+//   warp 1: MMA issuer: the next item's scores are issued behind this item's last second product, so they
+//           are ready when the softmax warps have stored the context
+//   warps 2-17: softmax; packed batches: warps 18, 19 clear the last V tile's rows beyond the sequence
+// Bound by the exponential unit (16 a clock: 1024 cycles per block) and the passes around it.
+// 16 sequences x 16 heads x 512 keys: 59.5 us with two groups of warps on items of their own and the scores
+// formed twice; 49.5 us in this form with eight softmax warps (two per scheduler do not cover the
+// tensor-memory reads and the fences); 48.3 us with sixteen, 46.2 with elected copying and issuing threads
+// (64 x 12 x 256 keys 48.8, 12 x 16 x 384 24.2, 21 x 12 x 232 20.7).
+// In steps of BERT-Large at 16 x (256..512) keys, packed tiles dealt out longest first: 56.8 -> 52.1 us a layer.
+// The row's maximum is the reference of the exponentials, so that the largest probability is exactly 1 in bf16 and
+// no context exceeds the largest value.  A form with two groups of warps that read the scores once, relative to the
+// largest of a row's first 32, took 42.6 us (64 x 12 x 256 keys 40.6); its context was up to 1.27 times as far from
+// float64 (a key of weight 0.3 past the first 32) and overflowed where values are large.
+constexpr int AR_RING = 8;
+constexpr int AR_TABLE = 256;  // items of a block described in shared memory; any beyond are read from memory
+constexpr int AR_WARPS = 16;  // softmax warps: four per TMEM lane quarter
+constexpr int AR_THREADS = 64 + 32 * AR_WARPS;
 
-__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+// 16 consecutive accumulator columns of this lane's row
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
-      ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
-        "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
-        "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
       : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+// Hand-over between the four warps of a lane quarter (pair_sync for more partners).
+__device__ __forceinline__ bool quad_sync(volatile int* flags, int me, int seq, int lane, volatile int* abort_flag, int* status) {
+  __syncwarp();
+  int ok = 1;
+  if (lane == 0) {
+    __threadfence_block();
+    flags[me] = seq;
+    const long long t0 = now_cycles();
+    uint32_t spins = 0;
+    const int first = me & ~3;
+    while (flags[first] < seq || flags[first + 1] < seq || flags[first + 2] < seq || flags[first + 3] < seq) {
+      if ((++spins & 255u) == 0u) {
+        if (*abort_flag) { ok = 0; break; }
+        if (now_cycles() - t0 > *reinterpret_cast<volatile long long*>(abort_flag + 1)) {
+          *abort_flag = 1;
+          atomicOr(status, ST_WAIT_TIMEOUT);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    __threadfence_block();
+  }
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  return ok != 0;
 }
 
 template <bool kPacked>
-__global__ void __launch_bounds__(AR_THREADS, 1)
+__global__ void __launch_bounds__(AR_THREADS + (kPacked ? 32 * CLEAR_WARPS : 0), 1)
 attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = warp < 2 ? 0 : warp < 10 ? (warp - 2) >> 2 : 1;  // the group a warp works for
-  uint8_t* q_smem = smem + (size_t)g * AR_GROUP_TILES * AT_TILE_BYTES;
-  uint8_t* ring_smem = q_smem + AT_TILE_BYTES;
-  uint8_t* p_smem = ring_smem + AR_RING * AT_TILE_BYTES;
-  int4* table0 = (int4*)(smem + 2 * AR_GROUP_TILES * AT_TILE_BYTES);
-  int4* table = table0 + g * AR_TABLE;
-  uint64_t* bars0 = (uint64_t*)(table0 + 2 * AR_TABLE);
-  uint64_t* bars = bars0 + g * AR_BARS;
-  const uint32_t qfull = smem_u32(&bars[0]), qempty = smem_u32(&bars[1]), sfull = smem_u32(&bars[2]), sempty = smem_u32(&bars[3]);
-  const uint32_t pready = smem_u32(&bars[4]), pfree = smem_u32(&bars[5]), ofull = smem_u32(&bars[6]), oempty = smem_u32(&bars[7]);
-  const uint32_t tfull0 = smem_u32(&bars[8]), tempty0 = smem_u32(&bars[8 + AR_RING]);
-  uint32_t* tmem_slot = (uint32_t*)(bars0 + 2 * AR_BARS);
+  uint8_t* ring_smem = smem + AT_TILE_BYTES;                  // Q first
+  uint8_t* p_smem = ring_smem + AR_RING * AT_TILE_BYTES;      // two blocks of P, 32 KB each
+  float* xch = (float*)(p_smem + 4 * AT_TILE_BYTES);          // [2][AR_WARPS][32] maxima, sums
+  int4* table = (int4*)(xch + 2 * AR_WARPS * 32);             // [AR_TABLE] items of this block
+  volatile int* xflag = (volatile int*)(table + AR_TABLE);
+  uint64_t* bars = (uint64_t*)(xflag + AR_WARPS);
+  const uint32_t qfull = smem_u32(&bars[0]), qempty = smem_u32(&bars[1]);
+  const uint32_t tfull0 = smem_u32(&bars[2]), tempty0 = smem_u32(&bars[2 + AR_RING]);
+  const uint32_t sfull = smem_u32(&bars[2 + 2 * AR_RING]);
+  const uint32_t pready0 = smem_u32(&bars[3 + 2 * AR_RING]), pfree0 = smem_u32(&bars[5 + 2 * AR_RING]);  // [2] each
+  const uint32_t ofull = smem_u32(&bars[7 + 2 * AR_RING]), oempty = smem_u32(&bars[8 + 2 * AR_RING]);
+  const uint32_t clean0 = smem_u32(&bars[9 + 2 * AR_RING]);  // [AR_RING]
+  uint32_t* tmem_slot = (uint32_t*)(bars + 9 + 3 * AR_RING);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int k = 0; k < 2; k++) {
-      uint64_t* b = bars0 + k * AR_BARS;
-      for (int a = 0; a < AR_BARS; a++) {
-        const bool by_group = a == 3 || a == 4 || a == 7;  // sempty, pready, oempty
-        mbar_init(smem_u32(&b[a]), by_group ? AT_GROUP_WARPS : 1);
-      }
+    mbar_init(qfull, 1); mbar_init(qempty, 1); mbar_init(sfull, 1); mbar_init(ofull, 1);
+    mbar_init(oempty, AR_WARPS);
+    for (int s = 0; s < AR_RING; s++) {
+      mbar_init(tfull0 + 8 * s, 1);
+      mbar_init(tempty0 + 8 * s, 1 + (kPacked ? CLEAR_WARPS : 0));
+      mbar_init(clean0 + 8 * s, CLEAR_WARPS);
     }
+    for (int b = 0; b < 2; b++) { mbar_init(pready0 + 8 * b, AR_WARPS); mbar_init(pfree0 + 8 * b, 1); }
+    for (int i = 0; i < AR_WARPS; i++) xflag[i] = 0;
     *abort_flag = 0;
     *reinterpret_cast<volatile long long*>(abort_flag + 1) = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -917,19 +944,12 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const uint32_t tmem_base = *tmem_slot;
   pdl_begin();
   // Items: packed batches list the query tiles that exist, those of the longest sequences first, so that
-  // dealing them out leaves the groups level; otherwise the query tile is the slow index.
+  // dealing them out leaves the CTAs level; otherwise the query tile is the slow index.
   const int nzh = p.items / ((p.S + 127) >> 7);
   const int n_items = kPacked ? p.rows[2] * p.heads : p.items;
-  const int step = 2 * (int)gridDim.x;
-  // every second row of the deal goes the other way round
-  auto place = [&](int k, int i) {
-    const int at = (int)blockIdx.x + k * (int)gridDim.x;
-    return i * step + (i & 1 ? step - 1 - at : at);
-  };
-  auto count = [&](int k) { const int full = n_items / step; return full + (place(k, full) < n_items ? 1 : 0); };
-  const int n_my = count(g);
-  auto describe = [&](int k, int i) -> int4 {  // {first row of the sequence, its length, sequence, query tile and head}
-    const int w = place(k, i);
+  const int n_my = (int)blockIdx.x < n_items ? (n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  auto describe = [&](int i) -> int4 {  // {first row of the sequence, its length, sequence, query tile and head}
+    const int w = (int)blockIdx.x + i * (int)gridDim.x;
     int zo, zi, qt;
     if (kPacked) {
       const int e = w / p.heads;
@@ -945,289 +965,243 @@ attn_fwd_rows_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     return make_int4(kPacked ? p.cu[zo] : zo * p.S, min(max(len, 1), p.S), zo, qt << 24 | zi);
   };
   // Every role needs these words at the start of every item, and read from memory one after another they held up each
-  // item by 0.7 us.  So all are fetched once; a block of one item a group has nothing to gain.
-  const int most = max(count(0), count(1));
-  const int listed = most > 1 ? min(most, AR_TABLE) : 0;
+  // item by 0.7 us (64 sequences x 12 heads x 256 keys: 50.0 us without lengths, 58.6 with).  So all are fetched once;
+  // a block of a single item has nothing to gain (5 x 12 x 256: 8.5 us, 9.0 by way of the table).
+  const int listed = n_my > 1 ? min(n_my, AR_TABLE) : 0;
   if (listed) {
-    for (int t = threadIdx.x; t < 2 * listed; t += blockDim.x) {
-      const int k = t / listed, i = t - k * listed;
-      if (i < count(k)) table0[k * AR_TABLE + i] = describe(k, i);
-    }
+    for (int i = threadIdx.x; i < listed; i += blockDim.x) table[i] = describe(i);
     __syncthreads();
   }
-  auto item = [&](int i) -> int4 { return i < listed ? table[i] : describe(g, i); };
-  // A walk over the key blocks of the group's items, query tiles in the padding left out.
-  struct Cursor { int i, j, n; int4 it; };
-  auto advance = [&](Cursor& c) -> bool {
-    if (++c.j < c.n) return true;
-    while (++c.i < n_my) {
-      c.it = item(c.i);
-      if ((c.it.w >> 24) * 128 >= c.it.y) continue;
-      c.j = 0;
-      c.n = (c.it.y + 127) >> 7;
-      return true;
-    }
-    c.n = 0;
-    return false;
-  };
-  const Cursor start = {-1, 0, 0, make_int4(0, 0, 0, 0)};
+  auto item = [&](int i) -> int4 { return i < listed ? table[i] : describe(i); };
+  // column of the context accumulator, and the key block it lies in
+  auto o_block = [](int n) { return n == 4 ? 0 : 3; };
+  auto o_col = [](int n) { return n == 4 ? 0u : 448u; };
 
-  if ((warp == 0 || warp == 10) && !p.starve && elect_one()) {
-    // ------------------------------- TMA producers -------------------------------
+  if (warp == 0 && !p.starve && elect_one()) {
+    // ------------------------------- TMA producer -------------------------------
     bool ok = true;
-    uint32_t tt = 0, items = 0;
-    auto load = [&](const Cursor& c, bool is_v) {
-      const uint32_t slot = tt % AR_RING;
-      if (!mbar_wait(tempty0 + 8 * slot, ((tt / AR_RING) & 1) ^ 1, abort_flag, p.status)) { ok = false; return; }
-      mbar_expect_tx(tfull0 + 8 * slot, AT_TILE_BYTES);
-      const int* perm = is_v ? p.v_perm : p.k_perm;
-      int x[4];
-      x[0] = 0; x[perm[0]] = (kPacked ? c.it.x : 0) + c.j * 128; x[perm[1]] = c.it.w & 0xffffff; x[perm[2]] = kPacked ? 0 : c.it.z;
-      tma_load_4d(smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES), is_v ? &tmV : &tmK, tfull0 + 8 * slot, x[0], x[1], x[2], x[3]);
-      tt++;
-    };
-    auto load_key = [&](const Cursor& c) {
-      if (c.j == 0) {
-        if (!mbar_wait(qempty, (items & 1) ^ 1, abort_flag, p.status)) { ok = false; return; }
-        items++;
-        mbar_expect_tx(qfull, AT_TILE_BYTES);
-        int x[4];
-        x[0] = 0; x[p.q_perm[0]] = (kPacked ? c.it.x : 0) + (c.it.w >> 24) * 128; x[p.q_perm[1]] = c.it.w & 0xffffff;
-        x[p.q_perm[2]] = kPacked ? 0 : c.it.z;
-        tma_load_4d(smem_u32(q_smem), &tmQ, qfull, x[0], x[1], x[2], x[3]);
+    uint32_t tt = 0, ig = 0;
+    for (int i = 0; i < n_my && ok; i++) {
+      const int4 it = item(i);
+      const int len = it.y, zi = it.w & 0xffffff, qt = it.w >> 24;
+      if (qt * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      const int row0 = kPacked ? it.x : 0, zseq = kPacked ? 0 : it.z;
+      if (!mbar_wait(qempty, (ig & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+      ig++;
+      int c[4];
+      c[0] = 0; c[p.q_perm[0]] = row0 + qt * 128; c[p.q_perm[1]] = zi; c[p.q_perm[2]] = zseq;
+      mbar_expect_tx(qfull, AT_TILE_BYTES);
+      tma_load_4d(smem_u32(smem), &tmQ, qfull, c[0], c[1], c[2], c[3]);
+      for (int k = 0; k < 2 * n; k++, tt++) {
+        const bool is_v = k >= n;
+        const uint32_t slot = tt % AR_RING, round = tt / AR_RING;
+        if (!mbar_wait(tempty0 + 8 * slot, (round & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        mbar_expect_tx(tfull0 + 8 * slot, AT_TILE_BYTES);
+        const int* perm = is_v ? p.v_perm : p.k_perm;
+        c[0] = 0; c[perm[0]] = row0 + (is_v ? k - n : k) * 128; c[perm[1]] = zi; c[perm[2]] = zseq;
+        tma_load_4d(smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES), is_v ? &tmV : &tmK, tfull0 + 8 * slot, c[0], c[1], c[2], c[3]);
       }
-      load(c, false);
-    };
-    Cursor cs = start, cv = start;
-    if (advance(cs)) load_key(cs);
-    while (ok && advance(cv)) {
-      if (advance(cs)) load_key(cs);
-      if (ok) load(cv, true);
     }
     if (!ok || *abort_flag) {  // give the copies in flight time to land before the CTA leaves
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 4000000ll) {}
     }
-  } else if ((warp == 1 || warp == 11) && elect_one()) {
-    // ------------------------------- MMA issuers -------------------------------
+  } else if (warp == 1 && elect_one()) {
+    // ------------------------------- MMA issuer -------------------------------
     bool ok = true;
     const uint32_t hi = (uint32_t)(make_smem_desc(0, 16) >> 32);
     const uint32_t lbo_mn_lo = (uint32_t)make_smem_desc(0, 64 * BK * 2);
-    const uint32_t q_lo = (uint32_t)make_smem_desc(smem_u32(q_smem), 16);
-    const uint32_t p_lo = (uint32_t)make_smem_desc(smem_u32(p_smem), 16);
-    const uint32_t s_tmem = tmem_base + g * 128, o_tmem = tmem_base + AT_O_COL + g * 64;
-    uint32_t tt = 0, ns = 0, np = 0, qi = 0, oi = 0;  // ring tiles, score and second products, items of each
-    auto scores = [&](const Cursor& c) -> bool {       // S_j = Q K_j^T
-      const uint32_t slot = tt % AR_RING;
-      if (c.j == 0 && !mbar_wait(qfull, qi++ & 1, abort_flag, p.status)) return false;
-      if (!mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status)) return false;
-      if (!mbar_wait(sempty, (ns & 1) ^ 1, abort_flag, p.status)) return false;
-      tc_fence_after();
-      const uint32_t k_lo = (uint32_t)make_smem_desc(smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES), 16);
-#pragma unroll
-      for (int k = 0; k < BK / UMMA_K; k++) {
-        const uint64_t ad = ((uint64_t)hi << 32) | (q_lo + k * (UMMA_K * 2 / 16));
-        const uint64_t bd = ((uint64_t)hi << 32) | (k_lo + k * (UMMA_K * 2 / 16));
-        tc_mma(s_tmem, ad, bd, p.idesc_s, k > 0 ? 1u : 0u);
-      }
-      tc_commit(sfull);
-      tc_commit(tempty0 + 8 * slot);
-      if (c.j == c.n - 1) tc_commit(qempty);
-      ns++;
-      tt++;
-      return true;
-    };
-    auto context = [&](const Cursor& c) -> bool {      // C (+)= P_j V_j
-      const uint32_t slot = tt % AR_RING;
-      const int keys = c.it.y - c.j * 128;             // left of the sequence
-      if (c.j == 0 && !mbar_wait(oempty, (oi++ & 1) ^ 1, abort_flag, p.status)) return false;
-      if (!mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status) || !mbar_wait(pready, np & 1, abort_flag, p.status))
-        return false;
-      tc_fence_after();
-      const uint32_t v_lo = lbo_mn_lo | ((smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES) & 0x3FFFFu) >> 4);
-#pragma unroll
-      for (int kb = 0; kb < 2; kb++)
+    const uint32_t q_lo = (uint32_t)make_smem_desc(smem_u32(smem), 16);
+    uint32_t tt = 0, pv = 0, ig = 0;  // ring tiles, second products, items
+    uint32_t cleaned = 0;             // parity of every slot's clean barrier
+    int n_prev = 0;
+    for (int i = 0; i < n_my && ok; i++) {
+      const int4 it = item(i);
+      const int len = it.y;
+      if ((it.w >> 24) * 128 >= len) continue;
+      const int n = (len + 127) >> 7;
+      if (!mbar_wait(qfull, ig & 1, abort_flag, p.status)) { ok = false; break; }
+      auto scores = [&](int j) -> bool {  // S_j = Q K_j^T
+        const uint32_t pos = tt + j, slot = pos % AR_RING;
+        if (!mbar_wait(tfull0 + 8 * slot, (pos / AR_RING) & 1, abort_flag, p.status)) return false;
+        tc_fence_after();
+        const uint32_t k_lo = (uint32_t)make_smem_desc(smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES), 16);
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; k++) {
-          if (kPacked && kb * BK + k * UMMA_K >= keys) continue;
-          const uint64_t ad = ((uint64_t)hi << 32) | (p_lo + kb * (AT_TILE_BYTES / 16) + k * (UMMA_K * 2 / 16));
-          const uint64_t bd = ((uint64_t)hi << 32) | (v_lo + kb * (AT_TILE_BYTES / 2 / 16) + k * (UMMA_K * 128 / 16));
-          tc_mma(o_tmem, ad, bd, p.idesc_o, (c.j > 0 || kb > 0 || k > 0) ? 1u : 0u);
+          const uint64_t ad = ((uint64_t)hi << 32) | (q_lo + k * (UMMA_K * 2 / 16));
+          const uint64_t bd = ((uint64_t)hi << 32) | (k_lo + k * (UMMA_K * 2 / 16));
+          tc_mma(tmem_base + j * 128, ad, bd, p.idesc_s, k > 0 ? 1u : 0u);
         }
-      tc_commit(pfree);
-      tc_commit(tempty0 + 8 * slot);
-      if (c.j == c.n - 1) tc_commit(ofull);
-      np++;
-      tt++;
-      return true;
-    };
-    Cursor cs = start, cv = start;
-    if (advance(cs)) ok = scores(cs);
-    while (ok && advance(cv)) {
-      if (advance(cs)) ok = scores(cs);
-      if (ok) ok = context(cv);
+        tc_commit(tempty0 + 8 * slot);
+        return true;
+      };
+      // The scores of the item before have been read (its P blocks were waited for below); only the block
+      // its context lies in has to wait until that context has been read.
+      const int held = n_prev ? o_block(n_prev) : -1;
+      for (int j = 0; j < n && ok; j++)
+        if (j != held) ok = scores(j);
+      if (ok && n_prev && !mbar_wait(oempty, (ig & 1) ^ 1, abort_flag, p.status)) ok = false;
+      if (ok && held >= 0 && held < n) ok = scores(held);
+      if (!ok) break;
+      tc_commit(sfull);
+      tc_commit(qempty);
+      tt += n;
+      for (int j = 0; j < n; j++, pv++, tt++) {  // C (+)= P_j V_j
+        const uint32_t slot = tt % AR_RING, b = pv & 1;
+        const bool edge = kPacked && (j + 1) * 128 > len;
+        if (!mbar_wait(pready0 + 8 * b, (pv >> 1) & 1, abort_flag, p.status) ||
+            !mbar_wait(edge ? clean0 + 8 * slot : tfull0 + 8 * slot, edge ? (cleaned >> slot) & 1 : (tt / AR_RING) & 1, abort_flag,
+                       p.status)) { ok = false; break; }
+        if (edge) cleaned ^= 1u << slot;
+        tc_fence_after();
+        const uint32_t p_lo = (uint32_t)make_smem_desc(smem_u32(p_smem + b * 2 * AT_TILE_BYTES), 16);
+        const uint32_t v_lo = lbo_mn_lo | ((smem_u32(ring_smem + (size_t)slot * AT_TILE_BYTES) & 0x3FFFFu) >> 4);
+#pragma unroll
+        for (int kb = 0; kb < 2; kb++)
+#pragma unroll
+          for (int k = 0; k < BK / UMMA_K; k++) {
+            const uint64_t ad = ((uint64_t)hi << 32) | (p_lo + kb * (AT_TILE_BYTES / 16) + k * (UMMA_K * 2 / 16));
+            const uint64_t bd = ((uint64_t)hi << 32) | (v_lo + kb * (AT_TILE_BYTES / 2 / 16) + k * (UMMA_K * 128 / 16));
+            tc_mma(tmem_base + o_col(n), ad, bd, p.idesc_o, (j > 0 || kb > 0 || k > 0) ? 1u : 0u);
+          }
+        tc_commit(pfree0 + 8 * b);
+        tc_commit(tempty0 + 8 * slot);
+      }
+      if (ok) tc_commit(ofull);
+      ig++;
+      n_prev = n;
     }
     if (!ok || *abort_flag) {  // make sure no MMA is still writing tensor memory before it is freed
       tc_commit(sfull);
       const long long t0 = now_cycles();
       while (now_cycles() - t0 < 2000000ll) {}
     }
-  } else if (warp >= 2 && warp < 10) {
-    // ------------------------------- softmax groups -------------------------------
-    const int q = warp & 3;       // TMEM lane quarter this warp may read
-    const int r = q * 32 + lane;  // query row this thread owns
+  } else if (kPacked && warp >= 2 + AR_WARPS) {
+    // ------------------------------- clearing of rows beyond the sequence -------------------------------
+    bool ok = true;
+    uint32_t tt = 0;
+    for (int i = 0; i < n_my && ok; i++) {
+      const int len = item(i).y, n = (len + 127) >> 7;
+      for (int k = 0; k < 2 * n; k++, tt++) {
+        const uint32_t slot = tt % AR_RING;
+        if (!mbar_wait(tfull0 + 8 * slot, (tt / AR_RING) & 1, abort_flag, p.status)) { ok = false; break; }
+        if (k == 2 * n - 1 && len < n * 128) {
+          clear_tile_rows(ring_smem + (size_t)slot * AT_TILE_BYTES, len - (n - 1) * 128, 128, threadIdx.x - AR_THREADS);
+          clear_done(clean0 + 8 * slot, lane);
+        }
+        if (lane == 0) mbar_arrive(tempty0 + 8 * slot);
+      }
+    }
+  } else if (warp >= 2) {
+    // ------------------------------- softmax warps -------------------------------
+    const int q = warp & 3, part = (warp - 2) >> 2;  // columns part * 32 .. of every key block
+    const int me = q * 4 + part;
+    const int r = q * 32 + lane;
     const float sl2 = p.scale * 1.4426950408889634f;
     const float2 k2 = splat2(sl2);
-    const uint32_t srow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)g * 128;
-    const uint32_t orow = tmem_base + ((uint32_t)(q * 32) << 16) + AT_O_COL + (uint32_t)g * 64;
-    uint8_t* prow = p_smem + r * 128;
+    const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16);
+    float* xsum = xch + AR_WARPS * 32;
     bool ok = true;
-    uint32_t nb = 0, ni = 0;  // key blocks and items so far
+    uint32_t pv = 0, ig = 0;
     for (int i = 0; i < n_my && ok; i++) {
       const int4 it = item(i);
       const int row0 = it.x, len = it.y, zi = it.w & 0xffffff, qt = it.w >> 24;
-      const bool row_ok = qt * 128 + r < (kPacked ? len : p.S);  // rows of the sequence that exist
-      bf16* crow = p.C + (long long)(row0 + qt * 128 + r) * p.c_ld + zi * p.c_bi;
+      const int rlim = kPacked ? len : p.S;  // rows of the sequence that exist
+      bf16* crow = p.C + (long long)(row0 + qt * 128 + r) * p.c_ld + zi * p.c_bi + part * 16;
+      const bool row_ok = qt * 128 + r < rlim;
       if (qt * 128 >= len) {
         // a query tile in the padding: zero context rows (finite, so that masked reads stay harmless)
         if (row_ok)
-          for (int e = 0; e < 8; e++) *reinterpret_cast<uint4*>(crow + 8 * e) = make_uint4(0, 0, 0, 0);
+          for (int e = 0; e < 2; e++) *reinterpret_cast<uint4*>(crow + 8 * e) = make_uint4(0, 0, 0, 0);
         continue;
       }
       const int n = (len + 127) >> 7;
-      float ref = 0.f;                          // the exponentials' reference
-      float2 sum = make_float2(0.f, 0.f), sumr = make_float2(0.f, 0.f);  // of the exponentials, and rounded
-      for (int j = 0; j < n && ok; j++, nb++) {
-        if (!mbar_wait(sfull, nb & 1, abort_flag, p.status)) { ok = false; break; }
-        tc_fence_after();
-        bool waited = false, again;
-        float2 part, partr;
-        do {
-          again = false;
-          part = partr = make_float2(0.f, 0.f);
-          float top = -INFINITY;                // largest score of the block
-          uint32_t s[2][32];
-          tc_ld32_issue(srow, s[0]);
+      if (!mbar_wait(sfull, ig & 1, abort_flag, p.status)) { ok = false; break; }
+      tc_fence_after();
+      uint32_t s[32];
+      auto load = [&](int j) {  // this thread's 32 scores of block j, keys beyond the sequence at -inf
+        tc_ld32_issue(trow + j * 128 + part * 32, s);
+        tc_ld32_wait(s);
+        const int k0 = j * 128 + part * 32;
+        if (k0 + 32 > len) {
 #pragma unroll
-          for (int c = 0; c < 4; c++) {
-            uint32_t(&x)[32] = s[c & 1];
-            tc_ld32_wait(x);
-            if (c < 3) tc_ld32_issue(srow + (c + 1) * 32, s[(c + 1) & 1]);
-            const int k0 = j * 128 + c * 32;
-            if (k0 + 32 > len) {                // keys beyond the sequence
-#pragma unroll
-              for (int e = 0; e < 32; e++)
-                if (k0 + e >= len) x[e] = 0xff800000u;
-            }
-            float m0 = -INFINITY, m1 = top;     // three-input maxima
-#pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-              m0 = fmaxf(fmaxf(m0, __uint_as_float(x[e])), __uint_as_float(x[e + 1]));
-              m1 = fmaxf(fmaxf(m1, __uint_as_float(x[e + 2])), __uint_as_float(x[e + 3]));
-            }
-            top = fmaxf(m0, m1);
-            if (j == 0 && c == 0 && !waited) ref = fmaxf(top, -1e30f);
-            if (c == 3) {
-              const bool over = (top - ref) * sl2 > 64.f;
-              if (__any_sync(0xffffffffu, over)) {
-                // a new reference for this warp's rows that need one; P of this block has not been handed over
-                const float to = over ? top : ref, f = fast_exp2((ref - to) * sl2);
-                ref = to;
-                sum = __fmul2_rn(sum, splat2(f));
-                sumr = __fmul2_rn(sumr, splat2(f));
-                if (j > 0) {                    // the products of the blocks before have completed: P was free
-#pragma unroll
-                  for (int h = 0; h < 2; h++) {
-                    tc_ld32_issue(orow + h * 32, s[0]);
-                    tc_ld32_wait(s[0]);
-#pragma unroll
-                    for (int e = 0; e < 32; e++) s[0][e] = __float_as_uint(__uint_as_float(s[0][e]) * f);
-                    tc_st32(orow + h * 32, s[0]);
-                  }
-                }
-                again = true;
-                break;
-              }
-              tc_fence_before();                // the scores have been read
-              __syncwarp();
-              if (lane == 0) mbar_arrive(sempty);
-            }
-            const float2 nm2 = splat2(-ref * sl2);
-            uint32_t h[16];
-#pragma unroll
-            for (int e = 0; e < 16; e++) {
-              const float2 a = __ffma2_rn(make_float2(__uint_as_float(x[2 * e]), __uint_as_float(x[2 * e + 1])), k2, nm2);
-              const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y));
-              part = __fadd2_rn(part, ea);
-              const __nv_bfloat162 pa = __float22bfloat162_rn(ea);
-              h[e] = *reinterpret_cast<const uint32_t*>(&pa);
-              partr = __fadd2_rn(partr, bf162_to_f2(h[e]));
-            }
-            if (!waited) {                      // the block before has been multiplied: P may be written
-              waited = true;
-              ok = __all_sync(0xffffffffu, mbar_wait(pfree, (nb & 1) ^ 1, abort_flag, p.status));
-            }
-#pragma unroll
-            for (int u = 0; u < 4; u++)
-              *reinterpret_cast<uint4*>(prow + (c >> 1) * AT_TILE_BYTES + ((((c & 1) * 4 + u) ^ (r & 7)) << 4)) =
-                  make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
-          }
-        } while (again && ok);
-        if (!ok) break;
-        sum = __fadd2_rn(sum, part);
-        sumr = __fadd2_rn(sumr, partr);
-        if (kPacked && q == 0 && j == n - 1 && (len & 15)) {
-          // position of the block's V tile in the ring: after the next block's K tile, if there is one
-          const uint32_t pos = 2 * nb + (i == n_my - 1 ? 1 : 2), slot = pos % AR_RING;
-          ok = __all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * slot, (pos / AR_RING) & 1, abort_flag, p.status));
-          if (!ok) break;
-          uint4* rows = reinterpret_cast<uint4*>(ring_smem + (size_t)slot * AT_TILE_BYTES);
-          const int end = ((len + 15) & ~15) - j * 128;
-          for (int v = (len - j * 128) * 8 + lane; v < end * 8; v += 32) rows[v] = make_uint4(0, 0, 0, 0);
+          for (int e = 0; e < 32; e++)
+            if (k0 + e >= len) s[e] = 0xff800000u;
         }
+      };
+      // pass 1: the row's maximum
+      float mx = -INFINITY;
+      for (int j = 0; j < n; j++) {
+        load(j);
+        float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < 32; e += 4) {
+          m0 = fmaxf(m0, __uint_as_float(s[e]));
+          m1 = fmaxf(m1, __uint_as_float(s[e + 1]));
+          m2 = fmaxf(m2, __uint_as_float(s[e + 2]));
+          m3 = fmaxf(m3, __uint_as_float(s[e + 3]));
+        }
+        mx = fmaxf(mx, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)));
+      }
+      xch[me * 32 + lane] = mx;
+      if (!quad_sync(xflag, me, (int)ig * 2 + 1, lane, abort_flag, p.status)) { ok = false; break; }
+#pragma unroll
+      for (int o = 0; o < 4; o++) mx = fmaxf(mx, xch[(q * 4 + o) * 32 + lane]);  // finite: one key is valid
+      // pass 2: exponentials, their sum, and P_j
+      const float2 nm2 = splat2(-mx * sl2);
+      float2 l0 = make_float2(0.f, 0.f);
+      for (int j = 0; j < n; j++, pv++) {
+        load(j);
+#pragma unroll
+        for (int e = 0; e < 16; e++) {
+          const float2 a = __ffma2_rn(make_float2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), k2, nm2);
+          const float2 ea = make_float2(fast_exp2(a.x), fast_exp2(a.y));
+          l0 = __fadd2_rn(l0, ea);
+          const __nv_bfloat162 pa = __float22bfloat162_rn(ea);
+          s[e] = *reinterpret_cast<const uint32_t*>(&pa);
+        }
+        const uint32_t b = pv & 1;
+        if (!mbar_wait(pfree0 + 8 * b, ((pv >> 1) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+        uint8_t* prow = p_smem + (b * 2 + (part >> 1)) * AT_TILE_BYTES + r * 128;
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+          *reinterpret_cast<uint4*>(prow + ((((part & 1) * 4 + c) ^ (r & 7)) << 4)) = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
         tc_fence_before();
-        fence_proxy_async_smem();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(pready);
+        if (lane == 0) mbar_arrive(pready0 + 8 * b);
       }
       if (!ok) break;
-      const float total = sum.x + sum.y;
-      if (p.lse && row_ok) p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = ref * sl2 + log2f(total);
-      if (!mbar_wait(ofull, ni & 1, abort_flag, p.status)) { ok = false; break; }
-      ni++;
+      xsum[me * 32 + lane] = l0.x + l0.y;
+      if (!quad_sync(xflag, me, (int)ig * 2 + 2, lane, abort_flag, p.status)) { ok = false; break; }
+      float sum = 0.f;
+#pragma unroll
+      for (int o = 0; o < 4; o++) sum += xsum[(q * 4 + o) * 32 + lane];
+      if (p.lse && part == 0 && row_ok) p.lse[zi * p.lse_ld + row0 + qt * 128 + r] = mx * sl2 + log2f(sum);
+      // the context: 16 of the row's 64 columns
+      if (!mbar_wait(ofull, ig & 1, abort_flag, p.status)) { ok = false; break; }
+      ig++;
       tc_fence_after();
-      uint32_t v[2][32];
-      tc_ld32_issue(orow, v[0]);
-      tc_ld32_issue(orow + 32, v[1]);
-      tc_ld32_wait(v[0]);
-      tc_ld32_wait(v[1]);
+      uint32_t v[16];
+      tc_ld16(trow + o_col(n) + part * 16, v);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(oempty);
       if (row_ok) {
-        const float2 il = splat2(1.0f / (sumr.x + sumr.y));
+        const float2 il = splat2(1.0f / sum);
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          float2 w[16];
+        for (int e = 0; e < 2; e++) {
+          uint4 o;
+          __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
-          for (int e = 0; e < 16; e++)
-            w[e] = __fmul2_rn(make_float2(__uint_as_float(v[h][2 * e]), __uint_as_float(v[h][2 * e + 1])), il);
-          if (p.fast_c) {
-            store_row32_bf16(crow + 32 * h, w);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 4; e++) {
-              uint4 o;
-              __nv_bfloat162* b = reinterpret_cast<__nv_bfloat162*>(&o);
-#pragma unroll
-              for (int t = 0; t < 4; t++) b[t] = __float22bfloat162_rn(w[4 * e + t]);
-              *reinterpret_cast<uint4*>(crow + 32 * h + 8 * e) = o;
-            }
-          }
+          for (int t = 0; t < 4; t++)
+            h[t] = __float22bfloat162_rn(__fmul2_rn(make_float2(__uint_as_float(v[8 * e + 2 * t]), __uint_as_float(v[8 * e + 2 * t + 1])), il));
+          *reinterpret_cast<uint4*>(crow + 8 * e) = o;
         }
       }
     }
-    if (kPacked) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
+    if (kPacked && warp < 2 + NUM_EPI_WARPS) zero_tail_rows(p.C, p.c_ld, p.heads * 64, p.rows);
   }
 
   tc_fence_before();
@@ -2063,12 +2037,12 @@ int attn_fwd_launch(const void* qkv, void* probs, void* ctx, const int* seq_lens
   if (rc) return rc;
   for (int i = 0; i < 3; i++) { p.q_perm[i] = mq.perm[i]; p.k_perm[i] = mk.perm[i]; p.v_perm[i] = mv.perm[i]; }
   if (long_rows && probs == nullptr) {
-    const size_t smem_rows = (size_t)2 * AR_GROUP_TILES * AT_TILE_BYTES + 2 * AR_TABLE * 16 + 2 * AR_BARS * 8 + 32 + 1024;
+    const size_t smem_rows = (size_t)(1 + AR_RING + 4) * AT_TILE_BYTES + 2 * AR_WARPS * 32 * 4 + AR_TABLE * 16 + 1024 + 512;
     if ((int)smem_rows > smem_optin) { snprintf(err, 256, "attention: not enough shared memory"); return MSLT_ERR_CUDA; }
     const auto kernel = cu ? attn_fwd_rows_kernel<true> : attn_fwd_rows_kernel<false>;
     rc = attn_opt_in(kernel, &adev->attr_rows[cu != nullptr], smem_optin, err);
     if (rc) return rc;
-    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, AR_THREADS, smem_rows, st, mq.map, mk.map, mv.map, p);
+    launch_pdl(kernel, p.items < num_sms ? p.items : num_sms, AR_THREADS + (cu ? 32 * CLEAR_WARPS : 0), smem_rows, st, mq.map, mk.map, mv.map, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { snprintf(err, 256, "attention: launch failed: %s", cudaGetErrorString(e)); return MSLT_ERR_CUDA; }
     g_attn_launches++;
