@@ -90,9 +90,13 @@ __device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int r
   const uint32_t base = f32_smem(tile);
   if (p.splits == 1) __syncthreads();
   else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-  const int share = BMT / p.splits;
-  for (int idx = threadIdx.x; idx < share * (BNT / 4); idx += NT) {
-    const int r = rank * share + idx / (BNT / 4), c = (idx % (BNT / 4)) * 4;
+  // Beyond the output nothing is read: a read that no store waits for could be under way at the meeting below.
+  // (Tested piece by piece it keeps the reads of neighbouring pieces apart: 1 % of the split-operand kernel.)
+  const int share = BMT / p.splits, c = ((int)threadIdx.x % (BNT / 4)) * 4;
+  static_assert(NT % (BNT / 4) == 0, "a thread's pieces lie in the same columns");
+  const int rows = n0 + c < p.d.N ? min(share, p.d.M - m0 - rank * share) : 0;
+  for (int idx = threadIdx.x; idx < rows * (BNT / 4); idx += NT) {
+    const int r = rank * share + idx / (BNT / 4);
     const uint32_t at = base + (uint32_t)(r * PITCH + c) * 4u;
     Extra4 x;
     if (KG > 1) x = idx == (int)threadIdx.x ? mine : load_extra4(p, zoff, m0 + r, n0 + c);
@@ -117,7 +121,8 @@ __device__ __forceinline__ void cluster_add_and_finish(const F32Params& p, int r
     }
     epilogue4<(KG > 1)>(p, zoff, m0 + r, n0 + c, s, x);
   }
-  // no block leaves while its tile is read (nothing is ordered by this, so stores on their way do not hold it up)
+  // No block leaves while its tile is read.  The meeting orders no memory, so stores on their way do not hold it up;
+  // every read of a peer has returned by then, because what is stored was formed from it.
   if (p.splits > 1) asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait;" ::: "memory");
 }
 

@@ -287,6 +287,18 @@ def test_fp32_tiles_and_cluster_splits(shape, majors, form):
     _run(0, *shape, *majors, bias=not wgrad, d_fp32=True, accumulate=wgrad, form=(3, tile, tile, groups, splits))
 
 
+@pytest.mark.parametrize("shape,planes", [
+    ((1, 1, 2100), False), ((3, 41, 4000), False), ((33, 2, 1500), False), ((65, 66, 3000), False), ((130, 250, 2500), False),
+    ((129, 136, 4104), True), ((2, 304, 2064), True)])
+def test_fp32_clusters_with_little_output(shape, planes):
+    """Blocks of a cluster each finish a share of the tile's rows.  Here most shares, or their last columns, lie beyond
+    the output: such blocks read nothing from the others and leave at once, while theirs is still read."""
+    from paper_2011_13635_b200 import binding as Bd
+    for majors, kw in ((("k", "k"), dict(bias=True)), (("mn", "mn"), dict(accumulate=True)), (("k", "mn"), dict(residual=True))):
+        _run(0, *shape, *majors, d_fp32=True, planes=planes, **kw)
+        assert Bd.mslt_debug_last_gemm_form()[4] > 1
+
+
 @pytest.mark.parametrize("shape,majors,kw,form", [
     ((664, 1040, 16), ("k", "k"), dict(bias=True, act=1, aux_out=True), (32, 4, 1)),
     ((976, 744, 24), ("k", "k"), dict(residual=True), (32, 1, 1)),
