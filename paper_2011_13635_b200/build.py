@@ -2,8 +2,10 @@
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 import sys
+import tempfile
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -29,6 +31,22 @@ def needs_build() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _compile(src: str, obj: str):
+    return [_nvcc(), *[f for f in NVCC_FLAGS if f != "--use_fast_math=false"], "-Xptxas=-v", "-c",
+            os.path.join(CSRC, src), "-o", obj]
+
+
+def resource_usage(src: str) -> dict:
+    """Compiles one source file and returns what ptxas reports: {mangled kernel name: (registers, spilled bytes)}."""
+    with tempfile.TemporaryDirectory() as tmp:
+        r = subprocess.run(_compile(src, os.path.join(tmp, "out.o")), stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+    if r.returncode:
+        raise RuntimeError(f"nvcc failed on {src}")
+    found = re.findall(r"entry function '(\w+)'.*?(\d+) bytes spill stores, (\d+) bytes spill loads.*?Used (\d+) registers",
+                       r.stdout.decode(), re.S)
+    return {name: (int(regs), int(stores) + int(loads)) for name, stores, loads, regs in found}
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compiles every .cu of the library into one shared object; returns its path."""
     if not force and not needs_build():
@@ -39,11 +57,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     procs = []
     for src in SOURCES:
         obj = os.path.join(odir, src.replace(".cu", ".o"))
-        cmd = [_nvcc(), *[f for f in NVCC_FLAGS if f != "--use_fast_math=false"], "-c",
-               os.path.join(CSRC, src), "-o", obj]
-        if verbose:
-            cmd.insert(1, "-Xptxas=-v")
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
+        procs.append((src, subprocess.Popen(_compile(src, obj), stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
         objs.append(obj)
     for src, p in procs:
         out, _ = p.communicate()

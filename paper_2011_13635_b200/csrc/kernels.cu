@@ -70,36 +70,44 @@ __device__ __forceinline__ void ln_finish_row(float (&x)[LN_MAXE], int lane, int
   }
 }
 
+// A load that stays ahead of a wait behind it (the compiler may move one of constant data past it).
+__device__ __forceinline__ float4 load_now(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 // One warp normalises ROWS consecutive rows at once: all their 16-byte loads are issued before
 // the first reduction, which keeps enough bytes in flight to approach HBM bandwidth, and gamma /
 // beta are fetched once per column vector for all ROWS rows.  NV = 16-byte vectors per lane.
-template <typename T, int NV, int ROWS>
+//
+// kEarly: gamma and beta are parameters that no kernel of this call writes, so they are asked for ahead of the wait
+// for the preceding kernel (evaluation of one sequence, 25 such launches: 483 -> 452 us).  Held across the reductions
+// they cost a thread 50 registers (hidden 768: 74 -> 124, 1024: 96 -> 155), a third of the warps that fit, so this form
+// serves launches whose blocks are all resident at once (see launch_ln_fwd).
+template <typename T, int NV, int ROWS, bool kEarly>
 __global__ void __launch_bounds__(256)
 ln_fwd_kernel(const T* __restrict__ z, const float* __restrict__ gamma, const float* __restrict__ beta,
               T* __restrict__ y, float* __restrict__ stats, int rows, int H, float eps,
-              const int* __restrict__ rows_dev, int early) {
+              const int* __restrict__ rows_dev) {
   constexpr int VN = VecT<T>::N;
   typedef typename VecT<T>::Raw Raw;
   const int lane = threadIdx.x & 31;
-  // early: gamma and beta are parameters that no kernel of this call writes, so they are asked for ahead of the
-  // wait for the preceding kernel (evaluation of one sequence, 25 such launches: 483 -> 452 us)
-  float gv[NV * VN], bv[NV * VN];
-  auto load_affine = [&]() {
+  float gv[kEarly ? NV : 1][VN], bv[kEarly ? NV : 1][VN];
+  auto load_affine = [&](int c, float (&g)[VN], float (&b)[VN]) {
 #pragma unroll
-    for (int i = 0; i < NV; i++) {
-      const int c = (lane + 32 * i) * VN;
-      if (c < H) {
-#pragma unroll
-        for (int e = 0; e < VN; e += 4) {
-          const float4 g4 = *reinterpret_cast<const float4*>(gamma + c + e);
-          const float4 b4 = *reinterpret_cast<const float4*>(beta + c + e);
-          gv[i * VN + e] = g4.x; gv[i * VN + e + 1] = g4.y; gv[i * VN + e + 2] = g4.z; gv[i * VN + e + 3] = g4.w;
-          bv[i * VN + e] = b4.x; bv[i * VN + e + 1] = b4.y; bv[i * VN + e + 2] = b4.z; bv[i * VN + e + 3] = b4.w;
-        }
-      }
+    for (int e = 0; e < VN; e += 4) {
+      const float4 g4 = kEarly ? load_now(gamma + c + e) : *reinterpret_cast<const float4*>(gamma + c + e);
+      const float4 b4 = kEarly ? load_now(beta + c + e) : *reinterpret_cast<const float4*>(beta + c + e);
+      g[e] = g4.x; g[e + 1] = g4.y; g[e + 2] = g4.z; g[e + 3] = g4.w;
+      b[e] = b4.x; b[e + 1] = b4.y; b[e + 2] = b4.z; b[e + 3] = b4.w;
     }
   };
-  if (early) load_affine();
+  if (kEarly) {
+#pragma unroll
+    for (int i = 0; i < NV; i++)
+      if ((lane + 32 * i) * VN < H) load_affine((lane + 32 * i) * VN, gv[i], bv[i]);
+  }
   pdl_begin();
   if (rows_dev != nullptr) rows = rows_dev[1];
   const int row0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * ROWS;
@@ -112,7 +120,6 @@ ln_fwd_kernel(const T* __restrict__ z, const float* __restrict__ gamma, const fl
       const int c = (lane + 32 * i) * VN;
       if (c < H && row0 + r < rows) raw[r][i] = VecT<T>::load_raw(z + (int64_t)(row0 + r) * H + c);
     }
-  if (!early) load_affine();
   // One reduction round for both moments: sums of (x - x0) and (x - x0)^2 with x0 the first element
   // of the row, which keeps the subtraction var = E[d^2] - E[d]^2 well conditioned (x0 lies within
   // the spread of the row).
@@ -171,7 +178,8 @@ ln_fwd_kernel(const T* __restrict__ z, const float* __restrict__ gamma, const fl
   for (int i = 0; i < NV; i++) {
     const int c = (lane + 32 * i) * VN;
     if (c < H) {
-      const float *g = gv + i * VN, *b = bv + i * VN;
+      float(&g)[VN] = gv[kEarly ? i : 0], (&b)[VN] = bv[kEarly ? i : 0];
+      if (!kEarly) load_affine(c, g, b);
 #pragma unroll
       for (int r = 0; r < ROWS; r++) {
         if (row0 + r < rows) {
@@ -1652,9 +1660,17 @@ void launch_ln_fwd(bool bf, const void* z, const float* gamma, const float* beta
   if (rows <= 0) return;
   const int vn = bf ? 8 : 4;
   const int nv = (H + 32 * vn - 1) / (32 * vn);
+  // Early reads pay where no block waits for another to leave: 4 blocks of 128 threads an SM are resident at up to 124
+  // registers (hidden 768), 3 at 155 (1024), 2 above.  Evaluation by 9 layers, early | late: 768 wide, 480 blocks 856 |
+  // 884 us, 608 blocks 1050 | 1043; 1024 wide, 448 blocks 1180 | 1158.  Of a packed batch only the blocks that find
+  // rows stay, so half as many again are let in: 609 of which 430 stay, a step 2697 | 2743.
+  auto use_early = [&](int nv_, int blocks) {
+    const int resident = (nv_ <= 3 ? 4 : nv_ <= 4 ? 3 : 2) * 148;
+    return early && blocks <= (rows_dev ? resident * 3 / 2 : resident);
+  };
 #define LN_FWD(NV, ROWS)                                                                             \
-  DISPATCH_T(bf, (launch_pdl(ln_fwd_kernel<T, NV, ROWS>, div_up(rows, 4 * ROWS), 128, 0, st,                   \
-                     (const T*)z, gamma, beta, (T*)y, stats, rows, H, eps, rows_dev, early ? 1 : 0)))
+  DISPATCH_T(bf, (launch_pdl(use_early(NV, div_up(rows, 4 * ROWS)) ? ln_fwd_kernel<T, NV, ROWS, true> : ln_fwd_kernel<T, NV, ROWS, false>, \
+                     div_up(rows, 4 * ROWS), 128, 0, st, (const T*)z, gamma, beta, (T*)y, stats, rows, H, eps, rows_dev)))
   if (nv <= 1) LN_FWD(1, 4);
   else if (nv <= 2) LN_FWD(2, 2);
   else if (nv <= 3) LN_FWD(3, 2);
