@@ -581,9 +581,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if constexpr (kMode != EPI_GENERIC && !kSoftmax) {
       // The specialised flavours.  What keeps a tile's epilogue short enough to hide behind the
       // next tile's main loop: the work-item coordinates advance by mixed-radix addition (no
-      // division per tile); the bias of the NEXT tile is fetched while this tile is worked on; the
-      // TMEM read of the next chunk is in flight while the current chunk is converted and stored;
-      // and a lane stores its row segment straight from registers.
+      // division per tile); the bias of the NEXT tile is asked for when this one is done and arrives
+      // while that one is multiplied; the TMEM read of the next chunk is in flight while the current
+      // chunk is converted; and the result leaves through the copy engine or, where a tile store does
+      // not fit, as row segments straight from registers.
       constexpr bool kHasXf = kMode == EPI_RESIDUAL || kMode == EPI_DGELU;
       const bf16* xsrc = kMode == EPI_DGELU ? p.aux : kMode == EPI_RESIDUAL ? p.residual : nullptr;
       // This warp's i-th chunk, in units of 32 columns.  The two warps of a quarter interleave
@@ -607,12 +608,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       begin();
       if (!p.early && w_first < total_work) fetch_bias(at.nt, bcur);
       for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
-        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = p.part ? at.sp : p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
+        // Results by split, which are fp32, are addressed like a batch.  The store flavours spill 160 bytes with the test
+        // in them (us, with | without: 2400 x 2304 x 768 13.3 | 13.05, 4096 x 2304 x 768 15.5 | 15.2, 16384 x 768 x 768
+        // 20.3 | 19.9); GELU on pairs, where it is never true, spills 28 without it.
+        const bool by_split = (kMode == EPI_F32 || (kMode == EPI_GELU && kPair)) && p.part != 0;
+        const int zo = p.hdiv == 1 ? at.z : at.z / p.hdiv, zi = by_split ? at.sp : p.hdiv == 1 ? 0 : at.z - zo * p.hdiv;
         const uint32_t acc = tile & 1, use = tile >> 1;
         const int m_warp = at.mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp
         const int m = m_warp + lane;
         const bool row_ok = m < p.M;
-        const long long zoff = zo * p.d_bo + zi * (p.part ? p.part : p.d_bi);
+        const long long zoff = zo * p.d_bo + zi * (by_split ? p.part : p.d_bi);
         const long long off0 = zoff + (long long)m * p.ldd;
         const int n_base = at.nt * p.bn;
         const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 256;
@@ -630,10 +635,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
           }
         };
-        // the next work item and its bias (the loads travel while this tile is worked on)
         at.advance(p.n_tiles, m_tiles, p.batch);
-        const int nt2 = at.nt, mt2 = at.mt, z2 = at.z;
         if constexpr (kHasXf) {
+          const int nt2 = at.nt, mt2 = at.mt, z2 = at.z;
           // the next tile's rows of the extra operand start on their way to L2: they come from memory where
           // the operand is as large as the output.  This, the accumulator reads issued early and the interleaved
           // polynomials came in together; apart (us at 16384 rows; all three | without this | without early reads |
@@ -728,13 +732,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         } else {
           release_acc();
         }
-        if (w + w_step < total_work) fetch_bias(nt2, bcur);
+        // the next tile's bias travels until its products are there
+        if (w + w_step < total_work) fetch_bias(at.nt, bcur);
       }
     } else {
     begin();
     for (int w = w_first; w < total_work && ok; w += w_step, tile++) {
+      at.start(w, w_step, p.n_tiles, m_tiles, p.batch);  // these flavours have no registers to carry the digits in
       const int z = at.z, mt = at.mt, nt = at.nt;
-      at.advance(p.n_tiles, m_tiles, p.batch);
       const int zo = z / p.hdiv, zi = z - zo * p.hdiv;
       const uint32_t acc = tile & 1, use = tile >> 1;
       const int m_warp = mt * mt_rows + (int)cta_rank * BM + q * 32;  // first row of this warp

@@ -96,3 +96,14 @@ def test_layernorm_of_many_rows_leaves_room_for_warps():
         forms = {k: v for k, v in used.items() if f"ln_fwd_kernelI13__nv_bfloat16Li{vectors}E" in k}
         assert min(regs for regs, spilled in forms.values()) <= limit, forms
         assert all(spilled == 0 for regs, spilled in forms.values()), forms
+
+
+def test_contraction_flavours_do_not_spill():
+    """The epilogue warps of the specialised flavours run in the 168 registers that 384 threads leave them; what the
+    general one (6) needs beyond that goes to memory."""
+    from paper_2011_13635_b200 import build
+    used = build.resource_usage("gemm_tc.cu")
+    forms = {re.search(r"gemm_tc_kernelILi(\d+)ELb\dELi\dE", k)[0]: v for k, v in used.items() if "gemm_tc_kernel" in k}
+    assert len(forms) == 22
+    spilled = {k: v for k, v in forms.items() if v[1] and "ILi6E" not in k}
+    assert not spilled
