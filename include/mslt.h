@@ -356,6 +356,16 @@ int mslt_debug_set_gemm_variant(int32_t variant);
 int mslt_debug_last_gemm_form(int32_t out[5]);
 
 /*
+ * One contraction with the options that only the library's own steps use, for tests; synchronises.  d_rows (dtype 1,
+ * device, may be NULL): how many of the M rows hold anything, or with rows_are_k of the K; rows of the result beyond
+ * it are not written, operands between it and the next multiple of 128 of k must be zero.  b_static: B is not written
+ * by the two kernels before this one and may be read early.  parts (host, may be NULL; dtype 1, one fp32 output that is
+ * not accumulated, without rows, act, bias or residual): each split of k leaves its own result, M * ldd elements after
+ * the one before, and *parts receives their number, at most 8. */
+int mslt_debug_gemm_in_step(const mslt_gemm_desc* desc, void* cuda_stream, int32_t* d_status, const int32_t* d_rows,
+                            int32_t rows_are_k, int32_t b_static, int32_t* parts);
+
+/*
  * Memory-safety check for tests: every buffer the library carves out of the workspace is followed
  * by a 256-byte guard band that no kernel may write and that is zero from mslt_create on.  Counts
  * the guard bands that are no longer zero (*bad_out, host; 0 = no stray write).  Synchronises. */

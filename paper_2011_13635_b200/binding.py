@@ -61,7 +61,7 @@ EXPORTS = ["mslt_query_bytes", "mslt_create", "mslt_destroy", "mslt_add_layers",
            "mslt_op_layernorm_bwd", "mslt_op_softmax", "mslt_op_softmax_bwd", "mslt_op_colsum",
            "mslt_op_attention", "mslt_op_attention_bwd", "mslt_op_attention_lse", "mslt_op_attention_lse_bwd",
            "mslt_debug_starve_next_gemm", "mslt_debug_starve_next_attention", "mslt_debug_check_guards",
-           "mslt_debug_set_gemm_variant", "mslt_debug_last_gemm_form"]
+           "mslt_debug_set_gemm_variant", "mslt_debug_last_gemm_form", "mslt_debug_gemm_in_step"]
 
 lib.mslt_last_error.restype = C.c_char_p
 lib.mslt_last_error.argtypes = [C.c_void_p]
@@ -123,6 +123,7 @@ lib.mslt_debug_starve_next_gemm.argtypes = [C.c_int32]
 lib.mslt_debug_starve_next_attention.argtypes = [C.c_int32]
 lib.mslt_debug_set_gemm_variant.argtypes = [C.c_int32]
 lib.mslt_debug_last_gemm_form.argtypes = [C.POINTER(C.c_int32)]
+lib.mslt_debug_gemm_in_step.argtypes = [C.POINTER(GemmDesc), C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
 lib.mslt_debug_check_guards.argtypes = [C.c_void_p, C.POINTER(C.c_int32)]
 lib.mslt_op_layernorm.argtypes = [C.c_int32, _P, _P, _P, _P, _P, C.c_int32, C.c_int32, C.c_float, _P, C.c_int32]
 lib.mslt_op_layernorm_bwd.argtypes = [C.c_int32, _P, _P, _P, _P, _P, _P, _P, _P, C.c_int32, C.c_int32, _P, C.c_int32]
@@ -163,6 +164,15 @@ def mslt_op_gemm(desc: GemmDesc, stream: int, status) -> None:
 
 def mslt_op_gemm_enqueue(desc: GemmDesc, stream: int, status) -> None:
     _check(lib.mslt_op_gemm_enqueue(C.byref(desc), C.c_void_p(stream), C.c_void_p(_ptr(status))))
+
+
+def mslt_debug_gemm_in_step(desc: GemmDesc, stream: int, status, rows=None, rows_are_k: bool = False,
+                            b_static: bool = False, parts: bool = False) -> int:
+    """rows: int32 CUDA tensor of one element or None.  Returns the number of results."""
+    n = C.c_int32(1)
+    _check(lib.mslt_debug_gemm_in_step(C.byref(desc), stream, status.data_ptr(), _ptr(rows), int(rows_are_k), int(b_static),
+                                       C.byref(n) if parts else None))
+    return n.value
 
 
 def mslt_debug_last_gemm_form() -> tuple:

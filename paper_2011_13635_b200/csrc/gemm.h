@@ -15,7 +15,7 @@ namespace mslt {
 // rows (dtype 1 only, may be null): device count <= M, or <= K with rows_are_k, of the rows that hold
 // anything; work is cut to it (row results beyond it are not written).  b_static: B is written by neither
 // of the two kernels before this one in the stream (weights inside a step), so it may be read early.
-// parts (fp32 output, not accumulated): the splits of k leave a result each, M * ldd elements after the one before,
+// parts (one fp32 output of all rows, not accumulated, alpha its only epilogue): the splits of k leave a result each, M * ldd elements after the one before,
 // instead of adding to one; their number (at most kMaxParts) is returned, the caller adds them in order.
 constexpr int kMaxParts = 8;
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows = nullptr,

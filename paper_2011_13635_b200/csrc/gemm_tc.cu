@@ -1073,8 +1073,8 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const int num_sms = di.num_sms, smem_optin = di.smem_optin;
   if (!status) { snprintf(err, 256, "gemm: the tensor-core kernel needs a device status word"); return MSLT_ERR_ARG; }
   // every argument check comes before a form is chosen: there is none for an epilogue that does not exist
-  if (parts && (!d.d_fp32 || d.accumulate || d.batch != 1 || d.split_k > kMaxParts)) {
-    snprintf(err, 256, "gemm: results by split need one fp32 output that is not accumulated");
+  if (parts && (!d.d_fp32 || d.accumulate || d.batch != 1 || d.split_k > kMaxParts || rows || d.act || d.bias || d.residual)) {
+    snprintf(err, 256, "gemm: results by split need one fp32 output of all rows that is not accumulated, at most %d splits and no epilogue", kMaxParts);
     return MSLT_ERR_ARG;
   }
   if (d.split_k > 1 && !(d.d_fp32 && (d.accumulate || parts))) {
@@ -1151,7 +1151,9 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.seq_lens = d.seq_lens;
   p.rows = rows;
   p.rows_are_k = rows_are_k;
-  p.early = b_static && !starve ? 1 : 0;
+  // Tiles asked for before the device row count is known are those of the first item as the host sees it.  The count
+  // changes which k a split covers where rows are k, and which batch or split an item belongs to where there are several.
+  p.early = b_static && !starve && (!rows || (!rows_are_k && d.batch * p.splits == 1)) ? 1 : 0;
   p.wait_limit = WAIT_LIMIT_CYCLES;
   if (starve) {  // armed by mslt_debug_starve_next_gemm
     p.starve = 1;

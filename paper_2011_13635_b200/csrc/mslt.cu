@@ -1462,6 +1462,17 @@ int mslt_op_gemm(const mslt_gemm_desc* d, void* cuda_stream, int32_t* d_status) 
   return read_gemm_status(d_status, (cudaStream_t)cuda_stream);
 }
 
+int mslt_debug_gemm_in_step(const mslt_gemm_desc* d, void* cuda_stream, int32_t* d_status, const int32_t* d_rows, int32_t rows_are_k,
+                            int32_t b_static, int32_t* parts) {
+  TRY(check_gemm_desc(d));
+  if (!d_status) return fail(MSLT_ERR_ARG, "null pointer");
+  char err[256] = "";
+  int rc = gemm_launch(*d, d_status, (cudaStream_t)cuda_stream, err, d_rows, rows_are_k, b_static != 0, parts);
+  if (rc) return fail(rc, "%s", err);
+  CUDA_TRY(cudaGetLastError());
+  return read_gemm_status(d_status, (cudaStream_t)cuda_stream);
+}
+
 int mslt_debug_last_gemm_form(int32_t out[5]) {
   if (!out) return fail(MSLT_ERR_ARG, "null pointer");
   const GemmForm& f = g_gemm_form;

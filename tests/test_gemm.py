@@ -416,6 +416,99 @@ def test_bf16_descriptors_without_a_kernel_are_refused(N, kw):
         assert ei.value.code == -1
 
 
+def _in_step_operands(M, N, K, batch=1, majors="kk", d_fp32=True):
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(M + N + K)
+    make = lambda rows, major: torch.randn((batch, rows, K) if major == "k" else (batch, K, rows), device="cuda",  # noqa: E731
+                                           generator=gen).bfloat16()
+    A, B = make(M, majors[0]), make(N, majors[1])
+    d = Bd.GemmDesc()
+    d.dtype, d.M, d.N, d.K, d.batch, d.hdiv, d.alpha = 1, M, N, K, batch, 1, 1.0
+    d.A, d.a_bo = A.data_ptr(), M * K
+    d.a_rs, d.a_ks = (K, 1) if majors[0] == "k" else (1, M)
+    d.B, d.b_bo = B.data_ptr(), N * K
+    d.b_rs, d.b_ks = (K, 1) if majors[1] == "k" else (1, N)
+    d.d_fp32, d.ldd = int(d_fp32), (N + 7) // 8 * 8
+    d.d_bo = M * d.ldd
+    return d, A, B
+
+
+@pytest.mark.parametrize("M,N,K,split_k", [(2560, 768, 30520, 7), (300, 1032, 4104, 8), (33, 192, 1040, 0), (520, 100, 2048, 3), (40, 64, 64, 0)])
+def test_bf16_results_by_split(M, N, K, split_k):
+    """Each split's sum over its own k, in its own result: added in their order they give the product, and nothing
+    beyond the number that is reported is written.  k is cut at multiples of 128, the last split takes the rest."""
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    d, A, B = _in_step_operands(M, N, K)
+    D = torch.full((9, M, d.ldd), 7.0, device="cuda")
+    d.D, d.split_k = D.data_ptr(), split_k
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    parts = Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, parts=True)
+    assert parts == Bd.mslt_debug_last_gemm_form()[4] and parts <= 8 and parts <= max(split_k, 1 if K < 512 else 8)
+    per = (-(-K // 128) + parts - 1) // parts * 128 if split_k else None
+    a, b = A[0].double(), B[0].double()
+    top = (a @ b.t()).abs().max().item()
+    if per:
+        for i in range(parts):
+            want = a[:, i * per:(i + 1) * per] @ b[:, i * per:(i + 1) * per].t()
+            assert (D[i, :, :N].double() - want).abs().max().item() < 2e-5 * top
+    assert (D[:parts, :, :N].double().sum(0) - a @ b.t()).abs().max().item() < 2e-5 * top
+    assert bool((D[parts:] == 7.0).all()) and bool((D[:, :, N:] == 7.0).all())
+
+
+@pytest.mark.parametrize("kw", [dict(bias=True), dict(act=1), dict(act=2), dict(residual=True), dict(accumulate=1), dict(d_fp32=0),
+                                dict(split_k=9), dict(rows=True), dict(batch=2)], ids=str)
+def test_bf16_results_by_split_without_a_kernel_are_refused(kw):
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    kw = dict(kw)
+    rows = torch.full((1,), 64, dtype=torch.int32, device="cuda") if kw.pop("rows", False) else None
+    d, A, B = _in_step_operands(64, 64, 1024, batch=kw.pop("batch", 1))
+    D = torch.zeros((9, 2, 64, 64), device="cuda")
+    extra = torch.zeros((2, 64, 64), device="cuda")
+    d.D = D.data_ptr()
+    if kw.pop("bias", False):
+        d.bias = extra.data_ptr()
+    if kw.pop("residual", False):
+        d.residual = extra.data_ptr()
+    d.aux = extra.data_ptr()
+    for k, v in kw.items():
+        setattr(d, k, v)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    with pytest.raises(Bd.MsltError) as ei:
+        Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, rows=rows, parts=True)
+    assert ei.value.code == -1
+
+
+@pytest.mark.parametrize("M,N,K,batch,count,rows_are_k,d_fp32", [
+    (520, 768, 768, 1, 300, False, False), (520, 768, 768, 1, 1, False, False), (4096, 768, 200, 1, 130, False, False),
+    (520, 136, 192, 3, 130, False, False), (1040, 264, 72, 2, 1040, False, True),
+    (768, 264, 4096, 1, 1000, True, True), (3072, 768, 8192, 1, 128, True, True), (136, 72, 2048, 1, 2048, True, True)])
+def test_bf16_weights_read_early_beside_a_device_row_count(M, N, K, batch, count, rows_are_k, d_fp32):
+    """b_static with a row count that only the device knows: the tiles of B that are asked for early are the ones that
+    are multiplied, whatever the count does to the split of k and to the place of a batch in the list of tiles."""
+    import torch
+    from paper_2011_13635_b200 import binding as Bd
+    d, A, B = _in_step_operands(M, N, K, batch, ("mn", "mn") if rows_are_k else ("k", "k"), d_fp32)
+    if rows_are_k:
+        A[:, count:] = 0
+        B[:, count:] = 0
+        d.accumulate = 1
+        want = (A[0].double().t() @ B[0].double())[None]
+    else:
+        want = A.double() @ B.double().transpose(1, 2)
+    D = torch.full((batch, M, d.ldd), 0.0 if rows_are_k else 7.0, device="cuda", dtype=torch.float32 if d_fp32 else torch.bfloat16)
+    d.D = D.data_ptr()
+    rows = torch.full((1,), count, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, rows=rows, rows_are_k=rows_are_k, b_static=True)
+    have = M if rows_are_k else count
+    err = (D[:, :have, :N].double() - want[:, :have]).abs().max().item() / want.abs().max().item()
+    assert err < (2e-5 if d_fp32 else 6e-3)
+    assert rows_are_k or bool((D[:, -(-count // 256) * 256:] == 7.0).all())
+
+
 def test_fp32_more_rows_than_narrow_tiles_can_index():
     """Over 65535 x 32 rows only the tiles of more rows fit the launch grid."""
     _run(0, 65535 * 32 + 70, 8, 8, "k", "k", bias=True, d_fp32=True, form=(3, 64, 64, 1, 1))
