@@ -361,7 +361,7 @@ int mslt_debug_last_gemm_form(int32_t out[5]);
  * it are not written, operands between it and the next multiple of 128 of k must be zero.  b_static: B is not written
  * by the two kernels before this one and may be read early.  parts (host, may be NULL; dtype 1, one fp32 output that is
  * not accumulated, without rows, act, bias or residual): each split of k leaves its own result, M * ldd elements after
- * the one before, and *parts receives their number, at most 8. */
+ * the one before; *parts is how many there is room for (8 are used at most) and receives their number. */
 int mslt_debug_gemm_in_step(const mslt_gemm_desc* desc, void* cuda_stream, int32_t* d_status, const int32_t* d_rows,
                             int32_t rows_are_k, int32_t b_static, int32_t* parts);
 

@@ -167,12 +167,12 @@ def mslt_op_gemm_enqueue(desc: GemmDesc, stream: int, status) -> None:
 
 
 def mslt_debug_gemm_in_step(desc: GemmDesc, stream: int, status, rows=None, rows_are_k: bool = False,
-                            b_static: bool = False, parts: bool = False) -> int:
-    """rows: int32 CUDA tensor of one element or None.  Returns the number of results."""
-    n = C.c_int32(1)
+                            b_static: bool = False, parts: int = 0) -> int:
+    """rows: int32 CUDA tensor of one element or None; parts: room for results by split.  Returns their number."""
+    n = C.c_int32(parts)
     _check(lib.mslt_debug_gemm_in_step(C.byref(desc), stream, status.data_ptr(), _ptr(rows), int(rows_are_k), int(b_static),
                                        C.byref(n) if parts else None))
-    return n.value
+    return n.value if parts else 1
 
 
 def mslt_debug_last_gemm_form() -> tuple:

@@ -21,12 +21,13 @@ int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err
     return MSLT_ERR_ARG;
   }
   int rc;
+  const int room = parts ? *parts : 0;
   if (parts) *parts = 1;
   if (d.dtype == 1) {
     // MSLT_BF16_CUDA_CORES=1 routes bf16 products to the CUDA-core kernel: a debugging aid for
     // telling a tensor-core kernel fault from an orchestration fault, never a silent fallback.
     static const bool cuda_cores = getenv("MSLT_BF16_CUDA_CORES") && atoi(getenv("MSLT_BF16_CUDA_CORES")) == 1;
-    rc = cuda_cores ? gemm_simt_launch(d, st, err) : gemm_tc_launch(d, status, st, err, rows, rows_are_k, b_static, parts);
+    rc = cuda_cores ? gemm_simt_launch(d, st, err) : gemm_tc_launch(d, status, st, err, rows, rows_are_k, b_static, parts, room);
   } else if (d.dtype == 0) {
     rc = gemm_f32_launch(d, st, err, b_static);
   } else {

@@ -16,7 +16,8 @@ namespace mslt {
 // anything; work is cut to it (row results beyond it are not written).  b_static: B is written by neither
 // of the two kernels before this one in the stream (weights inside a step), so it may be read early.
 // parts (one fp32 output of all rows, not accumulated, alpha its only epilogue): the splits of k leave a result each, M * ldd elements after the one before,
-// instead of adding to one; their number (at most kMaxParts) is returned, the caller adds them in order.
+// instead of adding to one; in: how many there is room for (kMaxParts are used at most), out: their number.  The caller
+// adds them in order.
 constexpr int kMaxParts = 8;
 int gemm_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows = nullptr,
                 int rows_are_k = 0, bool b_static = false, int* parts = nullptr);
@@ -35,7 +36,7 @@ int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void*
                       cudaStream_t st, char* err);
 int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
-                   bool b_static, int* parts);
+                   bool b_static, int* parts, int room);
 // The form for few tiles (gemm_tc_small.cu): split count and estimated time, 0 where it does not apply.
 int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, double* t);
 int gemm_tc_small_launch(const mslt_gemm_desc& d, int splits, bool early, int* status, cudaStream_t st, char* err,

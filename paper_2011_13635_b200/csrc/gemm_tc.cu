@@ -1053,7 +1053,7 @@ static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, i
 }
 
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
-                   bool b_static, int* parts) {
+                   bool b_static, int* parts, int room) {
   // the test hook is used up by this call even if an argument check below rejects it
   const bool starve = g_starve_next.exchange(0) != 0;
   int dev = 0;
@@ -1073,8 +1073,8 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const int num_sms = di.num_sms, smem_optin = di.smem_optin;
   if (!status) { snprintf(err, 256, "gemm: the tensor-core kernel needs a device status word"); return MSLT_ERR_ARG; }
   // every argument check comes before a form is chosen: there is none for an epilogue that does not exist
-  if (parts && (!d.d_fp32 || d.accumulate || d.batch != 1 || d.split_k > kMaxParts || rows || d.act || d.bias || d.residual)) {
-    snprintf(err, 256, "gemm: results by split need one fp32 output of all rows that is not accumulated, at most %d splits and no epilogue", kMaxParts);
+  if (parts && (!d.d_fp32 || d.accumulate || d.batch != 1 || room < 1 || d.split_k > std::min(room, kMaxParts) || rows || d.act || d.bias || d.residual)) {
+    snprintf(err, 256, "gemm: results by split need one fp32 output of all rows that is not accumulated, no epilogue, and room (at most %d are used)", kMaxParts);
     return MSLT_ERR_ARG;
   }
   if (d.split_k > 1 && !(d.d_fp32 && (d.accumulate || parts))) {
@@ -1092,7 +1092,7 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   p.a_mn = (d.a_rs == 1 && d.a_ks != 1) ? 1 : 0;
   p.b_mn = (d.b_rs == 1 && d.b_ks != 1) ? 1 : 0;
   const int variant = g_tile_variant.load();
-  const int max_splits = d.split_k != 0 || !d.d_fp32 ? 0 : d.accumulate ? 16 : parts ? kMaxParts : 0;
+  const int max_splits = d.split_k != 0 || !d.d_fp32 ? 0 : d.accumulate ? 16 : parts ? std::min(room, kMaxParts) : 0;
   bool pair = false;
   int splits = d.split_k > 1 ? d.split_k : 1, ksub = 1;
   // Where the row count is known on the device only, the form is chosen for part of what the launch has to reckon with:

@@ -309,7 +309,9 @@ void plan_workspace(const mslt_arch& a, const std::vector<Tensor>& tensors, char
   w.dlogits = take(R * Vp * E);
   w.nll = (float*)take(R * 4);
   w.dtm = take(R * H * E); w.dgt = take(R * H * E); w.dhm = take(R * H * E);
-  w.dtm32 = (float*)take(R * H * 4 * (a.dtype == 1 ? kMaxParts : 1));
+  // The fp32 sums of the head's input gradient (bf16) lie in the logits, which nothing reads once the loss has been taken;
+  // there is room for Vp / H of them.
+  w.dtm32 = a.dtype == 0 || Vp >= H ? w.logits : (float*)take(R * H * 4);
   if (a.nsp) {
     const int64_t Bm = a.max_batch;
     w.nsp_rowsrc = (int*)take(Bm * 4);
@@ -703,6 +705,9 @@ int head_forward(mslt_ctx* c, const void* x, int R, bool save) {
   return 0;
 }
 
+// How many results [R, H] of fp32 there is room for (see plan_workspace).
+int dtm_room(const mslt_ctx* c) { return std::min(kMaxParts, std::max(1, c->Vp / c->a.hidden)); }
+
 // Split count of the vocabulary-long contraction of the head's input gradient: the number that fills
 // the last wave of 256 x 256 tiles on CTA pairs.  Fixed here rather than left to the contraction's
 // own estimate, because this sum is rounded to bf16 and feeds the whole backward pass: with a fixed
@@ -713,7 +718,7 @@ int dtm_splits(const mslt_ctx* c, int R) {
   const long long tiles = (long long)((R + 255) / 256) * ((H + 255) / 256), units = c->num_sms / 2;
   int splits = 1;
   double best = 0.;
-  for (int sp = 1; sp <= kMaxParts && sp * 256 <= V; sp++) {
+  for (int sp = 1; sp <= dtm_room(c) && sp * 256 <= V; sp++) {
     if (sp > 1 && tiles >= 2 * units) break;
     const long long waves = (tiles * sp + units - 1) / units;
     const double e = (double)(tiles * sp) / (double)(waves * units);
@@ -735,7 +740,7 @@ int head_backward(mslt_ctx* c, int B, int S, int P, bool full) {
       // with fp32 partial sums, added in their order, then round once to bf16
       g.d.D = w.dtm32; g.d.ldd = H; g.d.d_fp32 = 1;
       g.d.split_k = dtm_splits(c, R);
-      int parts = 1;
+      int parts = dtm_room(c);
       TRY(run_gemm(c, g.d, nullptr, 0, false, false, false, false, &parts));
       KL(PC_OTHER, (4.0 * parts + 2.0) * R * H, launch_sum_parts(w.dtm32, (int64_t)R * H, parts, w.dtm, (int64_t)R * H, c->st));
     } else {

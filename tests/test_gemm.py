@@ -434,8 +434,10 @@ def _in_step_operands(M, N, K, batch=1, majors="kk", d_fp32=True):
     return d, A, B
 
 
-@pytest.mark.parametrize("M,N,K,split_k", [(2560, 768, 30520, 7), (300, 1032, 4104, 8), (33, 192, 1040, 0), (520, 100, 2048, 3), (40, 64, 64, 0)])
-def test_bf16_results_by_split(M, N, K, split_k):
+@pytest.mark.parametrize("M,N,K,split_k,room", [
+    (2560, 768, 30520, 7, 8), (300, 1032, 4104, 8, 39), (33, 192, 1040, 0, 5), (33, 192, 1040, 0, 2), (33, 192, 4104, 0, 1),
+    (520, 100, 2048, 3, 3), (40, 64, 64, 0, 8)])
+def test_bf16_results_by_split(M, N, K, split_k, room):
     """Each split's sum over its own k, in its own result: added in their order they give the product, and nothing
     beyond the number that is reported is written.  k is cut at multiples of 128, the last split takes the rest."""
     import torch
@@ -444,8 +446,8 @@ def test_bf16_results_by_split(M, N, K, split_k):
     D = torch.full((9, M, d.ldd), 7.0, device="cuda")
     d.D, d.split_k = D.data_ptr(), split_k
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    parts = Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, parts=True)
-    assert parts == Bd.mslt_debug_last_gemm_form()[4] and parts <= 8 and parts <= max(split_k, 1 if K < 512 else 8)
+    parts = Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, parts=room)
+    assert parts == Bd.mslt_debug_last_gemm_form()[4] and parts <= min(room, 8) and parts <= max(split_k, 1 if K < 512 else 8)
     per = (-(-K // 128) + parts - 1) // parts * 128 if split_k else None
     a, b = A[0].double(), B[0].double()
     top = (a @ b.t()).abs().max().item()
@@ -458,11 +460,12 @@ def test_bf16_results_by_split(M, N, K, split_k):
 
 
 @pytest.mark.parametrize("kw", [dict(bias=True), dict(act=1), dict(act=2), dict(residual=True), dict(accumulate=1), dict(d_fp32=0),
-                                dict(split_k=9), dict(rows=True), dict(batch=2)], ids=str)
+                                dict(split_k=9), dict(split_k=4, room=3), dict(room=-1), dict(rows=True), dict(batch=2)], ids=str)
 def test_bf16_results_by_split_without_a_kernel_are_refused(kw):
     import torch
     from paper_2011_13635_b200 import binding as Bd
     kw = dict(kw)
+    room = kw.pop("room", 8)
     rows = torch.full((1,), 64, dtype=torch.int32, device="cuda") if kw.pop("rows", False) else None
     d, A, B = _in_step_operands(64, 64, 1024, batch=kw.pop("batch", 1))
     D = torch.zeros((9, 2, 64, 64), device="cuda")
@@ -477,7 +480,7 @@ def test_bf16_results_by_split_without_a_kernel_are_refused(kw):
         setattr(d, k, v)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     with pytest.raises(Bd.MsltError) as ei:
-        Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, rows=rows, parts=True)
+        Bd.mslt_debug_gemm_in_step(d, torch.cuda.current_stream().cuda_stream, status, rows=rows, parts=room)
     assert ei.value.code == -1
 
 

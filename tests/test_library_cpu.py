@@ -86,6 +86,18 @@ def test_fp32_workspace_holds_planes_only_where_a_product_uses_them(binding):
     assert bytes_of(0, *base) > 2 * bytes_of(1, *base)
 
 
+@pytest.mark.parametrize("hidden,heads,vocab", [(768, 12, 30522), (1024, 16, 30522), (768, 12, 500)])
+def test_workspace_a_masked_slot_takes(binding, hidden, heads, vocab):
+    """A caller that keeps a workspace of a size queried once depends on it.  A slot takes its rows of the head (seven of
+    the hidden size in bf16), logits in fp32 and their gradient, five words, and at most one fp32 row for sums."""
+    sizes = []
+    for pred in (64, 128):
+        a = binding.Arch(hidden, heads, 4 * hidden, vocab, 512, 3, 12, 16, 128, pred, 1, 1e-12)
+        sizes.append(binding.mslt_query_bytes(a)[1])
+    padded = (vocab + 7) // 8 * 8
+    assert sizes[1] - sizes[0] <= 16 * 64 * (7 * 2 * hidden + 6 * padded + 20 + 4 * hidden)
+
+
 def test_layernorm_of_many_rows_leaves_room_for_warps():
     """Where blocks wait for others to leave, the registers of a thread decide how many bytes are on their way.  65536 of
     them are 6 blocks of 128 threads at 80 (hidden 768) and 5 at 96 (1024); with gamma and beta held across the

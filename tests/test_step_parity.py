@@ -246,6 +246,13 @@ def test_packed_batch_of_few_rows(batch, rest):
     m.close()
 
 
+@pytest.mark.parametrize("vocab,trainable", [(500, 1), (768, 2), (1700, 1)])
+def test_vocabulary_not_much_wider_than_the_hidden_state(vocab, trainable):
+    """The sums of the head's input gradient lie in the logits' memory: none fit beside a row of 500 logits, one in 768,
+    two in 1704."""
+    _run(I.scaled(I.CONFIGS["base_stage"], layers=2, trainable=trainable, batch=2, vocab=vocab), steps=2, lr=1e-4)
+
+
 @pytest.mark.parametrize("dtype,seq,varlen,pred", [("fp32", 40, None, 5), ("fp32", 72, (20, 72), 33), ("bf16", 136, (40, 136), 9),
                                                    ("bf16", 64, None, 40)])
 def test_slots_that_name_a_position_twice(dtype, seq, varlen, pred):
