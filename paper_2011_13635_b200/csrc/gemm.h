@@ -37,8 +37,15 @@ int gemm_f32x3_launch(const mslt_gemm_desc& d, const void* planes_a, const void*
 int gemm_simt_launch(const mslt_gemm_desc& d, cudaStream_t st, char* err);
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
                    bool b_static, int* parts, int room);
-// The form for few tiles (gemm_tc_small.cu): split count and estimated time, 0 where it does not apply.
-int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, double* t);
+// Shares of its rows that a product may turn out to have where only the device knows; one alone where the host does.
+struct Fills {
+  int n;
+  double share[3];
+  static int of(int rows, double share) { const int r = (int)(share * rows); return r < 1 ? 1 : r; }
+};
+constexpr Fills kFull = {1, {1.}}, kUnknownFill = {3, {0.4, 0.7, 1.}};
+// The form for few tiles (gemm_tc_small.cu): split count and estimated time (the mean over fills), 0 where it does not apply.
+int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, const Fills& fills, double* t);
 int gemm_tc_small_launch(const mslt_gemm_desc& d, int splits, bool early, int* status, cudaStream_t st, char* err,
                          const int* rows, bool starve);
 

@@ -1016,8 +1016,13 @@ std::mutex g_dev_mu;
 //   an epilogue that overlaps the next tile's loop, one more at the end;
 //   start-up (pairs have a cluster to set up); singles slow down a little when many waves of them
 //   contend for L2, where a pair fetches a third less per flop.
-static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, int max_splits, bool* pair, int* bn,
-                          int* ksub, int* splits) {
+// Where the row count (of k with rows_are_k) is known on the device only, the form is the best one for the middle of
+// fills, and its mean time over them is returned, for the comparison with the few-tile kernel.  Measured on 21 packed
+// batches (evaluations and steps, 1 x 128 to 128 x 128 and 8 x 512 to 16 x 512 tokens), each full, 0.95, 0.7, 0.4 and 0.1
+// filled: the form that is best on the mean of the fills is 1.3 % slower at 0.7 (5 % at worst) and 1.5 to 1.8 % faster at the
+// others (9 % at best).  Lengths between a quarter or a half of the longest and the longest leave 0.62 to 0.75 of a batch.
+static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, int max_splits, const Fills& fills, int rows_are_k,
+                            bool* pair, int* bn, int* ksub, int* splits) {
   struct Form { bool pair; int bn, ksub; double per_k; };
   static const Form forms[] = {{false, 64, 2, 0.202}, {false, 128, 2, 0.280}, {false, 192, 1, 0.362}, {false, 256, 1, 0.413},
                                {true, 128, 2, 0.240}, {true, 192, 2, 0.317}, {true, 256, 2, 0.383}};
@@ -1029,7 +1034,21 @@ static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, i
   else if (d.residual) { e0 = 1.2; e1 = 6.6; }
   const bool b_mn = d.b_rs == 1 && d.b_ks != 1;
   const bool pairs_ok = d.M > BM && d.act != 3 && num_sms % 2 == 0 && variant != 1;
-  const int kblocks = (d.K + BK - 1) / BK, fixed_splits = *splits;
+  const double likely = fills.share[fills.n / 2];
+  auto k_blocks = [&](double share) { return ((rows_are_k ? Fills::of(d.K, share) : d.K) + BK - 1) / BK; };
+  const int kblocks = k_blocks(1.), likely_blocks = k_blocks(likely), fixed_splits = *splits;
+  auto time = [&](const Form& f, int ks, int sp, double share) {
+    const int rows = f.pair ? 2 * BM : BM, units = f.pair ? num_sms / 2 : num_sms;
+    const int m = rows_are_k ? d.M : Fills::of(d.M, share);
+    const long long tiles = (long long)((m + rows - 1) / rows) * ((d.N + f.bn - 1) / f.bn) * d.batch;
+    const double epi = e0 + e1 * f.bn / 256.;
+    const double waves = (double)((tiles * sp + units - 1) / units);
+    const int kb = ((k_blocks(share) + sp - 1) / sp + ks - 1) / ks * ks;
+    const double loop = kb * f.per_k + 0.66;
+    const double crowd = f.pair ? 1. : 1. + 0.004 * (waves - 1 < 4 ? waves - 1 : 4);
+    return (f.pair ? 2.4 : 1.0) + waves * (loop > epi ? loop : epi) * crowd + (loop < epi ? loop : epi);
+  };
+  const Form* form = nullptr;
   double best = 1e30;
   for (const Form& f : forms) {
     if (f.bn > 64 && f.bn >= d.N + 64) continue;            // no wider than the output needs
@@ -1037,19 +1056,15 @@ static double choose_tiling(const mslt_gemm_desc& d, int num_sms, int variant, i
     if (f.pair && (!pairs_ok || (b_mn && f.bn % 128))) continue;  // row-contiguous B comes in 64-wide boxes
     if (!f.pair && variant == 2 && pairs_ok && d.N > 64) continue;
     const int ks = d.act == 3 || kblocks == 1 ? 1 : f.ksub;
-    const int rows = f.pair ? 2 * BM : BM, units = f.pair ? num_sms / 2 : num_sms;
-    const long long tiles = (long long)((d.M + rows - 1) / rows) * ((d.N + f.bn - 1) / f.bn) * d.batch;
-    const double epi = e0 + e1 * f.bn / 256.;
-    for (int sp = fixed_splits; sp == fixed_splits || (sp <= max_splits && sp * 4 <= kblocks); sp++) {
-      const double waves = (double)((tiles * sp + units - 1) / units);
-      const int kb = ((kblocks + sp - 1) / sp + ks - 1) / ks * ks;
-      const double loop = kb * f.per_k + 0.66;
-      const double crowd = f.pair ? 1. : 1. + 0.004 * (waves - 1 < 4 ? waves - 1 : 4);
-      const double t = (f.pair ? 2.4 : 1.0) + waves * (loop > epi ? loop : epi) * crowd + (loop < epi ? loop : epi);
-      if (t < best) { best = t; *pair = f.pair; *bn = f.bn; *ksub = f.pair ? 2 : ks; *splits = sp; }
+    for (int sp = fixed_splits; sp == fixed_splits || (sp <= max_splits && sp * 4 <= likely_blocks); sp++) {
+      const double t = time(f, ks, sp, likely);
+      if (t < best) { best = t; form = &f; *pair = f.pair; *bn = f.bn; *ksub = f.pair ? 2 : ks; *splits = sp; }
     }
   }
-  return best;
+  if (fills.n == 1 || !form) return best;
+  double mean = 0.;
+  for (int i = 0; i < fills.n; i++) mean += time(*form, *ksub, *splits, fills.share[i]) / fills.n;
+  return mean;
 }
 
 int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* err, const int* rows, int rows_are_k,
@@ -1095,16 +1110,10 @@ int gemm_tc_launch(const mslt_gemm_desc& d, int* status, cudaStream_t st, char* 
   const int max_splits = d.split_k != 0 || !d.d_fp32 ? 0 : d.accumulate ? 16 : parts ? std::min(room, kMaxParts) : 0;
   bool pair = false;
   int splits = d.split_k > 1 ? d.split_k : 1, ksub = 1;
-  // Where the row count is known on the device only, the form is chosen for part of what the launch has to reckon with:
-  // lengths between a quarter or a half of the longest and the longest leave 0.62 to 0.75 of a batch.
-  mslt_gemm_desc likely = d;
-  if (rows) {
-    int& n = rows_are_k ? likely.K : likely.M;
-    n = std::max(1, (int)(0.7 * n));
-  }
-  const double estimate = choose_tiling(likely, num_sms, variant, max_splits, &pair, &p.bn, &ksub, &splits);
+  const Fills fills = rows ? kUnknownFill : kFull;
+  const double estimate = choose_tiling(d, num_sms, variant, max_splits, fills, rows_are_k, &pair, &p.bn, &ksub, &splits);
   double t_small = 0.;
-  const int s_small = variant == 0 && g_store_variant.load() == 0 && !rows_are_k ? gemm_tc_small_plan(likely, num_sms, &t_small) : 0;
+  const int s_small = variant == 0 && g_store_variant.load() == 0 && !rows_are_k ? gemm_tc_small_plan(d, num_sms, fills, &t_small) : 0;
   if (s_small && t_small < estimate) return gemm_tc_small_launch(d, s_small, b_static, status, st, err, rows, starve);
   const int tile_m = pair ? 2 * BM : BM;
   p.m_tiles = (d.M + tile_m - 1) / tile_m;

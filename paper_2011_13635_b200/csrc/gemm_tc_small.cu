@@ -258,22 +258,35 @@ std::mutex g_attr_mu;
 }  // namespace
 
 // Split count with the least estimated time (microseconds, *t), or 0 where the kernel does not apply.
-int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, double* t) {
+int gemm_tc_small_plan(const mslt_gemm_desc& d, int num_sms, const Fills& fills, double* t) {
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
   if (d.batch != 1 || d.d_fp32 || d.act == 3 || d.N % 8 || d.ldd % 8 || !al16(d.D) || !al16(d.aux) || !al16(d.residual) ||
       !al16(d.bias) || (d.act == 2 && !d.aux))
     return 0;
-  const long long tiles = (long long)((d.M + BM - 1) / BM) * ((d.N + TS_BN - 1) / TS_BN);
   const int kb = (d.K + BK - 1) / BK;
   int best = 0;
   for (int s = 1; s <= 8; s *= 2) {
     const int per = (kb + s - 1) / s;
     if (s > 1 && per < 2) continue;
-    if (tiles * s > (s >= 4 ? num_sms * (s == 4 ? 8 : 7) / 9 : num_sms)) continue;  // one wave (200 KB blocks in clusters of 4 and 8: 132 and 120 of 148 at once)
-    // fitted to the launches named at the top of the file: start and end, rounds, the exchange in the
-    // cluster, rows of the epilogue, blocks that share L2
-    const double c = 3.4 + 0.23 * per + (s > 1 ? 0.3 + 0.1 * s : 0.) + (d.M < BM ? d.M : BM) / 128. + 0.4 * tiles * s / num_sms;
-    if (!best || c < *t) { best = s; *t = c; }
+    // blocks that run at once (200 KB of shared memory each; in clusters of 4 and 8 they leave SMs of a GPC unused)
+    const int units = s >= 4 ? num_sms * (s == 4 ? 8 : 7) / 9 : num_sms;
+    double mean = 0.;
+    bool fits = false;
+    for (int i = 0; i < fills.n; i++) {
+      const int m = Fills::of(d.M, fills.share[i]);
+      const long long blocks = (long long)((m + BM - 1) / BM) * ((d.N + TS_BN - 1) / TS_BN) * s;
+      const long long waves = (blocks + units - 1) / units;
+      fits |= waves <= 1;
+      // fitted to the launches named at the top of the file: start and end, rounds, the exchange in the
+      // cluster, rows of the epilogue, blocks that share L2
+      const double c = 3.4 + 0.23 * per + (s > 1 ? 0.3 + 0.1 * s : 0.) + (m < BM ? m : BM) / 128. + 0.4 * (waves > 1 ? units : blocks) / num_sms;
+      mean += c * waves / fills.n;
+    }
+    // Made for one wave.  Where the rows are known on the device only, some fill has to give one, and every fill counts with
+    // the waves it takes: evaluation of 8 x 128 tokens by 9 layers, split of k chosen for 0.7 of the rows alone | so, full
+    // 687 | 555 us, 0.7 filled 562 | 531, 0.4 filled 507 | 518.
+    if (!fits) continue;
+    if (!best || mean < *t) { best = s; *t = mean; }
   }
   return best;
 }
