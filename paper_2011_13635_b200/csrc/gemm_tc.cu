@@ -12,10 +12,10 @@
 //              steps; tcgen05.commit hands shared-memory stages back to the producers and
 //              accumulators over to the epilogue.
 //   warps 4-11: epilogue.  Two warps per 32-lane quarter of TMEM read the accumulator with
-//              tcgen05.ld, apply scale, bias, GELU / GELU', residual, and store bf16 or fp32
-//              (plain, or as vector reductions for split-k) through a swizzled staging buffer so
-//              that global stores are whole row segments.  Two accumulators of up to 256 columns
-//              let the epilogue of one tile overlap the main loop of the next.
+//              tcgen05.ld, apply scale, bias, GELU / GELU', residual, and leave bf16 or fp32 (plain,
+//              or added to what is there for split-k) in a swizzled staging tile that the copy engine
+//              stores; where a tile store does not fit, as whole row segments.  Two accumulators of up
+//              to 256 columns let the epilogue of one tile overlap the main loop of the next.
 // Operands may be k-contiguous ("K-major") or row-contiguous ("MN-major"); the second form is
 // what input-gradient and weight-gradient products need, and is fed to the tensor cores through
 // the MN-major shared-memory descriptor, so no transposed copies exist anywhere.
@@ -1007,7 +1007,9 @@ std::mutex g_dev_mu;
 
 // Tile form and k split of one product.  The estimate below (microseconds) was fitted to 1500 timed
 // launches of all forms: every product shape of BERT-Base at 64 to 16384 rows and its weight
-// gradients.  Over those shapes the form it picks is on average 0.7 % slower than the fastest one.
+// gradients.  Over those shapes the form it picked was on average 0.7 % slower than the fastest one.  The kernels under it
+// have changed since (elected threads, early weights, fp32 results as tile stores: 4 to 20 % of single launches) and it
+// has not been fitted again.
 // Against the rule it replaces (256 columns, or 128 where that fills the SMs better, and pairs from
 // 30 GFLOP on): 64 x 768 x 768 10.8 -> 6.1 us, 1024 x 768 x 3072 20.8 -> 14.5, 4096 x 768 x 768
 // 16.4 -> 13.3, 4096 x 768 x 3072 30.1 -> 25.4, 2304 x 768 x 2400 (weight gradient) 16.1 -> 14.6,
